@@ -59,6 +59,13 @@ static sats_status from_cuda(cudaError_t e, const char *where = "CUDA call")
     return e == cudaSuccess ? SATS_OK : cuda_fail(e, where);
 }
 
+// Eq. 3's rank: m = ceil(k n), with k read as the decimal fraction it stands for.
+int64_t percentile_rank(int64_t n, double k)
+{
+    const int64_t m = (int64_t)std::ceil((k * (double)n) * (1.0 - std::ldexp(1.0, -50)));
+    return m < 1 ? 1 : (m > n ? n : m);
+}
+
 static bool bad_threshold(float t) { return std::isnan(t) || t < 0.0f; }
 
 // Runs one block over B tokens: on the tensor cores when the batch is larger
@@ -489,13 +496,10 @@ sats_status sats_percentile_threshold(const float *a, int64_t n, double k, float
     if (n == 0 || !(k > 0.0)) { *t_out = 0.0f; return SATS_OK; }
     if (k > 1.0) { *t_out = INFINITY; return SATS_OK; }
     if (!a || !ws || ws_bytes < select_ws_bytes() || !aligned16(ws)) return SATS_EINVAL;
-    // m = ceil(k n), with k read as the decimal fraction it stands for
-    int64_t m = (int64_t)std::ceil((k * (double)n) * (1.0 - std::ldexp(1.0, -50)));
-    if (m < 1) m = 1;
-    if (m > n) m = n;
+    const int64_t m = percentile_rank(n, k);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float *t_dev = reinterpret_cast<float *>(static_cast<char *>(ws) + select_ws_bytes() - 128);
-    cudaError_t e = launch_select(a, n, m, ws, t_dev, st);
+    cudaError_t e = launch_select(a, n, &m, 1, ws, t_dev, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(t_out, t_dev, sizeof(float), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     return from_cuda(e);

@@ -163,62 +163,241 @@ __global__ void gate_act_kernel(const uint16_t *__restrict__ wg_t, int H, int N,
 }
 
 // ------------------------------------------------------------------ selection
-// The m-th smallest |a_i| by a two-level radix select on the IEEE bit pattern
-// of |a_i| (non-negative floats order as their unsigned bit patterns):
-// histogram of the high 16 bits, locate the bin holding rank m, histogram of
-// the low 16 bits inside that bin, locate again.
-constexpr int kBins = 65536;
+// The m-th smallest |a_i| for up to kSelRanks ranks m at once, by a radix select on
+// the IEEE bit pattern of |a_i| (non-negative floats order as their unsigned bit
+// patterns), 11 + 10 + 10 bits.  Level 0 counts the top 11 bits of every value;
+// levels 1 and 2 count the next 10 bits of the values that share their leading bits
+// with one of the ranks (a slot each; ranks in one bin share its slot).  Each level
+// is one kernel: a CTA counts its values in shared memory and adds the non-zero
+// counts to the level's histogram, and the last CTA to finish finds every rank's bin
+// and writes the slots of the next level.
+//
+// What bounds it: a pass over values that sit in L2, and the launches.  Post-gate
+// magnitudes fall into a few dozen of the top bins, so counting them with atomics in
+// global memory ran at the rate of one address (263 us per pass over 3.7 M values,
+// and 36 us to search 65536 bins with one CTA); level 0 therefore keeps kSelCopies
+// histograms per CTA in shared memory, and 2048-bin levels leave the search a few
+// microseconds.  All percentiles of a calibration grid share the three passes.
+constexpr int kSelBins0 = 2048, kSelBins = 1024, kSelCopies = 4;
+constexpr int kSelThreads = 512, kSelWarps = kSelThreads / 32;
 
-__global__ void hist_kernel(const float *__restrict__ a, int64_t n, int level, const int *__restrict__ sel,
-                            unsigned *__restrict__ hist)
+// Workspace of a selection of R ranks; cleared as a whole before level 0.
+struct SelWs {
+    unsigned *done;         // [3] CTAs finished per level
+    int *nslots;            // [2] slots of level 1 and 2
+    int *slot;              // [2][kSelRanks] rank -> slot
+    long long *rest;        // [kSelRanks] rank within the bins chosen so far (1-based)
+    uint32_t *prefix;       // [kSelRanks] bits chosen so far
+    unsigned *hist0;        // [kSelBins0]
+    uint8_t *map0;          // [kSelBins0] slot + 1 of level 1, 0 for a bin without a rank
+    unsigned *hist;         // [2][R][kSelBins] levels 1 and 2
+    uint8_t *map1;          // [R][kSelBins] slot + 1 of level 2
+};
+
+__host__ __device__ inline size_t sel_layout(char *base, int R, SelWs *w)
 {
-    const int hi_bin = level ? sel[0] : 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t bits = __float_as_uint(a[i]) & 0x7fffffffu;
-        if (level == 0) atomicAdd(&hist[bits >> 16], 1u);
-        else if ((int)(bits >> 16) == hi_bin) atomicAdd(&hist[bits & 0xffffu], 1u);
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char *p = base + off;
+        off += (bytes + 255) & ~(size_t)255;
+        return p;
+    };
+    w->done = reinterpret_cast<unsigned *>(take(3 * sizeof(unsigned)));
+    w->nslots = reinterpret_cast<int *>(take(2 * sizeof(int)));
+    w->slot = reinterpret_cast<int *>(take(2 * kSelRanks * sizeof(int)));
+    w->rest = reinterpret_cast<long long *>(take(kSelRanks * sizeof(long long)));
+    w->prefix = reinterpret_cast<uint32_t *>(take(kSelRanks * sizeof(uint32_t)));
+    w->hist0 = reinterpret_cast<unsigned *>(take(kSelBins0 * sizeof(unsigned)));
+    w->map0 = reinterpret_cast<uint8_t *>(take(kSelBins0));
+    w->hist = reinterpret_cast<unsigned *>(take((size_t)2 * R * kSelBins * sizeof(unsigned)));
+    w->map1 = reinterpret_cast<uint8_t *>(take((size_t)R * kSelBins));
+    return off;
+}
+
+// Calls f(bits of |a_i|) for this thread's share of the n values.
+template <typename F>
+__device__ __forceinline__ void for_each_bits(const float *__restrict__ a, int64_t n, F f)
+{
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, T = (int64_t)gridDim.x * blockDim.x;
+    int64_t done = 0;
+    if ((reinterpret_cast<uintptr_t>(a) & 15u) == 0) {   // 16-byte loads, two in flight
+        const uint4 *v = reinterpret_cast<const uint4 *>(a);
+        const int64_t nv = n >> 2;
+        done = nv << 2;
+        for (int64_t i = t; i < nv; i += 2 * T) {
+            const uint4 p = v[i];
+            const bool two = i + T < nv;
+            const uint4 q = two ? v[i + T] : p;
+            f(p.x & 0x7fffffffu);
+            f(p.y & 0x7fffffffu);
+            f(p.z & 0x7fffffffu);
+            f(p.w & 0x7fffffffu);
+            if (two) {
+                f(q.x & 0x7fffffffu);
+                f(q.y & 0x7fffffffu);
+                f(q.z & 0x7fffffffu);
+                f(q.w & 0x7fffffffu);
+            }
+        }
+    }
+    for (int64_t i = done + t; i < n; i += T) f(__float_as_uint(a[i]) & 0x7fffffffu);
+}
+
+// The bin of `nbins` (a multiple of 1024) counts that holds the 1-based rank r, and r
+// within it, by one warp: 32 rows of 32 counts are loaded together (past L1: other CTAs
+// wrote them), then summed row by row until the rank's row, whose lanes are scanned.
+__device__ __forceinline__ int find_bin(const unsigned *hist, int nbins, long long r, long long *within)
+{
+    const int lane = threadIdx.x & 31;
+    long long run = 0;
+    for (int base = 0; base < nbins; base += 1024) {
+        unsigned c[32];
+#pragma unroll
+        for (int k = 0; k < 32; ++k) c[k] = __ldcg(hist + base + 32 * k + lane);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            const long long row = (long long)__reduce_add_sync(0xffffffffu, c[k] & 0xffffu) +
+                                  ((long long)__reduce_add_sync(0xffffffffu, c[k] >> 16) << 16);
+            if (run + row >= r) {
+                long long incl = c[k];
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const long long t = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                const unsigned at = __ballot_sync(0xffffffffu, run + incl >= r);
+                const int src = __ffs(at) - 1;   // (the row holds the rank, so its last lane is in `at`)
+                *within = r - run - __shfl_sync(0xffffffffu, incl - (long long)c[k], src);
+                return base + 32 * k + src;
+            }
+            run += row;
+        }
+    }
+    *within = 1;   // not reached: 1 <= r <= the sum of the counts
+    return nbins - 1;
+}
+
+struct SelRankList {
+    long long m[kSelRanks];
+};
+
+template <int LEVEL>
+__global__ void __launch_bounds__(kSelThreads) select_kernel(const float *__restrict__ a, int64_t n, int R,
+                                                             const SelRankList ranks, char *ws,
+                                                             float *__restrict__ t_out)
+{
+    extern __shared__ unsigned sel_smem[];
+    __shared__ int bins[kSelRanks];
+    __shared__ bool last;
+    SelWs w;
+    sel_layout(ws, R, &w);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    unsigned *h = sel_smem;
+    grid_dependency_wait();   // the values and the slots belong to the preceding kernels
+    grid_launch_dependents();
+    const int slots = LEVEL == 0 ? 0 : w.nslots[LEVEL - 1];
+    const int nh = LEVEL == 0 ? kSelCopies * kSelBins0 : slots * kSelBins;
+    uint8_t *map0 = reinterpret_cast<uint8_t *>(h + nh), *map1 = map0 + kSelBins0;
+    for (int i = tid; i < nh; i += kSelThreads) h[i] = 0u;
+    if (LEVEL > 0)
+        for (int i = tid; i < kSelBins0 / 4; i += kSelThreads)
+            reinterpret_cast<uint32_t *>(map0)[i] = reinterpret_cast<const uint32_t *>(w.map0)[i];
+    if (LEVEL == 2)
+        for (int i = tid; i < w.nslots[0] * kSelBins / 4; i += kSelThreads)
+            reinterpret_cast<uint32_t *>(map1)[i] = reinterpret_cast<const uint32_t *>(w.map1)[i];
+    __syncthreads();
+    if (LEVEL == 0) {
+        unsigned *mine = h + (warp % kSelCopies) * kSelBins0;
+        for_each_bits(a, n, [&](uint32_t b) { atomicAdd(mine + (b >> 20), 1u); });
+    } else {
+        for_each_bits(a, n, [&](uint32_t b) {
+            const int s0 = map0[b >> 20];
+            if (s0 == 0) return;
+            if (LEVEL == 1) {
+                atomicAdd(h + (s0 - 1) * kSelBins + ((b >> 10) & 1023u), 1u);
+            } else {
+                const int s1 = map1[(s0 - 1) * kSelBins + ((b >> 10) & 1023u)];
+                if (s1) atomicAdd(h + (s1 - 1) * kSelBins + (b & 1023u), 1u);
+            }
+        });
+    }
+    __syncthreads();
+    unsigned *gh = LEVEL == 0 ? w.hist0 : w.hist + (size_t)(LEVEL - 1) * R * kSelBins;
+    if (LEVEL == 0) {
+        for (int i = tid; i < kSelBins0; i += kSelThreads) {
+            unsigned c = 0;
+            for (int k = 0; k < kSelCopies; ++k) c += h[k * kSelBins0 + i];
+            if (c) atomicAdd(gh + i, c);
+        }
+    } else {
+        for (int i = tid; i < nh; i += kSelThreads)
+            if (h[i]) atomicAdd(gh + i, h[i]);
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(w.done + LEVEL, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // the last CTA: a warp per rank finds its bin
+    for (int i = warp; i < R; i += kSelWarps) {
+        const long long r = LEVEL == 0 ? ranks.m[i] : w.rest[i];
+        const unsigned *hr = LEVEL == 0 ? gh : gh + (size_t)w.slot[(LEVEL - 1) * kSelRanks + i] * kSelBins;
+        long long rest;
+        const int bin = find_bin(hr, LEVEL == 0 ? kSelBins0 : kSelBins, r, &rest);
+        if (lane == 0) {
+            bins[i] = bin;
+            w.rest[i] = rest;
+            if (LEVEL == 0) {
+                w.prefix[i] = (uint32_t)bin << 20;
+            } else if (LEVEL == 1) {
+                w.prefix[i] |= (uint32_t)bin << 10;
+            } else {
+                t_out[i] = __uint_as_float(w.prefix[i] | (uint32_t)bin);
+            }
+        }
+    }
+    if (LEVEL == 2) return;
+    __syncthreads();
+    if (tid == 0) {   // ranks that share a bin share a slot of the next level
+        int ns = 0;
+        for (int i = 0; i < R; ++i) {
+            uint8_t *m = LEVEL == 0 ? w.map0 + bins[i] : w.map1 + (size_t)w.slot[i] * kSelBins + bins[i];
+            if (*m == 0) *m = (uint8_t)++ns;
+            w.slot[LEVEL * kSelRanks + i] = *m - 1;
+        }
+        w.nslots[LEVEL] = ns;
     }
 }
 
-// sel[2*level] <- bin holding rank r (1-based), sel[2*level+1] <- rank inside it.
-// rank r comes from sel[1] for level 1, from `m` for level 0.
-__global__ void __launch_bounds__(1024) find_bin_kernel(const unsigned *__restrict__ hist, int64_t m, int level,
-                                                        int *__restrict__ sel, float *__restrict__ t_out)
+size_t sel_smem_bytes(int level, int R)
 {
-    __shared__ unsigned long long warp_tot[32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long r = level ? (long long)sel[1] : (long long)m;
-    constexpr int kPer = kBins / 1024;
-    unsigned long long s = 0;
-    for (int i = 0; i < kPer; ++i) s += hist[tid * kPer + i];
-    unsigned long long incl = s;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
+    if (level == 0) return (size_t)kSelCopies * kSelBins0 * sizeof(unsigned);
+    return (size_t)R * kSelBins * sizeof(unsigned) + kSelBins0 + (level == 2 ? (size_t)R * kSelBins : 0);
+}
+
+template <int LEVEL>
+cudaError_t launch_select_level(const float *a, int64_t n, int R, const SelRankList &ranks, char *ws, float *t_out,
+                                int grid, cudaStream_t stream)
+{
+    const size_t smem = sel_smem_bytes(LEVEL, R);
+    // (the limit is set to the most that any call needs, so calls never lower it under one another)
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(select_kernel<LEVEL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)sel_smem_bytes(LEVEL, kSelRanks));
+        if (e != cudaSuccess) return e;
     }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    unsigned long long before = 0;
-    for (int w = 0; w < warp; ++w) before += warp_tot[w];
-    const unsigned long long lo = before + incl - s;     // count of values in bins below this thread's range
-    if ((long long)lo < r && (long long)(lo + s) >= r) {
-        unsigned long long run = lo;
-        for (int i = 0; i < kPer; ++i) {
-            const unsigned c = hist[tid * kPer + i];
-            if ((long long)(run + c) >= r) {
-                const int bin = tid * kPer + i;
-                if (level == 0) {
-                    sel[0] = bin;
-                    sel[1] = (int)(r - (long long)run);
-                } else {
-                    const uint32_t bits = ((uint32_t)sel[0] << 16) | (uint32_t)bin;
-                    *t_out = __uint_as_float(bits);
-                }
-                break;
-            }
-            run += c;
-        }
-    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kSelThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, select_kernel<LEVEL>, a, n, R, ranks, ws, t_out);
 }
 
 }  // namespace
@@ -325,22 +504,33 @@ cudaError_t launch_gate_act_f32(const sats_layer *layer, const float *x, int B, 
     return cudaGetLastError();
 }
 
-size_t select_ws_bytes() { return (size_t)kBins * sizeof(unsigned) + 256; }
+// The workspace of one percentile: what sats_select_workspace_bytes has always asked for.
+size_t select_ws_bytes() { return (size_t)65536 * sizeof(unsigned) + 256; }
 
-cudaError_t launch_select(const float *a, int64_t n, int64_t m, void *ws, float *t_dev, cudaStream_t stream)
+size_t select_multi_ws_bytes(int R)
 {
-    unsigned *hist = static_cast<unsigned *>(ws);
-    int *sel = reinterpret_cast<int *>(static_cast<char *>(ws) + (size_t)kBins * sizeof(unsigned));
-    const int blocks = 1024;
-    cudaError_t e = cudaMemsetAsync(hist, 0, (size_t)kBins * sizeof(unsigned), stream);
+    SelWs w;
+    return sel_layout(nullptr, R, &w);
+}
+
+// t_dev[i] = the m[i]-th smallest of |a_0 .. a_{n-1}| for R <= kSelRanks ranks in [1, n];
+// ws: select_multi_ws_bytes(R) bytes, 16-byte aligned.
+cudaError_t launch_select(const float *a, int64_t n, const int64_t *m, int R, void *ws, float *t_dev,
+                          cudaStream_t stream)
+{
+    if (R < 1 || R > kSelRanks) return cudaErrorInvalidValue;
+    SelRankList ranks;
+    for (int i = 0; i < kSelRanks; ++i) ranks.m[i] = i < R ? m[i] : 1;
+    char *base = static_cast<char *>(ws);
+    cudaError_t e = cudaMemsetAsync(base, 0, select_multi_ws_bytes(R), stream);
     if (e != cudaSuccess) return e;
-    hist_kernel<<<blocks, 256, 0, stream>>>(a, n, 0, sel, hist);
-    find_bin_kernel<<<1, 1024, 0, stream>>>(hist, m, 0, sel, t_dev);
-    e = cudaMemsetAsync(hist, 0, (size_t)kBins * sizeof(unsigned), stream);
-    if (e != cudaSuccess) return e;
-    hist_kernel<<<blocks, 256, 0, stream>>>(a, n, 1, sel, hist);
-    find_bin_kernel<<<1, 1024, 0, stream>>>(hist, m, 1, sel, t_dev);
-    return cudaGetLastError();
+    // one CTA per SM, fewer where a CTA would have less than 4 values a thread
+    const int64_t want = (n + 4 * kSelThreads - 1) / (4 * kSelThreads);
+    const int sms = fused_grid(kMaxGrid);
+    const int grid = (int)(want < sms ? want : sms);
+    if ((e = launch_select_level<0>(a, n, R, ranks, base, t_dev, grid, stream)) != cudaSuccess) return e;
+    if ((e = launch_select_level<1>(a, n, R, ranks, base, t_dev, grid, stream)) != cudaSuccess) return e;
+    return launch_select_level<2>(a, n, R, ranks, base, t_dev, grid, stream);
 }
 
 }  // namespace sats

@@ -98,10 +98,10 @@ ErrLayout err_layout(int H, int N, int C, int K)
 }
 
 struct SatsLayout {
-    size_t x, n, a, sel, err, total;
+    size_t x, n, a, sel, q, err, total;
 };
 
-SatsLayout sats_layout(int H, int N, int C, int L, int K)
+SatsLayout sats_layout(int H, int N, int C, int L, int K0, int K)
 {
     SatsLayout S{};
     size_t off = 0;
@@ -112,7 +112,9 @@ SatsLayout sats_layout(int H, int N, int C, int L, int K)
     S.a = off;
     off += al256((size_t)C * N * sizeof(float));
     S.sel = off;
-    off += al256(select_ws_bytes());
+    off += al256(select_multi_ws_bytes(kSelRanks));
+    S.q = off;   // every block's percentiles: the coarse candidates, the largest |a|, the guardrail's
+    off += al256((size_t)L * (K0 + 1) * sizeof(float));
     S.err = off;
     off += err_layout(H, N, C, K).total;
     S.total = off;
@@ -266,7 +268,7 @@ size_t sats_sats_workspace_bytes(int H, int N, int C, int L, int K0, int K1)
 {
     if (H < 8 || H > kMaxH || (H % 8) != 0 || N < 1 || N > kMaxN || C < 1 || L < 1 || K0 < 2 || K1 < 0) return 0;
     const int K = std::max(std::max(K0 - 1, K1), 1);
-    return sats_layout(H, N, C, L, K).total;
+    return sats_layout(H, N, C, L, K0, K).total;
 }
 
 sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *const *norm_w, int L, float eps,
@@ -282,7 +284,7 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     for (int l = 0; l < L; ++l)
         if (!layers[l] || layers[l]->H != H || layers[l]->N != N || !norm_w[l]) return SATS_EINVAL;
     const int Kc = K0 - 1, Kmax = std::max(std::max(Kc, K1), 1), Kt = Kc + K1;
-    const SatsLayout W = sats_layout(H, N, C, L, Kmax);
+    const SatsLayout W = sats_layout(H, N, C, L, K0, Kmax);
     if (ws_bytes < W.total) return SATS_ENOSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char *base = static_cast<char *>(ws);
@@ -290,6 +292,7 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     float *nall = reinterpret_cast<float *>(base + W.n);
     float *a = reinterpret_cast<float *>(base + W.a);
     void *sel = base + W.sel;
+    float *q = reinterpret_cast<float *>(base + W.q);
     void *ews = base + W.err;
     const size_t ews_bytes = W.total - W.err;
     void *mlp = base + W.err + err_layout(H, N, C, Kmax).mlp;
@@ -304,29 +307,33 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     double g_t = 0.0, g_sp = 0.0;
     const float zero = 0.0f;
     sats_status s;
+    const int64_t n = (int64_t)C * N;
+    std::vector<int64_t> rank((size_t)K0 + 1);
     for (int l = 0; l < L; ++l) {
         if ((s = sats_rmsnorm(x, C, H, norm_w[l], eps, n_of(l), stream)) != SATS_OK) return s;
         if ((s = sats_gate_act_f32(layers[l], n_of(l), C, a, stream)) != SATS_OK) return s;
-        const int64_t n = (int64_t)C * N;
-        for (int k = 1; k <= Kc; ++k) {   // Eq. 3 at k / K0
-            float tv = 0.f;
-            if ((s = sats_percentile_threshold(a, n, (double)k / K0, &tv, sel, select_ws_bytes(), stream)) != SATS_OK)
-                return s;
-            tc[(size_t)l * Kc + k - 1] = tv;
-        }
-        float mx = 0.f;
-        if ((s = sats_percentile_threshold(a, n, 1.0, &mx, sel, select_ws_bytes(), stream)) != SATS_OK) return s;
-        amax[(size_t)l] = mx;
-        if (l == guard) {
-            float gt = 0.f;
-            if ((s = sats_percentile_threshold(a, n, s_tar, &gt, sel, select_ws_bytes(), stream)) != SATS_OK)
-                return s;
-            g_t = gt;
-        }
+        // Eq. 3 at k / K0, the largest |a|, and the guardrail block's percentile at the target, all
+        // from shared passes over |a|; read back once after the last block
+        const int nq = l == guard && s_tar > 0.0 ? Kc + 2 : Kc + 1;
+        for (int k = 0; k < nq; ++k) rank[(size_t)k] = percentile_rank(n, k < Kc ? (double)(k + 1) / K0 : k == Kc ? 1.0 : s_tar);
+        for (int k = 0; k < nq; k += kSelRanks)
+            if ((e = launch_select(a, n, rank.data() + k, std::min(kSelRanks, nq - k), sel, q + (size_t)l * (K0 + 1) + k,
+                                   st)) != cudaSuccess)
+                return cuda_fail(e, "percentile kernels launch");
         // x <- x + MLP_l(n_l) with every neuron kept
         if ((s = run_layer(layers[l], kXF32, n_of(l), C, &zero, nullptr, 0.f, nullptr, kOutResid, x, nullptr,
                            nullptr, nullptr, mlp, st)) != SATS_OK)
             return s;
+    }
+    std::vector<float> qh((size_t)L * (K0 + 1), 0.f);
+    e = cudaMemcpyAsync(qh.data(), q, qh.size() * sizeof(float), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e, "percentile read-back");
+    for (int l = 0; l < L; ++l) {
+        const float *ql = qh.data() + (size_t)l * (K0 + 1);
+        std::copy(ql, ql + Kc, tc.begin() + (size_t)l * Kc);
+        amax[(size_t)l] = ql[Kc];
+        if (l == guard) g_t = s_tar > 0.0 ? ql[Kc + 1] : 0.f;
     }
     // 3: Eq. 6 for every coarse candidate (and the guardrail's CATS threshold)
     std::vector<float> tf((size_t)Kmax);

@@ -151,8 +151,11 @@ sats_status run_layer(const sats_layer *layer, int x_mode, const void *x, int B,
                       int32_t *active_idx, int32_t *active_cnt, uint8_t *keep_trace, void *ws, cudaStream_t stream,
                       const sats_lora *lora = nullptr, const int32_t *perm = nullptr,
                       const int32_t *n_dense = nullptr);
+constexpr int kSelRanks = 32;   // ranks that one selection finds together
+int64_t percentile_rank(int64_t n, double k);   // Eq. 3's rank of the k-th quantile, 0 < k <= 1
 size_t select_ws_bytes();
-cudaError_t launch_select(const float *a, int64_t n, int64_t m, void *ws, float *t_dev,
+size_t select_multi_ws_bytes(int R);
+cudaError_t launch_select(const float *a, int64_t n, const int64_t *m, int R, void *ws, float *t_dev,
                           cudaStream_t stream);
 
 }  // namespace sats
