@@ -18,6 +18,11 @@
 namespace sats {
 namespace {
 
+constexpr int kErrGroup = 32;     // candidate thresholds per group of Eq. 6
+// Rows of h per group (candidates x inputs): enough to fill the GPU for several waves, and at most
+// about 470 MB of rows at the largest layers' 14336 neurons
+constexpr int kErrRows = 8192;
+
 size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // out[b] = x[b] / sqrt(mean_i x[b][i]^2 + eps) * w  (one CTA per row).
@@ -73,28 +78,215 @@ __global__ void __launch_bounds__(256) err_accum_kernel(const float *__restrict_
     }
 }
 
-struct ErrLayout {
-    size_t mlp, yd, yk, idx, cnt, acc, total;
+// Candidates of one group: the threshold of each, or NaN for the dense output (every neuron).
+struct Candidates {
+    float t[kErrGroup];
 };
+
+// Row (k, c) of the dropped neurons' h, in bf16 parts: h where |a| < t_k, 0 elsewhere, for the K
+// candidates of a group; counts[k] += the neurons dropped.  h (hi, lo) and a are [C][ld], the rows
+// [K][C][ld]; ld is a multiple of 8, and columns N .. ld - 1 are never read as neurons.  Grid: (C,
+// column blocks of 8 x 256).  Bound by its writes (4 K C N bytes, mostly into L2).
+__global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict__ a, const uint16_t *__restrict__ hhi,
+                                                        const uint16_t *__restrict__ hlo, int C, int N, int ld,
+                                                        const Candidates cand, int K, uint16_t *__restrict__ rhi,
+                                                        uint16_t *__restrict__ rlo, unsigned long long *counts)
+{
+    __shared__ unsigned dropped[kErrGroup];
+    if (threadIdx.x < kErrGroup) dropped[threadIdx.x] = 0u;
+    grid_dependency_wait();   // h and a are the gate/up kernel's
+    grid_launch_dependents();
+    __syncthreads();
+    const int c = blockIdx.x, n0 = (blockIdx.y * 256 + threadIdx.x) * 8;
+    const bool in = n0 < N;
+    float av[8];
+    uint4 hh = make_uint4(0u, 0u, 0u, 0u), hl = hh;
+    if (in) {
+        const size_t at = (size_t)c * ld + n0;
+        const float4 p = *reinterpret_cast<const float4 *>(a + at), q = *reinterpret_cast<const float4 *>(a + at + 4);
+        av[0] = p.x; av[1] = p.y; av[2] = p.z; av[3] = p.w;
+        av[4] = q.x; av[5] = q.y; av[6] = q.z; av[7] = q.w;
+        hh = *reinterpret_cast<const uint4 *>(hhi + at);
+        hl = *reinterpret_cast<const uint4 *>(hlo + at);
+    }
+    for (int k = 0; k < K; ++k) {
+        const float t = cand.t[k];
+        unsigned m[4] = {0u, 0u, 0u, 0u}, cnt = 0u;
+        if (in) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                // not kept (Eqs. 4-5: a neuron is kept if |a| >= t); true for every a when t is NaN
+                const bool drop = n0 + e < N && !(fabsf(av[e]) >= t);
+                cnt += drop ? 1u : 0u;
+                m[e / 2] |= drop ? (e & 1 ? 0xffff0000u : 0xffffu) : 0u;
+            }
+            const size_t at = ((size_t)k * C + c) * ld + n0;
+            *reinterpret_cast<uint4 *>(rhi + at) = make_uint4(hh.x & m[0], hh.y & m[1], hh.z & m[2], hh.w & m[3]);
+            *reinterpret_cast<uint4 *>(rlo + at) = make_uint4(hl.x & m[0], hl.y & m[1], hl.z & m[2], hl.w & m[3]);
+        }
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(dropped + k, cnt);
+    }
+    __syncthreads();
+    if (threadIdx.x < K && dropped[threadIdx.x]) atomicAdd(counts + threadIdx.x, (unsigned long long)dropped[threadIdx.x]);
+}
+
+// A sum of squares carried as an unevaluated pair of floats (error-free product and sum), about
+// 48 bits: this GPU's 64-bit rate is 1/64 of its 32-bit one.
+struct SquareSum {
+    float hi = 0.f, lo = 0.f;
+    __device__ void add(float v)
+    {
+        const float p = __fmul_rn(v, v), pe = __fmaf_rn(v, v, -p);
+        const float s = __fadd_rn(hi, p), b = __fadd_rn(s, -hi);
+        lo += (__fadd_rn(hi, -__fadd_rn(s, -b)) + __fadd_rn(p, -b)) + pe;
+        hi = s;
+    }
+    __device__ double value() const { return (double)hi + (double)lo; }
+};
+
+// Token c, candidate k: acc[k] += ||d_kc|| / (||y_c|| + eps), with d = y - y~_t (the dropped
+// neurons' output, rows [K][C][H]) and y the dense output [C][H].  Grid: (C, K).
+__global__ void __launch_bounds__(256) drop_err_kernel(const float *__restrict__ y, const float *__restrict__ d, int C,
+                                                       int H, float eps, double *__restrict__ acc)
+{
+    const int c = blockIdx.x, k = blockIdx.y;
+    const float4 *yr = reinterpret_cast<const float4 *>(y + (size_t)c * H);
+    const float4 *dr = reinterpret_cast<const float4 *>(d + ((size_t)k * C + c) * H);
+    SquareSum sd, sy;
+    for (int i = threadIdx.x; i < (H >> 2); i += 256) {   // H is a multiple of 8
+        const float4 p = dr[i], q = yr[i];
+        sd.add(p.x); sd.add(p.y); sd.add(p.z); sd.add(p.w);
+        sy.add(q.x); sy.add(q.y); sy.add(q.z); sy.add(q.w);
+    }
+    __shared__ double r0[8], r1[8];
+    double ds, ys;
+    auto reduce = [&](double dd, double yy) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            dd += __shfl_xor_sync(0xffffffffu, dd, o);
+            yy += __shfl_xor_sync(0xffffffffu, yy, o);
+        }
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) {
+            r0[threadIdx.x >> 5] = dd;
+            r1[threadIdx.x >> 5] = yy;
+        }
+        __syncthreads();
+        ds = ys = 0.0;
+        for (int i = 0; i < 8; ++i) {
+            ds += r0[i];
+            ys += r1[i];
+        }
+    };
+    reduce(sd.value(), sy.value());
+    auto in_range = [](double v) { return v > 1e-24 && v < 1e36; };
+    if (!in_range(ds) || !in_range(ys)) {   // 32-bit squares may have over- or underflown
+        double dd = 0.0, yy = 0.0;
+        for (int i = threadIdx.x; i < H; i += 256) {
+            const double p = d[((size_t)k * C + c) * H + i], q = y[(size_t)c * H + i];
+            dd += p * p;
+            yy += q * q;
+        }
+        reduce(dd, yy);
+    }
+    if (threadIdx.x == 0) atomicAdd(acc + k, sqrt(ds) / (sqrt(ys) + (double)eps));
+}
+
+// Workspace of Eq. 6.  Batches on the fused kernel (at most two tokens) compare whole outputs
+// (yd, yk, idx, cnt); batches on the tensor cores project the dropped neurons of a group of
+// candidates (a, rows, y: the dense output, then the group's).
+struct ErrLayout {
+    size_t mlp, yd, yk, idx, cnt, a, rhi, rlo, y, acc, total;
+};
+
+// Candidates per group: at most kErrGroup, and about kErrRows rows of h at most (but one candidate's).
+int err_group(int C, int K)
+{
+    const int fit = kErrRows / C;
+    return std::max(1, std::min(std::min(fit, kErrGroup), K + 1));
+}
 
 ErrLayout err_layout(int H, int N, int C, int K)
 {
     ErrLayout L{};
     size_t off = 0;
-    L.mlp = off;
-    off += al256(ws_layout(H, N, C).total);
-    L.yd = off;
-    off += al256((size_t)C * H * sizeof(float));
-    L.yk = off;
-    off += al256((size_t)C * H * sizeof(float));
-    L.idx = off;
-    off += al256((size_t)C * N * sizeof(int32_t));
-    L.cnt = off;
-    off += al256((size_t)C * sizeof(int32_t));
-    L.acc = off;
-    off += al256((size_t)2 * (K > 0 ? K : 1) * sizeof(double));
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off += al256(bytes);
+        return at;
+    };
+    L.mlp = take(ws_layout(H, N, C).total);
+    if (use_tc_path(H, C)) {
+        const size_t ldn = ((size_t)N + 7) & ~(size_t)7, rows = (size_t)err_group(C, K) * C;
+        L.a = take((size_t)C * ldn * sizeof(float));
+        L.rhi = take(rows * ldn * 2);
+        L.rlo = take(rows * ldn * 2);
+        L.y = take((rows + C) * H * sizeof(float));
+        L.acc = take((size_t)(K + 1) * (sizeof(double) + sizeof(unsigned long long)));
+    } else {
+        L.yd = take((size_t)C * H * sizeof(float));
+        L.yk = take((size_t)C * H * sizeof(float));
+        L.idx = take((size_t)C * N * sizeof(int32_t));
+        L.cnt = take((size_t)C * sizeof(int32_t));
+        L.acc = take((size_t)2 * (K > 0 ? K : 1) * sizeof(double));
+    }
     L.total = off;
     return L;
+}
+
+// Eq. 6 on the tensor cores: h = a u of every neuron once, then y - y~_t = (h where |a| < t)
+// W_down directly, for all candidates of a group as the rows of one GEMM.  That is one pass over
+// W_gate and W_up and one over W_down per group instead of both per candidate (20 passes of 72 us
+// for 19 candidates of 64 inputs on the Llama-shaped layer), and the small difference is formed
+// without cancellation.  What bounds it: the down projection's MMAs (two per product: h's high and
+// low parts).
+sats_status layer_err_tc(const sats_layer *layer, const float *x, int C, const float *t, int K, float eps, double *err,
+                         double *sp, char *base, const ErrLayout &W, cudaStream_t st)
+{
+    const int H = layer->H, N = layer->N, ld = layer->ldn;
+    const WsLayout M = ws_layout(H, N, C);
+    char *mlp = base + W.mlp;
+    int *ctl = reinterpret_cast<int *>(mlp + M.ctl);
+    float *a = reinterpret_cast<float *>(base + W.a), *y = reinterpret_cast<float *>(base + W.y);
+    uint16_t *rhi = reinterpret_cast<uint16_t *>(base + W.rhi), *rlo = reinterpret_cast<uint16_t *>(base + W.rlo);
+    double *acc = reinterpret_cast<double *>(base + W.acc);
+    unsigned long long *counts = reinterpret_cast<unsigned long long *>(acc + K + 1);
+    cudaError_t e = clear_fused_state(mlp, H, N, C, st);
+    const size_t acc_bytes = (size_t)(K + 1) * (sizeof(double) + sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, acc_bytes, st);
+    if (e != cudaSuccess) return cuda_fail(e, "layer error workspace clear");
+    const uint16_t *hhi = nullptr, *hlo = nullptr;
+    if (run_tc_gate_up(layer, x, C, mlp + M.tc, &hhi, &hlo, a, ctl, st) != cudaSuccess) return SATS_ECUDA;
+    const int group = err_group(C, K);
+    // candidate 0 is the dense output; its rows stay at the front of y for every group
+    for (int k0 = 0; k0 <= K; k0 += group) {
+        const int kg = std::min(group, K + 1 - k0);
+        Candidates cand;
+        for (int k = 0; k < kg; ++k) cand.t[k] = k0 + k == 0 ? NAN : t[k0 + k - 1];
+        float *out = k0 == 0 ? y : y + (size_t)C * H;
+        if ((e = cudaMemsetAsync(out, 0, (size_t)kg * C * H * sizeof(float), st)) != cudaSuccess)
+            return cuda_fail(e, "layer error output clear");
+        drop_rows_kernel<<<dim3(C, (ld / 8 + 255) / 256), 256, 0, st>>>(a, hhi, hlo, C, N, ld, cand, kg, rhi, rlo,
+                                                                       counts + k0);
+        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "dropped rows kernel launch");
+        if (run_tc_down(layer, rhi, rlo, kg * C, out, ctl, st) != cudaSuccess) return SATS_ECUDA;
+        drop_err_kernel<<<dim3(C, kg), 256, 0, st>>>(y, out, C, H, eps, acc + k0);
+        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "error reduction kernel launch");
+    }
+    std::vector<char> h(acc_bytes);
+    e = cudaMemcpyAsync(h.data(), acc, acc_bytes, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e, "layer error read-back");
+    const sats_status s = sats_get_error(mlp, M.total, st);
+    if (s != SATS_OK) return s;
+    const double *ha = reinterpret_cast<const double *>(h.data());
+    const unsigned long long *hc = reinterpret_cast<const unsigned long long *>(h.data() + (size_t)(K + 1) * sizeof(double));
+    for (int k = 0; k < K; ++k) {
+        err[k] = ha[k + 1] / C;
+        sp[k] = (double)hc[k + 1] / ((double)C * N);
+    }
+    return SATS_OK;
 }
 
 struct SatsLayout {
@@ -171,6 +363,7 @@ sats_status sats_layer_err(const sats_layer *layer, const float *x, int C, const
     if (K == 0) return SATS_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char *base = static_cast<char *>(ws);
+    if (use_tc_path(H, C)) return layer_err_tc(layer, x, C, t, K, eps, err, sp, base, W, st);
     void *mlp = base + W.mlp;
     float *yd = reinterpret_cast<float *>(base + W.yd), *yk = reinterpret_cast<float *>(base + W.yk);
     int32_t *idx = reinterpret_cast<int32_t *>(base + W.idx), *cnt = reinterpret_cast<int32_t *>(base + W.cnt);

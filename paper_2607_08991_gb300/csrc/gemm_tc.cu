@@ -179,6 +179,7 @@ struct SkinnyGuParams {
     uint8_t *keep;                // [M][keep_stride] or nullptr
     int keep_stride;
     uint8_t *keep_trace;          // [M][N] or nullptr
+    float *a_out;                 // [M][ldh] fp32: SiLU(g) of every neuron (the calibration's masks), or nullptr
     int *ctl;
     float *zero;                  // y [M][H] to clear for the down projection's additions, or nullptr
     int zero_count;               // M H (a multiple of 8)
@@ -353,6 +354,7 @@ __global__ void __launch_bounds__(kSkinnyMaxThreads, 1)
                     p.hact_lo[(size_t)j * p.ldh + n] = bf16_bits(h - __uint_as_float((uint32_t)hb << 16));
                     if (p.keep) p.keep[(size_t)j * p.keep_stride + n] = keep ? 1 : 0;
                     if (p.keep_trace) p.keep_trace[(size_t)(p.perm ? p.perm[j] : j) * p.N + n] = keep ? 1 : 0;
+                    if (p.a_out) p.a_out[(size_t)j * p.ldh + n] = a;
                 }
             }
         }
@@ -1177,6 +1179,248 @@ bool use_tc_path(int H, int B) { return B > fused_tokens_per_pass(H); }
 
 size_t tc_workspace_bytes(int H, int N, int B) { return tc_layout(H, N, B).total; }
 
+namespace {
+using namespace tc;
+
+// What the gate/up kernels of one batch are given besides the layer.
+struct GateUpArgs {
+    const uint16_t *xhi, *xlo;   // bf16 activations [B][H]; xlo: their low parts, or nullptr (bf16 activations)
+    int B;
+    float t_l;
+    const uint8_t *dense_flags;
+    const int32_t *perm, *n_dense;
+    uint16_t *hact, *hact_lo;
+    uint8_t *keep;               // [B][keep_stride] or nullptr
+    uint8_t *keep_trace;
+    float *a_out;                // [B][ldn] (skinny kernel only) or nullptr
+    float *zero;                 // y [B][H] to clear, or nullptr
+    int *ctl;
+};
+
+cudaError_t fail(cudaError_t err, const char *where)
+{
+    cuda_fail(err, where);
+    return err;
+}
+
+int keep_stride_of(int N) { return (N + 15) & ~15; }
+
+cudaError_t launch_gate_up_skinny(const sats_layer *layer, const GateUpArgs &a, cudaStream_t stream)
+{
+    const int H = layer->H, N = layer->N, R = layer->tc_R, B = a.B;
+    const bool split = a.xlo != nullptr;
+    const int NT = (B + 15) & ~15;
+    CUtensorMap mX, mX2;
+    if (!make_map(&mX, a.xhi, B, H, (uint64_t)H * 2, NT) ||
+        !make_map(&mX2, split ? a.xlo : a.xhi, B, H, (uint64_t)H * 2, NT))
+        return fail(cudaErrorInvalidValue, "tensor map encoding");
+    SkinnyGuParams gp{};
+    gp.w = layer->gu_blk;
+    gp.M = B;
+    gp.N = N;
+    gp.R = R;
+    gp.KBh = layer->tc_kbh;
+    gp.NT = NT;
+    gp.split = split ? 1 : 0;
+    gp.t_l = a.t_l;
+    gp.dense_flags = a.dense_flags;
+    gp.perm = a.perm;
+    gp.n_dense = a.n_dense;
+    gp.hact = a.hact;
+    gp.hact_lo = a.hact_lo;
+    gp.ldh = layer->ldn;
+    gp.keep = a.keep;
+    gp.keep_stride = keep_stride_of(N);
+    gp.keep_trace = a.keep_trace;
+    gp.a_out = a.a_out;
+    gp.ctl = a.ctl;
+    gp.zero = a.zero;
+    gp.zero_count = B * H;
+    // stage: gate + up rows, then the token tile(s).  The up tile's MMA reads 128 rows from
+    // row R; past 2R they are other data of the ring (rows R..127 of D are not used), and the
+    // ring ends with enough room for the last stage's read.
+    gp.a_bytes = 2 * R * kTileBytes;
+    gp.x_bytes = NT * kTileBytes;
+    gp.stage_bytes = gp.a_bytes + gp.x_bytes * (split ? 2 : 1);
+    const int over = (R + BM) * kTileBytes - gp.stage_bytes;
+    const int slack = over > 0 ? ((over + 1023) & ~1023) : 0;
+    gp.stages = stages_for(gp.stage_bytes, kSmemBudget - slack);
+    gp.ring_bytes = gp.stages * gp.stage_bytes + slack;
+    gp.merge = split && NT <= 128 ? 1 : 0;
+    gp.tmem_cols = tmem_cols_for((gp.merge ? 4 : 2) * NT);
+    cudaError_t e = set_smem(gu_skinny_kernel, smem_for(1, gp.ring_bytes), cfg_gu_skinny);
+    if (e != cudaSuccess) return fail(e, "shared-memory attribute");
+    // epilogue groups: one per 16-token column block, at most kSkinnyMaxGroups (the epilogue
+    // runs after the last MMA, so its time adds to the call's)
+    const int groups = NT / 16 < kSkinnyMaxGroups ? NT / 16 : kSkinnyMaxGroups;
+    e = launch_pdl_cfg(gu_skinny_kernel, dim3(layer->tc_T), 64 + 128 * groups, smem_for(1, gp.ring_bytes), stream, mX,
+                       mX2, gp);
+    return e == cudaSuccess ? e : fail(e, "gate/up kernel launch");
+}
+
+cudaError_t launch_gate_up_wide(const sats_layer *layer, const GateUpArgs &a, cudaStream_t stream)
+{
+    const int H = layer->H, N = layer->N, R = layer->tc_R, B = a.B, sms = sm_count();
+    const bool split = a.xlo != nullptr;
+    CUtensorMap mX, mX2;
+    if (!make_map(&mX, a.xhi, B, H, (uint64_t)H * 2, BM) ||
+        !make_map(&mX2, split ? a.xlo : a.xhi, B, H, (uint64_t)H * 2, BM))
+        return fail(cudaErrorInvalidValue, "tensor map encoding");
+    const int mtiles = (B + BM - 1) / BM;
+    WideGuParams gp{};
+    gp.w = layer->gu_blk;
+    gp.M = B;
+    gp.N = N;
+    gp.R = R;
+    gp.KBh = layer->tc_kbh;
+    gp.T = layer->tc_T;
+    gp.Rw = wide_rows(N, R, mtiles, sms, split);
+    gp.mtiles = mtiles;
+    gp.tiles = mtiles * ((N + gp.Rw - 1) / gp.Rw);
+    gp.tmem_cols = tmem_cols_for(4 * gp.Rw);
+    gp.split = split ? 1 : 0;
+    gp.t_l = a.t_l;
+    gp.dense_flags = a.dense_flags;
+    gp.perm = a.perm;
+    gp.n_dense = a.n_dense;
+    gp.hact = a.hact;
+    gp.hact_lo = a.hact_lo;
+    gp.ldh = layer->ldn;
+    gp.keep = a.keep;
+    gp.keep_stride = keep_stride_of(N);
+    gp.keep_trace = a.keep_trace;
+    gp.ctl = a.ctl;
+    gp.zero = a.zero;
+    gp.zero_count = (long long)B * H;
+    gp.stage_bytes = BM * kTileBytes * (split ? 2 : 1) + 2 * gp.Rw * kTileBytes;
+    gp.stages = stages_for(gp.stage_bytes, wide_budget());
+    // epilogue groups: the tile's 16-neuron column blocks split evenly over at most kWideGuGroups
+    const int blocks16 = gp.Rw / 16, per_group = (blocks16 + kWideGuGroups - 1) / kWideGuGroups;
+    const int gu_groups = (blocks16 + per_group - 1) / per_group;
+    static std::atomic<int> cfg_gu[64];
+    cudaError_t e = set_smem(gu_wide_kernel, smem_for(gp.stages, gp.stage_bytes), cfg_gu);
+    if (e != cudaSuccess) return fail(e, "shared-memory attribute");
+    gu_wide_kernel<<<dim3(gp.tiles < sms ? gp.tiles : sms), 64 + 128 * gu_groups, smem_for(gp.stages, gp.stage_bytes),
+                     stream>>>(mX, mX2, gp);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? e : fail(e, "gate/up kernel launch");
+}
+
+// out[row perm[m] or m] += (hact + hact_lo)[m] W_down for M rows of h (row stride layer->ldn).
+cudaError_t launch_down_skinny(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
+                               const int32_t *perm, int *ctl, cudaStream_t stream)
+{
+    const int N = layer->N, ldn = layer->ldn, sms = sm_count();
+    const int NT = (M + 15) & ~15;
+    CUtensorMap mH, mH2;
+    if (!make_map(&mH, hact, M, N, (uint64_t)ldn * 2, NT) || !make_map(&mH2, hact_lo, M, N, (uint64_t)ldn * 2, NT))
+        return fail(cudaErrorInvalidValue, "tensor map encoding");
+    SkinnyDownParams dp{};
+    dp.w = layer->wd_blk;
+    dp.M = M;
+    dp.H = layer->H;
+    dp.NT = NT;
+    dp.KBn = layer->tc_kbn;
+    dp.units = layer->tc_dt * layer->tc_kbn;
+    dp.out = out;
+    dp.perm = perm;
+    dp.ctl = ctl;
+    dp.a_bytes = BM * kTileBytes;
+    dp.stage_bytes = dp.a_bytes + 2 * NT * kTileBytes;
+    dp.stages = stages_for(dp.stage_bytes);
+    dp.merge = NT <= 128 ? 1 : 0;
+    dp.tmem_cols = tmem_cols_for((dp.merge ? 4 : 2) * NT);
+    static std::atomic<int> cfg_dn[64];
+    cudaError_t e = set_smem(down_skinny_kernel, smem_for(dp.stages, dp.stage_bytes), cfg_dn);
+    if (e != cudaSuccess) return fail(e, "shared-memory attribute");
+    e = launch_pdl(down_skinny_kernel, dim3(dp.units < sms ? dp.units : sms), smem_for(dp.stages, dp.stage_bytes),
+                   stream, mH, mH2, dp);
+    return e == cudaSuccess ? e : fail(e, "down kernel launch");
+}
+
+// As launch_down_skinny, in the prefill orientation: 256 output columns per unit when the hidden
+// tiles pair up; the neuron range split so that the persistent CTAs' units come out even; every
+// unit adds into the output.
+cudaError_t launch_down_wide(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
+                             const int32_t *perm, int *ctl, cudaStream_t stream)
+{
+    const int N = layer->N, ldn = layer->ldn, sms = sm_count();
+    CUtensorMap mH, mH2;
+    if (!make_map(&mH, hact, M, N, (uint64_t)ldn * 2, BM) || !make_map(&mH2, hact_lo, M, N, (uint64_t)ldn * 2, BM))
+        return fail(cudaErrorInvalidValue, "tensor map encoding");
+    WideDownParams dp{};
+    dp.w = layer->wd_blk;
+    dp.M = M;
+    dp.H = layer->H;
+    dp.KBn = layer->tc_kbn;
+    dp.dtiles = (layer->tc_dt % 2 == 0) ? 2 : 1;
+    dp.mtiles = (M + BM - 1) / BM;
+    dp.dcols = layer->tc_dt / dp.dtiles;
+    const int splits = wide_down_splits(dp.mtiles * dp.dcols, dp.KBn, sms);
+    dp.kb_per_split = (dp.KBn + splits - 1) / splits;
+    dp.units = dp.mtiles * dp.dcols * splits;
+    dp.out = out;
+    dp.perm = perm;
+    dp.ctl = ctl;
+    dp.stage_bytes = BM * kTileBytes * (2 + dp.dtiles);
+    dp.stages = stages_for(dp.stage_bytes, wide_budget());
+    dp.tmem_cols = tmem_cols_for(2 * BM * dp.dtiles);
+    static std::atomic<int> cfg_dn[64];
+    cudaError_t e = set_smem(down_wide_kernel, smem_for(dp.stages, dp.stage_bytes), cfg_dn);
+    if (e != cudaSuccess) return fail(e, "shared-memory attribute");
+    down_wide_kernel<<<dim3(dp.units < sms ? dp.units : sms), 64 + 128 * kWideDownGroups,
+                       smem_for(dp.stages, dp.stage_bytes), stream>>>(mH, mH2, dp);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? e : fail(e, "down kernel launch");
+}
+
+// Which orientation a batch's gate/up takes.
+bool skinny_batch(int B, bool split) { return B <= (split ? kMaxSkinnySplit : kMaxSkinny); }
+}  // namespace
+
+// Gate and up projections of B fp32 inputs with every neuron kept: h in bf16 parts and a =
+// SiLU(x W_gate) (row stride layer->ldn), for the calibration's masks.  tc_ws: the tensor-core
+// region of a workspace for B tokens; a_out [B][ldn].  In passes of up to kGateUpTokens tokens
+// of the skinny kernel, whose epilogue has a thread per neuron and writes a in whole lines.
+constexpr int kGateUpTokens = 128;
+
+cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void *tc_ws, const uint16_t **hact,
+                           const uint16_t **hact_lo, float *a_out, int *ctl, cudaStream_t stream)
+{
+    const int H = layer->H;
+    const size_t ldn = layer->ldn;
+    const TcLayout W = tc_layout(H, layer->N, B);
+    uint8_t *base = static_cast<uint8_t *>(tc_ws);
+    uint16_t *xhi = reinterpret_cast<uint16_t *>(base + W.xhi), *xlo = reinterpret_cast<uint16_t *>(base + W.xlo);
+    uint16_t *hhi = reinterpret_cast<uint16_t *>(base + W.hact), *hlo = reinterpret_cast<uint16_t *>(base + W.hact_lo);
+    *hact = hhi;
+    *hact_lo = hlo;
+    cudaError_t e = launch_pdl_threads(split_kernel, dim3(B), 256, stream, x, H, static_cast<const float *>(nullptr), 0.f,
+                                       xhi, xlo, static_cast<const int32_t *>(nullptr));
+    if (e != cudaSuccess) return fail(e, "split kernel launch");
+    const int passes = (B + kGateUpTokens - 1) / kGateUpTokens, per = (B + passes - 1) / passes;
+    for (int m0 = 0; m0 < B; m0 += per) {
+        GateUpArgs a{};
+        a.xhi = xhi + (size_t)m0 * H;
+        a.xlo = xlo + (size_t)m0 * H;
+        a.B = B - m0 < per ? B - m0 : per;
+        a.hact = hhi + m0 * ldn;
+        a.hact_lo = hlo + m0 * ldn;
+        a.a_out = a_out + m0 * ldn;
+        a.ctl = ctl;
+        if ((e = launch_gate_up_skinny(layer, a, stream)) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// out[m] += (hact + hact_lo)[m] W_down for M rows of h (row stride layer->ldn).
+cudaError_t run_tc_down(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
+                        int *ctl, cudaStream_t stream)
+{
+    return M <= kMaxSkinny ? launch_down_skinny(layer, hact, hact_lo, M, out, nullptr, ctl, stream)
+                           : launch_down_wide(layer, hact, hact_lo, M, out, nullptr, ctl, stream);
+}
+
 // The thresholded MLP for a batch of B tokens on the tensor cores.
 //   x: bf16 [B][H] (x_mode kXBf16) or fp32 [B][H] (kXF32 / kXResidNorm, then
 //   split into bf16 hi + lo, after RMSNorm with norm_w for kXResidNorm).
@@ -1190,10 +1434,6 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
                          void *tc_ws, int *ctl, cudaStream_t stream, bool union_path)
 {
     using namespace tc;
-    auto fail = [](cudaError_t err, const char *where) {
-        cuda_fail(err, where);
-        return err;
-    };
     const int H = layer->H, N = layer->N, ldn = layer->ldn, R = layer->tc_R;
     const TcLayout W = tc_layout(H, N, B);
     uint8_t *base = static_cast<uint8_t *>(tc_ws);
@@ -1202,8 +1442,7 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
     uint16_t *hact = reinterpret_cast<uint16_t *>(base + W.hact);
     uint16_t *hact_lo = reinterpret_cast<uint16_t *>(base + W.hact_lo);
     uint8_t *keep = base + W.keep;
-    const int kstride = (N + 15) & ~15;
-    const int sms = sm_count();
+    const int kstride = keep_stride_of(N);
     const bool split = x_mode != kXBf16;
     if (perm && (!split || !n_dense || union_path)) return fail(cudaErrorInvalidValue, "routed batch arguments");
     const uint16_t *xa = split ? xhi : static_cast<const uint16_t *>(x);
@@ -1264,146 +1503,29 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
         e = launch_union_tail(layer, B, xa, split ? xlo : nullptr, uflag, ulist, ucount, a_keep, ldn, u, ldn, out, ctl,
                               stream);
         if (e != cudaSuccess) return fail(e, "union kernels launch");
-    } else if (B <= (split ? kMaxSkinnySplit : kMaxSkinny)) {
-        const int NT = (B + 15) & ~15;
-        CUtensorMap mX, mX2, mH, mH2;
-        if (!make_map(&mX, xa, B, H, (uint64_t)H * 2, NT) || !make_map(&mX2, split ? xlo : xa, B, H, (uint64_t)H * 2, NT) ||
-            !make_map(&mH, hact, B, N, (uint64_t)ldn * 2, NT) || !make_map(&mH2, hact_lo, B, N, (uint64_t)ldn * 2, NT))
-            return fail(cudaErrorInvalidValue, "tensor map encoding");
-        SkinnyGuParams gp{};
-        gp.w = layer->gu_blk;
-        gp.M = B;
-        gp.N = N;
-        gp.R = R;
-        gp.KBh = layer->tc_kbh;
-        gp.NT = NT;
-        gp.split = split ? 1 : 0;
-        gp.t_l = t_l;
-        gp.dense_flags = dense_flags;
-        gp.perm = perm;
-        gp.n_dense = n_dense;
-        gp.hact = hact;
-        gp.hact_lo = hact_lo;
-        gp.ldh = ldn;
-        gp.keep = active_idx ? keep : nullptr;
-        gp.keep_stride = kstride;
-        gp.keep_trace = keep_trace;
-        gp.ctl = ctl;
-        gp.zero = out_mode == kOutY ? out : nullptr;   // the down projection adds into y
-        gp.zero_count = B * H;
-        // stage: gate + up rows, then the token tile(s).  The up tile's MMA reads 128 rows from
-        // row R; past 2R they are other data of the ring (rows R..127 of D are not used), and the
-        // ring ends with enough room for the last stage's read.
-        gp.a_bytes = 2 * R * kTileBytes;
-        gp.x_bytes = NT * kTileBytes;
-        gp.stage_bytes = gp.a_bytes + gp.x_bytes * (split ? 2 : 1);
-        const int over = (R + BM) * kTileBytes - gp.stage_bytes;
-        const int slack = over > 0 ? ((over + 1023) & ~1023) : 0;
-        gp.stages = stages_for(gp.stage_bytes, kSmemBudget - slack);
-        gp.ring_bytes = gp.stages * gp.stage_bytes + slack;
-        gp.merge = split && NT <= 128 ? 1 : 0;
-        gp.tmem_cols = tmem_cols_for((gp.merge ? 4 : 2) * NT);
-        if ((e = set_smem(gu_skinny_kernel, smem_for(1, gp.ring_bytes), cfg_gu_skinny)) != cudaSuccess)
-            return fail(e, "shared-memory attribute");
-        // epilogue groups: one per 16-token column block, at most kSkinnyMaxGroups (the epilogue
-        // runs after the last MMA, so its time adds to the call's)
-        const int groups = NT / 16 < kSkinnyMaxGroups ? NT / 16 : kSkinnyMaxGroups;
-        e = launch_pdl_cfg(gu_skinny_kernel, dim3(layer->tc_T), 64 + 128 * groups, smem_for(1, gp.ring_bytes), stream,
-                           mX, mX2, gp);
-        if (e != cudaSuccess) return fail(e, "gate/up kernel launch");
-
-        SkinnyDownParams dp{};
-        dp.w = layer->wd_blk;
-        dp.M = B;
-        dp.H = H;
-        dp.NT = NT;
-        dp.KBn = layer->tc_kbn;
-        dp.units = layer->tc_dt * layer->tc_kbn;
-        dp.out = out;
-        dp.perm = perm;
-        dp.ctl = ctl;
-        dp.a_bytes = BM * kTileBytes;
-        dp.stage_bytes = dp.a_bytes + 2 * NT * kTileBytes;
-        dp.stages = stages_for(dp.stage_bytes);
-        dp.merge = NT <= 128 ? 1 : 0;
-        dp.tmem_cols = tmem_cols_for((dp.merge ? 4 : 2) * NT);
-        static std::atomic<int> cfg_dn[64];
-        if ((e = set_smem(down_skinny_kernel, smem_for(dp.stages, dp.stage_bytes), cfg_dn)) != cudaSuccess)
-            return fail(e, "shared-memory attribute");
-        e = launch_pdl(down_skinny_kernel, dim3(dp.units < sms ? dp.units : sms), smem_for(dp.stages, dp.stage_bytes),
-                       stream, mH, mH2, dp);
-        if (e != cudaSuccess) return fail(e, "down kernel launch");
     } else {
-        CUtensorMap mX, mX2, mH, mH2;
-        if (!make_map(&mX, xa, B, H, (uint64_t)H * 2, BM) ||
-            !make_map(&mX2, split ? xlo : xa, B, H, (uint64_t)H * 2, BM) ||
-            !make_map(&mH, hact, B, N, (uint64_t)ldn * 2, BM) || !make_map(&mH2, hact_lo, B, N, (uint64_t)ldn * 2, BM))
-            return fail(cudaErrorInvalidValue, "tensor map encoding");
-        const int mtiles = (B + BM - 1) / BM;
-
-        WideGuParams gp{};
-        gp.w = layer->gu_blk;
-        gp.M = B;
-        gp.N = N;
-        gp.R = R;
-        gp.KBh = layer->tc_kbh;
-        gp.T = layer->tc_T;
-        gp.Rw = wide_rows(N, R, mtiles, sms, split);
-        gp.mtiles = mtiles;
-        gp.tiles = mtiles * ((N + gp.Rw - 1) / gp.Rw);
-        gp.tmem_cols = tmem_cols_for(4 * gp.Rw);
-        gp.split = split ? 1 : 0;
-        gp.t_l = t_l;
-        gp.dense_flags = dense_flags;
-        gp.perm = perm;
-        gp.n_dense = n_dense;
-        gp.hact = hact;
-        gp.hact_lo = hact_lo;
-        gp.ldh = ldn;
-        gp.keep = active_idx ? keep : nullptr;
-        gp.keep_stride = kstride;
-        gp.keep_trace = keep_trace;
-        gp.ctl = ctl;
-        gp.zero = out_mode == kOutY ? out : nullptr;   // the down projection adds into y
-        gp.zero_count = (long long)B * H;
-        gp.stage_bytes = BM * kTileBytes * (split ? 2 : 1) + 2 * gp.Rw * kTileBytes;
-        gp.stages = stages_for(gp.stage_bytes, wide_budget());
-        // epilogue groups: the tile's 16-neuron column blocks split evenly over at most kWideGuGroups
-        const int blocks16 = gp.Rw / 16, per_group = (blocks16 + kWideGuGroups - 1) / kWideGuGroups;
-        const int gu_groups = (blocks16 + per_group - 1) / per_group;
-        static std::atomic<int> cfg_gu[64];
-        if ((e = set_smem(gu_wide_kernel, smem_for(gp.stages, gp.stage_bytes), cfg_gu)) != cudaSuccess)
-            return fail(e, "shared-memory attribute");
-        gu_wide_kernel<<<dim3(gp.tiles < sms ? gp.tiles : sms), 64 + 128 * gu_groups, smem_for(gp.stages, gp.stage_bytes),
-                         stream>>>(mX, mX2, gp);
-        if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "gate/up kernel launch");
-
-        // down projection: 256 output columns per unit when the hidden tiles pair up; the neuron
-        // range split so that the persistent CTAs' units come out even; every unit adds into the
-        // output (y cleared by the gate/up kernel, or the residual stream)
-        WideDownParams dp{};
-        dp.w = layer->wd_blk;
-        dp.M = B;
-        dp.H = H;
-        dp.KBn = layer->tc_kbn;
-        dp.dtiles = (layer->tc_dt % 2 == 0) ? 2 : 1;
-        dp.mtiles = mtiles;
-        dp.dcols = layer->tc_dt / dp.dtiles;
-        const int splits = wide_down_splits(mtiles * dp.dcols, dp.KBn, sms);
-        dp.kb_per_split = (dp.KBn + splits - 1) / splits;
-        dp.units = mtiles * dp.dcols * splits;
-        dp.out = out;
-        dp.perm = perm;
-        dp.ctl = ctl;
-        dp.stage_bytes = BM * kTileBytes * (2 + dp.dtiles);
-        dp.stages = stages_for(dp.stage_bytes, wide_budget());
-        dp.tmem_cols = tmem_cols_for(2 * BM * dp.dtiles);
-        static std::atomic<int> cfg_dn[64];
-        if ((e = set_smem(down_wide_kernel, smem_for(dp.stages, dp.stage_bytes), cfg_dn)) != cudaSuccess)
-            return fail(e, "shared-memory attribute");
-        down_wide_kernel<<<dim3(dp.units < sms ? dp.units : sms), 64 + 128 * kWideDownGroups,
-                           smem_for(dp.stages, dp.stage_bytes), stream>>>(mH, mH2, dp);
-        if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "down kernel launch");
+        GateUpArgs a{};
+        a.xhi = xa;
+        a.xlo = split ? xlo : nullptr;
+        a.B = B;
+        a.t_l = t_l;
+        a.dense_flags = dense_flags;
+        a.perm = perm;
+        a.n_dense = n_dense;
+        a.hact = hact;
+        a.hact_lo = hact_lo;
+        a.keep = active_idx ? keep : nullptr;
+        a.keep_trace = keep_trace;
+        a.zero = out_mode == kOutY ? out : nullptr;   // the down projection adds into y
+        a.ctl = ctl;
+        if (skinny_batch(B, split)) {
+            if ((e = launch_gate_up_skinny(layer, a, stream)) != cudaSuccess) return e;
+            e = launch_down_skinny(layer, hact, hact_lo, B, out, perm, ctl, stream);
+        } else {
+            if ((e = launch_gate_up_wide(layer, a, stream)) != cudaSuccess) return e;
+            e = launch_down_wide(layer, hact, hact_lo, B, out, perm, ctl, stream);
+        }
+        if (e != cudaSuccess) return e;
     }
     if (active_idx) {
         e = launch_pdl_threads(keep_list_kernel, dim3(B), 512, stream, static_cast<const uint8_t *>(keep), kstride, N,

@@ -135,6 +135,13 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
                          float eps, const uint8_t *dense_flags, const int32_t *perm, const int32_t *n_dense,
                          int out_mode, float *out, int32_t *active_idx, int32_t *active_cnt, uint8_t *keep_trace,
                          void *tc_ws, int *ctl, cudaStream_t stream, bool union_path = false);
+// The calibration's halves of it: gate and up of B fp32 inputs with every neuron kept (h in bf16
+// parts inside tc_ws, a = SiLU(x W_gate) in a_out, both with row stride ldn), and the down
+// projection of any M rows of h, added into out.
+cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void *tc_ws, const uint16_t **hact,
+                           const uint16_t **hact_lo, float *a_out, int *ctl, cudaStream_t stream);
+cudaError_t run_tc_down(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
+                        int *ctl, cudaStream_t stream);
 cudaError_t launch_wait_timeout(int *ctl, cudaStream_t stream);
 cudaError_t launch_route(const int32_t *ids, int B, const uint8_t *lut, int V, int32_t *perm,
                          int32_t *n_dense, uint8_t *flags, int32_t *status, cudaStream_t stream);
