@@ -10,6 +10,8 @@
 // host; the coarse-to-fine driver chains everything for a whole stack.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
+#include <cstring>
 #include <vector>
 
 #include "common.cuh"
@@ -605,19 +607,99 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
 namespace sats {
 namespace {
 
-// Eqs. 11-12, the sums: for every occurrence, d = max(0, l_sparse - l_base) into the token's total.
-__global__ void score_accum_kernel(const int32_t *__restrict__ ids, const float *__restrict__ lb,
-                                   const float *__restrict__ ls, int64_t n, int V, double *__restrict__ total,
-                                   unsigned *__restrict__ count, int32_t *__restrict__ status)
+// A warp's table of the token ids it has met: sums of the occurrences it has seen, added to the
+// device totals once at the end.  Token frequencies are far from even (a corpus' most common token
+// is several per cent of it), and atomics on one address go one after the other: 290 us for a
+// million occurrences added straight to global memory.  Tables of one warp need no atomics:
+// lanes with the same id take turns.  An id whose slot another id holds is added to the totals
+// directly.
+constexpr int kTallySlots = 512, kTallyWarps = 16;
+constexpr int kNoToken = -1;
+
+template <bool SUMS>
+struct Tally {
+    int id[kTallySlots];
+    unsigned count[kTallySlots];
+    double sum[SUMS ? kTallySlots : 1];
+};
+
+// Adds one occurrence per lane (id kNoToken: none) with excess loss v.
+template <bool SUMS>
+__device__ __forceinline__ void tally_add(Tally<SUMS> &T, int id, float v, double *__restrict__ total,
+                                          unsigned *__restrict__ count)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int id = ids[i];
-        if (id < 0 || id >= V) {
-            atomicOr(status, kStatusBadToken);
-            continue;
-        }
-        atomicAdd(total + id, (double)fmaxf(0.0f, ls[i] - lb[i]));
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned same = __match_any_sync(0xffffffffu, id);
+    const int slot = (int)(((unsigned)id * 2654435761u) >> (32 - 9));
+    static_assert(kTallySlots == 1 << 9, "slot hash width");
+    const unsigned turn = __popc(same & ((1u << lane) - 1u));   // of the lanes with this id
+    bool mine = false;
+    if (id != kNoToken && turn == 0 && T.id[slot] == kNoToken) T.id[slot] = id;   // one id wins an empty slot
+    __syncwarp();
+    if (id != kNoToken) mine = T.id[slot] == id;
+    if (id != kNoToken && !mine) {
+        if (SUMS) atomicAdd(total + id, (double)v);
         atomicAdd(count + id, 1u);
+    }
+    if (mine && turn == 0) T.count[slot] += (unsigned)__popc(same);
+    if (!SUMS) {
+        __syncwarp();
+        return;
+    }
+    const unsigned turns = __reduce_max_sync(0xffffffffu, mine ? turn + 1u : 0u);
+    for (unsigned k = 0; k < turns; ++k) {
+        if (mine && turn == k) T.sum[slot] += (double)v;
+        __syncwarp();
+    }
+}
+
+// Eqs. 11-12, the sums (SUMS): for every occurrence, d = max(0, l_sparse - l_base) into the token's
+// total, and the occurrences per token; without SUMS the occurrences only.
+template <bool SUMS>
+__global__ void __launch_bounds__(32 * kTallyWarps) tally_kernel(const int32_t *__restrict__ ids,
+                                                                 const float *__restrict__ lb,
+                                                                 const float *__restrict__ ls, int64_t n, int V,
+                                                                 double *__restrict__ total,
+                                                                 unsigned *__restrict__ count,
+                                                                 int32_t *__restrict__ status)
+{
+    extern __shared__ __align__(16) char tally_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    Tally<SUMS> &T = reinterpret_cast<Tally<SUMS> *>(tally_smem)[warp];
+    for (int i = lane; i < kTallySlots; i += 32) {
+        T.id[i] = kNoToken;
+        T.count[i] = 0u;
+        if (SUMS) T.sum[i] = 0.0;
+    }
+    __syncwarp();
+    constexpr int kAhead = 4;   // loads in flight per lane
+    const int64_t step = (int64_t)gridDim.x * kTallyWarps * 32;
+    for (int64_t base = ((int64_t)blockIdx.x * kTallyWarps + warp) * 32; base < n; base += kAhead * step) {
+        int id[kAhead];
+        float v[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            const int64_t i = base + k * step + lane;
+            id[k] = kNoToken;
+            v[k] = 0.f;
+            if (i < n) {
+                id[k] = ids[i];
+                if (SUMS) v[k] = fmaxf(0.0f, ls[i] - lb[i]);
+                if (id[k] < 0 || id[k] >= V) {
+                    atomicOr(status, kStatusBadToken);
+                    id[k] = kNoToken;
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) tally_add<SUMS>(T, id[k], v[k], total, count);
+    }
+    __syncwarp();
+    for (int i = lane; i < kTallySlots; i += 32) {
+        const int id = T.id[i];
+        if (id == kNoToken) continue;
+        if (SUMS) atomicAdd(total + id, T.sum[i]);
+        atomicAdd(count + id, T.count[i]);
     }
 }
 
@@ -629,16 +711,132 @@ __global__ void score_final_kernel(const double *__restrict__ total, const unsig
     if (v < V) score[v] = count[v] ? (float)(total[v] / count[v]) : INFINITY;
 }
 
-__global__ void freq_kernel(const int32_t *__restrict__ ids, int64_t m, int V, unsigned *__restrict__ freq,
-                            int32_t *__restrict__ status)
+// Eq. 14 on the device.  With the held-out occurrences' scores in increasing order, the candidates
+// around the target are the occurrence at rank K + 1 (K: the most occurrences that may lie below tau
+// for R(tau) <= r_tar) and the next larger score.  A radix search over the V scores, weighted by the
+// occurrences (11 + 11 + 10 bits of the ordered bit pattern; each level one kernel whose last CTA
+// picks the bin), finds the first; one more pass sums the occurrences below it and at it, and takes
+// the smallest score above it.  Sorting the scores on the host took 2 ms of the call.
+struct TauSearch {
+    unsigned done[3];
+    uint32_t prefix;                 // bits of the rank's score chosen so far
+    unsigned long long rest;         // rank within the chosen bins (1-based)
+    unsigned long long below, at;    // occurrences with a smaller score, with the same score
+    unsigned long long negative;     // occurrences with a score below 0
+    unsigned long long finite;       // occurrences with a score below +inf
+    uint32_t not_above;              // complement of the ordered bits of the smallest larger score (0: none)
+    uint32_t pad;
+    unsigned long long hist[3][2048];
+};
+
+// Floats in increasing order as unsigned numbers (-0 as +0).
+__device__ __forceinline__ uint32_t ordered_bits(float f)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        const int id = ids[i];
-        if (id < 0 || id >= V) {
-            atomicOr(status, kStatusBadToken);
-            continue;
+    const uint32_t b = __float_as_uint(f + 0.0f);
+    return (b & 0x80000000u) ? ~b : b | 0x80000000u;
+}
+
+constexpr int kTauThreads = 512;
+
+template <int LEVEL>
+__global__ void __launch_bounds__(kTauThreads) tau_level_kernel(const float *__restrict__ score,
+                                                                const unsigned *__restrict__ freq, int V,
+                                                                unsigned long long rank, TauSearch *S)
+{
+    constexpr int kShift = LEVEL == 0 ? 21 : LEVEL == 1 ? 10 : 0;
+    constexpr int kBins = LEVEL == 2 ? 1024 : 2048;
+    __shared__ unsigned long long h[kBins];
+    __shared__ unsigned long long warp_sum_s[kTauThreads / 32];
+    __shared__ bool last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < kBins; i += kTauThreads) h[i] = 0ull;
+    grid_dependency_wait();
+    grid_launch_dependents();
+    const uint32_t prefix = LEVEL == 0 ? 0u : S->prefix;
+    __syncthreads();
+    for (int v = blockIdx.x * kTauThreads + tid; v < V; v += gridDim.x * kTauThreads) {
+        const unsigned f = freq[v];
+        const uint32_t b = ordered_bits(score[v]);
+        const bool in = LEVEL == 0 || (LEVEL == 1 ? (b >> 21) == (prefix >> 21) : (b >> 10) == (prefix >> 10));
+        if (f && in) atomicAdd(h + ((b >> kShift) & (kBins - 1)), (unsigned long long)f);
+    }
+    __syncthreads();
+    for (int i = tid; i < kBins; i += kTauThreads)
+        if (h[i]) atomicAdd(&S->hist[LEVEL][i], h[i]);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(&S->done[LEVEL], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    constexpr int kPer = kBins / kTauThreads;
+    unsigned long long c[kPer], s = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        c[k] = __ldcg(&S->hist[LEVEL][tid * kPer + k]);
+        s += c[k];
+    }
+    unsigned long long incl = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) warp_sum_s[warp] = incl;
+    const unsigned long long r = LEVEL == 0 ? rank : S->rest;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) incl += warp_sum_s[w];
+    unsigned long long run = incl - s;
+    if (run < r && incl >= r) {   // one thread's bins hold the rank (1 <= rank <= the occurrences)
+        for (int k = 0; k < kPer; ++k) {
+            if (run + c[k] >= r) {
+                S->prefix = prefix | ((uint32_t)(tid * kPer + k) << kShift);
+                S->rest = r - run;
+                break;
+            }
+            run += c[k];
         }
-        atomicAdd(freq + id, 1u);
+    }
+}
+
+// The occurrences around the score at the rank (S->prefix), and those below 0 and below +inf.
+__global__ void __launch_bounds__(kTauThreads) tau_sums_kernel(const float *__restrict__ score,
+                                                               const unsigned *__restrict__ freq, int V, TauSearch *S)
+{
+    __shared__ unsigned long long sums[4];
+    __shared__ uint32_t not_above;
+    if (threadIdx.x < 4) sums[threadIdx.x] = 0ull;
+    if (threadIdx.x == 4) not_above = 0u;
+    grid_dependency_wait();
+    __syncthreads();
+    const uint32_t at = S->prefix, zero = 0x80000000u, inf = 0xff800000u;
+    unsigned long long s[4] = {0ull, 0ull, 0ull, 0ull};
+    uint32_t na = 0u;
+    for (int v = blockIdx.x * kTauThreads + threadIdx.x; v < V; v += gridDim.x * kTauThreads) {
+        const unsigned f = freq[v];
+        if (!f) continue;
+        const uint32_t b = ordered_bits(score[v]);
+        s[0] += b < at ? f : 0u;
+        s[1] += b == at ? f : 0u;
+        s[2] += b < zero ? f : 0u;
+        s[3] += b < inf ? f : 0u;
+        if (b > at) na = max(na, ~b);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+        if ((threadIdx.x & 31) == 0 && s[k]) atomicAdd(sums + k, s[k]);
+    }
+    na = __reduce_max_sync(0xffffffffu, na);
+    if ((threadIdx.x & 31) == 0 && na) atomicMax(&not_above, na);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (sums[0]) atomicAdd(&S->below, sums[0]);
+        if (sums[1]) atomicAdd(&S->at, sums[1]);
+        if (sums[2]) atomicAdd(&S->negative, sums[2]);
+        if (sums[3]) atomicAdd(&S->finite, sums[3]);
+        if (not_above) atomicMax(&S->not_above, not_above);
     }
 }
 
@@ -650,7 +848,7 @@ __global__ void lut_kernel(const float *__restrict__ score, int V, float tau, ui
 }
 
 struct ScoreLayout {
-    size_t status, total, count, total_bytes;
+    size_t status, search, total, count, total_bytes;
 };
 
 ScoreLayout score_layout(int V)
@@ -659,6 +857,8 @@ ScoreLayout score_layout(int V)
     size_t off = 0;
     S.status = off;
     off += 256;
+    S.search = off;   // sats_route_calibrate
+    off += al256(sizeof(TauSearch));
     S.total = off;
     off += al256((size_t)V * sizeof(double));
     S.count = off;
@@ -676,10 +876,42 @@ sats_status read_status_word(int32_t *word, cudaStream_t st)
     return (v & kStatusBadToken) ? SATS_EDEVICE : SATS_OK;
 }
 
-int grid_for(int64_t n)
+template <bool SUMS>
+cudaError_t launch_tally(const int32_t *ids, const float *lb, const float *ls, int64_t n, int V, double *total,
+                         unsigned *count, int32_t *status, cudaStream_t st)
 {
-    const int64_t g = (n + 255) / 256;
-    return (int)(g < 4096 ? (g > 0 ? g : 1) : 4096);
+    const size_t smem = sizeof(Tally<SUMS>) * kTallyWarps;
+    const cudaError_t e = cudaFuncSetAttribute(tally_kernel<SUMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int64_t want = (n + 32 * kTallyWarps - 1) / (32 * kTallyWarps);
+    const int sms = fused_grid(kMaxGrid);
+    tally_kernel<SUMS><<<(int)(want < sms ? want : sms), 32 * kTallyWarps, smem, st>>>(ids, lb, ls, n, V, total, count,
+                                                                                     status);
+    return cudaGetLastError();
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_search(void (*kernel)(KArgs...), int V, cudaStream_t st, Args... args)
+{
+    const int want = (V + 2 * kTauThreads - 1) / (2 * kTauThreads), sms = fused_grid(kMaxGrid);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(want < sms ? want : sms);
+    cfg.blockDim = dim3(kTauThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+float score_of(uint32_t ordered)
+{
+    const uint32_t b = (ordered & 0x80000000u) ? ordered & 0x7fffffffu : ~ordered;
+    float f;
+    std::memcpy(&f, &b, sizeof f);
+    return f;
 }
 
 }  // namespace
@@ -706,7 +938,8 @@ sats_status sats_token_scores(const int32_t *ids, const float *l_base, const flo
     unsigned *count = reinterpret_cast<unsigned *>(base + S.count);
     cudaError_t e = cudaMemsetAsync(ws, 0, S.total_bytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "score workspace clear");
-    if (n > 0) score_accum_kernel<<<grid_for(n), 256, 0, st>>>(ids, l_base, l_sparse, n, V, total, count, status);
+    if (n > 0 && (e = launch_tally<true>(ids, l_base, l_sparse, n, V, total, count, status, st)) != cudaSuccess)
+        return cuda_fail(e, "score kernel launch");
     score_final_kernel<<<(V + 255) / 256, 256, 0, st>>>(total, count, V, score);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "score kernel launch");
     return read_status_word(status, st);
@@ -722,30 +955,46 @@ sats_status sats_route_calibrate(const float *score, int V, const int32_t *heldo
     char *base = static_cast<char *>(ws);
     int32_t *status = reinterpret_cast<int32_t *>(base + S.status);
     unsigned *freq = reinterpret_cast<unsigned *>(base + S.count);
-    cudaError_t e = cudaMemsetAsync(status, 0, 256, st);
+    TauSearch *search = reinterpret_cast<TauSearch *>(base + S.search);
+    cudaError_t e = cudaMemsetAsync(status, 0, 256 + sizeof(TauSearch), st);   // (the search follows the status word)
     if (e == cudaSuccess) e = cudaMemsetAsync(freq, 0, (size_t)V * sizeof(unsigned), st);
     if (e != cudaSuccess) return cuda_fail(e, "held-out count clear");
-    if (m > 0) freq_kernel<<<grid_for(m), 256, 0, st>>>(heldout_ids, m, V, freq, status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "held-out count kernel launch");
-    sats_status s = read_status_word(status, st);
-    if (s != SATS_OK) return s;
-    // Eq. 14 on the host over the V scores: R(tau) = (held-out occurrences with score < tau) / m
-    std::vector<float> sc((size_t)V);
-    std::vector<unsigned> fr((size_t)V);
-    e = cudaMemcpyAsync(sc.data(), score, sc.size() * sizeof(float), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(fr.data(), freq, fr.size() * sizeof(unsigned), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(e, "score read-back");
-    std::vector<std::pair<float, unsigned>> occ;
-    for (int v = 0; v < V; ++v)
-        if (fr[(size_t)v]) occ.emplace_back(sc[(size_t)v], fr[(size_t)v]);
-    std::sort(occ.begin(), occ.end());
-    // candidates in increasing order: 0, each distinct finite held-out score, +inf; below(tau) is the
-    // number of held-out occurrences whose score is < tau
+    if (m > 0 && (e = launch_tally<false>(heldout_ids, nullptr, nullptr, m, V, nullptr, freq, status, st)) != cudaSuccess)
+        return cuda_fail(e, "held-out count kernel launch");
+    // K: the most occurrences c <= m with c / m <= r_tar (-1: none); R(tau) = (occurrences below tau) / m
     const double M = m > 0 ? (double)m : 1.0;
+    int64_t K = m;
+    if (!(r_tar >= 1.0)) {
+        K = r_tar < 0.0 ? -1 : (int64_t)(r_tar * M);
+        while (K >= 0 && (double)K / M > r_tar) --K;
+        while (K < m && (double)(K + 1) / M <= r_tar) ++K;
+    }
+    struct {
+        int32_t status;
+        char pad[252];
+        unsigned done[3];
+        uint32_t prefix;
+        unsigned long long rest, below, at, negative, finite;
+        uint32_t not_above, pad2;
+    } got;
+    static_assert(offsetof(TauSearch, hist) == sizeof(got) - 256, "layout of the search's results");
+    const unsigned long long rank = (unsigned long long)(K < 0 ? 1 : K >= m ? m : K + 1);   // 1-based
+    if (m > 0) {
+        e = launch_search(tau_level_kernel<0>, V, st, score, (const unsigned *)freq, V, rank, search);
+        if (e == cudaSuccess) e = launch_search(tau_level_kernel<1>, V, st, score, (const unsigned *)freq, V, rank, search);
+        if (e == cudaSuccess) e = launch_search(tau_level_kernel<2>, V, st, score, (const unsigned *)freq, V, rank, search);
+        if (e == cudaSuccess) e = launch_search(tau_sums_kernel, V, st, score, (const unsigned *)freq, V, search);
+        if (e != cudaSuccess) return cuda_fail(e, "threshold search kernels launch");
+    }
+    e = cudaMemcpyAsync(&got, status, sizeof got, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e, "threshold search read-back");
+    if (got.status & kStatusBadToken) return SATS_EDEVICE;
+    // The candidates are 0, each distinct finite positive held-out score, and +inf; R never falls from
+    // one to the next, so the nearest to the target is one of the two around it (a tie: the smaller).
     double best_gap = INFINITY, best_R = 0.0;
     float best_tau = 0.0f;
-    auto consider = [&](float tau, uint64_t below) {
+    auto consider = [&](float tau, uint64_t below) {   // in increasing order of tau
         const double R = (double)below / M;
         const double gap = std::fabs(R - r_tar);
         if (gap < best_gap) {
@@ -754,16 +1003,14 @@ sats_status sats_route_calibrate(const float *score, int V, const int32_t *heldo
             best_R = R;
         }
     };
-    uint64_t below = 0;
-    size_t i = 0;
-    while (i < occ.size() && occ[i].first < 0.0f) below += occ[i++].second;   // (scores are >= 0)
-    consider(0.0f, below);
-    while (i < occ.size() && std::isfinite(occ[i].first)) {
-        const float v = occ[i].first;
-        if (v > 0.0f) consider(v, below);   // R(v) counts the scores strictly below v
-        while (i < occ.size() && occ[i].first == v) below += occ[i++].second;
+    consider(0.0f, got.negative);
+    if (m > 0) {
+        const float at = score_of(got.prefix);
+        if (at > 0.0f && std::isfinite(at)) consider(at, got.below);
+        const float above = got.not_above ? score_of(~got.not_above) : INFINITY;
+        if (std::isfinite(above) && above > 0.0f) consider(above, got.below + got.at);
     }
-    consider(INFINITY, below);
+    consider(INFINITY, m > 0 ? got.finite : 0);
     *tau_out = best_tau;
     if (R_out) *R_out = best_R;
     if (lut) {
