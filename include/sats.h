@@ -240,7 +240,10 @@ SATS_API sats_status sats_sparse_mlp_union_f32(const sats_layer *layer, const fl
  *   u = x W_up + scale (x A_up) B_up,        h = keep ? a u : 0
  *   y = h W_down + scale (h A_down) B_down
  * in the decode kernel: the gate's low-rank term for every neuron, the up and
- * down terms only for kept neurons; batches run as passes of that kernel.
+ * down terms only for kept neurons.  Larger batches (where sats_uses_tensor_cores
+ * says so, from hidden size 96) stream the weights once through the tensor cores
+ * in that kernel's fp32 arithmetic: activations and h enter as three bf16 parts
+ * and sums are rounded every 32 products.
  * Arguments, index outputs, workspace and errors are those of sats_sparse_mlp
  * (x bf16) and sats_sparse_mlp_f32 (x fp32); the adapter must match the
  * layer's H and N (else SATS_ESHAPE).

@@ -79,7 +79,12 @@ sats_status run_layer(const sats_layer *layer, int x_mode, const void *x, int B,
     const int H = layer->H, N = layer->N;
     const WsLayout L = ws_layout(H, N, B);
     char *base = static_cast<char *>(ws);
-    if (!lora && use_tc_path(H, B)) {   // the LoRA variant runs in passes of the fused kernel at any batch
+    if (lora && lora_tc_ok(H, B)) {
+        const cudaError_t e = run_lora_tc(layer, lora, x_mode != kXBf16, x, B, *t_per_pass_l, out, active_idx, active_cnt,
+                                          base + L.tc, reinterpret_cast<int *>(base + L.ctl), stream);
+        return e == cudaSuccess ? SATS_OK : SATS_ECUDA;   // run_lora_tc recorded the failing step
+    }
+    if (!lora && use_tc_path(H, B)) {
         const cudaError_t e = run_tc_layer(layer, x_mode, x, B, *t_per_pass_l, norm_w, eps, perm ? nullptr : dense_flags,
                                            perm, n_dense, out_mode,
                                            out, active_idx, active_cnt, keep_trace, base + L.tc,
@@ -264,11 +269,13 @@ sats_status sats_lora_create(const sats_layer *layer, const void *A_gate, const 
                              static_cast<const uint16_t *>(A_up), static_cast<const uint16_t *>(B_up),
                              static_cast<const uint16_t *>(A_down), static_cast<const uint16_t *>(B_down), l->H, l->N,
                              r, l, st);
+    if (e == cudaSuccess) e = lora_pack_tc(layer, static_cast<const uint16_t *>(A_down), l, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         cudaFree(l->blk);
         cudaFree(l->agu);
         cudaFree(l->bd);
+        cudaFree(l->ad_blk);
         delete l;
         return cuda_fail(e, "adapter allocation or repacking");
     }
@@ -283,10 +290,11 @@ sats_status sats_lora_destroy(sats_lora *lora)
     const cudaError_t e1 = cudaFree(lora->blk);
     const cudaError_t e2 = cudaFree(lora->agu);
     const cudaError_t e3 = cudaFree(lora->bd);
+    const cudaError_t e4 = cudaFree(lora->ad_blk);
     delete lora;
     if (e1 != cudaSuccess) return cuda_fail(e1, "cudaFree");
     if (e2 != cudaSuccess) return cuda_fail(e2, "cudaFree");
-    return from_cuda(e3, "cudaFree");
+    return from_cuda(e3 != cudaSuccess ? e3 : e4, "cudaFree");
 }
 
 static sats_status lora_common(const sats_layer *layer, const sats_lora *lora, int x_mode, const void *x, int B,

@@ -348,6 +348,574 @@ cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, f
     return launch_pdl_cfg(gate_precise_kernel<F32>, dim3(mt, layer->tc_T), kPreciseThreads<F32>, smem, stream, mX, p);
 }
 
+// ---------------------------------------------------------------------- LoRA batches
+// The sparse path of a fine-tuned model (Sec. 4) for batches beyond one pass of the fused
+// kernel, in the arithmetic of that kernel:
+//   lora_z_kernel        z = x A_gate | x A_up, per slice of hidden rows
+//   lora_gate_up_kernel  g = x W_gate + s z B_gate[:, n], u likewise, h = keep ? SiLU(g) u : 0
+//   lora_down_kernel     y += h W_down, w += h A_down (one more tile of outputs)
+//   lora_out_kernel      y += s w B_down
+// W is streamed once for up to kLoraTok tokens, where the fused kernel streamed it once per pass
+// of one or two (129 us for four tokens on the Llama-shaped layer at 70 % sparsity, 267 us for
+// eight).  What bounds it: that stream; with at most 32 tokens the parts of an operand are the
+// rows of one tile, so a K step is one MMA per weight tile however many parts there are, and
+// their products are added in the epilogue.
+constexpr int kLoraTok = 32;
+constexpr int kLoraWRow = kMaxLoraRank;        // row pitch of w
+constexpr int kLoraZRow = 2 * kMaxLoraRank;    // row pitch of z
+constexpr int kLoraEpiThreads = 256;           // two groups of four warps, one per 16 tokens
+template <bool F32> constexpr int kLoraGuThreads = 64 + (F32 ? kConvThreads : 0) + kLoraEpiThreads;
+constexpr int kLoraDownThreads = 64 + kConvThreads + kLoraEpiThreads;
+
+// z[b][s][0 .. 2r) over the hidden rows of slice s.  Grid: (slices, B).
+template <typename X>
+__global__ void __launch_bounds__(256) lora_z_kernel(const X *__restrict__ x, int H, const uint16_t *__restrict__ agu,
+                                                     int r, float *__restrict__ z)
+{
+    __shared__ float red[256][9];
+    const int s = blockIdx.x, slices = gridDim.x, b = blockIdx.y, t = threadIdx.x;
+    const int C = r / 4, rows = 256 / C;   // 16-byte chunks of a row of agu (2r values), rows per pass
+    const int c = t % C, row = t / C;
+    const int h0 = (int)((long long)H * s / slices), h1 = (int)((long long)H * (s + 1) / slices);
+    grid_dependency_wait();
+    grid_launch_dependents();
+    float acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+    if (row < rows) {
+#pragma unroll 4
+        for (int h = h0 + row; h < h1; h += rows) {
+            float xv;
+            if constexpr (sizeof(X) == 2) xv = __uint_as_float((uint32_t)x[(size_t)b * H + h] << 16);
+            else xv = x[(size_t)b * H + h];
+            float w[8];
+            unpack8(*reinterpret_cast<const uint4 *>(agu + (size_t)h * 2 * r + 8 * c), w);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] = fmaf(xv, w[e], acc[e]);
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) red[t][e] = acc[e];
+    __syncthreads();
+    if (t < 2 * r) {
+        float sum = 0.f;
+        for (int k = 0; k < rows; ++k) sum += red[k * C + t / 8][t % 8];
+        z[((size_t)b * slices + s) * kLoraZRow + t] = sum;
+    }
+}
+
+struct LoraGuParams {
+    const uint16_t *w;      // gu_blk
+    const float *x;         // fp32 activations [B][H] (bf16 ones come by TMA)
+    int B, H, N, R, KBh;
+    int NT;                 // tokens per tile (16 or 32)
+    int halves;             // accumulators per K block and weight matrix: K = 32 each (2) or 64 (1)
+    float t_l, scale;
+    const uint16_t *blk;    // adapter columns per neuron: B_gate, B_up, A_down
+    int r;
+    const float *z;         // [B][slices][kLoraZRow]
+    int slices;
+    float *h;               // [B][ldh] fp32
+    int ldh;
+    uint8_t *keep;          // [B][keep_stride] or nullptr
+    int keep_stride;
+    float *y;               // [B][H], cleared here for the down kernel's additions
+    float *wsum;            // [B][kLoraWRow], likewise
+    int *ctl;
+    int stages, stage_bytes, w_bytes, ring_bytes;
+    uint32_t tmem_cols;
+};
+
+// One tile of NT tokens and R neurons per CTA, as gate_precise_kernel; grid: token tiles x neuron tiles.
+template <bool F32>
+__global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
+    lora_gate_up_kernel(const __grid_constant__ CUtensorMap tmX, const LoraGuParams p)
+{
+    constexpr int kEpi0 = 2 + (F32 ? kConvThreads / 32 : 0);
+    constexpr int kXParts = F32 ? kParts : 1;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *ring = align1024(smem_raw);
+    uint8_t *parts = ring + p.ring_bytes;
+    uint64_t *full = reinterpret_cast<uint64_t *>(parts + (F32 ? kPartStages * kParts * p.NT * kTileBytes : 0));
+    uint64_t *empty = full + kMaxStages;
+    uint64_t *pfull = empty + kMaxStages;
+    uint64_t *pempty = pfull + kPartStages;
+    uint64_t *acc_full = pempty + kPartStages;   // [2]
+    uint64_t *acc_empty = acc_full + 2;          // [2]
+    uint64_t *mma_done = acc_empty + 2;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
+    __shared__ int abort_flag, issued_s, consumed_s;
+    __shared__ float zs[kLoraTok][kLoraZRow];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int R = p.R, NT = p.NT, S = p.stages, KBh = p.KBh, halves = p.halves;
+    const int NX = kXParts * NT;   // accumulator columns: the parts side by side
+    const int m0 = (int)blockIdx.x * NT, t = blockIdx.y;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int s = 0; s < kPartStages; ++s) {
+            mbar_init(&pfull[s], kConvThreads);
+            mbar_init(&pempty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], kLoraEpiThreads);
+        }
+        mbar_init(mma_done, 1);
+        abort_flag = 0;
+        issued_s = 0;
+        consumed_s = 0;
+        mbar_init_fence();
+    }
+    if (warp == 1) tmem_alloc(tmem_slot, p.tmem_cols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    grid_launch_dependents();
+
+    if (warp == 0 && lane == 0) {
+        const uint32_t load_bytes = (uint32_t)p.w_bytes + (F32 ? 0u : (uint32_t)(NT * kTileBytes));
+        const uint64_t once = l2_policy_evict_first();
+        auto load_w = [&](int s, int kb) {
+            const uint16_t *src = p.w + ((size_t)t * KBh + kb) * 2 * R * BK;
+            if (gridDim.x == 1) bulk_load(ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s], once);
+            else bulk_load_shared(ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s]);
+        };
+        const int npre = KBh < S ? KBh : S;
+        for (int i = 0; i < npre; ++i) {
+            mbar_arrive_expect_tx(&full[i], load_bytes);
+            load_w(i, i);
+        }
+        if (!F32) grid_dependency_wait();
+        int kb = 0;
+        for (int s = 0, ph = 0; kb < KBh; ++kb) {
+            if (kb >= npre) {
+                if (!mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
+                mbar_arrive_expect_tx(&full[s], load_bytes);
+                load_w(s, kb);
+            }
+            if (!F32) tma_load(ring + (size_t)s * p.stage_bytes + p.w_bytes, &tmX, kb * BK, m0, &full[s]);
+            if (++s == S) { s = 0; ph ^= 1; }
+        }
+        issued_s = kb;
+    } else if (warp == 1 && lane == 0) {
+        const uint32_t idesc = instr_desc(BM, NX);
+        const int per = 4 / halves;   // K = 16 steps per accumulator
+        int kb = 0;
+        for (int s = 0, ph = 0; kb < KBh; ++kb) {
+            const int buf = kb & 1, ps = kb % kPartStages;
+            if (!mbar_wait(&acc_empty[buf], (uint32_t)((kb >> 1) & 1) ^ 1u, &abort_flag) ||
+                !mbar_wait(&full[s], (uint32_t)ph, &abort_flag) ||
+                (F32 && !mbar_wait(&pfull[ps], (uint32_t)((kb / kPartStages) & 1), &abort_flag))) {
+                set_timeout(p.ctl, &abort_flag);
+                break;
+            }
+            tc_fence_after();
+            const uint32_t st = smem_addr(ring + (size_t)s * p.stage_bytes);
+            const uint32_t xs = F32 ? smem_addr(parts + (size_t)ps * kParts * NT * kTileBytes) : st + p.w_bytes;
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk) {
+                const uint32_t d = tmem + (uint32_t)((buf * halves + kk / per) * 2 * NX), acc = kk % per ? 1u : 0u;
+                const uint64_t b = smem_desc(xs + kk * 32);
+                mma_bf16(d, smem_desc(st + kk * 32), b, idesc, acc);
+                mma_bf16(d + NX, smem_desc(st + R * kTileBytes + kk * 32), b, idesc, acc);
+            }
+            mma_commit(&empty[s]);
+            if (F32) mma_commit(&pempty[ps]);
+            mma_commit(&acc_full[buf]);
+            if (++s == S) { s = 0; ph ^= 1; }
+        }
+        consumed_s = kb;
+        mma_commit(mma_done);
+    } else if (F32 && warp >= 2 && warp < kEpi0) {
+        grid_dependency_wait();
+        auto load = [&](int r, int c, int kb, float4 &lo, float4 &hi) {
+            const int m = m0 + r, k = kb * BK + c * 8;
+            if (m < p.B && k < p.H) {   // H is a multiple of 8
+                const float4 *src = reinterpret_cast<const float4 *>(p.x + (size_t)m * p.H + k);
+                lo = src[0];
+                hi = src[1];
+            }
+        };
+        if (!cut_tiles<kLoraTok>(parts, NT, KBh, pfull, pempty, &abort_flag, load)) set_timeout(p.ctl, &abort_flag);
+    } else if (warp >= kEpi0) {
+        const int et = threadIdx.x - 32 * kEpi0;
+        const int quad = warp & 3, grp = (warp - kEpi0) >> 2;
+        const int c0 = 16 * grp;
+        const int n = t * R + 32 * quad + lane;
+        const bool busy = c0 < NT && 32 * quad < R;   // (uniform in the warp)
+        const uint32_t lane0 = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0;
+        float acc[2][16];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int e = 0; e < 16; ++e) acc[q][e] = 0.f;
+        bool ok = true;
+        for (int kb = 0; kb < KBh; ++kb) {
+            const int buf = kb & 1;
+            if (!mbar_wait(&acc_full[buf], (uint32_t)((kb >> 1) & 1), &abort_flag)) {
+                set_timeout(p.ctl, &abort_flag);
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            if (busy) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    float sum[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) sum[e] = 0.f;
+                    for (int f = 0; f < halves; ++f) {
+                        float v[kXParts][16];
+#pragma unroll
+                        for (int k = 0; k < kXParts; ++k)
+                            tmem_ld16(lane0 + (uint32_t)(((buf * halves + f) * 2 + q) * NX + k * NT), v[k]);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            float w = v[kXParts - 1][e];   // the small parts first
+#pragma unroll
+                            for (int k = kXParts - 2; k >= 0; --k) w += v[k][e];
+                            sum[e] += w;
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) acc[q][e] += sum[e];
+                }
+            }
+            tc_fence_before();
+            mbar_arrive(&acc_empty[buf]);
+        }
+        grid_dependency_wait();   // z, and y, w, h and the keep bytes may still be in use by the preceding kernels
+        const int ctas = (int)(gridDim.x * gridDim.y), cta = (int)(blockIdx.y * gridDim.x + blockIdx.x);
+        for (long long i = (long long)cta * kLoraEpiThreads + et; i < (long long)p.B * (p.H >> 2);
+             i += (long long)ctas * kLoraEpiThreads)
+            reinterpret_cast<float4 *>(p.y)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = cta * kLoraEpiThreads + et; i < p.B * kLoraWRow; i += ctas * kLoraEpiThreads) p.wsum[i] = 0.f;
+        const int r = p.r, r2 = 2 * r;
+        for (int i = et; i < NT * r2; i += kLoraEpiThreads) {
+            const int j = i / r2, c = i % r2;
+            float v = 0.f;
+            if (m0 + j < p.B)
+                for (int k = 0; k < p.slices; ++k) v += p.z[((size_t)(m0 + j) * p.slices + k) * kLoraZRow + c];
+            zs[j][c] = v;
+        }
+        named_barrier(1, kLoraEpiThreads);
+        if (ok && busy && 32 * quad + lane < R && n < p.N) {
+            float lg[16], lu[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) lg[e] = lu[e] = 0.f;
+            const uint16_t *col = p.blk + (size_t)n * 3 * r;
+            for (int q0 = 0; q0 < r; q0 += 8) {
+                float bg[8], bu[8];
+                unpack8(*reinterpret_cast<const uint4 *>(col + q0), bg);
+                unpack8(*reinterpret_cast<const uint4 *>(col + r + q0), bu);
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        lg[e] = fmaf(zs[c0 + e][q0 + q], bg[q], lg[e]);
+                        lu[e] = fmaf(zs[c0 + e][r + q0 + q], bu[q], lu[e]);
+                    }
+            }
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const int j = m0 + c0 + e;
+                if (j < p.B && c0 + e < NT) {
+                    const float g = fmaf(p.scale, lg[e], acc[0][e]);
+                    const float u = fmaf(p.scale, lu[e], acc[1][e]);
+                    const float a = g / (1.0f + expf(-g));   // SiLU, Eq. 2
+                    const bool keep = fabsf(a) >= p.t_l;     // Eqs. 4-5
+                    p.h[(size_t)j * p.ldh + n] = keep ? a * u : 0.f;
+                    if (p.keep) p.keep[(size_t)j * p.keep_stride + n] = keep ? 1 : 0;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int never = 0;
+        if (abort_flag)
+            for (int k = consumed_s; k < issued_s; ++k) mbar_wait(&full[k % S], (uint32_t)((k / S) & 1), &never);
+        mbar_wait(mma_done, 0u, &never);
+    }
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, p.tmem_cols);
+    }
+}
+
+struct LoraDownParams {
+    const uint16_t *w;      // wd_blk
+    const uint16_t *ad;     // ad_blk: A_down as one more hidden tile of kMaxLoraRank rows
+    const float *h;         // [B][ldh] fp32
+    int ldh, B, H, N;
+    int NT, halves;
+    int KBn, dt, units;     // units = (dt + 1) KBn: (hidden tile or A_down, neuron block) pairs
+    int r;
+    float *y;               // [B][H], added to
+    float *wsum;            // [B][kLoraWRow], added to
+    int *ctl;
+    int stages, ring_bytes;
+    uint32_t tmem_cols;
+};
+
+// CTA c takes units [c U / G, (c + 1) U / G) in order for the tokens of tile blockIdx.y; consecutive
+// units of one output tile are summed in registers and added into y (or w).
+__global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const LoraDownParams p)
+{
+    constexpr int kEpi0 = 2 + kConvThreads / 32;
+    constexpr int kA = BM * kTileBytes;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *ring = align1024(smem_raw);
+    uint8_t *parts = ring + p.ring_bytes;
+    uint64_t *full = reinterpret_cast<uint64_t *>(parts + kPartStages * kParts * p.NT * kTileBytes);
+    uint64_t *empty = full + kMaxStages;
+    uint64_t *pfull = empty + kMaxStages;
+    uint64_t *pempty = pfull + kPartStages;
+    uint64_t *acc_full = pempty + kPartStages;   // [2]
+    uint64_t *acc_empty = acc_full + 2;          // [2]
+    uint64_t *mma_done = acc_empty + 2;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
+    __shared__ int abort_flag, issued_s, consumed_s;
+    __shared__ float tr[kLoraEpiThreads / 32][16][33];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int NT = p.NT, S = p.stages, KBn = p.KBn, halves = p.halves, NX = kParts * NT;
+    const int m0 = (int)blockIdx.y * NT;
+    const int u0 = (int)((long long)blockIdx.x * p.units / gridDim.x);
+    const int u1 = (int)((long long)(blockIdx.x + 1) * p.units / gridDim.x);
+    const int nu = u1 - u0;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int s = 0; s < kPartStages; ++s) {
+            mbar_init(&pfull[s], kConvThreads);
+            mbar_init(&pempty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], kLoraEpiThreads);
+        }
+        mbar_init(mma_done, 1);
+        abort_flag = 0;
+        issued_s = 0;
+        consumed_s = 0;
+        mbar_init_fence();
+    }
+    if (warp == 1) tmem_alloc(tmem_slot, p.tmem_cols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    grid_launch_dependents();
+
+    if (warp == 0 && lane == 0) {
+        // nothing but weights is copied, so the whole stream runs ahead of the preceding kernel's end
+        const uint64_t once = l2_policy_evict_first();
+        int i = 0;
+        for (int s = 0, ph = 0; i < nu; ++i) {
+            if (!mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
+            const int u = u0 + i, d = u / KBn;
+            const bool ad = d == p.dt;
+            const uint32_t bytes = (uint32_t)((ad ? kMaxLoraRank : BM) * kTileBytes);
+            const uint16_t *src = ad ? p.ad + (size_t)(u - d * KBn) * kMaxLoraRank * BK : p.w + (size_t)u * BM * BK;
+            mbar_arrive_expect_tx(&full[s], bytes);
+            if (gridDim.y == 1) bulk_load(ring + (size_t)s * kA, src, bytes, &full[s], once);
+            else bulk_load_shared(ring + (size_t)s * kA, src, bytes, &full[s]);
+            if (++s == S) { s = 0; ph ^= 1; }
+        }
+        issued_s = i;
+    } else if (warp == 1 && lane == 0) {
+        const uint32_t idesc = instr_desc(BM, NX);
+        const int per = 4 / halves;
+        int i = 0;
+        for (int s = 0, ph = 0; i < nu; ++i) {
+            const int buf = i & 1, ps = i % kPartStages;
+            if (!mbar_wait(&acc_empty[buf], (uint32_t)((i >> 1) & 1) ^ 1u, &abort_flag) ||
+                !mbar_wait(&full[s], (uint32_t)ph, &abort_flag) ||
+                !mbar_wait(&pfull[ps], (uint32_t)((i / kPartStages) & 1), &abort_flag)) {
+                set_timeout(p.ctl, &abort_flag);
+                break;
+            }
+            tc_fence_after();
+            const uint32_t st = smem_addr(ring + (size_t)s * kA);
+            const uint32_t hs = smem_addr(parts + (size_t)ps * kParts * NT * kTileBytes);
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk)
+                mma_bf16(tmem + (uint32_t)((buf * halves + kk / per) * NX), smem_desc(st + kk * 32),
+                         smem_desc(hs + kk * 32), idesc, kk % per ? 1u : 0u);
+            mma_commit(&empty[s]);
+            mma_commit(&pempty[ps]);
+            mma_commit(&acc_full[buf]);
+            if (++s == S) { s = 0; ph ^= 1; }
+        }
+        consumed_s = i;
+        mma_commit(mma_done);
+    } else if (warp >= 2 && warp < kEpi0) {
+        grid_dependency_wait();   // h is written by the preceding gate/up kernel
+        auto load = [&](int r, int c, int step, float4 &lo, float4 &hi) {
+            const int m = m0 + r, k = ((u0 + step) % KBn) * BK + c * 8;
+            if (m >= p.B || k >= p.N) return;
+            const float *src = p.h + (size_t)m * p.ldh + k;   // (ldh is a multiple of 8)
+            if (k + 8 <= p.N) {
+                lo = reinterpret_cast<const float4 *>(src)[0];
+                hi = reinterpret_cast<const float4 *>(src)[1];
+            } else {   // columns past N hold anything
+                const int left = p.N - k;
+                lo.x = src[0];
+                if (left > 1) lo.y = src[1];
+                if (left > 2) lo.z = src[2];
+                if (left > 3) lo.w = src[3];
+                if (left > 4) hi.x = src[4];
+                if (left > 5) hi.y = src[5];
+                if (left > 6) hi.z = src[6];
+            }
+        };
+        if (!cut_tiles<kLoraTok>(parts, NT, nu, pfull, pempty, &abort_flag, load)) set_timeout(p.ctl, &abort_flag);
+    } else if (warp >= kEpi0) {
+        grid_dependency_wait();   // y and w are cleared by the preceding kernel
+        const int quad = warp & 3, grp = (warp - kEpi0) >> 2;
+        const int c0 = 16 * grp;
+        const bool busy = c0 < NT;
+        const uint32_t lane0 = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0;
+        float(*T)[33] = tr[warp - kEpi0];
+        const int te = lane >> 1, r0 = (lane & 1) * 16;   // this lane's token in the block, first row
+        float acc[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[e] = 0.f;
+        for (int i = 0; i < nu; ++i) {
+            const int buf = i & 1, u = u0 + i, d = u / KBn;
+            if (!mbar_wait(&acc_full[buf], (uint32_t)((i >> 1) & 1), &abort_flag)) {
+                set_timeout(p.ctl, &abort_flag);
+                break;
+            }
+            tc_fence_after();
+            if (busy) {
+                float sum[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) sum[e] = 0.f;
+                for (int f = 0; f < halves; ++f) {
+                    float v[kParts][16];
+#pragma unroll
+                    for (int k = 0; k < kParts; ++k)
+                        tmem_ld16(lane0 + (uint32_t)((buf * halves + f) * NX + k * NT), v[k]);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) sum[e] += (v[2][e] + v[1][e]) + v[0][e];
+                }
+#pragma unroll
+                for (int e = 0; e < 16; ++e) acc[e] += sum[e];
+            }
+            tc_fence_before();
+            mbar_arrive(&acc_empty[buf]);
+            if (i + 1 < nu && (u + 1) / KBn == d) continue;
+            // the last unit of this output tile: 32 rows x 16 tokens through shared memory, so that each
+            // lane adds four vectors of four hidden units of one token
+            if (busy && d < p.dt) {
+#pragma unroll
+                for (int e = 0; e < 16; ++e) T[e][lane] = acc[e];
+                __syncwarp();
+                const int j = m0 + c0 + te, h0 = d * BM + 32 * quad + r0;
+                if (j < p.B && c0 + te < NT) {
+                    float *dst = p.y + (size_t)j * p.H + h0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)   // H is a multiple of 8: a vector is in range or not at all
+                        if (h0 + 4 * k < p.H)
+                            red_add_v4(dst + 4 * k, T[te][r0 + 4 * k], T[te][r0 + 4 * k + 1], T[te][r0 + 4 * k + 2],
+                                       T[te][r0 + 4 * k + 3]);
+                }
+                __syncwarp();
+            } else if (busy && quad == 0 && lane < p.r) {   // row q of A_down's tile
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+                    if (m0 + c0 + e < p.B && c0 + e < NT) atomicAdd(p.wsum + (size_t)(m0 + c0 + e) * kLoraWRow + lane, acc[e]);
+            }
+#pragma unroll
+            for (int e = 0; e < 16; ++e) acc[e] = 0.f;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int never = 0;
+        if (abort_flag)
+            for (int k = consumed_s; k < issued_s; ++k) mbar_wait(&full[k % S], (uint32_t)((k / S) & 1), &never);
+        mbar_wait(mma_done, 0u, &never);
+    }
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, p.tmem_cols);
+    }
+}
+
+// y[b] += scale w[b] B_down.  Grid: (blocks of 8 x 128 hidden units, B).
+__global__ void __launch_bounds__(128) lora_out_kernel(const float *__restrict__ wsum, const uint16_t *__restrict__ bd,
+                                                       int H, int r, float scale, float *__restrict__ y)
+{
+    const int b = blockIdx.y, h = (blockIdx.x * 128 + threadIdx.x) * 8;
+    grid_dependency_wait();
+    grid_launch_dependents();
+    if (h >= H) return;
+    float acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+#pragma unroll 8
+    for (int q = 0; q < r; ++q) {
+        float w[8];
+        unpack8(*reinterpret_cast<const uint4 *>(bd + (size_t)q * H + h), w);
+        const float v = scale * wsum[(size_t)b * kLoraWRow + q];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = fmaf(v, w[e], acc[e]);
+    }
+    float4 *dst = reinterpret_cast<float4 *>(y + (size_t)b * H + h);
+    const float4 p = dst[0], q = dst[1];
+    dst[0] = make_float4(p.x + acc[0], p.y + acc[1], p.z + acc[2], p.w + acc[3]);
+    dst[1] = make_float4(q.x + acc[4], q.y + acc[5], q.z + acc[6], q.w + acc[7]);
+}
+
+// A_down [N][r] as tiles [kb][q][64] of kMaxLoraRank rows (row q, neuron kb 64 + c), 128-byte swizzled;
+// rows past r and neurons past N are zero.
+__global__ void pack_ad_kernel(const uint16_t *__restrict__ Ad, int N, int r, int KBn, uint16_t *__restrict__ dst)
+{
+    const size_t total = (size_t)KBn * kMaxLoraRank * BK;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+        const int c = (int)(i % BK), q = (int)(i / BK % kMaxLoraRank), kb = (int)(i / BK / kMaxLoraRank);
+        const int n = kb * BK + c;
+        dst[(i / BK) * BK + (size_t)(((c / 8) ^ (q & 7)) * 8) + c % 8] = (n < N && q < r) ? Ad[(size_t)n * r + q] : (uint16_t)0;
+    }
+}
+
+template <bool F32>
+cudaError_t launch_lora_gate_up(LoraGuParams &p, const sats_layer *layer, const void *x, int mt, cudaStream_t stream)
+{
+    p.w_bytes = 2 * p.R * kTileBytes;
+    p.stage_bytes = p.w_bytes + (F32 ? 0 : p.NT * kTileBytes);
+    const int parts = F32 ? kPartStages * kParts * p.NT * kTileBytes : 0;
+    // the up tile's MMA reads 128 rows from row R (rows R..127 of D are not used)
+    const int over = (p.R + BM) * kTileBytes - p.stage_bytes;
+    const int slack = over > 0 ? ((over + 1023) & ~1023) : 0;
+    p.stages = stages_for(p.stage_bytes, kSmemBudget - parts - slack);
+    p.ring_bytes = p.stages * p.stage_bytes + slack;
+    p.halves = F32 && p.NT > 16 ? 1 : 2;
+    p.tmem_cols = tmem_cols_for(2 * p.halves * 2 * (F32 ? kParts : 1) * p.NT);
+    CUtensorMap mX{};
+    if (!F32 && !make_map(&mX, x, (uint64_t)p.B, (uint64_t)p.H, (uint64_t)p.H * 2, (uint32_t)p.NT))
+        return cudaErrorInvalidValue;
+    static std::atomic<int> cfg[64];
+    const size_t smem = smem_for(1, p.ring_bytes + parts);
+    const cudaError_t e = set_smem(lora_gate_up_kernel<F32>, smem, cfg);
+    if (e != cudaSuccess) return e;
+    return launch_pdl_cfg(lora_gate_up_kernel<F32>, dim3(mt, layer->tc_T), kLoraGuThreads<F32>, smem, stream, mX, p);
+}
+
 }  // namespace
 }  // namespace tc
 
@@ -359,6 +927,108 @@ cudaError_t launch_gate_act(const sats_layer *layer, const uint16_t *x, int B, f
 cudaError_t launch_gate_act_f32(const sats_layer *layer, const float *x, int B, float *a, cudaStream_t stream)
 {
     return tc::launch_gate_precise<true>(layer, x, B, a, stream);
+}
+
+// Scratch of a LoRA batch inside the tensor-core region of a workspace: z and w where the other
+// paths keep bf16 copies of x (4 H bytes per token), h in fp32 where they keep its two parts.
+static int lora_slices(int H) { return H / 128 < 1 ? 1 : (H / 128 > 8 ? 8 : H / 128); }
+
+bool lora_tc_ok(int H, int B)
+{
+    const int need = lora_slices(H) * tc::kLoraZRow * 4 + tc::kLoraWRow * 4;
+    return use_tc_path(H, B) && B <= 65535 && need <= 4 * H;   // (B is a grid dimension)
+}
+
+cudaError_t lora_pack_tc(const sats_layer *layer, const uint16_t *Ad, sats_lora *l, cudaStream_t stream)
+{
+    const cudaError_t e = cudaMalloc(&l->ad_blk, (size_t)layer->tc_kbn * kMaxLoraRank * tc::BK * 2);
+    if (e != cudaSuccess) return e;
+    tc::pack_ad_kernel<<<256, 256, 0, stream>>>(Ad, l->N, l->r, layer->tc_kbn, l->ad_blk);
+    return cudaGetLastError();
+}
+
+cudaError_t run_lora_tc(const sats_layer *layer, const sats_lora *lora, bool x_f32, const void *x, int B, float t_l,
+                        float *y, int32_t *active_idx, int32_t *active_cnt, void *tc_ws, int *ctl, cudaStream_t stream)
+{
+    using namespace tc;
+    const int H = layer->H, N = layer->N;
+    const TcRegions W = tc_regions(H, N, B);
+    char *base = static_cast<char *>(tc_ws);
+    const int slices = lora_slices(H);
+    float *z = reinterpret_cast<float *>(base + W.x);
+    float *wsum = z + (size_t)B * slices * kLoraZRow;
+    float *h = reinterpret_cast<float *>(base + W.h);
+    uint8_t *keep = reinterpret_cast<uint8_t *>(base + W.keep);
+    auto failed = [](cudaError_t e, const char *where) {
+        cuda_fail(e, where);
+        return e;
+    };
+    cudaError_t e =
+        x_f32 ? launch_pdl_threads(lora_z_kernel<float>, dim3(slices, B), 256, stream, static_cast<const float *>(x), H,
+                                   static_cast<const uint16_t *>(lora->agu), lora->r, z)
+              : launch_pdl_threads(lora_z_kernel<uint16_t>, dim3(slices, B), 256, stream,
+                                   static_cast<const uint16_t *>(x), H, static_cast<const uint16_t *>(lora->agu),
+                                   lora->r, z);
+    if (e != cudaSuccess) return failed(e, "adapter input kernel launch");
+
+    const int mt = (B + kLoraTok - 1) / kLoraTok;
+    LoraGuParams gp{};
+    gp.w = layer->gu_blk;
+    gp.x = x_f32 ? static_cast<const float *>(x) : nullptr;
+    gp.B = B;
+    gp.H = H;
+    gp.N = N;
+    gp.R = layer->tc_R;
+    gp.KBh = layer->tc_kbh;
+    gp.NT = ((B + mt - 1) / mt + 15) & ~15;
+    gp.t_l = t_l;
+    gp.scale = lora->scale;
+    gp.blk = lora->blk;
+    gp.r = lora->r;
+    gp.z = z;
+    gp.slices = slices;
+    gp.h = h;
+    gp.ldh = layer->ldn;
+    gp.keep = active_idx ? keep : nullptr;
+    gp.keep_stride = (N + 15) & ~15;
+    gp.y = y;
+    gp.wsum = wsum;
+    gp.ctl = ctl;
+    e = x_f32 ? launch_lora_gate_up<true>(gp, layer, x, mt, stream) : launch_lora_gate_up<false>(gp, layer, x, mt, stream);
+    if (e != cudaSuccess) return failed(e, "adapted gate/up kernel launch");
+
+    LoraDownParams dp{};
+    dp.w = layer->wd_blk;
+    dp.ad = lora->ad_blk;
+    dp.h = h;
+    dp.ldh = layer->ldn;
+    dp.B = B;
+    dp.H = H;
+    dp.N = N;
+    dp.NT = gp.NT;
+    dp.halves = 2;
+    dp.KBn = layer->tc_kbn;
+    dp.dt = layer->tc_dt;
+    dp.units = (dp.dt + 1) * dp.KBn;
+    dp.r = lora->r;
+    dp.y = y;
+    dp.wsum = wsum;
+    dp.ctl = ctl;
+    const int parts = kPartStages * kParts * dp.NT * kTileBytes;
+    dp.stages = stages_for(BM * kTileBytes, kSmemBudget - parts);
+    dp.ring_bytes = dp.stages * BM * kTileBytes;
+    dp.tmem_cols = tmem_cols_for(2 * dp.halves * kParts * dp.NT);
+    static std::atomic<int> cfg[64];
+    const size_t smem = smem_for(1, dp.ring_bytes + parts);
+    if ((e = set_smem(lora_down_kernel, smem, cfg)) != cudaSuccess) return failed(e, "shared-memory attribute");
+    const int sms = sm_count();
+    e = launch_pdl_cfg(lora_down_kernel, dim3(dp.units < sms ? dp.units : sms, mt), kLoraDownThreads, smem, stream, dp);
+    if (e != cudaSuccess) return failed(e, "adapted down kernel launch");
+    e = launch_pdl_threads(lora_out_kernel, dim3((H + 1023) / 1024, B), 128, stream, static_cast<const float *>(wsum),
+                           static_cast<const uint16_t *>(lora->bd), H, lora->r, lora->scale, y);
+    if (e != cudaSuccess) return failed(e, "adapter output kernel launch");
+    if (active_idx) return launch_keep_lists(keep, gp.keep_stride, B, N, active_idx, active_cnt, nullptr, stream);
+    return cudaSuccess;
 }
 
 }  // namespace sats

@@ -1179,6 +1179,21 @@ bool use_tc_path(int H, int B) { return B > fused_tokens_per_pass(H); }
 
 size_t tc_workspace_bytes(int H, int N, int B) { return tc_layout(H, N, B).total; }
 
+TcRegions tc_regions(int H, int N, int B)
+{
+    const TcLayout L = tc_layout(H, N, B);   // (xhi and xlo, hact and hact_lo are neighbours)
+    return {L.xhi, L.hact, L.keep};
+}
+
+cudaError_t launch_keep_lists(const uint8_t *keep, int stride, int B, int N, int32_t *active_idx, int32_t *active_cnt,
+                              const int32_t *perm, cudaStream_t stream)
+{
+    const cudaError_t e = tc::launch_pdl_threads(tc::keep_list_kernel, dim3(B), 512, stream, keep, stride, N, active_idx,
+                                                 active_cnt, perm);
+    if (e != cudaSuccess) cuda_fail(e, "kept-list kernel launch");
+    return e;
+}
+
 namespace {
 using namespace tc;
 
@@ -1527,11 +1542,7 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
         }
         if (e != cudaSuccess) return e;
     }
-    if (active_idx) {
-        e = launch_pdl_threads(keep_list_kernel, dim3(B), 512, stream, static_cast<const uint8_t *>(keep), kstride, N,
-                               active_idx, active_cnt, perm);
-        if (e != cudaSuccess) return fail(e, "kept-list kernel launch");
-    }
+    if (active_idx) return launch_keep_lists(keep, kstride, B, N, active_idx, active_cnt, perm, stream);
     return cudaSuccess;
 }
 

@@ -34,6 +34,7 @@ struct sats_lora {
     uint16_t *blk = nullptr;      // [ceil(N / 8)][8][3 r]: neuron j's B_gate[:, j], B_up[:, j], A_down[j, :]
     uint16_t *agu = nullptr;      // [H][2 r]: A_gate[h, :], A_up[h, :]
     uint16_t *bd = nullptr;       // [r][H]: B_down
+    uint16_t *ad_blk = nullptr;   // [ceil(N / 64)][32][64]: A_down as a weight tile of the down projection (batches)
 };
 
 namespace sats {
@@ -142,6 +143,20 @@ cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void 
                            const uint16_t **hact_lo, float *a_out, int *ctl, cudaStream_t stream);
 cudaError_t run_tc_down(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
                         int *ctl, cudaStream_t stream);
+// Byte offsets of the tensor-core region's parts that other paths reuse: the bf16 copies of x
+// (4 H B bytes), h (4 ldn B bytes), the keep bytes (N rounded up to 16, per token).
+struct TcRegions {
+    size_t x, h, keep;
+};
+TcRegions tc_regions(int H, int N, int B);
+cudaError_t launch_keep_lists(const uint8_t *keep, int stride, int B, int N, int32_t *active_idx, int32_t *active_cnt,
+                              const int32_t *perm, cudaStream_t stream);
+// gemm_f32.cu: LoRA batches beyond one pass of the fused kernel.  lora_pack_tc allocates and fills
+// ad_blk; lora_tc_ok says whether a batch's scratch fits its workspace (hidden sizes of 96 and more).
+bool lora_tc_ok(int H, int B);
+cudaError_t lora_pack_tc(const sats_layer *layer, const uint16_t *Ad, sats_lora *l, cudaStream_t stream);
+cudaError_t run_lora_tc(const sats_layer *layer, const sats_lora *lora, bool x_f32, const void *x, int B, float t_l,
+                        float *y, int32_t *active_idx, int32_t *active_cnt, void *tc_ws, int *ctl, cudaStream_t stream);
 cudaError_t launch_wait_timeout(int *ctl, cudaStream_t stream);
 cudaError_t launch_route(const int32_t *ids, int B, const uint8_t *lut, int V, int32_t *perm,
                          int32_t *n_dense, uint8_t *flags, int32_t *status, cudaStream_t stream);

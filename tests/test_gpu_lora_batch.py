@@ -1,0 +1,61 @@
+"""LoRA batches beyond one pass of the fused kernel, at token counts around the tile edges, neuron
+counts that do not fill a tile or a K block, the smallest hidden size of the path and every rank,
+against the oracle element by element.  The bound is fp32 arithmetic's (both matrix products are
+summed in segments of 32 rounded once each, a few units of 2^-24): 1e-6 relative, which a plain
+accumulator chain on the tensor cores (1e-5) or h rounded to two bf16 parts (4e-6) does not meet."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_08991_gb300 import inputs
+from tests import _parity as P
+from tests.test_gpu_lora import _call, _setup, _threshold
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sats():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2607_08991_gb300 import sats as s
+    return s
+
+
+@pytest.mark.parametrize("H,N,B,r,f32", [
+    (96, 5, 3, 8, False),        # the smallest hidden size, one ragged tile
+    (96, 200, 4, 32, True),
+    (512, 1408, 16, 16, True),   # a full tile of 16 tokens
+    (1032, 777, 17, 24, False),  # two token blocks, a hidden size that ends inside a K block
+    (1032, 777, 32, 24, True),   # a full tile of 32 tokens
+    (4096, 1009, 33, 16, False), # two token tiles
+    (4096, 1009, 40, 16, True),
+    (8192, 130, 2, 8, True),     # hidden 8192: one token per fused pass, so two take this path
+    (64, 100, 5, 8, False),      # below the path: passes of the fused kernel
+])
+def test_batches_match_oracle(sats, oracle, H, N, B, r, f32):
+    scale = 0.75
+    w, lo, layer, lora = _setup(sats, H, N, r, scale, seed=11)
+    t = _threshold(oracle, w, H, 0.6)
+    ws = sats.Workspace(H, N, B)
+    if f32:
+        xf = inputs.activations_f32(B, H, seed=inputs.SEED_X + 31)
+        x64, xdev = xf.astype(np.float64), P.dev(xf)
+    else:
+        xb = inputs.activations_bf16(B, H, seed=inputs.SEED_X + 31)
+        x64, xdev = oracle.bf16_to_f64(xb), P.dev_u16(xb)
+    for _ in range(2):   # a second call on the same workspace
+        y, keep = _call(sats, layer, lora, xdev, t, B, H, N, ws)
+        y_ref, a_ref, keep_ref, _ = oracle.sparse_mlp_lora(x64, w.Wg, w.Wu, w.Wd, lo, scale, t, keep_hint=keep,
+                                                           band_rel=P.BAND_REL)
+        P.assert_keep_match(keep, keep_ref, a_ref, t)
+        assert np.linalg.norm(y - y_ref) <= 1e-6 * np.linalg.norm(y_ref)
+    # without the lists, on a workspace that other calls have used
+    y2 = torch.full((B, H), float("nan"), device="cuda")
+    if not f32:
+        sats.sparse_mlp(layer, xdev, t, y2, ws)
+    sats.sparse_mlp_lora(layer, lora, xdev, t, y2, ws)
+    assert sats.get_error(ws) == sats.OK
+    assert np.linalg.norm(y2.cpu().numpy() - y_ref) <= 1e-6 * np.linalg.norm(y_ref)
+    lora.close()
+    layer.close()
