@@ -43,31 +43,58 @@ struct PreciseGateParams {
     uint32_t tmem_cols;    // four accumulators of NT columns
 };
 
-// x = the sum of three bf16 values, cut off the top 8 significant bits at a time.  (x - top is
-// exact; the comparison keeps an infinity from becoming inf - inf.)
-__device__ __forceinline__ float cut_bf16(float &x)
-{
-    const float top = __uint_as_float(__float_as_uint(x) & 0xffff0000u);
-    x = top == x ? 0.f : x - top;
-    return top;
-}
+__device__ __forceinline__ float bf16_top(float x) { return __uint_as_float(__float_as_uint(x) & 0xffff0000u); }
 
 __device__ __forceinline__ uint32_t pack_tops(float lo, float hi)
 {
     return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 
-// Eight fp32 values -> one 16-byte chunk of each part.
+// Eight fp32 values -> one 16-byte chunk of each part: the top 8 significant bits, the next 8, the
+// last 8 (each difference x - top is exact, so the parts' sum is x).
 __device__ __forceinline__ void cut8(const float4 &p, const float4 &q, uint4 (&part)[kParts])
 {
     float v[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+    uint32_t out[kParts][4];
+    uint32_t most = 0u;
 #pragma unroll
-    for (int i = 0; i < kParts; ++i) {
-        float t[8];
+    for (int e = 0; e < 8; ++e) most = max(most, __float_as_uint(v[e]) & 0x7fffffffu);
+    if (most < 0x7f800000u) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) t[e] = cut_bf16(v[e]);
-        part[i] = make_uint4(pack_tops(t[0], t[1]), pack_tops(t[2], t[3]), pack_tops(t[4], t[5]), pack_tops(t[6], t[7]));
+        for (int e = 0; e < 4; ++e) {
+            const f32x2 minus1 = pack2(-1.f, -1.f);
+            f32x2 r = pack2(v[2 * e], v[2 * e + 1]);
+#pragma unroll
+            for (int i = 0; i < kParts; ++i) {
+                const float2 f = unpack2(r);
+                out[i][e] = pack_tops(f.x, f.y);
+                if (i + 1 < kParts) r = ffma2(pack2(bf16_top(f.x), bf16_top(f.y)), minus1, r);
+            }
+        }
+    } else {   // infinities keep out of the differences (inf - inf), NaN stays NaN in every part
+#pragma unroll
+        for (int i = 0; i < kParts; ++i) {
+            float t[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                t[e] = bf16_top(v[e]);
+                v[e] = t[e] == v[e] ? 0.f : v[e] - t[e];
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) out[i][e] = pack_tops(t[2 * e], t[2 * e + 1]);
+        }
     }
+#pragma unroll
+    for (int i = 0; i < kParts; ++i) part[i] = make_uint4(out[i][0], out[i][1], out[i][2], out[i][3]);
+}
+
+// One arrival per warp once all its lanes have read their TMEM columns: hundreds of threads
+// arriving one by one on a barrier cost more than a K block's MMAs.
+__device__ __forceinline__ void warp_arrive_tmem(uint64_t *bar, int lane)
+{
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
 }
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -81,34 +108,45 @@ __device__ __forceinline__ bool cut_tiles(uint8_t *parts, int NT, int steps, uin
                                           volatile int *abort, Load load)
 {
     constexpr int kUnits = (TOK * 8 + kConvThreads - 1) / kConvThreads;
+    // steps whose units are in flight: a load takes as long as several small tiles' MMAs, and the
+    // registers of a large tile hold one step
+    constexpr int kAhead = TOK <= 32 ? 4 : TOK <= 64 ? 2 : 1;
     const int ct = threadIdx.x - 64, nu = NT * 8;
-    float4 lo[kUnits], hi[kUnits];
-    auto fetch = [&](int i, int step) {
+    float4 lo[kAhead][kUnits], hi[kAhead][kUnits];
+    auto fetch = [&](int a, int i, int step) {
         const int u = ct + kConvThreads * i;
-        lo[i] = hi[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (u < nu) load(u >> 3, u & 7, step, lo[i], hi[i]);
+        lo[a][i] = hi[a][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (u < nu && step < steps) load(u >> 3, u & 7, step, lo[a][i], hi[a][i]);
     };
 #pragma unroll
-    for (int i = 0; i < kUnits; ++i)
-        if (steps > 0) fetch(i, 0);
-    for (int step = 0; step < steps; ++step) {
-        const int ps = step % kPartStages;
-        if (!mbar_wait(&pempty[ps], (uint32_t)((step / kPartStages) & 1) ^ 1u, abort)) return false;
-        uint8_t *dst = parts + (size_t)ps * kParts * NT * kTileBytes;
+    for (int a = 0; a < kAhead; ++a)
 #pragma unroll
-        for (int i = 0; i < kUnits; ++i) {
-            const int u = ct + kConvThreads * i, r = u >> 3, c = u & 7;
-            uint4 part[kParts];
-            cut8(lo[i], hi[i], part);
-            if (step + 1 < steps) fetch(i, step + 1);
-            if (u < nu) {
+        for (int i = 0; i < kUnits; ++i) fetch(a, i, a);
+    for (int base = 0; base < steps; base += kAhead) {
 #pragma unroll
-                for (int q = 0; q < kParts; ++q)
-                    *reinterpret_cast<uint4 *>(dst + (size_t)(q * NT + r) * kTileBytes + ((c ^ (r & 7)) << 4)) = part[q];
+        for (int a = 0; a < kAhead; ++a) {
+            const int step = base + a;
+            if (step >= steps) break;
+            const int ps = step % kPartStages;
+            if (!mbar_wait(&pempty[ps], (uint32_t)((step / kPartStages) & 1) ^ 1u, abort)) return false;
+            uint8_t *dst = parts + (size_t)ps * kParts * NT * kTileBytes;
+#pragma unroll
+            for (int i = 0; i < kUnits; ++i) {
+                const int u = ct + kConvThreads * i, r = u >> 3, c = u & 7;
+                uint4 part[kParts];
+                cut8(lo[a][i], hi[a][i], part);
+                fetch(a, i, step + kAhead);
+                if (u < nu) {
+#pragma unroll
+                    for (int q = 0; q < kParts; ++q)
+                        *reinterpret_cast<uint4 *>(dst + (size_t)(q * NT + r) * kTileBytes + ((c ^ (r & 7)) << 4)) =
+                            part[q];
+                }
             }
+            fence_async_smem();   // the MMAs read the tile through the async proxy
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0) mbar_arrive(&pfull[ps]);
         }
-        fence_async_smem();   // the MMAs read the tile through the async proxy
-        mbar_arrive(&pfull[ps]);
     }
     return true;
 }
@@ -116,13 +154,15 @@ __device__ __forceinline__ bool cut_tiles(uint8_t *parts, int NT, int steps, uin
 // a = SiLU(x W_gate) for one tile of NT tokens and R neurons per CTA (neurons are the MMA's
 // M, tokens its N).  Grid: token tiles x neuron tiles, the token tiles of one neuron tile
 // next to each other, so that its weights come from L2 for all but the first of them.
-template <bool F32>
+// TOK: the most tokens of a tile (64 leaves registers for a second level of sums and for loads two
+// steps ahead with fp32 activations).
+template <bool F32, int TOK>
 __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     gate_precise_kernel(const __grid_constant__ CUtensorMap tmX, const PreciseGateParams p)
 {
     constexpr int kEpi0 = 2 + (F32 ? kConvThreads / 32 : 0);        // first epilogue warp
     constexpr int G = (kPreciseThreads<F32> / 32 - kEpi0) / 4;           // epilogue groups of four warps
-    constexpr int kBlocks = (kPreciseTok / 16 + G - 1) / G;         // 16-token blocks per thread
+    constexpr int kBlocks = (TOK / 16 + G - 1) / G;         // 16-token blocks per thread
     constexpr int kXParts = F32 ? kParts : 1;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *ring = align1024(smem_raw);
@@ -147,12 +187,12 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
             mbar_init(&empty[s], 1);
         }
         for (int s = 0; s < kPartStages; ++s) {
-            mbar_init(&pfull[s], kConvThreads);
+            mbar_init(&pfull[s], kConvThreads / 32);
             mbar_init(&pempty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 128 * G);
+            mbar_init(&acc_empty[b], 4 * G);
         }
         mbar_init(mma_done, 1);
         abort_flag = 0;
@@ -234,20 +274,21 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                 hi = src[1];
             }
         };
-        if (!cut_tiles<kPreciseTok>(parts, NT, KBh, pfull, pempty, &abort_flag, load)) abort_flag = 1;
+        if (!cut_tiles<TOK>(parts, NT, KBh, pfull, pempty, &abort_flag, load)) abort_flag = 1;
     } else if (warp >= kEpi0) {
         const int quad = warp & 3, grp = (warp - kEpi0) >> 2;
         const uint32_t lane0 = tmem + ((uint32_t)(32 * quad) << 16);
         const int n = t * R + 32 * quad + lane;
         // acc: totals; sub: the sums of up to kSubBlocks K blocks, added to the totals together, so that
-        // a total takes few roundings at its full size (bf16: 64 more registers than fp32's have)
-        float acc[kBlocks][16], sub[F32 ? 1 : kBlocks][16];
+        // a total takes few roundings at its full size (where the registers hold both)
+        constexpr bool kTwoLevel = kBlocks <= 2;
+        float acc[kBlocks][16], sub[kTwoLevel ? kBlocks : 1][16];
 #pragma unroll
         for (int k = 0; k < kBlocks; ++k)
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
                 acc[k][e] = 0.f;
-                if (!F32) sub[F32 ? 0 : k][e] = 0.f;
+                if (kTwoLevel) sub[kTwoLevel ? k : 0][e] = 0.f;
             }
         bool ok = true;
         for (int kb = 0; kb < KBh; ++kb) {
@@ -267,21 +308,20 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                         tmem_ld_wait();
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
-                            if (F32) acc[k][o + e] += v0[e] + v1[e];
-                            else sub[F32 ? 0 : k][o + e] += v0[e] + v1[e];
+                            if (kTwoLevel) sub[kTwoLevel ? k : 0][o + e] += v0[e] + v1[e];
+                            else acc[k][o + e] += v0[e] + v1[e];
                         }
                     }
                 }
             }
-            tc_fence_before();
-            mbar_arrive(&acc_empty[buf]);
-            if (!F32 && (kb % kSubBlocks == kSubBlocks - 1 || kb + 1 == KBh)) {
+            warp_arrive_tmem(&acc_empty[buf], lane);
+            if (kTwoLevel && (kb % kSubBlocks == kSubBlocks - 1 || kb + 1 == KBh)) {
 #pragma unroll
                 for (int k = 0; k < kBlocks; ++k)
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
-                        acc[k][e] += sub[F32 ? 0 : k][e];
-                        sub[F32 ? 0 : k][e] = 0.f;
+                        acc[k][e] += sub[kTwoLevel ? k : 0][e];
+                        sub[kTwoLevel ? k : 0][e] = 0.f;
                     }
             }
         }
@@ -315,7 +355,7 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     }
 }
 
-template <bool F32>
+template <bool F32, int TOK>
 cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, float *a, cudaStream_t stream)
 {
     PreciseGateParams p{};
@@ -343,9 +383,9 @@ cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, f
         return cudaErrorInvalidValue;
     static std::atomic<int> cfg[64];
     const size_t smem = smem_for(1, p.ring_bytes + parts);
-    const cudaError_t e = set_smem(gate_precise_kernel<F32>, smem, cfg);
+    const cudaError_t e = set_smem(gate_precise_kernel<F32, TOK>, smem, cfg);
     if (e != cudaSuccess) return e;
-    return launch_pdl_cfg(gate_precise_kernel<F32>, dim3(mt, layer->tc_T), kPreciseThreads<F32>, smem, stream, mX, p);
+    return launch_pdl_cfg(gate_precise_kernel<F32, TOK>, dim3(mt, layer->tc_T), kPreciseThreads<F32>, smem, stream, mX, p);
 }
 
 // ---------------------------------------------------------------------- LoRA batches
@@ -457,12 +497,12 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
             mbar_init(&empty[s], 1);
         }
         for (int s = 0; s < kPartStages; ++s) {
-            mbar_init(&pfull[s], kConvThreads);
+            mbar_init(&pfull[s], kConvThreads / 32);
             mbar_init(&pempty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], kLoraEpiThreads);
+            mbar_init(&acc_empty[b], kLoraEpiThreads / 32);
         }
         mbar_init(mma_done, 1);
         abort_flag = 0;
@@ -587,8 +627,7 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
                     for (int e = 0; e < 16; ++e) acc[q][e] += sum[e];
                 }
             }
-            tc_fence_before();
-            mbar_arrive(&acc_empty[buf]);
+            warp_arrive_tmem(&acc_empty[buf], lane);
         }
         grid_dependency_wait();   // z, and y, w, h and the keep bytes may still be in use by the preceding kernels
         const int ctas = (int)(gridDim.x * gridDim.y), cta = (int)(blockIdx.y * gridDim.x + blockIdx.x);
@@ -697,12 +736,12 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
             mbar_init(&empty[s], 1);
         }
         for (int s = 0; s < kPartStages; ++s) {
-            mbar_init(&pfull[s], kConvThreads);
+            mbar_init(&pfull[s], kConvThreads / 32);
             mbar_init(&pempty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], kLoraEpiThreads);
+            mbar_init(&acc_empty[b], kLoraEpiThreads / 32);
         }
         mbar_init(mma_done, 1);
         abort_flag = 0;
@@ -814,8 +853,7 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
 #pragma unroll
                 for (int e = 0; e < 16; ++e) acc[e] += sum[e];
             }
-            tc_fence_before();
-            mbar_arrive(&acc_empty[buf]);
+            warp_arrive_tmem(&acc_empty[buf], lane);
             if (i + 1 < nu && (u + 1) / KBn == d) continue;
             // the last unit of this output tile: 32 rows x 16 tokens through shared memory, so that each
             // lane adds four vectors of four hidden units of one token
@@ -921,12 +959,13 @@ cudaError_t launch_lora_gate_up(LoraGuParams &p, const sats_layer *layer, const 
 
 cudaError_t launch_gate_act(const sats_layer *layer, const uint16_t *x, int B, float *a, cudaStream_t stream)
 {
-    return tc::launch_gate_precise<false>(layer, x, B, a, stream);
+    return tc::launch_gate_precise<false, tc::kPreciseTok>(layer, x, B, a, stream);
 }
 
 cudaError_t launch_gate_act_f32(const sats_layer *layer, const float *x, int B, float *a, cudaStream_t stream)
 {
-    return tc::launch_gate_precise<true>(layer, x, B, a, stream);
+    return B <= 64 ? tc::launch_gate_precise<true, 64>(layer, x, B, a, stream)
+                   : tc::launch_gate_precise<true, tc::kPreciseTok>(layer, x, B, a, stream);
 }
 
 // Scratch of a LoRA batch inside the tensor-core region of a workspace: z and w where the other
