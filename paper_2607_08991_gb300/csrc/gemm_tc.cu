@@ -179,7 +179,7 @@ struct SkinnyGuParams {
     uint8_t *keep;                // [M][keep_stride] or nullptr
     int keep_stride;
     uint8_t *keep_trace;          // [M][N] or nullptr
-    float *a_out;                 // [M][ldh] fp32: SiLU(g) of every neuron (the calibration's masks), or nullptr
+    float *a_out;                 // ACT: [M][ldh] fp32: SiLU(g) of every neuron (the calibration's masks)
     int *ctl;
     float *zero;                  // y [M][H] to clear for the down projection's additions, or nullptr
     int zero_count;               // M H (a multiple of 8)
@@ -196,7 +196,9 @@ struct SkinnyGuParams {
 // lane r, column j (gate) and NT + j (up).  Grid: tc_T CTAs.  In gate-only mode
 // only the gate rows are read and multiplied.  The epilogue runs once all MMAs
 // are done, on G groups of four warps (blockDim 64 + 128 G): group g takes the
-// 16-token column blocks g, g + G, ... of every row (G = 1 in gate-only mode).
+// 16-token column blocks g, g + G, ... of every row (G = 1 in gate-only mode).  ACT: SiLU(g) is written too
+// (a template flag: tested per element in the epilogue it cost 1-2.5 % of calls of 100-250 tokens).
+template <bool ACT>
 __global__ void __launch_bounds__(kSkinnyMaxThreads, 1)
     gu_skinny_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmX2,
                      const SkinnyGuParams p)
@@ -354,7 +356,7 @@ __global__ void __launch_bounds__(kSkinnyMaxThreads, 1)
                     p.hact_lo[(size_t)j * p.ldh + n] = bf16_bits(h - __uint_as_float((uint32_t)hb << 16));
                     if (p.keep) p.keep[(size_t)j * p.keep_stride + n] = keep ? 1 : 0;
                     if (p.keep_trace) p.keep_trace[(size_t)(p.perm ? p.perm[j] : j) * p.N + n] = keep ? 1 : 0;
-                    if (p.a_out) p.a_out[(size_t)j * p.ldh + n] = a;
+                    if (ACT) p.a_out[(size_t)j * p.ldh + n] = a;
                 }
             }
         }
@@ -1263,13 +1265,15 @@ cudaError_t launch_gate_up_skinny(const sats_layer *layer, const GateUpArgs &a, 
     gp.ring_bytes = gp.stages * gp.stage_bytes + slack;
     gp.merge = split && NT <= 128 ? 1 : 0;
     gp.tmem_cols = tmem_cols_for((gp.merge ? 4 : 2) * NT);
-    cudaError_t e = set_smem(gu_skinny_kernel, smem_for(1, gp.ring_bytes), cfg_gu_skinny);
+    static std::atomic<int> cfg_act[64];
+    cudaError_t e = a.a_out ? set_smem(gu_skinny_kernel<true>, smem_for(1, gp.ring_bytes), cfg_act)
+                            : set_smem(gu_skinny_kernel<false>, smem_for(1, gp.ring_bytes), cfg_gu_skinny);
     if (e != cudaSuccess) return fail(e, "shared-memory attribute");
     // epilogue groups: one per 16-token column block, at most kSkinnyMaxGroups (the epilogue
     // runs after the last MMA, so its time adds to the call's)
     const int groups = NT / 16 < kSkinnyMaxGroups ? NT / 16 : kSkinnyMaxGroups;
-    e = launch_pdl_cfg(gu_skinny_kernel, dim3(layer->tc_T), 64 + 128 * groups, smem_for(1, gp.ring_bytes), stream, mX,
-                       mX2, gp);
+    e = launch_pdl_cfg(a.a_out ? gu_skinny_kernel<true> : gu_skinny_kernel<false>, dim3(layer->tc_T), 64 + 128 * groups,
+                       smem_for(1, gp.ring_bytes), stream, mX, mX2, gp);
     return e == cudaSuccess ? e : fail(e, "gate/up kernel launch");
 }
 
@@ -1510,9 +1514,9 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
         gp.ring_bytes = gp.stages * gp.stage_bytes + slack;
         gp.merge = split && NT <= 128 ? 1 : 0;
         gp.tmem_cols = tmem_cols_for(gp.merge ? 2 * NT : NT);
-        if ((e = set_smem(gu_skinny_kernel, smem_for(1, gp.ring_bytes), cfg_gu_skinny)) != cudaSuccess)
+        if ((e = set_smem(gu_skinny_kernel<false>, smem_for(1, gp.ring_bytes), cfg_gu_skinny)) != cudaSuccess)
             return fail(e, "shared-memory attribute");
-        e = launch_pdl_cfg(gu_skinny_kernel, dim3(layer->tc_T), 64 + 128, smem_for(1, gp.ring_bytes), stream, mX, mX2,
+        e = launch_pdl_cfg(gu_skinny_kernel<false>, dim3(layer->tc_T), 64 + 128, smem_for(1, gp.ring_bytes), stream, mX, mX2,
                            gp);
         if (e != cudaSuccess) return fail(e, "gate kernel launch");
         e = launch_union_tail(layer, B, xa, split ? xlo : nullptr, uflag, ulist, ucount, a_keep, ldn, u, ldn, out, ctl,
