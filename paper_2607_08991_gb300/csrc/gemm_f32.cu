@@ -702,6 +702,7 @@ struct LoraDownParams {
     int *ctl;
     int stages, ring_bytes;
     uint32_t tmem_cols;
+    KeepLists lists;        // the kept lists to write, if any
 };
 
 // CTA c takes units [c U / G, (c + 1) U / G) in order for the tokens of tile blockIdx.y; consecutive
@@ -820,7 +821,11 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
         };
         if (!cut_tiles<kLoraTok>(parts, NT, nu, pfull, pempty, &abort_flag, load)) set_timeout(p.ctl, &abort_flag);
     } else if (warp >= kEpi0) {
-        grid_dependency_wait();   // y and w are cleared by the preceding kernel
+        grid_dependency_wait();   // y and w are cleared, and the keep bytes written, by the preceding kernel
+        __shared__ int warp_sums[kLoraEpiThreads / 32];
+        if (blockIdx.y == 0)
+            for (int m = blockIdx.x; p.lists.idx && m < p.B; m += gridDim.x)
+                write_keep_list(p.lists, m, (int)threadIdx.x - 32 * kEpi0, kLoraEpiThreads, warp_sums, 1);
         const int quad = warp & 3, grp = (warp - kEpi0) >> 2;
         const int c0 = 16 * grp;
         const bool busy = c0 < NT;
@@ -1052,6 +1057,7 @@ cudaError_t run_lora_tc(const sats_layer *layer, const sats_lora *lora, bool x_f
     dp.r = lora->r;
     dp.y = y;
     dp.wsum = wsum;
+    dp.lists = {keep, gp.keep_stride, N, active_idx, active_cnt, nullptr};
     dp.ctl = ctl;
     const int parts = kPartStages * kParts * dp.NT * kTileBytes;
     dp.stages = stages_for(BM * kTileBytes, kSmemBudget - parts);
@@ -1065,9 +1071,7 @@ cudaError_t run_lora_tc(const sats_layer *layer, const sats_lora *lora, bool x_f
     if (e != cudaSuccess) return failed(e, "adapted down kernel launch");
     e = launch_pdl_threads(lora_out_kernel, dim3((H + 1023) / 1024, B), 128, stream, static_cast<const float *>(wsum),
                            static_cast<const uint16_t *>(lora->bd), H, lora->r, lora->scale, y);
-    if (e != cudaSuccess) return failed(e, "adapter output kernel launch");
-    if (active_idx) return launch_keep_lists(keep, gp.keep_stride, B, N, active_idx, active_cnt, nullptr, stream);
-    return cudaSuccess;
+    return e == cudaSuccess ? e : failed(e, "adapter output kernel launch");
 }
 
 }  // namespace sats

@@ -382,6 +382,7 @@ struct SkinnyDownParams {
     int stages, stage_bytes, a_bytes;
     int merge;                    // NT <= 128: one MMA of N = 2 NT over h's high and low parts
     uint32_t tmem_cols;           // two accumulators of NX columns (NX = 2 NT merged, else NT)
+    KeepLists lists;              // the kept lists to write, if any
 };
 
 // CTA c handles units [c U / G, (c+1) U / G) in order; consecutive units of one
@@ -502,6 +503,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int j = (int)threadIdx.x - 64; j < NT; j += (int)blockDim.x - 64)
             tok_s[j] = j < p.M ? (p.perm ? p.perm[j] : j) : 0;
         named_barrier(1, (int)blockDim.x - 64);   // the epilogue warps only
+        __shared__ int warp_sums[4];
+        for (int m = blockIdx.x; p.lists.idx && m < p.M; m += gridDim.x)
+            write_keep_list(p.lists, m, (int)threadIdx.x - 64, kThreads - 64, warp_sums, 1);
         const int lb = 32 * (warp & 3);
         const int te = lane >> 1, r0 = (lane & 1) * 16;   // this lane's token in the block, first row
         int q = 0;
@@ -850,6 +854,7 @@ struct WideDownParams {
     int *ctl;
     int stages, stage_bytes;
     uint32_t tmem_cols;   // two accumulator buffers of 128 dtiles columns
+    KeepLists lists;      // the kept lists to write, if any
 };
 
 // Persistent: CTA c takes units c, c + G, c + 2G, ...; unit u is the 128-token
@@ -995,6 +1000,9 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
         consumed_s = i;
         mma_commit(mma_done);
     } else if (warp >= 2) {
+        __shared__ int warp_sums[kWideMaxThreads / 32];
+        for (int m = blockIdx.x; p.lists.idx && m < p.M; m += gridDim.x)
+            write_keep_list(p.lists, m, (int)threadIdx.x - 64, (int)blockDim.x - 64, warp_sums, 1);
         // thread = token row of the unit's tile; group g of four warps takes the 16-column blocks
         // g, g + G, ...
         const int lb = 32 * (warp & 3);
@@ -1046,58 +1054,14 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
 }
 
 // ---------------------------------------------------------------------- kept lists
-// Row m's ascending kept list from its keep bytes (one CTA per row), written as
-// the list of token perm[m] (token m without a permutation).  Thread t takes the
-// 16-byte vectors [t per, (t + 1) per) of the row: it counts their kept bytes, a
-// block scan gives its first position, and it writes its entries in order.  Two
-// passes over the row in all (the second from L1/L2), one block scan.
-__global__ void __launch_bounds__(512) keep_list_kernel(const uint8_t *__restrict__ keep, int stride, int N,
-                                                        int32_t *__restrict__ idx, int32_t *__restrict__ cnt,
-                                                        const int32_t *__restrict__ perm)
+// The kept lists on their own, one CTA per row (the union path, and where lists_inside says no).
+__global__ void __launch_bounds__(512) keep_list_kernel(const KeepLists L)
 {
-    grid_dependency_wait();   // the keep bytes are written by the preceding kernel
-    grid_launch_dependents();
-    const int m = blockIdx.x;
-    const int tok = perm ? perm[m] : m;
-    const uint4 *k = reinterpret_cast<const uint4 *>(keep + (size_t)m * stride);   // stride: a multiple of 16
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int nv = (N + 15) >> 4;
-    const int per = (nv + 511) >> 9;
-    const int v0 = t * per, v1 = min(nv, v0 + per);
-    // the kept bytes (0 or 1) of vector v as a 16-bit mask; bytes at or past N are not counted
-    auto mask16 = [&](int v) {
-        const uint4 q = k[v];
-        const uint32_t wq[4] = {q.x, q.y, q.z, q.w};
-        uint32_t bits = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            bits |= ((wq[i] & 1u) | ((wq[i] >> 7) & 2u) | ((wq[i] >> 14) & 4u) | ((wq[i] >> 21) & 8u)) << (4 * i);
-        const int rest = N - 16 * v;
-        return rest >= 16 ? bits : bits & ((1u << rest) - 1u);
-    };
-    int c = 0;
-    for (int v = v0; v < v1; ++v) c += __popc(mask16(v));
     __shared__ int warp_sums[16];
-    int incl = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += x;
-    }
-    if (lane == 31) warp_sums[w] = incl;
-    __syncthreads();
-    int pos = incl - c, total = 0;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        if (i < w) pos += warp_sums[i];
-        total += warp_sums[i];
-    }
-    int32_t *out = idx + (size_t)tok * N;
-    for (int v = v0; v < v1; ++v)
-        for (uint32_t bits = mask16(v); bits; bits &= bits - 1u) out[pos++] = 16 * v + __ffs(bits) - 1;
-    if (t == 0 && cnt) cnt[tok] = total;
+    grid_dependency_wait();   // the keep bytes are written by a preceding kernel
+    grid_launch_dependents();
+    write_keep_list(L, blockIdx.x, (int)threadIdx.x, 512, warp_sums, 0);
 }
-
 
 }  // namespace
 }  // namespace tc
@@ -1187,17 +1151,18 @@ TcRegions tc_regions(int H, int N, int B)
     return {L.xhi, L.hact, L.keep};
 }
 
-cudaError_t launch_keep_lists(const uint8_t *keep, int stride, int B, int N, int32_t *active_idx, int32_t *active_cnt,
-                              const int32_t *perm, cudaStream_t stream)
-{
-    const cudaError_t e = tc::launch_pdl_threads(tc::keep_list_kernel, dim3(B), 512, stream, keep, stride, N, active_idx,
-                                                 active_cnt, perm);
-    if (e != cudaSuccess) cuda_fail(e, "kept-list kernel launch");
-    return e;
-}
-
 namespace {
 using namespace tc;
+
+// Whether the down projection's CTAs (grid of them) write the kept lists, or a kernel of their own does
+// afterwards.  Inside, the lists are written by idle epilogue warps, row after row of a CTA's share, before
+// its first accumulator: free (8 tokens of the Llama-shaped layer 63.7 -> 59.0 us, 2048 tokens' lists 25 us)
+// unless a small layer's CTA has several rows and no long stream to hide them (hidden 512 / intermediate 1408,
+// 333 tokens: 24.9 us with a kernel of their own, 28.9 inside; hidden 1168 / intermediate 2391: 42.1 and 39.1).
+bool lists_inside(const sats_layer *layer, int M, int grid)
+{
+    return M <= grid || (long long)layer->H * layer->N >= 1LL << 21;
+}
 
 // What the gate/up kernels of one batch are given besides the layer.
 struct GateUpArgs {
@@ -1221,6 +1186,12 @@ cudaError_t fail(cudaError_t err, const char *where)
 }
 
 int keep_stride_of(int N) { return (N + 15) & ~15; }
+
+cudaError_t launch_keep_lists(const KeepLists &lists, int M, cudaStream_t stream)
+{
+    const cudaError_t e = launch_pdl_threads(keep_list_kernel, dim3(M), 512, stream, lists);
+    return e == cudaSuccess ? e : fail(e, "kept-list kernel launch");
+}
 
 cudaError_t launch_gate_up_skinny(const sats_layer *layer, const GateUpArgs &a, cudaStream_t stream)
 {
@@ -1327,7 +1298,7 @@ cudaError_t launch_gate_up_wide(const sats_layer *layer, const GateUpArgs &a, cu
 
 // out[row perm[m] or m] += (hact + hact_lo)[m] W_down for M rows of h (row stride layer->ldn).
 cudaError_t launch_down_skinny(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
-                               const int32_t *perm, int *ctl, cudaStream_t stream)
+                               const int32_t *perm, const KeepLists &lists, int *ctl, cudaStream_t stream)
 {
     const int N = layer->N, ldn = layer->ldn, sms = sm_count();
     const int NT = (M + 15) & ~15;
@@ -1344,6 +1315,9 @@ cudaError_t launch_down_skinny(const sats_layer *layer, const uint16_t *hact, co
     dp.out = out;
     dp.perm = perm;
     dp.ctl = ctl;
+    const int grid = dp.units < sms ? dp.units : sms;
+    const bool inside = lists.idx && lists_inside(layer, M, grid);
+    if (inside) dp.lists = lists;
     dp.a_bytes = BM * kTileBytes;
     dp.stage_bytes = dp.a_bytes + 2 * NT * kTileBytes;
     dp.stages = stages_for(dp.stage_bytes);
@@ -1352,16 +1326,17 @@ cudaError_t launch_down_skinny(const sats_layer *layer, const uint16_t *hact, co
     static std::atomic<int> cfg_dn[64];
     cudaError_t e = set_smem(down_skinny_kernel, smem_for(dp.stages, dp.stage_bytes), cfg_dn);
     if (e != cudaSuccess) return fail(e, "shared-memory attribute");
-    e = launch_pdl(down_skinny_kernel, dim3(dp.units < sms ? dp.units : sms), smem_for(dp.stages, dp.stage_bytes),
+    e = launch_pdl(down_skinny_kernel, dim3(grid), smem_for(dp.stages, dp.stage_bytes),
                    stream, mH, mH2, dp);
-    return e == cudaSuccess ? e : fail(e, "down kernel launch");
+    if (e != cudaSuccess) return fail(e, "down kernel launch");
+    return lists.idx && !inside ? launch_keep_lists(lists, M, stream) : cudaSuccess;
 }
 
 // As launch_down_skinny, in the prefill orientation: 256 output columns per unit when the hidden
 // tiles pair up; the neuron range split so that the persistent CTAs' units come out even; every
 // unit adds into the output.
 cudaError_t launch_down_wide(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
-                             const int32_t *perm, int *ctl, cudaStream_t stream)
+                             const int32_t *perm, const KeepLists &lists, int *ctl, cudaStream_t stream)
 {
     const int N = layer->N, ldn = layer->ldn, sms = sm_count();
     CUtensorMap mH, mH2;
@@ -1381,16 +1356,20 @@ cudaError_t launch_down_wide(const sats_layer *layer, const uint16_t *hact, cons
     dp.out = out;
     dp.perm = perm;
     dp.ctl = ctl;
+    const int grid = dp.units < sms ? dp.units : sms;
+    const bool inside = lists.idx && lists_inside(layer, M, grid);
+    if (inside) dp.lists = lists;
     dp.stage_bytes = BM * kTileBytes * (2 + dp.dtiles);
     dp.stages = stages_for(dp.stage_bytes, wide_budget());
     dp.tmem_cols = tmem_cols_for(2 * BM * dp.dtiles);
     static std::atomic<int> cfg_dn[64];
     cudaError_t e = set_smem(down_wide_kernel, smem_for(dp.stages, dp.stage_bytes), cfg_dn);
     if (e != cudaSuccess) return fail(e, "shared-memory attribute");
-    down_wide_kernel<<<dim3(dp.units < sms ? dp.units : sms), 64 + 128 * kWideDownGroups,
+    down_wide_kernel<<<dim3(grid), 64 + 128 * kWideDownGroups,
                        smem_for(dp.stages, dp.stage_bytes), stream>>>(mH, mH2, dp);
     e = cudaGetLastError();
-    return e == cudaSuccess ? e : fail(e, "down kernel launch");
+    if (e != cudaSuccess) return fail(e, "down kernel launch");
+    return lists.idx && !inside ? launch_keep_lists(lists, M, stream) : cudaSuccess;
 }
 
 // Which orientation a batch's gate/up takes.
@@ -1436,8 +1415,8 @@ cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void 
 cudaError_t run_tc_down(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
                         int *ctl, cudaStream_t stream)
 {
-    return M <= kMaxSkinny ? launch_down_skinny(layer, hact, hact_lo, M, out, nullptr, ctl, stream)
-                           : launch_down_wide(layer, hact, hact_lo, M, out, nullptr, ctl, stream);
+    return M <= kMaxSkinny ? launch_down_skinny(layer, hact, hact_lo, M, out, nullptr, KeepLists{}, ctl, stream)
+                           : launch_down_wide(layer, hact, hact_lo, M, out, nullptr, KeepLists{}, ctl, stream);
 }
 
 // The thresholded MLP for a batch of B tokens on the tensor cores.
@@ -1462,6 +1441,7 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
     uint16_t *hact_lo = reinterpret_cast<uint16_t *>(base + W.hact_lo);
     uint8_t *keep = base + W.keep;
     const int kstride = keep_stride_of(N);
+    const KeepLists lists = {keep, kstride, N, active_idx, active_cnt, perm};
     const bool split = x_mode != kXBf16;
     if (perm && (!split || !n_dense || union_path)) return fail(cudaErrorInvalidValue, "routed batch arguments");
     const uint16_t *xa = split ? xhi : static_cast<const uint16_t *>(x);
@@ -1522,6 +1502,7 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
         e = launch_union_tail(layer, B, xa, split ? xlo : nullptr, uflag, ulist, ucount, a_keep, ldn, u, ldn, out, ctl,
                               stream);
         if (e != cudaSuccess) return fail(e, "union kernels launch");
+        if (active_idx) return launch_keep_lists(lists, B, stream);
     } else {
         GateUpArgs a{};
         a.xhi = xa;
@@ -1539,14 +1520,13 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
         a.ctl = ctl;
         if (skinny_batch(B, split)) {
             if ((e = launch_gate_up_skinny(layer, a, stream)) != cudaSuccess) return e;
-            e = launch_down_skinny(layer, hact, hact_lo, B, out, perm, ctl, stream);
+            e = launch_down_skinny(layer, hact, hact_lo, B, out, perm, lists, ctl, stream);
         } else {
             if ((e = launch_gate_up_wide(layer, a, stream)) != cudaSuccess) return e;
-            e = launch_down_wide(layer, hact, hact_lo, B, out, perm, ctl, stream);
+            e = launch_down_wide(layer, hact, hact_lo, B, out, perm, lists, ctl, stream);
         }
         if (e != cudaSuccess) return e;
     }
-    if (active_idx) return launch_keep_lists(keep, kstride, B, N, active_idx, active_cnt, perm, stream);
     return cudaSuccess;
 }
 

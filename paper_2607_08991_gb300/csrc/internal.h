@@ -149,8 +149,6 @@ struct TcRegions {
     size_t x, h, keep;
 };
 TcRegions tc_regions(int H, int N, int B);
-cudaError_t launch_keep_lists(const uint8_t *keep, int stride, int B, int N, int32_t *active_idx, int32_t *active_cnt,
-                              const int32_t *perm, cudaStream_t stream);
 // gemm_f32.cu: LoRA batches beyond one pass of the fused kernel.  lora_pack_tc allocates and fills
 // ad_blk; lora_tc_ok says whether a batch's scratch fits its workspace (hidden sizes of 96 and more).
 bool lora_tc_ok(int H, int B);

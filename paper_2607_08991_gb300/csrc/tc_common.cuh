@@ -171,6 +171,64 @@ __device__ __forceinline__ void set_timeout(int *ctl, volatile int *abort_flag)
     atomicOr(ctl + kCtlStatus, kStatusTimeout);
 }
 
+// ---------------------------------------------------------------------- kept lists
+// The ascending kept lists of a batch, from the keep bytes of the gate/up epilogue (0 or 1 per row
+// and neuron): row m's list is written as the list of token perm[m] (token m without a permutation).
+// The down projections' epilogue warps write them while their first MMAs run.
+struct KeepLists {
+    const uint8_t *keep;
+    int stride;             // a multiple of 16
+    int N;
+    int32_t *idx;           // [tokens][N], or nullptr: no lists
+    int32_t *cnt;           // [tokens] or nullptr
+    const int32_t *perm;
+};
+
+// Row m, by `threads` (a multiple of 32) threads that share hardware barrier `bar`; t is the thread's
+// number among them, warp_sums holds an int per warp.  Thread t takes the 16-byte vectors [t per,
+// (t + 1) per) of the row: it counts their kept bytes, a scan gives its first position, and it writes
+// its entries in order (two passes over the row, the second from L1/L2).
+__device__ __forceinline__ void write_keep_list(const KeepLists &L, int m, int t, int threads, int *warp_sums, int bar)
+{
+    const int tok = L.perm ? L.perm[m] : m;
+    const uint4 *k = reinterpret_cast<const uint4 *>(L.keep + (size_t)m * L.stride);
+    const int lane = t & 31, w = t >> 5;
+    const int nv = (L.N + 15) >> 4;
+    const int per = (nv + threads - 1) / threads;
+    const int v0 = min(nv, t * per), v1 = min(nv, v0 + per);
+    // the kept bytes of vector v as a 16-bit mask; bytes at or past N are not counted
+    auto mask16 = [&](int v) {
+        const uint4 q = k[v];
+        const uint32_t wq[4] = {q.x, q.y, q.z, q.w};
+        uint32_t bits = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            bits |= ((wq[i] & 1u) | ((wq[i] >> 7) & 2u) | ((wq[i] >> 14) & 4u) | ((wq[i] >> 21) & 8u)) << (4 * i);
+        const int rest = L.N - 16 * v;
+        return rest >= 16 ? bits : bits & ((1u << rest) - 1u);
+    };
+    int c = 0;
+    for (int v = v0; v < v1; ++v) c += __popc(mask16(v));
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    if (lane == 31) warp_sums[w] = incl;
+    named_barrier(bar, threads);
+    int pos = incl - c, total = 0;
+    for (int i = 0; i < threads >> 5; ++i) {
+        if (i < w) pos += warp_sums[i];
+        total += warp_sums[i];
+    }
+    int32_t *out = L.idx + (size_t)tok * L.N;
+    for (int v = v0; v < v1; ++v)
+        for (uint32_t bits = mask16(v); bits; bits &= bits - 1u) out[pos++] = 16 * v + __ffs(bits) - 1;
+    if (t == 0 && L.cnt) L.cnt[tok] = total;
+    named_barrier(bar, threads);   // warp_sums may be written again
+}
+
 // ---------------------------------------------------------------------- host
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 {
