@@ -111,12 +111,17 @@ def _check(s: int, where: str):
         raise SatsError(s, where)
 
 
-def _stream(stream: Optional[torch.cuda.Stream]):
-    st = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(st.cuda_stream)
+# The calls below pass addresses as plain integers (ctypes converts them by the declared argument
+# types) and ask torch for the current stream's handle itself: a one-token call on a small layer takes
+# the GPU 6 to 7 us, and building a Stream and a c_void_p object per argument took the host longer.
+
+def _stream(stream: Optional[torch.cuda.Stream]) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
-def _ptr(t: Optional[torch.Tensor], name: str, elem: Optional[int] = None):
+def _ptr(t: Optional[torch.Tensor], name: str, elem: Optional[int] = None) -> Optional[int]:
     if t is None:
         return None
     if not t.is_cuda:
@@ -125,7 +130,7 @@ def _ptr(t: Optional[torch.Tensor], name: str, elem: Optional[int] = None):
         raise ValueError("%s must be contiguous" % name)
     if elem is not None and t.element_size() != elem:
         raise ValueError("%s must have %d-byte elements" % (name, elem))
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 class Layer:
@@ -180,7 +185,7 @@ def sparse_mlp(layer: Layer, x: torch.Tensor, t_l: float, y: torch.Tensor, ws: W
     B = x.shape[0]
     _check(lib().sats_sparse_mlp(layer.handle, _ptr(x, "x", 2), B, float(t_l), _ptr(y, "y", 4),
                                  _ptr(active_idx, "active_idx", 4), _ptr(active_cnt, "active_cnt", 4),
-                                 ws.ptr, ws.nbytes, _stream(stream)), "sats_sparse_mlp")
+                                 ws.buf.data_ptr(), ws.nbytes, _stream(stream)), "sats_sparse_mlp")
 
 
 def sparse_mlp_f32(layer: Layer, x: torch.Tensor, t_l: float, y: torch.Tensor, ws: Workspace,
@@ -189,7 +194,7 @@ def sparse_mlp_f32(layer: Layer, x: torch.Tensor, t_l: float, y: torch.Tensor, w
     B = x.shape[0]
     _check(lib().sats_sparse_mlp_f32(layer.handle, _ptr(x, "x", 4), B, float(t_l), _ptr(y, "y", 4),
                                      _ptr(active_idx, "active_idx", 4), _ptr(active_cnt, "active_cnt", 4),
-                                     ws.ptr, ws.nbytes, _stream(stream)), "sats_sparse_mlp_f32")
+                                     ws.buf.data_ptr(), ws.nbytes, _stream(stream)), "sats_sparse_mlp_f32")
 
 
 class Lora:
@@ -227,12 +232,12 @@ def sparse_mlp_lora(layer: Layer, lora: Lora, x: torch.Tensor, t_l: float, y: to
     if x.dtype == torch.float32:
         _check(lib().sats_sparse_mlp_lora_f32(layer.handle, lora.handle, _ptr(x, "x", 4), B, float(t_l),
                                               _ptr(y, "y", 4), _ptr(active_idx, "active_idx", 4),
-                                              _ptr(active_cnt, "active_cnt", 4), ws.ptr, ws.nbytes,
+                                              _ptr(active_cnt, "active_cnt", 4), ws.buf.data_ptr(), ws.nbytes,
                                               _stream(stream)), "sats_sparse_mlp_lora_f32")
     else:
         _check(lib().sats_sparse_mlp_lora(layer.handle, lora.handle, _ptr(x, "x", 2), B, float(t_l),
                                           _ptr(y, "y", 4), _ptr(active_idx, "active_idx", 4),
-                                          _ptr(active_cnt, "active_cnt", 4), ws.ptr, ws.nbytes, _stream(stream)),
+                                          _ptr(active_cnt, "active_cnt", 4), ws.buf.data_ptr(), ws.nbytes, _stream(stream)),
                "sats_sparse_mlp_lora")
 
 
@@ -244,11 +249,11 @@ def sparse_mlp_union(layer: Layer, x: torch.Tensor, t_l: float, y: torch.Tensor,
     if x.dtype == torch.float32:
         _check(lib().sats_sparse_mlp_union_f32(layer.handle, _ptr(x, "x", 4), B, float(t_l), _ptr(y, "y", 4),
                                                _ptr(active_idx, "active_idx", 4), _ptr(active_cnt, "active_cnt", 4),
-                                               ws.ptr, ws.nbytes, _stream(stream)), "sats_sparse_mlp_union_f32")
+                                               ws.buf.data_ptr(), ws.nbytes, _stream(stream)), "sats_sparse_mlp_union_f32")
     else:
         _check(lib().sats_sparse_mlp_union(layer.handle, _ptr(x, "x", 2), B, float(t_l), _ptr(y, "y", 4),
                                            _ptr(active_idx, "active_idx", 4), _ptr(active_cnt, "active_cnt", 4),
-                                           ws.ptr, ws.nbytes, _stream(stream)), "sats_sparse_mlp_union")
+                                           ws.buf.data_ptr(), ws.nbytes, _stream(stream)), "sats_sparse_mlp_union")
 
 
 def sparse_mlp_fixed_scratch(layer: Layer, x: torch.Tensor, t_l: float, y: torch.Tensor,
@@ -293,7 +298,7 @@ def mlp_stack(layers: Sequence[Layer], norm_w: Sequence[torch.Tensor], t: Sequen
     ts = (ctypes.c_float * L)(*[float(v) for v in t])
     _check(lib().sats_mlp_stack(hs, nws, ts, L, float(eps), _ptr(token_ids, "token_ids", 4), _ptr(lut, "lut", 1),
                                 0 if lut is None else lut.numel(), _ptr(x, "x", 4), x.shape[0],
-                                _ptr(keep_trace, "keep_trace", 1), ws.ptr, ws.nbytes, _stream(stream)),
+                                _ptr(keep_trace, "keep_trace", 1), ws.buf.data_ptr(), ws.nbytes, _stream(stream)),
            "sats_mlp_stack")
 
 
@@ -371,7 +376,7 @@ def sats_calibrate(layers: Sequence[Layer], norm_w: Sequence[torch.Tensor], eps:
     ws = torch.empty(n + 256, dtype=torch.uint8, device=x_cal.device)
     off = (-ws.data_ptr()) % 256
     hs = (ctypes.c_void_p * L)(*[l.handle.value for l in layers])
-    nws = (ctypes.c_void_p * L)(*[_ptr(w, "norm_w", 4).value for w in norm_w])
+    nws = (ctypes.c_void_p * L)(*[_ptr(w, "norm_w", 4) for w in norm_w])
     tout = (ctypes.c_float * L)()
     b = ctypes.c_double()
     S = ctypes.c_double()
@@ -421,12 +426,12 @@ def route_calibrate(score: torch.Tensor, heldout_ids: torch.Tensor, r_tar: float
 def selftest_wait_timeout(ws: Workspace, stream: Optional[torch.cuda.Stream] = None):
     """Runs the library's bounded device waits against conditions nothing satisfies; the
     next get_error(ws) reads ETIMEOUT (takes about 4 s)."""
-    _check(lib().sats_selftest_wait_timeout(ws.ptr, ws.nbytes, _stream(stream)), "sats_selftest_wait_timeout")
+    _check(lib().sats_selftest_wait_timeout(ws.buf.data_ptr(), ws.nbytes, _stream(stream)), "sats_selftest_wait_timeout")
 
 
 def get_error(ws: Workspace, stream: Optional[torch.cuda.Stream] = None) -> int:
     """Returns the device status of the workspace (OK, EDEVICE or ETIMEOUT) and clears it."""
-    return int(lib().sats_get_error(ws.ptr, ws.nbytes, _stream(stream)))
+    return int(lib().sats_get_error(ws.buf.data_ptr(), ws.nbytes, _stream(stream)))
 
 
 def get_status_word(dev_status: torch.Tensor, stream: Optional[torch.cuda.Stream] = None) -> int:
