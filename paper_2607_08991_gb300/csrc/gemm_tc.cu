@@ -40,7 +40,7 @@
 // owns the TMEM allocation and lane 0 issues the MMAs, warps 2 .. 4 G + 1 run the
 // epilogue in G groups of four (warp w reads TMEM lanes 32 (w mod 4) .. 32 (w mod
 // 4) + 31; the groups split the accumulator's columns; G = 1 in the down kernel of
-// batched decode, up to six in its gate/up kernel, four in the prefill kernels).
+// batched decode, up to seven in its gate/up kernel, four in the prefill kernels).
 // Every wait is bounded in time and sets the status word when it gives up.
 #include "tc_common.cuh"
 
