@@ -607,6 +607,15 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
 namespace sats {
 namespace {
 
+// Where token v's total and count are kept: neighbouring ids go to different cache lines.  Ids are often
+// given out by frequency, and additions to one line queue up behind one another (a million occurrences,
+// Zipf ids in order of rank: 57 us, most of it on the first few lines).
+constexpr int kSpread = 64;
+
+__host__ __device__ inline int spread_rows(int V) { return (V + kSpread - 1) / kSpread; }
+
+__device__ __forceinline__ int spread(int v, int rows) { return (v & (kSpread - 1)) * rows + v / kSpread; }
+
 // A warp's table of the token ids it has met: sums of the occurrences it has seen, added to the
 // device totals once at the end.  Token frequencies are far from even (a corpus' most common token
 // is several per cent of it), and atomics on one address go one after the other: 290 us for a
@@ -626,7 +635,7 @@ struct Tally {
 // Adds one occurrence per lane (id kNoToken: none) with excess loss v.
 template <bool SUMS>
 __device__ __forceinline__ void tally_add(Tally<SUMS> &T, int id, float v, double *__restrict__ total,
-                                          unsigned *__restrict__ count)
+                                          unsigned *__restrict__ count, int rows)
 {
     const unsigned lane = threadIdx.x & 31u;
     const unsigned same = __match_any_sync(0xffffffffu, id);
@@ -638,8 +647,8 @@ __device__ __forceinline__ void tally_add(Tally<SUMS> &T, int id, float v, doubl
     __syncwarp();
     if (id != kNoToken) mine = T.id[slot] == id;
     if (id != kNoToken && !mine) {
-        if (SUMS) atomicAdd(total + id, (double)v);
-        atomicAdd(count + id, 1u);
+        if (SUMS) atomicAdd(total + spread(id, rows), (double)v);
+        atomicAdd(count + spread(id, rows), 1u);
     }
     if (mine && turn == 0) T.count[slot] += (unsigned)__popc(same);
     if (!SUMS) {
@@ -672,6 +681,7 @@ __global__ void __launch_bounds__(32 * kTallyWarps) tally_kernel(const int32_t *
         if (SUMS) T.sum[i] = 0.0;
     }
     __syncwarp();
+    const int rows = spread_rows(V);
     constexpr int kAhead = 4;   // loads in flight per lane
     const int64_t step = (int64_t)gridDim.x * kTallyWarps * 32;
     for (int64_t base = ((int64_t)blockIdx.x * kTallyWarps + warp) * 32; base < n; base += kAhead * step) {
@@ -692,14 +702,31 @@ __global__ void __launch_bounds__(32 * kTallyWarps) tally_kernel(const int32_t *
             }
         }
 #pragma unroll
-        for (int k = 0; k < kAhead; ++k) tally_add<SUMS>(T, id[k], v[k], total, count);
+        for (int k = 0; k < kAhead; ++k) tally_add<SUMS>(T, id[k], v[k], total, count, rows);
     }
-    __syncwarp();
-    for (int i = lane; i < kTallySlots; i += 32) {
-        const int id = T.id[i];
-        if (id == kNoToken) continue;
-        if (SUMS) atomicAdd(total + id, T.sum[i]);
-        atomicAdd(count + id, T.count[i]);
+    __syncthreads();
+    // the CTA's tables together, a thread per slot: common tokens have the slot in every table
+    const Tally<SUMS> *all = reinterpret_cast<const Tally<SUMS> *>(tally_smem);
+    for (int i = threadIdx.x; i < kTallySlots; i += 32 * kTallyWarps) {
+        int first = kNoToken;
+        unsigned c = 0u;
+        double v = 0.0;
+        for (int w = 0; w < kTallyWarps; ++w) {
+            const int id = all[w].id[i];
+            if (id == kNoToken) continue;
+            if (first == kNoToken) first = id;
+            if (id == first) {
+                c += all[w].count[i];
+                if (SUMS) v += all[w].sum[i];
+            } else {
+                if (SUMS) atomicAdd(total + spread(id, rows), all[w].sum[i]);
+                atomicAdd(count + spread(id, rows), all[w].count[i]);
+            }
+        }
+        if (first != kNoToken) {
+            if (SUMS) atomicAdd(total + spread(first, rows), v);
+            atomicAdd(count + spread(first, rows), c);
+        }
     }
 }
 
@@ -708,7 +735,19 @@ __global__ void score_final_kernel(const double *__restrict__ total, const unsig
                                    float *__restrict__ score)
 {
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < V) score[v] = count[v] ? (float)(total[v] / count[v]) : INFINITY;
+    if (v >= V) return;
+    const int at = spread(v, spread_rows(V));
+    const unsigned c = count[at];
+    if (c == 0u) {
+        score[v] = INFINITY;
+        return;
+    }
+    // total / c rounded to fp32, with one 64-bit multiply-add instead of a 64-bit division (this GPU has
+    // few 64-bit units): a quotient q in fp32 and its remainder's share
+    const double t = total[at];
+    const float cf = (float)c, q = (float)t / cf;
+    if (q > 1e-30f && q < 1e38f) score[v] = q + (float)__fma_rn(-(double)q, (double)c, t) / cf;
+    else score[v] = (float)(t / (double)c);   // 0, and the ends of fp32's range
 }
 
 // Eq. 14 on the device.  With the held-out occurrences' scores in increasing order, the candidates
@@ -753,9 +792,10 @@ __global__ void __launch_bounds__(kTauThreads) tau_level_kernel(const float *__r
     grid_dependency_wait();
     grid_launch_dependents();
     const uint32_t prefix = LEVEL == 0 ? 0u : S->prefix;
+    const int rows = spread_rows(V);
     __syncthreads();
     for (int v = blockIdx.x * kTauThreads + tid; v < V; v += gridDim.x * kTauThreads) {
-        const unsigned f = freq[v];
+        const unsigned f = freq[spread(v, rows)];
         const uint32_t b = ordered_bits(score[v]);
         const bool in = LEVEL == 0 || (LEVEL == 1 ? (b >> 21) == (prefix >> 21) : (b >> 10) == (prefix >> 10));
         if (f && in) atomicAdd(h + ((b >> kShift) & (kBins - 1)), (unsigned long long)f);
@@ -809,11 +849,12 @@ __global__ void __launch_bounds__(kTauThreads) tau_sums_kernel(const float *__re
     if (threadIdx.x == 4) not_above = 0u;
     grid_dependency_wait();
     __syncthreads();
+    const int rows = spread_rows(V);
     const uint32_t at = S->prefix, zero = 0x80000000u, inf = 0xff800000u;
     unsigned long long s[4] = {0ull, 0ull, 0ull, 0ull};
     uint32_t na = 0u;
     for (int v = blockIdx.x * kTauThreads + threadIdx.x; v < V; v += gridDim.x * kTauThreads) {
-        const unsigned f = freq[v];
+        const unsigned f = freq[spread(v, rows)];
         if (!f) continue;
         const uint32_t b = ordered_bits(score[v]);
         s[0] += b < at ? f : 0u;
@@ -860,9 +901,9 @@ ScoreLayout score_layout(int V)
     S.search = off;   // sats_route_calibrate
     off += al256(sizeof(TauSearch));
     S.total = off;
-    off += al256((size_t)V * sizeof(double));
+    off += al256((size_t)kSpread * spread_rows(V) * sizeof(double));
     S.count = off;
-    off += al256((size_t)V * sizeof(unsigned));
+    off += al256((size_t)kSpread * spread_rows(V) * sizeof(unsigned));
     S.total_bytes = off;
     return S;
 }
@@ -957,7 +998,7 @@ sats_status sats_route_calibrate(const float *score, int V, const int32_t *heldo
     unsigned *freq = reinterpret_cast<unsigned *>(base + S.count);
     TauSearch *search = reinterpret_cast<TauSearch *>(base + S.search);
     cudaError_t e = cudaMemsetAsync(status, 0, 256 + sizeof(TauSearch), st);   // (the search follows the status word)
-    if (e == cudaSuccess) e = cudaMemsetAsync(freq, 0, (size_t)V * sizeof(unsigned), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(freq, 0, (size_t)kSpread * spread_rows(V) * sizeof(unsigned), st);
     if (e != cudaSuccess) return cuda_fail(e, "held-out count clear");
     if (m > 0 && (e = launch_tally<false>(heldout_ids, nullptr, nullptr, m, V, nullptr, freq, status, st)) != cudaSuccess)
         return cuda_fail(e, "held-out count kernel launch");
