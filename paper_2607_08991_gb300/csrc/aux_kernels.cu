@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kRouteThreads) route_kernel(const int32_t *ids
 // histograms per CTA in shared memory, and 2048-bin levels leave the search a few
 // microseconds.  All percentiles of a calibration grid share the three passes.
 constexpr int kSelBins0 = 2048, kSelBins = 1024, kSelCopies = 4;
-constexpr int kSelThreads = 512, kSelWarps = kSelThreads / 32;
+constexpr int kSelThreads = 1024, kSelWarps = kSelThreads / 32;
 
 // Workspace of a selection of R ranks; cleared as a whole before level 0.
 struct SelWs {

@@ -2,11 +2,11 @@
 // on the GPU, with the same kernels that run the thresholded MLP.
 //
 // Eq. 6, Err_l(t) = E_x[ ||y(x) - y~_t(x)|| / (||y(x)|| + eps) ], is evaluated for
-// many candidate thresholds at once per block: the dense output once, then one
-// thresholded pass per candidate (the fused kernel or the tensor-core path,
-// whichever the batch of calibration inputs takes), each followed by a small
-// reduction kernel that adds the per-token relative distortion and realised
-// sparsity into device accumulators.  Eqs. 7-10 (budget selection) run on the
+// many candidate thresholds at once per block: on the tensor cores from one pass
+// over the gate and up projections and one GEMM over the dropped neurons of all
+// candidates, for one or two inputs from the fused kernel's outputs (the dense one,
+// then one per candidate); small reduction kernels add the per-token relative
+// distortion and realised sparsity into device accumulators.  Eqs. 7-10 (budget selection) run on the
 // host; the coarse-to-fine driver chains everything for a whole stack.
 #include <algorithm>
 #include <cmath>
@@ -24,6 +24,7 @@ constexpr int kErrGroup = 32;     // candidate thresholds per group of Eq. 6
 // Rows of h per group (candidates x inputs): enough to fill the GPU for several waves, and at most
 // about 470 MB of rows at the largest layers' 14336 neurons
 constexpr int kErrRows = 8192;
+constexpr size_t kErrKeep = (size_t)1 << 30;
 
 size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -80,9 +81,11 @@ __global__ void __launch_bounds__(256) err_accum_kernel(const float *__restrict_
     }
 }
 
-// Candidates of one group: the threshold of each, or NaN for the dense output (every neuron).
+// Candidates of one group: the threshold of each; with dev, candidate k's is dev[at[k]].
 struct Candidates {
     float t[kErrGroup];
+    int at[kErrGroup];
+    const float *dev;
 };
 
 // Row (k, c) of the dropped neurons' h, in bf16 parts: h where |a| < t_k, 0 elsewhere, for the K
@@ -112,12 +115,12 @@ __global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict_
         hl = *reinterpret_cast<const uint4 *>(hlo + at);
     }
     for (int k = 0; k < K; ++k) {
-        const float t = cand.t[k];
+        const float t = cand.dev ? cand.dev[cand.at[k]] : cand.t[k];
         unsigned m[4] = {0u, 0u, 0u, 0u}, cnt = 0u;
         if (in) {
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                // not kept (Eqs. 4-5: a neuron is kept if |a| >= t); true for every a when t is NaN
+                // not kept (Eqs. 4-5: a neuron is kept if |a| >= t)
                 const bool drop = n0 + e < N && !(fabsf(av[e]) >= t);
                 cnt += drop ? 1u : 0u;
                 m[e / 2] |= drop ? (e & 1 ? 0xffff0000u : 0xffffu) : 0u;
@@ -133,16 +136,28 @@ __global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict_
     if (threadIdx.x < K && dropped[threadIdx.x]) atomicAdd(counts + threadIdx.x, (unsigned long long)dropped[threadIdx.x]);
 }
 
-// A sum of squares carried as an unevaluated pair of floats (error-free product and sum), about
+// A sum of squares carried as an unevaluated pair of floats (error-free product and sums), about
 // 48 bits: this GPU's 64-bit rate is 1/64 of its 32-bit one.
 struct SquareSum {
     float hi = 0.f, lo = 0.f;
+    __device__ void join(float v, float rest)   // += v + rest, |rest| far below |v|
+    {
+        const float s = __fadd_rn(hi, v), b = __fadd_rn(s, -hi);
+        lo += (__fadd_rn(hi, -__fadd_rn(s, -b)) + __fadd_rn(v, -b)) + rest;
+        hi = s;
+    }
     __device__ void add(float v)
     {
-        const float p = __fmul_rn(v, v), pe = __fmaf_rn(v, v, -p);
-        const float s = __fadd_rn(hi, p), b = __fadd_rn(s, -hi);
-        lo += (__fadd_rn(hi, -__fadd_rn(s, -b)) + __fadd_rn(p, -b)) + pe;
-        hi = s;
+        const float p = __fmul_rn(v, v);
+        join(p, __fmaf_rn(v, v, -p));
+    }
+    __device__ void over_warp()
+    {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+            join(h, l);
+        }
     }
     __device__ double value() const { return (double)hi + (double)lo; }
 };
@@ -161,43 +176,43 @@ __global__ void __launch_bounds__(256) drop_err_kernel(const float *__restrict__
         sd.add(p.x); sd.add(p.y); sd.add(p.z); sd.add(p.w);
         sy.add(q.x); sy.add(q.y); sy.add(q.z); sy.add(q.w);
     }
-    __shared__ double r0[8], r1[8];
-    double ds, ys;
-    auto reduce = [&](double dd, double yy) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            dd += __shfl_xor_sync(0xffffffffu, dd, o);
-            yy += __shfl_xor_sync(0xffffffffu, yy, o);
-        }
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) {
-            r0[threadIdx.x >> 5] = dd;
-            r1[threadIdx.x >> 5] = yy;
-        }
-        __syncthreads();
-        ds = ys = 0.0;
-        for (int i = 0; i < 8; ++i) {
-            ds += r0[i];
-            ys += r1[i];
-        }
-    };
-    reduce(sd.value(), sy.value());
+    __shared__ float part[2][8][2];
+    __shared__ double sums[2];
+    sd.over_warp();
+    sy.over_warp();
+    if ((threadIdx.x & 31) == 0) {
+        const int w = threadIdx.x >> 5;
+        part[0][w][0] = sd.hi; part[0][w][1] = sd.lo;
+        part[1][w][0] = sy.hi; part[1][w][1] = sy.lo;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        SquareSum s;
+        for (int w = 0; w < 8; ++w) s.join(part[threadIdx.x][w][0], part[threadIdx.x][w][1]);
+        sums[threadIdx.x] = s.value();
+    }
+    __syncthreads();
     auto in_range = [](double v) { return v > 1e-24 && v < 1e36; };
-    if (!in_range(ds) || !in_range(ys)) {   // 32-bit squares may have over- or underflown
+    if (!in_range(sums[0]) || !in_range(sums[1])) {   // 32-bit squares may have over- or underflown
         double dd = 0.0, yy = 0.0;
         for (int i = threadIdx.x; i < H; i += 256) {
             const double p = d[((size_t)k * C + c) * H + i], q = y[(size_t)c * H + i];
             dd += p * p;
             yy += q * q;
         }
-        reduce(dd, yy);
+        __syncthreads();   // every thread has read the sums
+        if (threadIdx.x < 2) sums[threadIdx.x] = 0.0;
+        __syncthreads();
+        atomicAdd(&sums[0], dd);
+        atomicAdd(&sums[1], yy);
+        __syncthreads();
     }
-    if (threadIdx.x == 0) atomicAdd(acc + k, sqrt(ds) / (sqrt(ys) + (double)eps));
+    if (threadIdx.x == 0) atomicAdd(acc + k, sqrt(sums[0]) / (sqrt(sums[1]) + (double)eps));
 }
 
 // Workspace of Eq. 6.  Batches on the fused kernel (at most two tokens) compare whole outputs
 // (yd, yk, idx, cnt); batches on the tensor cores project the dropped neurons of a group of
-// candidates (a, rows, y: the dense output, then the group's).
+// candidates (a: ErrInputs, rows, y: the group's outputs).
 struct ErrLayout {
     size_t mlp, yd, yk, idx, cnt, a, rhi, rlo, y, acc, total;
 };
@@ -206,7 +221,7 @@ struct ErrLayout {
 int err_group(int C, int K)
 {
     const int fit = kErrRows / C;
-    return std::max(1, std::min(std::min(fit, kErrGroup), K + 1));
+    return std::max(1, std::min(std::min(fit, kErrGroup), K));
 }
 
 ErrLayout err_layout(int H, int N, int C, int K)
@@ -221,11 +236,11 @@ ErrLayout err_layout(int H, int N, int C, int K)
     L.mlp = take(ws_layout(H, N, C).total);
     if (use_tc_path(H, C)) {
         const size_t ldn = ((size_t)N + 7) & ~(size_t)7, rows = (size_t)err_group(C, K) * C;
-        L.a = take((size_t)C * ldn * sizeof(float));
+        L.a = take((size_t)C * H * 4 + (size_t)C * ldn * 8);   // ErrInputs
         L.rhi = take(rows * ldn * 2);
         L.rlo = take(rows * ldn * 2);
-        L.y = take((rows + C) * H * sizeof(float));
-        L.acc = take((size_t)(K + 1) * (sizeof(double) + sizeof(unsigned long long)));
+        L.y = take(rows * H * sizeof(float));
+        L.acc = take((size_t)std::max(K, 1) * (sizeof(double) + sizeof(unsigned long long)));   // ErrSums
     } else {
         L.yd = take((size_t)C * H * sizeof(float));
         L.yk = take((size_t)C * H * sizeof(float));
@@ -243,56 +258,126 @@ ErrLayout err_layout(int H, int N, int C, int K)
 // for 19 candidates of 64 inputs on the Llama-shaped layer), and the small difference is formed
 // without cancellation.  What bounds it: the down projection's MMAs (two per product: h's high and
 // low parts).
-sats_status layer_err_tc(const sats_layer *layer, const float *x, int C, const float *t, int K, float eps, double *err,
-                         double *sp, char *base, const ErrLayout &W, cudaStream_t st)
+struct ErrSums {
+    double *err;                     // [K]
+    unsigned long long *dropped;     // [K]
+    static size_t bytes(int K) { return (size_t)K * (sizeof(double) + sizeof(unsigned long long)); }
+    ErrSums(void *p, int K) : err(static_cast<double *>(p)), dropped(reinterpret_cast<unsigned long long *>(err + K)) {}
+};
+
+// What the candidates of one block are formed from.
+struct ErrInputs {
+    float *y;                // [C][H]: the dense output
+    float *a;                // [C][ldn]: SiLU(x W_gate)
+    uint16_t *hhi, *hlo;     // [C][ldn]: a u of every neuron
+    static size_t bytes(int H, int N, int C) { return al256((size_t)C * H * 4 + (size_t)C * ((N + 7) & ~7) * 8); }
+    ErrInputs(void *p, int H, int N, int C)
+        : y(static_cast<float *>(p)), a(y + (size_t)C * H),
+          hhi(reinterpret_cast<uint16_t *>(a + (size_t)C * ((N + 7) & ~7))), hlo(hhi + (size_t)C * ((N + 7) & ~7)) {}
+};
+
+// The rows of kg candidates (cand) and their product with W_down, into out [kg][C][H].
+sats_status enqueue_rows(const sats_layer *layer, const ErrInputs &in, int C, const Candidates &cand, int kg,
+                         unsigned long long *dropped, float *out, char *base, const ErrLayout &W, cudaStream_t st)
 {
     const int H = layer->H, N = layer->N, ld = layer->ldn;
-    const WsLayout M = ws_layout(H, N, C);
+    int *ctl = reinterpret_cast<int *>(base + W.mlp + ws_layout(H, N, C).ctl);
+    uint16_t *rhi = reinterpret_cast<uint16_t *>(base + W.rhi), *rlo = reinterpret_cast<uint16_t *>(base + W.rlo);
+    cudaError_t e = cudaMemsetAsync(out, 0, (size_t)kg * C * H * sizeof(float), st);
+    if (e != cudaSuccess) return cuda_fail(e, "layer error output clear");
+    drop_rows_kernel<<<dim3(C, (ld / 8 + 255) / 256), 256, 0, st>>>(in.a, in.hhi, in.hlo, C, N, ld, cand, kg, rhi, rlo,
+                                                                   dropped);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "dropped rows kernel launch");
+    return run_tc_down(layer, rhi, rlo, kg * C, out, ctl, st) == cudaSuccess ? SATS_OK : SATS_ECUDA;
+}
+
+// h, a and the dense output of one block's inputs x.  The dense output is projected on its own: a stack's next
+// block starts from it, and up to 256 inputs take the batched-decode kernel, whose shorter accumulator chains
+// are the more accurate ones.
+sats_status enqueue_err_inputs(const sats_layer *layer, const float *x, int C, const ErrInputs &in, char *base,
+                               const ErrLayout &W, cudaStream_t st)
+{
+    const WsLayout M = ws_layout(layer->H, layer->N, C);
     char *mlp = base + W.mlp;
     int *ctl = reinterpret_cast<int *>(mlp + M.ctl);
-    float *a = reinterpret_cast<float *>(base + W.a), *y = reinterpret_cast<float *>(base + W.y);
-    uint16_t *rhi = reinterpret_cast<uint16_t *>(base + W.rhi), *rlo = reinterpret_cast<uint16_t *>(base + W.rlo);
-    double *acc = reinterpret_cast<double *>(base + W.acc);
-    unsigned long long *counts = reinterpret_cast<unsigned long long *>(acc + K + 1);
-    cudaError_t e = clear_fused_state(mlp, H, N, C, st);
-    const size_t acc_bytes = (size_t)(K + 1) * (sizeof(double) + sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, acc_bytes, st);
-    if (e != cudaSuccess) return cuda_fail(e, "layer error workspace clear");
-    const uint16_t *hhi = nullptr, *hlo = nullptr;
-    if (run_tc_gate_up(layer, x, C, mlp + M.tc, &hhi, &hlo, a, ctl, st) != cudaSuccess) return SATS_ECUDA;
+    if (run_tc_gate_up(layer, x, C, mlp + M.tc, in.hhi, in.hlo, in.a, ctl, st) != cudaSuccess) return SATS_ECUDA;
+    const cudaError_t e = cudaMemsetAsync(in.y, 0, (size_t)C * layer->H * sizeof(float), st);
+    if (e != cudaSuccess) return cuda_fail(e, "layer error output clear");
+    return run_tc_down(layer, in.hhi, in.hlo, C, in.y, ctl, st) == cudaSuccess ? SATS_OK : SATS_ECUDA;
+}
+
+// Enqueues the sums for K candidates: thresholds t (host), or q[at(k)] on the device where q is given.
+// sums: cleared device memory of ErrSums::bytes(K).
+template <typename At>
+sats_status enqueue_err(const sats_layer *layer, const ErrInputs &in, int C, const float *t, const float *q, At at, int K,
+                        float eps, const ErrSums &sums, char *base, const ErrLayout &W, cudaStream_t st)
+{
+    float *out = reinterpret_cast<float *>(base + W.y);
     const int group = err_group(C, K);
-    // candidate 0 is the dense output; its rows stay at the front of y for every group
-    for (int k0 = 0; k0 <= K; k0 += group) {
-        const int kg = std::min(group, K + 1 - k0);
-        Candidates cand;
-        for (int k = 0; k < kg; ++k) cand.t[k] = k0 + k == 0 ? NAN : t[k0 + k - 1];
-        float *out = k0 == 0 ? y : y + (size_t)C * H;
-        if ((e = cudaMemsetAsync(out, 0, (size_t)kg * C * H * sizeof(float), st)) != cudaSuccess)
-            return cuda_fail(e, "layer error output clear");
-        drop_rows_kernel<<<dim3(C, (ld / 8 + 255) / 256), 256, 0, st>>>(a, hhi, hlo, C, N, ld, cand, kg, rhi, rlo,
-                                                                       counts + k0);
-        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "dropped rows kernel launch");
-        if (run_tc_down(layer, rhi, rlo, kg * C, out, ctl, st) != cudaSuccess) return SATS_ECUDA;
-        drop_err_kernel<<<dim3(C, kg), 256, 0, st>>>(y, out, C, H, eps, acc + k0);
-        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "error reduction kernel launch");
-    }
-    std::vector<char> h(acc_bytes);
-    e = cudaMemcpyAsync(h.data(), acc, acc_bytes, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(e, "layer error read-back");
-    const sats_status s = sats_get_error(mlp, M.total, st);
-    if (s != SATS_OK) return s;
-    const double *ha = reinterpret_cast<const double *>(h.data());
-    const unsigned long long *hc = reinterpret_cast<const unsigned long long *>(h.data() + (size_t)(K + 1) * sizeof(double));
-    for (int k = 0; k < K; ++k) {
-        err[k] = ha[k + 1] / C;
-        sp[k] = (double)hc[k + 1] / ((double)C * N);
+    for (int k0 = 0; k0 < K; k0 += group) {
+        const int kg = std::min(group, K - k0);
+        Candidates cand{};
+        cand.dev = q;
+        for (int k = 0; k < kg; ++k) {
+            cand.t[k] = q ? 0.f : t[k0 + k];
+            cand.at[k] = at(k0 + k);
+        }
+        const sats_status s = enqueue_rows(layer, in, C, cand, kg, sums.dropped + k0, out, base, W, st);
+        if (s != SATS_OK) return s;
+        drop_err_kernel<<<dim3(C, kg), 256, 0, st>>>(in.y, out, C, layer->H, eps, sums.err + k0);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(e, "error reduction kernel launch");
     }
     return SATS_OK;
 }
 
+// The means of a candidate table's rows from their sums (host copies).
+void err_means(const void *host_sums, int K, int C, int N, double *err, double *sp)
+{
+    const char *p = static_cast<const char *>(host_sums);
+    for (int k = 0; k < K; ++k) {
+        double e;
+        unsigned long long d;
+        std::memcpy(&e, p + sizeof(double) * k, sizeof e);
+        std::memcpy(&d, p + sizeof(double) * K + sizeof d * k, sizeof d);
+        err[k] = e / C;
+        sp[k] = (double)d / ((double)C * N);
+    }
+}
+
+sats_status layer_err_tc(const sats_layer *layer, const float *x, int C, const float *t, int K, float eps, double *err,
+                         double *sp, char *base, const ErrLayout &W, cudaStream_t st)
+{
+    char *mlp = base + W.mlp;
+    const size_t sum_bytes = ErrSums::bytes(K);
+    cudaError_t e = clear_fused_state(mlp, layer->H, layer->N, C, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(base + W.acc, 0, sum_bytes, st);
+    if (e != cudaSuccess) return cuda_fail(e, "layer error workspace clear");
+    const ErrInputs in(base + W.a, layer->H, layer->N, C);
+    sats_status s = enqueue_err_inputs(layer, x, C, in, base, W, st);
+    if (s == SATS_OK)
+        s = enqueue_err(layer, in, C, t, nullptr, [](int k) { return k; }, K, eps, ErrSums(base + W.acc, K), base, W, st);
+    if (s != SATS_OK) return s;
+    std::vector<char> h(sum_bytes);
+    e = cudaMemcpyAsync(h.data(), base + W.acc, sum_bytes, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e, "layer error read-back");
+    s = sats_get_error(mlp, ws_layout(layer->H, layer->N, C).total, st);
+    if (s != SATS_OK) return s;
+    err_means(h.data(), K, C, layer->N, err, sp);
+    return SATS_OK;
+}
+
+__global__ void __launch_bounds__(256) add_rows_kernel(float4 *__restrict__ x, const float4 *__restrict__ y, size_t n4)
+{
+    const size_t i = blockIdx.x * (size_t)256 + threadIdx.x;
+    if (i >= n4) return;
+    const float4 a = x[i], b = y[i];
+    x[i] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+
 struct SatsLayout {
-    size_t x, n, a, sel, q, err, total;
+    size_t x, n, a, sel, q, sums, in, in_each, err, total;   // in_each: 0 if the blocks share one
 };
 
 SatsLayout sats_layout(int H, int N, int C, int L, int K0, int K)
@@ -309,6 +394,13 @@ SatsLayout sats_layout(int H, int N, int C, int L, int K0, int K)
     off += al256(select_multi_ws_bytes(kSelRanks));
     S.q = off;   // every block's percentiles: the coarse candidates, the largest |a|, the guardrail's
     off += al256((size_t)L * (K0 + 1) * sizeof(float));
+    S.sums = off;   // every block's ErrSums
+    off += al256((size_t)L * ErrSums::bytes(K));
+    // every block's ErrInputs, kept from the coarse candidates for the fine ones, up to kErrKeep bytes
+    const size_t each = use_tc_path(H, C) ? ErrInputs::bytes(H, N, C) : 0;
+    S.in = off;
+    S.in_each = each * L <= kErrKeep ? each : 0;
+    off += S.in_each * L;
     S.err = off;
     off += err_layout(H, N, C, K).total;
     S.total = off;
@@ -462,7 +554,7 @@ sats_status sats_sats_select(const double *t, const double *err, const double *s
 size_t sats_sats_workspace_bytes(int H, int N, int C, int L, int K0, int K1)
 {
     if (H < 8 || H > kMaxH || (H % 8) != 0 || N < 1 || N > kMaxN || C < 1 || L < 1 || K0 < 2 || K1 < 0) return 0;
-    const int K = std::max(std::max(K0 - 1, K1), 1);
+    const int K = std::max(K0, K1);   // (the coarse candidates and the guardrail threshold)
     return sats_layout(H, N, C, L, K0, K).total;
 }
 
@@ -478,7 +570,7 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     const int H = layers[0] ? layers[0]->H : 0, N = layers[0] ? layers[0]->N : 0;
     for (int l = 0; l < L; ++l)
         if (!layers[l] || layers[l]->H != H || layers[l]->N != N || !norm_w[l]) return SATS_EINVAL;
-    const int Kc = K0 - 1, Kmax = std::max(std::max(Kc, K1), 1), Kt = Kc + K1;
+    const int Kc = K0 - 1, Kmax = std::max(Kc + 1, K1), Kt = Kc + K1;
     const SatsLayout W = sats_layout(H, N, C, L, K0, Kmax);
     if (ws_bytes < W.total) return SATS_ENOSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -488,15 +580,21 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     float *a = reinterpret_cast<float *>(base + W.a);
     void *sel = base + W.sel;
     float *q = reinterpret_cast<float *>(base + W.q);
-    void *ews = base + W.err;
+    char *ews = base + W.err;
+    const ErrLayout E = err_layout(H, N, C, Kmax);
+    char *sums = base + W.sums;
+    const size_t sum_bytes = ErrSums::bytes(Kmax);
+    const bool batched = use_tc_path(H, C);
+    auto inputs_of = [&](int l) { return ErrInputs(W.in_each ? base + W.in + l * W.in_each : ews + E.a, H, N, C); };
     const size_t ews_bytes = W.total - W.err;
-    void *mlp = base + W.err + err_layout(H, N, C, Kmax).mlp;
+    void *mlp = ews + E.mlp;
     auto n_of = [&](int l) { return nall + (size_t)l * C * H; };
     const int guard = guardrail ? L - 1 : -1;
 
     // 1-2: the dense stack gives each block's MLP inputs; coarse candidates from |SiLU(n W_gate)|
     cudaError_t e = cudaMemcpyAsync(x, x_cal, (size_t)C * H * sizeof(float), cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = clear_fused_state(mlp, H, N, C, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, W.in - W.q, st);   // (the sums follow the percentiles)
     if (e != cudaSuccess) return cuda_fail(e, "calibration set-up");
     std::vector<double> tc((size_t)L * Kc), amax((size_t)L), errc((size_t)L * Kc), spc((size_t)L * Kc);
     double g_t = 0.0, g_sp = 0.0;
@@ -509,19 +607,36 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
         if ((s = sats_gate_act_f32(layers[l], n_of(l), C, a, stream)) != SATS_OK) return s;
         // Eq. 3 at k / K0, the largest |a|, and the guardrail block's percentile at the target, all
         // from shared passes over |a|; read back once after the last block
+        float *ql = q + (size_t)l * (K0 + 1);
         const int nq = l == guard && s_tar > 0.0 ? Kc + 2 : Kc + 1;
-        for (int k = 0; k < nq; ++k) rank[(size_t)k] = percentile_rank(n, k < Kc ? (double)(k + 1) / K0 : k == Kc ? 1.0 : s_tar);
+        for (int k = 0; k < nq; ++k)
+            rank[(size_t)k] = percentile_rank(n, k < Kc ? (double)(k + 1) / K0 : k == Kc ? 1.0 : s_tar);
         for (int k = 0; k < nq; k += kSelRanks)
-            if ((e = launch_select(a, n, rank.data() + k, std::min(kSelRanks, nq - k), sel, q + (size_t)l * (K0 + 1) + k,
-                                   st)) != cudaSuccess)
+            if ((e = launch_select(a, n, rank.data() + k, std::min(kSelRanks, nq - k), sel, ql + k, st)) != cudaSuccess)
                 return cuda_fail(e, "percentile kernels launch");
+        if (batched) {
+            // 3: Eq. 6 for every coarse candidate (and, with them, the guardrail's CATS threshold), the
+            // thresholds read on the device; x <- x + MLP_l(n_l) takes the dense output from it
+            const int K = l == guard ? Kc + 1 : Kc;
+            if ((s = enqueue_err_inputs(layers[l], n_of(l), C, inputs_of(l), ews, E, st)) != SATS_OK) return s;
+            if ((s = enqueue_err(layers[l], inputs_of(l), C, nullptr, ql, [&](int k) { return k < Kc ? k : Kc + 1; }, K,
+                                 err_eps, ErrSums(sums + l * sum_bytes, K), ews, E, st)) != SATS_OK)
+                return s;
+            const size_t n4 = (size_t)C * H / 4;
+            add_rows_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(
+                reinterpret_cast<float4 *>(x), reinterpret_cast<const float4 *>(inputs_of(l).y), n4);
+            if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "residual kernel launch");
+            continue;
+        }
         // x <- x + MLP_l(n_l) with every neuron kept
         if ((s = run_layer(layers[l], kXF32, n_of(l), C, &zero, nullptr, 0.f, nullptr, kOutResid, x, nullptr,
                            nullptr, nullptr, mlp, st)) != SATS_OK)
             return s;
     }
     std::vector<float> qh((size_t)L * (K0 + 1), 0.f);
+    std::vector<char> hs((size_t)L * sum_bytes);
     e = cudaMemcpyAsync(qh.data(), q, qh.size() * sizeof(float), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && batched) e = cudaMemcpyAsync(hs.data(), sums, hs.size(), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "percentile read-back");
     for (int l = 0; l < L; ++l) {
@@ -530,25 +645,26 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
         amax[(size_t)l] = ql[Kc];
         if (l == guard) g_t = s_tar > 0.0 ? ql[Kc + 1] : 0.f;
     }
-    // 3: Eq. 6 for every coarse candidate (and the guardrail's CATS threshold)
+    if (batched && (s = sats_get_error(mlp, ws_layout(H, N, C).total, stream)) != SATS_OK) return s;
+    // 3 (without a batch): Eq. 6 block by block
     std::vector<float> tf((size_t)Kmax);
     std::vector<double> eb((size_t)Kmax), sb((size_t)Kmax);
     for (int l = 0; l < L; ++l) {
-        for (int k = 0; k < Kc; ++k) tf[(size_t)k] = (float)tc[(size_t)l * Kc + k];
-        if ((s = sats_layer_err(layers[l], n_of(l), C, tf.data(), Kc, err_eps, eb.data(), sb.data(), ews, ews_bytes,
-                                stream)) != SATS_OK)
-            return s;
+        const int K = l == guard ? Kc + 1 : Kc;
+        if (batched) {
+            err_means(hs.data() + l * sum_bytes, K, C, N, eb.data(), sb.data());
+        } else {
+            for (int k = 0; k < Kc; ++k) tf[(size_t)k] = (float)tc[(size_t)l * Kc + k];
+            if (l == guard) tf[(size_t)Kc] = (float)g_t;
+            if ((s = sats_layer_err(layers[l], n_of(l), C, tf.data(), K, err_eps, eb.data(), sb.data(), ews, ews_bytes,
+                                    stream)) != SATS_OK)
+                return s;
+        }
         for (int k = 0; k < Kc; ++k) {
             errc[(size_t)l * Kc + k] = eb[(size_t)k];
             spc[(size_t)l * Kc + k] = sb[(size_t)k];
         }
-        if (l == guard) {
-            const float gt = (float)g_t;
-            double ge = 0.0;
-            if ((s = sats_layer_err(layers[l], n_of(l), C, &gt, 1, err_eps, &ge, &g_sp, ews, ews_bytes, stream)) !=
-                SATS_OK)
-                return s;
-        }
+        if (l == guard) g_sp = sb[(size_t)Kc];
     }
     // 4: Eqs. 7-10 over the coarse candidates
     double b0 = 0.0, S0 = 0.0;
@@ -559,6 +675,9 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     // 5-6: K1 candidates strictly between the coarse neighbours of each block's choice, then
     // Eqs. 6-10 over coarse and fine candidates together
     std::vector<double> ta((size_t)L * Kt), ea((size_t)L * Kt), sa((size_t)L * Kt);
+    tf.assign((size_t)L * std::max(K1, 1), 0.f);
+    if (batched && K1 > 0 && (e = cudaMemsetAsync(sums, 0, (size_t)L * sum_bytes, st)) != cudaSuccess)
+        return cuda_fail(e, "layer error workspace clear");
     for (int l = 0; l < L; ++l) {
         double lo = 0.0, hi = amax[(size_t)l];
         bool above = false;
@@ -575,15 +694,29 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
             ea[(size_t)l * Kt + k] = errc[(size_t)l * Kc + k];
             sa[(size_t)l * Kt + k] = spc[(size_t)l * Kc + k];
         }
-        for (int k = 0; k < K1; ++k) tf[(size_t)k] = (float)(lo + (hi - lo) * (k + 1) / (K1 + 1));
-        if (K1 > 0 && (s = sats_layer_err(layers[l], n_of(l), C, tf.data(), K1, err_eps, eb.data(), sb.data(), ews,
-                                          ews_bytes, stream)) != SATS_OK)
-            return s;
         for (int k = 0; k < K1; ++k) {
-            ta[(size_t)l * Kt + Kc + k] = tf[(size_t)k];
-            ea[(size_t)l * Kt + Kc + k] = eb[(size_t)k];
-            sa[(size_t)l * Kt + Kc + k] = sb[(size_t)k];
+            const float t = (float)(lo + (hi - lo) * (k + 1) / (K1 + 1));
+            tf[(size_t)l * K1 + k] = t;
+            ta[(size_t)l * Kt + Kc + k] = t;
         }
+        if (K1 == 0) continue;
+        if (batched && W.in_each == 0 &&
+            (s = enqueue_err_inputs(layers[l], n_of(l), C, inputs_of(l), ews, E, st)) != SATS_OK)
+            return s;
+        s = batched ? enqueue_err(layers[l], inputs_of(l), C, tf.data() + (size_t)l * K1, nullptr, [](int k) { return k; },
+                                  K1, err_eps, ErrSums(sums + l * sum_bytes, K1), ews, E, st)
+                    : sats_layer_err(layers[l], n_of(l), C, tf.data() + (size_t)l * K1, K1, err_eps,
+                                     ea.data() + (size_t)l * Kt + Kc, sa.data() + (size_t)l * Kt + Kc, ews, ews_bytes,
+                                     stream);
+        if (s != SATS_OK) return s;
+    }
+    if (batched && K1 > 0) {
+        e = cudaMemcpyAsync(hs.data(), sums, hs.size(), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_fail(e, "layer error read-back");
+        if ((s = sats_get_error(mlp, ws_layout(H, N, C).total, stream)) != SATS_OK) return s;
+        for (int l = 0; l < L; ++l)
+            err_means(hs.data() + l * sum_bytes, K1, C, N, ea.data() + (size_t)l * Kt + Kc, sa.data() + (size_t)l * Kt + Kc);
     }
     double b = 0.0, S = 0.0;
     std::vector<double> tt((size_t)L);

@@ -1405,22 +1405,19 @@ bool skinny_batch(int B, bool split) { return B <= (split ? kMaxSkinnySplit : kM
 }  // namespace
 
 // Gate and up projections of B fp32 inputs with every neuron kept: h in bf16 parts and a =
-// SiLU(x W_gate) (row stride layer->ldn), for the calibration's masks.  tc_ws: the tensor-core
-// region of a workspace for B tokens; a_out [B][ldn].  In passes of up to kGateUpTokens tokens
+// SiLU(x W_gate) (all with row stride layer->ldn), for the calibration's masks.  tc_ws: the tensor-core
+// region of a workspace for B tokens.  In passes of up to kGateUpTokens tokens
 // of the skinny kernel, whose epilogue has a thread per neuron and writes a in whole lines.
 constexpr int kGateUpTokens = 128;
 
-cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void *tc_ws, const uint16_t **hact,
-                           const uint16_t **hact_lo, float *a_out, int *ctl, cudaStream_t stream)
+cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void *tc_ws, uint16_t *hhi, uint16_t *hlo,
+                           float *a_out, int *ctl, cudaStream_t stream)
 {
     const int H = layer->H;
     const size_t ldn = layer->ldn;
     const TcLayout W = tc_layout(H, layer->N, B);
     uint8_t *base = static_cast<uint8_t *>(tc_ws);
     uint16_t *xhi = reinterpret_cast<uint16_t *>(base + W.xhi), *xlo = reinterpret_cast<uint16_t *>(base + W.xlo);
-    uint16_t *hhi = reinterpret_cast<uint16_t *>(base + W.hact), *hlo = reinterpret_cast<uint16_t *>(base + W.hact_lo);
-    *hact = hhi;
-    *hact_lo = hlo;
     cudaError_t e = launch_pdl_threads(split_kernel, dim3(B), 256, stream, x, H, static_cast<const float *>(nullptr), 0.f,
                                        xhi, xlo, static_cast<const int32_t *>(nullptr));
     if (e != cudaSuccess) return fail(e, "split kernel launch");
