@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     uint64_t *mma_done = acc_empty + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
     __shared__ int abort_flag, issued_s, consumed_s;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const int R = p.R, NT = p.NT, S = p.stages, KBh = p.KBh;
     const int m0 = (int)blockIdx.x * NT, t = blockIdx.y;
     const int n_quads = (R + 31) / 32;   // TMEM lane quarters that hold neurons
@@ -207,18 +207,20 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     const uint32_t tmem = *tmem_slot;
     grid_launch_dependents();
 
+    // (one lane runs the load role here: 256 bf16 tokens took 69 us so and 75 with a whole warp)
     if (warp == 0 && lane == 0) {
+        const uint32_t lead = 1u;
         const uint32_t load_bytes = (uint32_t)p.w_bytes + (F32 ? 0u : (uint32_t)(NT * kTileBytes));
         // (each weight tile is read once with one token tile, else by its neighbours through L2)
         const uint64_t once = l2_policy_evict_first();
         auto load_w = [&](int s, int kb) {
             const uint16_t *src = p.w + (size_t)((size_t)t * KBh + kb) * 2 * R * BK;
-            if (gridDim.x == 1) bulk_load(ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s], once);
-            else bulk_load_shared(ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s]);
+            if (gridDim.x == 1) bulk_load_if(lead, ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s], once);
+            else bulk_load_shared_if(lead, ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s]);
         };
         const int npre = KBh < S ? KBh : S;
         for (int i = 0; i < npre; ++i) {   // the weights do not depend on the preceding kernel
-            mbar_arrive_expect_tx(&full[i], load_bytes);
+            mbar_expect_if(lead, &full[i], load_bytes);
             load_w(i, i);
         }
         if (!F32) grid_dependency_wait();
@@ -226,21 +228,22 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
         for (int s = 0, ph = 0; kb < KBh; ++kb) {
             if (kb >= npre) {
                 if (!mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { abort_flag = 1; break; }
-                mbar_arrive_expect_tx(&full[s], load_bytes);
+                mbar_expect_if(lead, &full[s], load_bytes);
                 load_w(s, kb);
             }
-            if (!F32) tma_load(ring + (size_t)s * p.stage_bytes + p.w_bytes, &tmX, kb * BK, m0, &full[s]);
+            if (!F32) tma_load_if(lead, ring + (size_t)s * p.stage_bytes + p.w_bytes, &tmX, kb * BK, m0, &full[s]);
             if (++s == S) { s = 0; ph ^= 1; }
         }
         issued_s = kb;
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+        const uint32_t lead = elect_one();
         const uint32_t idesc = instr_desc(BM, NT);
         int kb = 0;
         for (int s = 0, ph = 0; kb < KBh; ++kb) {
             const int buf = kb & 1, ps = kb % kPartStages;
             const uint32_t bph = (uint32_t)((kb >> 1) & 1);
-            if (!mbar_wait(&acc_empty[buf], bph ^ 1u, &abort_flag) || !mbar_wait(&full[s], (uint32_t)ph, &abort_flag) ||
-                (F32 && !mbar_wait(&pfull[ps], (uint32_t)((kb / kPartStages) & 1), &abort_flag))) {
+            if (!warp_wait(&acc_empty[buf], bph ^ 1u, &abort_flag) || !warp_wait(&full[s], (uint32_t)ph, &abort_flag) ||
+                (F32 && !warp_wait(&pfull[ps], (uint32_t)((kb / kPartStages) & 1), &abort_flag))) {
                 abort_flag = 1;
                 break;
             }
@@ -254,16 +257,16 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                 for (int q = kXParts - 1; q >= 0; --q)   // the smallest part first
 #pragma unroll
                     for (int kk = 2 * half; kk < 2 * half + 2; ++kk)
-                        mma_bf16(d, smem_desc(st + kk * 32), smem_desc(xs + q * NT * kTileBytes + kk * 32), idesc,
+                        mma_bf16_if(lead, d, smem_desc(st + kk * 32), smem_desc(xs + q * NT * kTileBytes + kk * 32), idesc,
                                  (q < kXParts - 1 || (kk & 1)) ? 1u : 0u);
             }
-            mma_commit(&empty[s]);
-            if (F32) mma_commit(&pempty[ps]);
-            mma_commit(&acc_full[buf]);
+            mma_commit_if(lead, &empty[s]);
+            if (F32) mma_commit_if(lead, &pempty[ps]);
+            mma_commit_if(lead, &acc_full[buf]);
             if (++s == S) { s = 0; ph ^= 1; }
         }
         consumed_s = kb;
-        mma_commit(mma_done);
+        mma_commit_if(lead, mma_done);
     } else if (F32 && warp >= 2 && warp < kEpi0) {
         grid_dependency_wait();
         auto load = [&](int r, int c, int kb, float4 &lo, float4 &hi) {
@@ -486,7 +489,7 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
     __shared__ int abort_flag, issued_s, consumed_s;
     __shared__ float zs[kLoraTok][kLoraZRow];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const int R = p.R, NT = p.NT, S = p.stages, KBh = p.KBh, halves = p.halves;
     const int NX = kXParts * NT;   // accumulator columns: the parts side by side
     const int m0 = (int)blockIdx.x * NT, t = blockIdx.y;
@@ -517,40 +520,42 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
     const uint32_t tmem = *tmem_slot;
     grid_launch_dependents();
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
+        const uint32_t lead = elect_one();
         const uint32_t load_bytes = (uint32_t)p.w_bytes + (F32 ? 0u : (uint32_t)(NT * kTileBytes));
         const uint64_t once = l2_policy_evict_first();
         auto load_w = [&](int s, int kb) {
             const uint16_t *src = p.w + ((size_t)t * KBh + kb) * 2 * R * BK;
-            if (gridDim.x == 1) bulk_load(ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s], once);
-            else bulk_load_shared(ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s]);
+            if (gridDim.x == 1) bulk_load_if(lead, ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s], once);
+            else bulk_load_shared_if(lead, ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s]);
         };
         const int npre = KBh < S ? KBh : S;
         for (int i = 0; i < npre; ++i) {
-            mbar_arrive_expect_tx(&full[i], load_bytes);
+            mbar_expect_if(lead, &full[i], load_bytes);
             load_w(i, i);
         }
         if (!F32) grid_dependency_wait();
         int kb = 0;
         for (int s = 0, ph = 0; kb < KBh; ++kb) {
             if (kb >= npre) {
-                if (!mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
-                mbar_arrive_expect_tx(&full[s], load_bytes);
+                if (!warp_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
+                mbar_expect_if(lead, &full[s], load_bytes);
                 load_w(s, kb);
             }
-            if (!F32) tma_load(ring + (size_t)s * p.stage_bytes + p.w_bytes, &tmX, kb * BK, m0, &full[s]);
+            if (!F32) tma_load_if(lead, ring + (size_t)s * p.stage_bytes + p.w_bytes, &tmX, kb * BK, m0, &full[s]);
             if (++s == S) { s = 0; ph ^= 1; }
         }
         issued_s = kb;
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+        const uint32_t lead = elect_one();
         const uint32_t idesc = instr_desc(BM, NX);
         const int per = 4 / halves;   // K = 16 steps per accumulator
         int kb = 0;
         for (int s = 0, ph = 0; kb < KBh; ++kb) {
             const int buf = kb & 1, ps = kb % kPartStages;
-            if (!mbar_wait(&acc_empty[buf], (uint32_t)((kb >> 1) & 1) ^ 1u, &abort_flag) ||
-                !mbar_wait(&full[s], (uint32_t)ph, &abort_flag) ||
-                (F32 && !mbar_wait(&pfull[ps], (uint32_t)((kb / kPartStages) & 1), &abort_flag))) {
+            if (!warp_wait(&acc_empty[buf], (uint32_t)((kb >> 1) & 1) ^ 1u, &abort_flag) ||
+                !warp_wait(&full[s], (uint32_t)ph, &abort_flag) ||
+                (F32 && !warp_wait(&pfull[ps], (uint32_t)((kb / kPartStages) & 1), &abort_flag))) {
                 set_timeout(p.ctl, &abort_flag);
                 break;
             }
@@ -561,16 +566,16 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
             for (int kk = 0; kk < BK / 16; ++kk) {
                 const uint32_t d = tmem + (uint32_t)((buf * halves + kk / per) * 2 * NX), acc = kk % per ? 1u : 0u;
                 const uint64_t b = smem_desc(xs + kk * 32);
-                mma_bf16(d, smem_desc(st + kk * 32), b, idesc, acc);
-                mma_bf16(d + NX, smem_desc(st + R * kTileBytes + kk * 32), b, idesc, acc);
+                mma_bf16_if(lead, d, smem_desc(st + kk * 32), b, idesc, acc);
+                mma_bf16_if(lead, d + NX, smem_desc(st + R * kTileBytes + kk * 32), b, idesc, acc);
             }
-            mma_commit(&empty[s]);
-            if (F32) mma_commit(&pempty[ps]);
-            mma_commit(&acc_full[buf]);
+            mma_commit_if(lead, &empty[s]);
+            if (F32) mma_commit_if(lead, &pempty[ps]);
+            mma_commit_if(lead, &acc_full[buf]);
             if (++s == S) { s = 0; ph ^= 1; }
         }
         consumed_s = kb;
-        mma_commit(mma_done);
+        mma_commit_if(lead, mma_done);
     } else if (F32 && warp >= 2 && warp < kEpi0) {
         grid_dependency_wait();
         auto load = [&](int r, int c, int kb, float4 &lo, float4 &hi) {
@@ -724,7 +729,7 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
     __shared__ int abort_flag, issued_s, consumed_s;
     __shared__ float tr[kLoraEpiThreads / 32][16][33];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const int NT = p.NT, S = p.stages, KBn = p.KBn, halves = p.halves, NX = kParts * NT;
     const int m0 = (int)blockIdx.y * NT;
     const int u0 = (int)((long long)blockIdx.x * p.units / gridDim.x);
@@ -757,31 +762,33 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
     const uint32_t tmem = *tmem_slot;
     grid_launch_dependents();
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
+        const uint32_t lead = elect_one();
         // nothing but weights is copied, so the whole stream runs ahead of the preceding kernel's end
         const uint64_t once = l2_policy_evict_first();
         int i = 0;
         for (int s = 0, ph = 0; i < nu; ++i) {
-            if (!mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
+            if (!warp_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
             const int u = u0 + i, d = u / KBn;
             const bool ad = d == p.dt;
             const uint32_t bytes = (uint32_t)((ad ? kMaxLoraRank : BM) * kTileBytes);
             const uint16_t *src = ad ? p.ad + (size_t)(u - d * KBn) * kMaxLoraRank * BK : p.w + (size_t)u * BM * BK;
-            mbar_arrive_expect_tx(&full[s], bytes);
-            if (gridDim.y == 1) bulk_load(ring + (size_t)s * kA, src, bytes, &full[s], once);
-            else bulk_load_shared(ring + (size_t)s * kA, src, bytes, &full[s]);
+            mbar_expect_if(lead, &full[s], bytes);
+            if (gridDim.y == 1) bulk_load_if(lead, ring + (size_t)s * kA, src, bytes, &full[s], once);
+            else bulk_load_shared_if(lead, ring + (size_t)s * kA, src, bytes, &full[s]);
             if (++s == S) { s = 0; ph ^= 1; }
         }
         issued_s = i;
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+        const uint32_t lead = elect_one();
         const uint32_t idesc = instr_desc(BM, NX);
         const int per = 4 / halves;
         int i = 0;
         for (int s = 0, ph = 0; i < nu; ++i) {
             const int buf = i & 1, ps = i % kPartStages;
-            if (!mbar_wait(&acc_empty[buf], (uint32_t)((i >> 1) & 1) ^ 1u, &abort_flag) ||
-                !mbar_wait(&full[s], (uint32_t)ph, &abort_flag) ||
-                !mbar_wait(&pfull[ps], (uint32_t)((i / kPartStages) & 1), &abort_flag)) {
+            if (!warp_wait(&acc_empty[buf], (uint32_t)((i >> 1) & 1) ^ 1u, &abort_flag) ||
+                !warp_wait(&full[s], (uint32_t)ph, &abort_flag) ||
+                !warp_wait(&pfull[ps], (uint32_t)((i / kPartStages) & 1), &abort_flag)) {
                 set_timeout(p.ctl, &abort_flag);
                 break;
             }
@@ -790,15 +797,15 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
             const uint32_t hs = smem_addr(parts + (size_t)ps * kParts * NT * kTileBytes);
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
-                mma_bf16(tmem + (uint32_t)((buf * halves + kk / per) * NX), smem_desc(st + kk * 32),
+                mma_bf16_if(lead, tmem + (uint32_t)((buf * halves + kk / per) * NX), smem_desc(st + kk * 32),
                          smem_desc(hs + kk * 32), idesc, kk % per ? 1u : 0u);
-            mma_commit(&empty[s]);
-            mma_commit(&pempty[ps]);
-            mma_commit(&acc_full[buf]);
+            mma_commit_if(lead, &empty[s]);
+            mma_commit_if(lead, &pempty[ps]);
+            mma_commit_if(lead, &acc_full[buf]);
             if (++s == S) { s = 0; ph ^= 1; }
         }
         consumed_s = i;
-        mma_commit(mma_done);
+        mma_commit_if(lead, mma_done);
     } else if (warp >= 2 && warp < kEpi0) {
         grid_dependency_wait();   // h is written by the preceding gate/up kernel
         auto load = [&](int r, int c, int step, float4 &lo, float4 &hi) {

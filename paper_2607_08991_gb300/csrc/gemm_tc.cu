@@ -36,8 +36,8 @@
 // The weights are read from tile-contiguous copies made at layer creation
 // (gu_blk, wd_blk), so that every TMA box is one contiguous DRAM read.
 //
-// Kernel layout (64 + 128 G threads): warp 0 lane 0 issues the TMA loads, warp 1
-// owns the TMEM allocation and lane 0 issues the MMAs, warps 2 .. 4 G + 1 run the
+// Kernel layout (64 + 128 G threads): warp 0 issues the TMA loads, warp 1 owns the
+// TMEM allocation and issues the MMAs (each through one elected lane), warps 2 .. 4 G + 1 run the
 // epilogue in G groups of four (warp w reads TMEM lanes 32 (w mod 4) .. 32 (w mod
 // 4) + 31; the groups split the accumulator's columns; G = 1 in the down kernel of
 // batched decode, up to seven in its gate/up kernel, four in the prefill kernels).
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kSkinnyMaxThreads, 1)
     uint64_t *acc_full = empty + kMaxStages;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_full + 1);
     __shared__ int abort_flag, issued_s, consumed_s;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const int t = blockIdx.x, R = p.R, NT = p.NT, S = p.stages;
     const int NX = p.merge ? 2 * NT : NT;   // accumulator columns per matrix: tokens, or their high then low parts
 
@@ -235,15 +235,16 @@ __global__ void __launch_bounds__(kSkinnyMaxThreads, 1)
     const uint32_t tmem = *tmem_slot;
     grid_launch_dependents();   // the down projection may start prefetching its weights
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
+        const uint32_t lead = elect_one();
         const uint32_t w_bytes = (uint32_t)((p.gate_only ? 1 : 2) * R * kTileBytes);
         const uint32_t load_bytes = w_bytes + (uint32_t)(p.x_bytes * (p.split ? 2 : 1));
         const uint64_t policy = l2_policy_evict_first();   // each weight tile is read by this CTA only
         // the weight tiles do not depend on the preceding kernel: start them before waiting for it
         const int npre = p.KBh < S ? p.KBh : S;
         for (int i = 0; i < npre; ++i) {
-            mbar_arrive_expect_tx(&full[i], load_bytes);
-            bulk_load(ring + (size_t)i * p.stage_bytes, p.w + (size_t)(t * p.KBh + i) * 2 * R * BK, w_bytes, &full[i],
+            mbar_expect_if(lead, &full[i], load_bytes);
+            bulk_load_if(lead, ring + (size_t)i * p.stage_bytes, p.w + (size_t)(t * p.KBh + i) * 2 * R * BK, w_bytes, &full[i],
                       policy);
         }
         grid_dependency_wait();   // x (and this call's buffers) may belong to the preceding kernel
@@ -251,23 +252,24 @@ __global__ void __launch_bounds__(kSkinnyMaxThreads, 1)
         for (int s = 0, ph = 0; kb < p.KBh; ++kb) {
             uint8_t *st = ring + (size_t)s * p.stage_bytes;
             if (kb >= npre) {
-                if (!mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
-                mbar_arrive_expect_tx(&full[s], load_bytes);
-                bulk_load(st, p.w + (size_t)(t * p.KBh + kb) * 2 * R * BK, w_bytes, &full[s], policy);
+                if (!warp_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
+                mbar_expect_if(lead, &full[s], load_bytes);
+                bulk_load_if(lead, st, p.w + (size_t)(t * p.KBh + kb) * 2 * R * BK, w_bytes, &full[s], policy);
             }
-            tma_load(st + p.a_bytes, &tmX, kb * BK, 0, &full[s]);
-            if (p.split) tma_load(st + p.a_bytes + p.x_bytes, &tmX2, kb * BK, 0, &full[s]);
+            tma_load_if(lead, st + p.a_bytes, &tmX, kb * BK, 0, &full[s]);
+            if (p.split) tma_load_if(lead, st + p.a_bytes + p.x_bytes, &tmX2, kb * BK, 0, &full[s]);
             if (++s == S) { s = 0; ph ^= 1; }
         }
         issued_s = kb;   // a break happens only before stage kb's loads are issued (kb >= npre)
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+        const uint32_t lead = elect_one();
         // x's high and low parts sit back to back in the stage (one 2 NT-row tile): merged,
         // one MMA of N = 2 NT covers both, its two column halves summed in the epilogue;
         // otherwise (N would pass 256) a second MMA adds the low part into the same columns
         const uint32_t idesc = instr_desc(BM, NX);
         int kb = 0;
         for (int s = 0, ph = 0; kb < p.KBh; ++kb) {
-            if (!mbar_wait(&full[s], (uint32_t)ph, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
+            if (!warp_wait(&full[s], (uint32_t)ph, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
             tc_fence_after();
             const uint32_t st = smem_addr(ring + (size_t)s * p.stage_bytes);
             const uint32_t xa = st + p.a_bytes;
@@ -277,19 +279,19 @@ __global__ void __launch_bounds__(kSkinnyMaxThreads, 1)
                 const uint64_t ag = smem_desc(st + kk * 32);
                 const uint64_t au = smem_desc(st + R * kTileBytes + kk * 32);
                 const uint64_t b = smem_desc(xa + kk * 32);
-                mma_bf16(tmem, ag, b, idesc, acc);
-                if (!p.gate_only) mma_bf16(tmem + NX, au, b, idesc, acc);
+                mma_bf16_if(lead, tmem, ag, b, idesc, acc);
+                if (!p.gate_only) mma_bf16_if(lead, tmem + NX, au, b, idesc, acc);
                 if (p.split && !p.merge) {
                     const uint64_t b2 = smem_desc(xa + p.x_bytes + kk * 32);
-                    mma_bf16(tmem, ag, b2, idesc, 1u);
-                    if (!p.gate_only) mma_bf16(tmem + NX, au, b2, idesc, 1u);
+                    mma_bf16_if(lead, tmem, ag, b2, idesc, 1u);
+                    if (!p.gate_only) mma_bf16_if(lead, tmem + NX, au, b2, idesc, 1u);
                 }
             }
-            mma_commit(&empty[s]);
+            mma_commit_if(lead, &empty[s]);
             if (++s == S) { s = 0; ph ^= 1; }
         }
         consumed_s = kb;
-        mma_commit(acc_full);
+        mma_commit_if(lead, acc_full);
     } else if (warp >= 2) {
         grid_dependency_wait();   // y, h and the keep bytes may still be in use by the preceding kernel
         if (p.zero) {
@@ -407,7 +409,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint64_t *mma_done = acc_empty + 2;        // every MMA of this CTA has completed
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
     __shared__ int abort_flag, issued_s, consumed_s;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const int S = p.stages, NT = p.NT, KBn = p.KBn;
     const int NX = p.merge ? 2 * NT : NT;
     const int u0 = (int)((long long)blockIdx.x * p.units / gridDim.x);
@@ -436,15 +438,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem = *tmem_slot;
     grid_launch_dependents();   // the next call's kernels may start their prologue as SMs free up
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
+        const uint32_t lead = elect_one();
         const uint32_t w_bytes = (uint32_t)(BM * kTileBytes);
         const uint32_t load_bytes = w_bytes + (uint32_t)(2 * NT * kTileBytes);
         const uint64_t policy = l2_policy_evict_first();
         // the weight tiles do not depend on the preceding kernel: start them first
         const int npre = nu < S ? nu : S;
         for (int i = 0; i < npre; ++i) {
-            mbar_arrive_expect_tx(&full[i], load_bytes);
-            bulk_load(ring + (size_t)i * p.stage_bytes, p.w + (size_t)(u0 + i) * BM * BK, w_bytes, &full[i], policy);
+            mbar_expect_if(lead, &full[i], load_bytes);
+            bulk_load_if(lead, ring + (size_t)i * p.stage_bytes, p.w + (size_t)(u0 + i) * BM * BK, w_bytes, &full[i], policy);
         }
         grid_dependency_wait();   // h is written by the preceding gate/up kernel
         int i = 0;
@@ -452,50 +455,56 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int u = u0 + i;
             uint8_t *st = ring + (size_t)s * p.stage_bytes;
             if (i >= npre) {
-                if (!mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
-                mbar_arrive_expect_tx(&full[s], load_bytes);
-                bulk_load(st, p.w + (size_t)u * BM * BK, w_bytes, &full[s], policy);
+                if (!warp_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
+                mbar_expect_if(lead, &full[s], load_bytes);
+                bulk_load_if(lead, st, p.w + (size_t)u * BM * BK, w_bytes, &full[s], policy);
             }
-            tma_load(st + p.a_bytes, &tmH, (u % KBn) * BK, 0, &full[s]);
-            tma_load(st + p.a_bytes + NT * kTileBytes, &tmH2, (u % KBn) * BK, 0, &full[s]);
+            tma_load_if(lead, st + p.a_bytes, &tmH, (u % KBn) * BK, 0, &full[s]);
+            tma_load_if(lead, st + p.a_bytes + NT * kTileBytes, &tmH2, (u % KBn) * BK, 0, &full[s]);
             if (++s == S) { s = 0; ph ^= 1; }
         }
         issued_s = i;   // a break happens only before stage i's loads are issued (i >= npre)
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+        const uint32_t lead = elect_one();
         const uint32_t idesc = instr_desc(BM, NX);
         int i = 0, q = 0;
         int s = 0, ph = 0;
-        for (int u = u0; u < u1 && !abort_flag;) {
+        bool stop = false;
+        for (int u = u0; u < u1 && !stop;) {
             const int seg_end = min(u1, (u / KBn + 1) * KBn);
             const int buf = q & 1;
-            if (!mbar_wait(&acc_empty[buf], (uint32_t)((q >> 1) & 1) ^ 1u, &abort_flag)) {
+            if (!warp_wait(&acc_empty[buf], (uint32_t)((q >> 1) & 1) ^ 1u, &abort_flag)) {
                 set_timeout(p.ctl, &abort_flag);
                 break;
             }
             tc_fence_after();
             bool first = true;
             for (; u < seg_end; ++u, ++i) {
-                if (!mbar_wait(&full[s], (uint32_t)ph, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
+                if (!warp_wait(&full[s], (uint32_t)ph, &abort_flag)) {
+                    set_timeout(p.ctl, &abort_flag);
+                    stop = true;
+                    break;
+                }
                 tc_fence_after();
                 const uint32_t st = smem_addr(ring + (size_t)s * p.stage_bytes);
 #pragma unroll
                 for (int kk = 0; kk < BK / 16; ++kk) {
                     const uint64_t w = smem_desc(st + kk * 32);
-                    mma_bf16(tmem + (uint32_t)(buf * NX), w, smem_desc(st + p.a_bytes + kk * 32), idesc,
+                    mma_bf16_if(lead, tmem + (uint32_t)(buf * NX), w, smem_desc(st + p.a_bytes + kk * 32), idesc,
                              (first && kk == 0) ? 0u : 1u);
                     if (!p.merge)
-                        mma_bf16(tmem + (uint32_t)(buf * NX), w, smem_desc(st + p.a_bytes + NT * kTileBytes + kk * 32),
+                        mma_bf16_if(lead, tmem + (uint32_t)(buf * NX), w, smem_desc(st + p.a_bytes + NT * kTileBytes + kk * 32),
                                  idesc, 1u);
                 }
                 first = false;
-                mma_commit(&empty[s]);
+                mma_commit_if(lead, &empty[s]);
                 if (++s == S) { s = 0; ph ^= 1; }
             }
-            mma_commit(&acc_full[buf]);
+            mma_commit_if(lead, &acc_full[buf]);
             ++q;
         }
         consumed_s = i;
-        mma_commit(mma_done);
+        mma_commit_if(lead, mma_done);
     } else if (warp >= 2) {
         // a warp's 32 rows x 16 tokens go through shared memory, so that each lane adds four
         // vectors of four consecutive hidden units of one token (vector reductions in L2)
@@ -612,7 +621,7 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
     uint64_t *mma_done = acc_empty + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
     __shared__ int abort_flag, issued_s, consumed_s;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const int R = p.R, Rw = p.Rw, S = p.stages, KBh = p.KBh;
     const int wofs = kA * (p.split ? 2 : 1);
 
@@ -637,13 +646,14 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
+        const uint32_t lead = elect_one();
         // a wide tile's gate (and up) rows lie in at most two tiles of gu_blk: la rows from row r0
         // of tile t0, then lb rows from the start of tile t0 + 1 (the host keeps Rw - gcd(Rw, R)
         // <= R).  R and Rw are multiples of 16, so each piece keeps its rows' swizzle phase.  Rows
         // past the last packed tile are not loaded: their columns of D belong to neurons >= N,
         // which the epilogue skips.  Offsets in rows of BK elements at K block 0, worked out
-        // once per tile: this one thread's per-stage work must stay well below a stage's MMAs.
+        // once per tile: the issuing warp's per-stage work must stay well below a stage's MMAs.
         struct Pieces {
             size_t a, b;
             int la, lb;
@@ -678,8 +688,8 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
             if (go) {
                 const size_t o = (size_t)pkb * kb_rows;
                 for (int g = 0; g < 2; ++g) {
-                    bulk_prefetch_l2(p.w + (pf.a + o + g * R) * BK, (uint32_t)(pf.la * kTileBytes));
-                    if (pf.lb) bulk_prefetch_l2(p.w + (pf.b + o + g * R) * BK, (uint32_t)(pf.lb * kTileBytes));
+                    bulk_prefetch_l2_if(lead, p.w + (pf.a + o + g * R) * BK, (uint32_t)(pf.la * kTileBytes));
+                    if (pf.lb) bulk_prefetch_l2_if(lead, p.w + (pf.b + o + g * R) * BK, (uint32_t)(pf.lb * kTileBytes));
                 }
             }
             if (++pkb == KBh) {
@@ -696,21 +706,21 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
             const Pieces pc = pieces_of(q / p.mtiles);
             const uint32_t load_bytes = (uint32_t)(wofs + 2 * (pc.la + pc.lb) * kTileBytes);
             for (int kb = 0; kb < KBh; ++kb, ++i) {
-                if (!mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) {
+                if (!warp_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) {
                     set_timeout(p.ctl, &abort_flag);
                     stop = true;
                     break;
                 }
                 uint8_t *st = ring + (size_t)s * p.stage_bytes;
-                mbar_arrive_expect_tx(&full[s], load_bytes);
-                tma_load(st, &tmX, kb * BK, m0, &full[s]);
-                if (p.split) tma_load(st + kA, &tmX2, kb * BK, m0, &full[s]);
+                mbar_expect_if(lead, &full[s], load_bytes);
+                tma_load_if(lead, st, &tmX, kb * BK, m0, &full[s]);
+                if (p.split) tma_load_if(lead, st + kA, &tmX2, kb * BK, m0, &full[s]);
                 const size_t o = (size_t)kb * kb_rows;
                 for (int g = 0; g < 2; ++g) {
                     uint8_t *dst = st + wofs + g * Rw * kTileBytes;
-                    bulk_load_shared(dst, p.w + (pc.a + o + g * R) * BK, (uint32_t)(pc.la * kTileBytes), &full[s]);
+                    bulk_load_shared_if(lead, dst, p.w + (pc.a + o + g * R) * BK, (uint32_t)(pc.la * kTileBytes), &full[s]);
                     if (pc.lb)
-                        bulk_load_shared(dst + pc.la * kTileBytes, p.w + (pc.b + o + g * R) * BK,
+                        bulk_load_shared_if(lead, dst + pc.la * kTileBytes, p.w + (pc.b + o + g * R) * BK,
                                          (uint32_t)(pc.lb * kTileBytes), &full[s]);
                 }
                 prefetch_ahead();
@@ -718,7 +728,8 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
             }
         }
         issued_s = i;
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+        const uint32_t lead = elect_one();
         // gate rows and up rows are adjacent in the stage: one MMA with N = 2Rw writes the gate
         // accumulator to columns [0, Rw) and the up accumulator to [Rw, 2Rw)
         const uint32_t idesc = instr_desc(BM, 2 * Rw);
@@ -726,14 +737,14 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
         bool stop = false;
         for (int q = blockIdx.x; q < p.tiles && !stop; q += gridDim.x, ++it) {
             const int buf = it & 1;
-            if (!mbar_wait(&acc_empty[buf], (uint32_t)((it >> 1) & 1) ^ 1u, &abort_flag)) {
+            if (!warp_wait(&acc_empty[buf], (uint32_t)((it >> 1) & 1) ^ 1u, &abort_flag)) {
                 set_timeout(p.ctl, &abort_flag);
                 break;
             }
             tc_fence_after();
             const uint32_t d = tmem + (uint32_t)(buf * 2 * Rw);
             for (int kb = 0; kb < KBh; ++kb, ++i) {
-                if (!mbar_wait(&full[s], (uint32_t)ph, &abort_flag)) {
+                if (!warp_wait(&full[s], (uint32_t)ph, &abort_flag)) {
                     set_timeout(p.ctl, &abort_flag);
                     stop = true;
                     break;
@@ -744,16 +755,16 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
 #pragma unroll
                 for (int kk = 0; kk < BK / 16; ++kk) {
                     const uint64_t w = smem_desc(wa + kk * 32);
-                    mma_bf16(d, smem_desc(st + kk * 32), w, idesc, (kb | kk) ? 1u : 0u);
-                    if (p.split) mma_bf16(d, smem_desc(st + kA + kk * 32), w, idesc, 1u);
+                    mma_bf16_if(lead, d, smem_desc(st + kk * 32), w, idesc, (kb | kk) ? 1u : 0u);
+                    if (p.split) mma_bf16_if(lead, d, smem_desc(st + kA + kk * 32), w, idesc, 1u);
                 }
-                mma_commit(&empty[s]);
+                mma_commit_if(lead, &empty[s]);
                 if (++s == S) { s = 0; ph ^= 1; }
             }
-            mma_commit(&acc_full[buf]);
+            mma_commit_if(lead, &acc_full[buf]);
         }
         consumed_s = i;
-        mma_commit(mma_done);
+        mma_commit_if(lead, mma_done);
     } else if (warp >= 2) {
         if (p.zero) {
             // this CTA's share of y, cleared for the down projection's additions while the first
@@ -882,7 +893,7 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
     uint64_t *mma_done = acc_empty + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
     __shared__ int abort_flag, issued_s, consumed_s;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const int S = p.stages, BN = BM * p.dtiles, KBn = p.KBn;
     const int per_split = p.mtiles * p.dcols;
     // unit u -> its token tile's first row, first hidden tile and K-block range
@@ -915,7 +926,8 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
+        const uint32_t lead = elect_one();
         const uint32_t load_bytes = (uint32_t)(2 * kA + BN * kTileBytes);
         // L2 prefetch kWidePrefetch stages ahead (this CTA's own sequence of units): the weight
         // tiles by the CTAs of the first two token tiles, the h tiles by every fourth unit column;
@@ -933,10 +945,10 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
             if (pu >= p.units) return;
             if (pf_w)
                 for (int q = 0; q < p.dtiles; ++q)
-                    bulk_prefetch_l2(p.w + ((size_t)(pd0 + q) * KBn + pkb) * BM * BK, (uint32_t)kA);
+                    bulk_prefetch_l2_if(lead, p.w + ((size_t)(pd0 + q) * KBn + pkb) * BM * BK, (uint32_t)kA);
             if (pf_h) {
-                tma_prefetch_l2(&tmH, pkb * BK, pm0);
-                tma_prefetch_l2(&tmH2, pkb * BK, pm0);
+                tma_prefetch_l2_if(lead, &tmH, pkb * BK, pm0);
+                tma_prefetch_l2_if(lead, &tmH2, pkb * BK, pm0);
             }
             if (++pkb == pkb1) {
                 pu += gridDim.x;
@@ -950,24 +962,25 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
             int m0, d0, kb0, kb1;
             unit(u, m0, d0, kb0, kb1);
             for (int kb = kb0; kb < kb1; ++kb, ++i) {
-                if (!mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) {
+                if (!warp_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) {
                     set_timeout(p.ctl, &abort_flag);
                     stop = true;
                     break;
                 }
                 uint8_t *st = ring + (size_t)s * p.stage_bytes;
-                mbar_arrive_expect_tx(&full[s], load_bytes);
-                tma_load(st, &tmH, kb * BK, m0, &full[s]);
-                tma_load(st + kA, &tmH2, kb * BK, m0, &full[s]);
+                mbar_expect_if(lead, &full[s], load_bytes);
+                tma_load_if(lead, st, &tmH, kb * BK, m0, &full[s]);
+                tma_load_if(lead, st + kA, &tmH2, kb * BK, m0, &full[s]);
                 for (int q = 0; q < p.dtiles; ++q)
-                    bulk_load_shared(st + 2 * kA + q * kA, p.w + ((size_t)(d0 + q) * KBn + kb) * BM * BK,
+                    bulk_load_shared_if(lead, st + 2 * kA + q * kA, p.w + ((size_t)(d0 + q) * KBn + kb) * BM * BK,
                                      (uint32_t)kA, &full[s]);
                 prefetch_ahead();
                 if (++s == S) { s = 0; ph ^= 1; }
             }
         }
         issued_s = i;
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+        const uint32_t lead = elect_one();
         const uint32_t idesc = instr_desc(BM, BN);
         int i = 0, s = 0, ph = 0, it = 0;
         bool stop = false;
@@ -975,14 +988,14 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
             int m0, d0, kb0, kb1;
             unit(u, m0, d0, kb0, kb1);
             const int buf = it & 1;
-            if (!mbar_wait(&acc_empty[buf], (uint32_t)((it >> 1) & 1) ^ 1u, &abort_flag)) {
+            if (!warp_wait(&acc_empty[buf], (uint32_t)((it >> 1) & 1) ^ 1u, &abort_flag)) {
                 set_timeout(p.ctl, &abort_flag);
                 break;
             }
             tc_fence_after();
             const uint32_t d = tmem + (uint32_t)(buf * BN);
             for (int kb = kb0; kb < kb1; ++kb, ++i) {
-                if (!mbar_wait(&full[s], (uint32_t)ph, &abort_flag)) {
+                if (!warp_wait(&full[s], (uint32_t)ph, &abort_flag)) {
                     set_timeout(p.ctl, &abort_flag);
                     stop = true;
                     break;
@@ -992,16 +1005,16 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
 #pragma unroll
                 for (int kk = 0; kk < BK / 16; ++kk) {
                     const uint64_t w = smem_desc(st + 2 * kA + kk * 32);
-                    mma_bf16(d, smem_desc(st + kk * 32), w, idesc, (kb > kb0 || kk) ? 1u : 0u);
-                    mma_bf16(d, smem_desc(st + kA + kk * 32), w, idesc, 1u);
+                    mma_bf16_if(lead, d, smem_desc(st + kk * 32), w, idesc, (kb > kb0 || kk) ? 1u : 0u);
+                    mma_bf16_if(lead, d, smem_desc(st + kA + kk * 32), w, idesc, 1u);
                 }
-                mma_commit(&empty[s]);
+                mma_commit_if(lead, &empty[s]);
                 if (++s == S) { s = 0; ph ^= 1; }
             }
-            mma_commit(&acc_full[buf]);
+            mma_commit_if(lead, &acc_full[buf]);
         }
         consumed_s = i;
-        mma_commit(mma_done);
+        mma_commit_if(lead, mma_done);
     } else if (warp >= 2) {
         __shared__ int warp_sums[kWideMaxThreads / 32];
         for (int m = blockIdx.x; p.lists.idx && m < p.M; m += gridDim.x)

@@ -70,20 +70,44 @@ __host__ __device__ constexpr uint32_t instr_desc(int M, int N)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
+// The load and MMA roles are run by whole warps, whose loops and operands are then uniform, and issued by one
+// elected lane.  With a role's loop in one lane's branch every address and descriptor had to be moved into uniform
+// registers before each instruction: about 100 cycles per MMA, commit or copy, more than the MMAs of a batched-
+// decode K block or the eight copies of a prefill stage leave (the same box, us; before -> MMA role -> both roles):
+// Llama-shaped layer 8 bf16 tokens 57.5 -> 54.3 -> 53.5 and 2048 610 -> 601 -> 560, hidden 8192 / intermediate 7168
+// 8 tokens 75 -> 61 -> 54, hidden 2048 / intermediate 8192 25.4 -> 22.5 -> 20.1.
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t lead;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(lead));
+    return lead;
+}
+
+// warp = threadIdx.x / 32, known to be the same in all its lanes.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
+// mbar_wait by all lanes of a warp, with one answer.
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, volatile int *abort)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
+}
+
+__device__ __forceinline__ void mma_bf16_if(uint32_t lead, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                            uint32_t acc)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(lead)
         : "memory");
 }
 
-// The mbarrier receives one arrival when all previously issued MMAs are done.
-__device__ __forceinline__ void mma_commit(uint64_t *bar)
+// The mbarrier receives one arrival when all MMAs that the elected lane issued before are done.
+__device__ __forceinline__ void mma_commit_if(uint32_t lead, uint64_t *bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 ::"r"(smem_addr(bar)) : "memory");
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 ::"r"(smem_addr(bar)), "r"(lead) : "memory");
 }
 
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -140,20 +164,57 @@ __device__ void drain_after_abort(uint64_t *full, int stages, int issued, int co
     mbar_wait(acc_full, 0u, &never);
 }
 
-// One 2D TMA tile load: inner coordinate c0 (elements, a multiple of 64), row c1.
-__device__ __forceinline__ void tma_load(void *dst, const CUtensorMap *map, int c0, int c1, uint64_t *bar)
+// The load role's instructions (lead: whether this lane issues them).
+__device__ __forceinline__ void mbar_expect_if(uint32_t lead, uint64_t *bar, uint32_t bytes)
 {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(smem_addr(dst)), "l"(map), "r"(c0), "r"(c1), "r"(smem_addr(bar))
-        : "memory");
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+                 "@q mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;\n\t}"
+                 ::"r"(smem_addr(bar)), "r"(bytes), "r"(lead) : "memory");
+}
+
+__device__ __forceinline__ void bulk_load_if(uint32_t lead, void *dst, const void *src, uint32_t bytes, uint64_t *bar,
+                                             uint64_t policy)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+                 "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+                 " [%0], [%1], %2, [%3], %4;\n\t}"
+                 ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)), "l"(policy), "r"(lead)
+                 : "memory");
+}
+
+__device__ __forceinline__ void bulk_load_shared_if(uint32_t lead, void *dst, const void *src, uint32_t bytes,
+                                                    uint64_t *bar)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
+                 "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t}"
+                 ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)), "r"(lead)
+                 : "memory");
+}
+
+__device__ __forceinline__ void bulk_prefetch_l2_if(uint32_t lead, const void *src, uint32_t bytes)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+                 "@q cp.async.bulk.prefetch.L2.global [%0], %1;\n\t}" ::"l"(src), "r"(bytes), "r"(lead) : "memory");
+}
+
+// One 2D TMA tile load: inner coordinate c0 (elements, a multiple of 64), row c1.
+__device__ __forceinline__ void tma_load_if(uint32_t lead, void *dst, const CUtensorMap *map, int c0, int c1,
+                                            uint64_t *bar)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+                 "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+                 " [%0], [%1, {%2, %3}], [%4];\n\t}"
+                 ::"r"(smem_addr(dst)), "l"(map), "r"(c0), "r"(c1), "r"(smem_addr(bar)), "r"(lead)
+                 : "memory");
 }
 
 // Starts bringing one TMA box (inner coordinate c0, row c1) of the tensor into L2;
 // no completion to wait for.
-__device__ __forceinline__ void tma_prefetch_l2(const CUtensorMap *map, int c0, int c1)
+__device__ __forceinline__ void tma_prefetch_l2_if(uint32_t lead, const CUtensorMap *map, int c0, int c1)
 {
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(c0), "r"(c1)
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %3, 0;\n\t"
+                 "@q cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];\n\t}"
+                 ::"l"(map), "r"(c0), "r"(c1), "r"(lead)
                  : "memory");
 }
 
