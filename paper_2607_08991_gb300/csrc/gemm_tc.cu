@@ -1180,29 +1180,6 @@ bool lists_inside(const sats_layer *layer, int M, int grid)
     return M <= grid || (long long)layer->H * layer->N >= 1LL << 21;
 }
 
-// Stage rings of the two batched-decode kernels, in bytes: about half of an SM's shared memory each for up to
-// 64 tokens, so that the next kernel's CTA starts beside this one and has its first weights in flight when this
-// one ends (four or five stages of 20 KB and more still cover the memory latency), else a whole SM's.
-// Llama-shaped layer, 8 tokens: 59.1 us with whole SMs, 58.0 with halves; hidden 2048 / intermediate 8192, 8 and
-// 64 tokens: 26.5 and 28.8, 25.4 and 27.6.  The blocks of a stack keep whole SMs: the next gate/up kernel there
-// waits behind the kernel that normalises the residual, and its deeper ring holds more weights by then (routed
-// Qwen-shaped block, 8 tokens: 54.2 us whole, 54.9 halves).  So do layers of a few MB, whose CTAs are short and
-// pile up on some SMs (hidden 1168 / intermediate 2391, 8 tokens: 15.5 us whole, 17.0 halves; hidden 1024 /
-// intermediate 4096: 15.0 and 15.2; hidden 2624 / intermediate 4251: 27.7 and 27.3).
-struct SkinnyRings {
-    int gu, down;
-};
-
-SkinnyRings skinny_rings(const sats_layer *layer, int NT, bool split, bool stack, int gu_slack)
-{
-    const int R = layer->tc_R;
-    if (stack || NT > 64 || (long long)layer->H * layer->N < 1LL << 23) return {kSmemBudget, kSmemBudget};
-    const int gu_stage = (2 * R + NT * (split ? 2 : 1)) * kTileBytes;
-    const int gu_stages = kSmemHalf / gu_stage < 4 ? 4 : kSmemHalf / gu_stage;
-    const int gu = gu_stages * gu_stage + gu_slack;
-    return {gu < kSmemBudget ? gu : kSmemBudget, 5 * (BM + 2 * NT) * kTileBytes};
-}
-
 // What the gate/up kernels of one batch are given besides the layer.
 struct GateUpArgs {
     const uint16_t *xhi, *xlo;   // bf16 activations [B][H]; xlo: their low parts, or nullptr (bf16 activations)
@@ -1215,7 +1192,6 @@ struct GateUpArgs {
     uint8_t *keep_trace;
     float *a_out;                // [B][ldn] (skinny kernel only) or nullptr
     float *zero;                 // y [B][H] to clear, or nullptr
-    bool stack;                  // a block of a stack
     int *ctl;
 };
 
@@ -1272,7 +1248,7 @@ cudaError_t launch_gate_up_skinny(const sats_layer *layer, const GateUpArgs &a, 
     gp.stage_bytes = gp.a_bytes + gp.x_bytes * (split ? 2 : 1);
     const int over = (R + BM) * kTileBytes - gp.stage_bytes;
     const int slack = over > 0 ? ((over + 1023) & ~1023) : 0;
-    gp.stages = stages_for(gp.stage_bytes, skinny_rings(layer, NT, split, a.stack, slack).gu - slack);
+    gp.stages = stages_for(gp.stage_bytes, kSmemBudget - slack);
     gp.ring_bytes = gp.stages * gp.stage_bytes + slack;
     gp.merge = split && NT <= 128 ? 1 : 0;
     gp.tmem_cols = tmem_cols_for((gp.merge ? 4 : 2) * NT);
@@ -1336,10 +1312,9 @@ cudaError_t launch_gate_up_wide(const sats_layer *layer, const GateUpArgs &a, cu
     return e == cudaSuccess ? e : fail(e, "gate/up kernel launch");
 }
 
-// out[row perm[m] or m] += (hact + hact_lo)[m] W_down for M rows of h (row stride layer->ldn); ring: bytes of
-// the stage ring.
+// out[row perm[m] or m] += (hact + hact_lo)[m] W_down for M rows of h (row stride layer->ldn).
 cudaError_t launch_down_skinny(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
-                               const int32_t *perm, const KeepLists &lists, int ring, int *ctl, cudaStream_t stream)
+                               const int32_t *perm, const KeepLists &lists, int *ctl, cudaStream_t stream)
 {
     const int N = layer->N, ldn = layer->ldn, sms = sm_count();
     const int NT = (M + 15) & ~15;
@@ -1361,7 +1336,7 @@ cudaError_t launch_down_skinny(const sats_layer *layer, const uint16_t *hact, co
     if (inside) dp.lists = lists;
     dp.a_bytes = BM * kTileBytes;
     dp.stage_bytes = dp.a_bytes + 2 * NT * kTileBytes;
-    dp.stages = stages_for(dp.stage_bytes, ring);
+    dp.stages = stages_for(dp.stage_bytes);
     dp.merge = NT <= 128 ? 1 : 0;
     dp.tmem_cols = tmem_cols_for((dp.merge ? 4 : 2) * NT);
     static std::atomic<int> cfg_dn[64];
@@ -1453,7 +1428,7 @@ cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void 
 cudaError_t run_tc_down(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
                         int *ctl, cudaStream_t stream)
 {
-    return M <= kMaxSkinny ? launch_down_skinny(layer, hact, hact_lo, M, out, nullptr, KeepLists{}, kSmemBudget, ctl, stream)
+    return M <= kMaxSkinny ? launch_down_skinny(layer, hact, hact_lo, M, out, nullptr, KeepLists{}, ctl, stream)
                            : launch_down_wide(layer, hact, hact_lo, M, out, nullptr, KeepLists{}, ctl, stream);
 }
 
@@ -1555,12 +1530,10 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
         a.keep = active_idx ? keep : nullptr;
         a.keep_trace = keep_trace;
         a.zero = out_mode == kOutY ? out : nullptr;   // the down projection adds into y
-        a.stack = x_mode == kXResidNorm;
         a.ctl = ctl;
         if (skinny_batch(B, split)) {
             if ((e = launch_gate_up_skinny(layer, a, stream)) != cudaSuccess) return e;
-            e = launch_down_skinny(layer, hact, hact_lo, B, out, perm, lists,
-                                   skinny_rings(layer, (B + 15) & ~15, split, a.stack, 0).down, ctl, stream);
+            e = launch_down_skinny(layer, hact, hact_lo, B, out, perm, lists, ctl, stream);
         } else {
             if ((e = launch_gate_up_wide(layer, a, stream)) != cudaSuccess) return e;
             e = launch_down_wide(layer, hact, hact_lo, B, out, perm, lists, ctl, stream);

@@ -35,7 +35,6 @@ constexpr int kWideMaxThreads = 64 + 128 * 4;
 constexpr int kSkinnyMaxGroups = 7;
 constexpr int kSkinnyMaxThreads = 64 + 128 * kSkinnyMaxGroups;  // of the batched-decode gate/up kernel
 constexpr int kSmemBudget = 196608;  // stage ring (one CTA per SM)
-constexpr int kSmemHalf = 106496;    // stage ring of a batched-decode kernel that shares its SM with the next one
 constexpr int kSmemWide = 225280;    // stage ring of the persistent prefill kernels, at most
 constexpr int kMaxStages = 8;
 constexpr int kMaxSkinny = 256;      // largest batch on the skinny orientation (MMA N <= 256)
