@@ -30,7 +30,7 @@ def sats():
     (1032, 777, 32, 24, True),   # a full tile of 32 tokens
     (4096, 1009, 33, 16, False), # two token tiles
     (4096, 1009, 40, 16, True),
-    (8192, 130, 2, 8, True),     # hidden 8192: one token per fused pass, so two take this path
+    (8192, 130, 3, 8, True),     # the largest hidden size (one token per fused pass; two would stay passes)
     (64, 100, 5, 8, False),      # below the path: passes of the fused kernel
 ])
 def test_batches_match_oracle(sats, oracle, H, N, B, r, f32):
