@@ -1256,9 +1256,11 @@ cudaError_t launch_gate_up_skinny(const sats_layer *layer, const GateUpArgs &a, 
     cudaError_t e = a.a_out ? set_smem(gu_skinny_kernel<true>, smem_for(1, gp.ring_bytes), cfg_act)
                             : set_smem(gu_skinny_kernel<false>, smem_for(1, gp.ring_bytes), cfg_gu_skinny);
     if (e != cudaSuccess) return fail(e, "shared-memory attribute");
-    // epilogue groups: one per 16-token column block, at most kSkinnyMaxGroups (the epilogue
-    // runs after the last MMA, so its time adds to the call's)
-    const int groups = NT / 16 < kSkinnyMaxGroups ? NT / 16 : kSkinnyMaxGroups;
+    // epilogue groups: one per 16-token column block, at most kSkinnyMaxGroups where the last of them saves
+    // a turn, else one less (the epilogue runs after the last MMA, so its time adds to the call's)
+    const int blocks16 = NT / 16, G = kSkinnyMaxGroups;
+    const int most = (blocks16 + G - 1) / G < (blocks16 + G - 2) / (G - 1) ? G : G - 1;
+    const int groups = blocks16 < most ? blocks16 : most;
     e = launch_pdl_cfg(a.a_out ? gu_skinny_kernel<true> : gu_skinny_kernel<false>, dim3(layer->tc_T), 64 + 128 * groups,
                        smem_for(1, gp.ring_bytes), stream, mX, mX2, gp);
     return e == cudaSuccess ? e : fail(e, "gate/up kernel launch");

@@ -31,7 +31,8 @@ constexpr int kWideDownGroups = 4;   // 256 columns: four 16-column blocks each
 constexpr int kWideMaxThreads = 64 + 128 * 4;
 // Epilogue groups of four warps of the batched-decode gate/up kernel, at most: seven (64 registers a
 // thread) take 97-112 and 193-224 tokens in one turn less than six (Llama-shaped layer, 112 bf16 / fp32
-// tokens 65.5 / 74.5 -> 63.9 / 73.0 us, 224 tokens 95.0 / 125.2 -> 91.9 / 122.5).
+// tokens 65.5 / 74.5 -> 63.9 / 73.0 us, 224 tokens 95.0 / 125.2 -> 91.9 / 122.5); elsewhere the seventh only
+// costs (hidden 1024 / intermediate 4096, 250 tokens 30.8 -> 31.3).
 constexpr int kSkinnyMaxGroups = 7;
 constexpr int kSkinnyMaxThreads = 64 + 128 * kSkinnyMaxGroups;  // of the batched-decode gate/up kernel
 constexpr int kSmemBudget = 196608;  // stage ring (one CTA per SM)
