@@ -116,31 +116,28 @@ __global__ void __launch_bounds__(kRouteThreads) route_kernel(const int32_t *ids
 // the IEEE bit pattern of |a_i| (non-negative floats order as their unsigned bit
 // patterns), 11 + 10 + 10 bits.  Level 0 counts the top 11 bits of every value;
 // levels 1 and 2 count the next 10 bits of the values that share their leading bits
-// with one of the ranks (a slot each; ranks in one bin share its slot).  Each level
-// is one kernel: a CTA counts its values in shared memory and adds the non-zero
-// counts to the level's histogram, and the last CTA to finish finds every rank's bin
-// and writes the slots of the next level.
+// with one of the ranks (a slot each; ranks in one bin share its slot).  At each level
+// a CTA counts its values in shared memory and adds the non-zero counts to the level's
+// histogram; once all CTAs have, every one of them finds every rank's bin by itself.
+// The three levels are one cooperative launch, whose CTAs meet twice.
 //
-// What bounds it: a pass over values that sit in L2, and the launches.  Post-gate
+// What bounds it: passes over values that sit in L2, and the meetings.  Post-gate
 // magnitudes fall into a few dozen of the top bins, so counting them with atomics in
 // global memory ran at the rate of one address (263 us per pass over 3.7 M values,
 // and 36 us to search 65536 bins with one CTA); level 0 therefore keeps kSelCopies
 // histograms per CTA in shared memory, and 2048-bin levels leave the search a few
 // microseconds.  All percentiles of a calibration grid share the three passes.
+// As three launches, the last CTA of each searching, a whole call took 37 / 45 / 46 / 59 us for
+// 39 k / 0.9 M / 3.7 M / 7.3 M values; as one it takes 33 / 35 / 43 / 47 (the kernel 20 us at 3.7 M, of which
+// the second and third pass are 2 each and a meeting with the additions before it about 4).
 constexpr int kSelBins0 = 2048, kSelBins = 1024, kSelCopies = 4;
 constexpr int kSelThreads = 1024, kSelWarps = kSelThreads / 32;
 
-// Workspace of a selection of R ranks; cleared as a whole before level 0.
+// Workspace of a selection of R ranks; cleared as a whole before it.
 struct SelWs {
-    unsigned *done;         // [3] CTAs finished per level
-    int *nslots;            // [2] slots of level 1 and 2
-    int *slot;              // [2][kSelRanks] rank -> slot
-    long long *rest;        // [kSelRanks] rank within the bins chosen so far (1-based)
-    uint32_t *prefix;       // [kSelRanks] bits chosen so far
+    int *done;              // [3] CTAs finished per level
     unsigned *hist0;        // [kSelBins0]
-    uint8_t *map0;          // [kSelBins0] slot + 1 of level 1, 0 for a bin without a rank
     unsigned *hist;         // [2][R][kSelBins] levels 1 and 2
-    uint8_t *map1;          // [R][kSelBins] slot + 1 of level 2
 };
 
 __host__ __device__ inline size_t sel_layout(char *base, int R, SelWs *w)
@@ -151,15 +148,9 @@ __host__ __device__ inline size_t sel_layout(char *base, int R, SelWs *w)
         off += (bytes + 255) & ~(size_t)255;
         return p;
     };
-    w->done = reinterpret_cast<unsigned *>(take(3 * sizeof(unsigned)));
-    w->nslots = reinterpret_cast<int *>(take(2 * sizeof(int)));
-    w->slot = reinterpret_cast<int *>(take(2 * kSelRanks * sizeof(int)));
-    w->rest = reinterpret_cast<long long *>(take(kSelRanks * sizeof(long long)));
-    w->prefix = reinterpret_cast<uint32_t *>(take(kSelRanks * sizeof(uint32_t)));
+    w->done = reinterpret_cast<int *>(take(3 * sizeof(int)));
     w->hist0 = reinterpret_cast<unsigned *>(take(kSelBins0 * sizeof(unsigned)));
-    w->map0 = reinterpret_cast<uint8_t *>(take(kSelBins0));
     w->hist = reinterpret_cast<unsigned *>(take((size_t)2 * R * kSelBins * sizeof(unsigned)));
-    w->map1 = reinterpret_cast<uint8_t *>(take((size_t)R * kSelBins));
     return off;
 }
 
@@ -192,162 +183,162 @@ __device__ __forceinline__ void for_each_bits(const float *__restrict__ a, int64
     for (int64_t i = done + t; i < n; i += T) f(__float_as_uint(a[i]) & 0x7fffffffu);
 }
 
-// The bin of `nbins` (a multiple of 1024) counts that holds the 1-based rank r, and r
-// within it, by one warp: 32 rows of 32 counts are loaded together (past L1: other CTAs
-// wrote them), then summed row by row until the rank's row, whose lanes are scanned.
-__device__ __forceinline__ int find_bin(const unsigned *hist, int nbins, long long r, long long *within)
+// Sum over the lanes up to this one.
+__device__ __forceinline__ long long warp_incl_scan(long long v)
 {
-    const int lane = threadIdx.x & 31;
-    long long run = 0;
-    for (int base = 0; base < nbins; base += 1024) {
-        unsigned c[32];
 #pragma unroll
-        for (int k = 0; k < 32; ++k) c[k] = __ldcg(hist + base + 32 * k + lane);
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            const long long row = (long long)__reduce_add_sync(0xffffffffu, c[k] & 0xffffu) +
-                                  ((long long)__reduce_add_sync(0xffffffffu, c[k] >> 16) << 16);
-            if (run + row >= r) {
-                long long incl = c[k];
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const long long t = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += t;
-                }
-                const unsigned at = __ballot_sync(0xffffffffu, run + incl >= r);
-                const int src = __ffs(at) - 1;   // (the row holds the rank, so its last lane is in `at`)
-                *within = r - run - __shfl_sync(0xffffffffu, incl - (long long)c[k], src);
-                return base + 32 * k + src;
-            }
-            run += row;
-        }
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long t = __shfl_up_sync(0xffffffffu, v, o);
+        if ((int)(threadIdx.x & 31) >= o) v += t;
     }
-    *within = 1;   // not reached: 1 <= r <= the sum of the counts
-    return nbins - 1;
+    return v;
+}
+
+// The bin of NBINS counts (in shared memory) that holds the 1-based rank r, and r within it, by one warp: each lane
+// sums NBINS / 32 counts, then the lanes share the counts of the lane that the rank falls in.
+template <int NBINS>
+__device__ __forceinline__ int find_bin(const unsigned *hist, long long r, long long *within)
+{
+    constexpr int kPer = NBINS / 32;
+    const int lane = threadIdx.x & 31;
+    long long sum = 0;
+#pragma unroll 8
+    for (int k = 0; k < kPer; ++k) sum += hist[lane * kPer + ((k + lane) & (kPer - 1))];   // (no two lanes in a bank)
+    const long long incl = warp_incl_scan(sum);
+    const unsigned at = __ballot_sync(0xffffffffu, incl >= r);
+    const int src = at ? __ffs(at) - 1 : 31;   // (1 <= r <= the sum of the counts)
+    long long run = __shfl_sync(0xffffffffu, incl - sum, src);
+#pragma unroll
+    for (int k = 0; k < kPer / 32; ++k) {
+        const long long v = hist[src * kPer + 32 * k + lane], in = run + warp_incl_scan(v);
+        const unsigned hit = __ballot_sync(0xffffffffu, in >= r);
+        if (hit) {
+            const int l = __ffs(hit) - 1;
+            *within = r - __shfl_sync(0xffffffffu, in - v, l);
+            return src * kPer + 32 * k + l;
+        }
+        run = __shfl_sync(0xffffffffu, in, 31);
+    }
+    *within = 1;   // not reached
+    return NBINS - 1;
+}
+
+// Counts that a CTA keeps in shared memory: level 0's copies, or a slot per rank.
+__host__ __device__ constexpr int sel_counts(int R)
+{
+    return kSelCopies * kSelBins0 > R * kSelBins ? kSelCopies * kSelBins0 : R * kSelBins;
 }
 
 struct SelRankList {
     long long m[kSelRanks];
 };
 
-template <int LEVEL>
+// All CTAs of the (cooperative) grid have added their counts of a level; false if they do not within kWaitLimitNs.
+__device__ __forceinline__ bool sel_meet(int *done, bool *met)
+{
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(done, 1);
+        const unsigned long long t0 = global_ns();
+        bool ok = true;
+        while (ld_acquire_gpu(done) < (int)gridDim.x)
+            if (global_ns() - t0 > kWaitLimitNs) { ok = false; break; }
+        *met = ok;
+    }
+    __syncthreads();
+    return *met;
+}
+
 __global__ void __launch_bounds__(kSelThreads) select_kernel(const float *__restrict__ a, int64_t n, int R,
                                                              const SelRankList ranks, char *ws,
                                                              float *__restrict__ t_out)
 {
     extern __shared__ unsigned sel_smem[];
-    __shared__ int bins[kSelRanks];
-    __shared__ bool last;
+    __shared__ int bins[kSelRanks], slot[kSelRanks], nslots;
+    __shared__ long long rest[kSelRanks];        // rank within the bins chosen so far (1-based)
+    __shared__ uint32_t prefix[kSelRanks];       // bits chosen so far
+    __shared__ bool met;
     SelWs w;
     sel_layout(ws, R, &w);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     unsigned *h = sel_smem;
-    grid_dependency_wait();   // the values and the slots belong to the preceding kernels
-    grid_launch_dependents();
-    const int slots = LEVEL == 0 ? 0 : w.nslots[LEVEL - 1];
-    const int nh = LEVEL == 0 ? kSelCopies * kSelBins0 : slots * kSelBins;
-    uint8_t *map0 = reinterpret_cast<uint8_t *>(h + nh), *map1 = map0 + kSelBins0;
-    for (int i = tid; i < nh; i += kSelThreads) h[i] = 0u;
-    if (LEVEL > 0)
-        for (int i = tid; i < kSelBins0 / 4; i += kSelThreads)
-            reinterpret_cast<uint32_t *>(map0)[i] = reinterpret_cast<const uint32_t *>(w.map0)[i];
-    if (LEVEL == 2)
-        for (int i = tid; i < w.nslots[0] * kSelBins / 4; i += kSelThreads)
-            reinterpret_cast<uint32_t *>(map1)[i] = reinterpret_cast<const uint32_t *>(w.map1)[i];
-    __syncthreads();
-    if (LEVEL == 0) {
-        unsigned *mine = h + (warp % kSelCopies) * kSelBins0;
-        for_each_bits(a, n, [&](uint32_t b) { atomicAdd(mine + (b >> 20), 1u); });
-    } else {
-        for_each_bits(a, n, [&](uint32_t b) {
-            const int s0 = map0[b >> 20];
-            if (s0 == 0) return;
-            if (LEVEL == 1) {
-                atomicAdd(h + (s0 - 1) * kSelBins + ((b >> 10) & 1023u), 1u);
-            } else {
-                const int s1 = map1[(s0 - 1) * kSelBins + ((b >> 10) & 1023u)];
-                if (s1) atomicAdd(h + (s1 - 1) * kSelBins + (b & 1023u), 1u);
-            }
-        });
+    uint8_t *map0 = reinterpret_cast<uint8_t *>(h + sel_counts(R));   // [kSelBins0] slot + 1 of level 1, or 0
+    uint8_t *map1 = map0 + kSelBins0;                                 // [R][kSelBins] slot + 1 of level 2, or 0
+    for (int i = tid; i < (kSelBins0 + R * kSelBins) / 4; i += kSelThreads) reinterpret_cast<uint32_t *>(map0)[i] = 0u;
+    if (tid < R) {
+        rest[tid] = ranks.m[tid];
+        prefix[tid] = 0u;
+        slot[tid] = 0;
     }
-    __syncthreads();
-    unsigned *gh = LEVEL == 0 ? w.hist0 : w.hist + (size_t)(LEVEL - 1) * R * kSelBins;
-    if (LEVEL == 0) {
-        for (int i = tid; i < kSelBins0; i += kSelThreads) {
-            unsigned c = 0;
-            for (int k = 0; k < kSelCopies; ++k) c += h[k * kSelBins0 + i];
-            if (c) atomicAdd(gh + i, c);
+#pragma unroll
+    for (int level = 0; level < 3; ++level) {
+        const int nh = level == 0 ? kSelCopies * kSelBins0 : nslots * kSelBins;
+        for (int i = tid; i < nh; i += kSelThreads) h[i] = 0u;
+        __syncthreads();
+        if (level == 0) {
+            unsigned *mine = h + (warp % kSelCopies) * kSelBins0;
+            for_each_bits(a, n, [&](uint32_t b) { atomicAdd(mine + (b >> 20), 1u); });
+        } else {
+            for_each_bits(a, n, [&](uint32_t b) {
+                const int s0 = map0[b >> 20];
+                if (s0 == 0) return;
+                if (level == 1) {
+                    atomicAdd(h + (s0 - 1) * kSelBins + ((b >> 10) & 1023u), 1u);
+                } else {
+                    const int s1 = map1[(s0 - 1) * kSelBins + ((b >> 10) & 1023u)];
+                    if (s1) atomicAdd(h + (s1 - 1) * kSelBins + (b & 1023u), 1u);
+                }
+            });
         }
-    } else {
-        for (int i = tid; i < nh; i += kSelThreads)
-            if (h[i]) atomicAdd(gh + i, h[i]);
-    }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) last = atomicAdd(w.done + LEVEL, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    // the last CTA: a warp per rank finds its bin
-    for (int i = warp; i < R; i += kSelWarps) {
-        const long long r = LEVEL == 0 ? ranks.m[i] : w.rest[i];
-        const unsigned *hr = LEVEL == 0 ? gh : gh + (size_t)w.slot[(LEVEL - 1) * kSelRanks + i] * kSelBins;
-        long long rest;
-        const int bin = find_bin(hr, LEVEL == 0 ? kSelBins0 : kSelBins, r, &rest);
-        if (lane == 0) {
-            bins[i] = bin;
-            w.rest[i] = rest;
-            if (LEVEL == 0) {
-                w.prefix[i] = (uint32_t)bin << 20;
-            } else if (LEVEL == 1) {
-                w.prefix[i] |= (uint32_t)bin << 10;
-            } else {
-                t_out[i] = __uint_as_float(w.prefix[i] | (uint32_t)bin);
+        __syncthreads();
+        unsigned *gh = level == 0 ? w.hist0 : w.hist + (size_t)(level - 1) * R * kSelBins;
+        if (level == 0) {
+            for (int i = tid; i < kSelBins0; i += kSelThreads) {
+                unsigned c = 0;
+                for (int k = 0; k < kSelCopies; ++k) c += h[k * kSelBins0 + i];
+                if (c) atomicAdd(gh + i, c);
+            }
+        } else {
+            for (int i = tid; i < nh; i += kSelThreads)
+                if (h[i]) atomicAdd(gh + i, h[i]);
+        }
+        if (!sel_meet(w.done + level, &met)) {
+            if (tid < R) t_out[tid] = __int_as_float(0x7fffffff);
+            return;
+        }
+        if (level == 2 && blockIdx.x != 0) return;
+        // all CTAs' counts (past L1: the other CTAs wrote them)
+        for (int i = tid; i < (level == 0 ? kSelBins0 : nh) / 4; i += kSelThreads)
+            reinterpret_cast<uint4 *>(h)[i] = __ldcg(reinterpret_cast<const uint4 *>(gh) + i);
+        __syncthreads();
+        for (int i = warp; i < R; i += kSelWarps) {   // a warp per rank finds its bin
+            long long within;
+            const int bin = level == 0 ? find_bin<kSelBins0>(h, rest[i], &within)
+                                       : find_bin<kSelBins>(h + slot[i] * kSelBins, rest[i], &within);
+            if (lane == 0) {
+                bins[i] = bin;
+                rest[i] = within;
+                prefix[i] |= (uint32_t)bin << (20 - 10 * level);
+                if (level == 2) t_out[i] = __uint_as_float(prefix[i]);
             }
         }
-    }
-    if (LEVEL == 2) return;
-    __syncthreads();
-    if (tid == 0) {   // ranks that share a bin share a slot of the next level
-        int ns = 0;
-        for (int i = 0; i < R; ++i) {
-            uint8_t *m = LEVEL == 0 ? w.map0 + bins[i] : w.map1 + (size_t)w.slot[i] * kSelBins + bins[i];
-            if (*m == 0) *m = (uint8_t)++ns;
-            w.slot[LEVEL * kSelRanks + i] = *m - 1;
+        if (level == 2) return;
+        __syncthreads();
+        if (tid == 0) {   // ranks that share a bin share a slot of the next level
+            int ns = 0;
+            for (int i = 0; i < R; ++i) {
+                uint8_t *m = level == 0 ? map0 + bins[i] : map1 + slot[i] * kSelBins + bins[i];
+                if (*m == 0) *m = (uint8_t)++ns;
+                slot[i] = *m - 1;
+            }
+            nslots = ns;
         }
-        w.nslots[LEVEL] = ns;
+        __syncthreads();
     }
 }
 
-size_t sel_smem_bytes(int level, int R)
-{
-    if (level == 0) return (size_t)kSelCopies * kSelBins0 * sizeof(unsigned);
-    return (size_t)R * kSelBins * sizeof(unsigned) + kSelBins0 + (level == 2 ? (size_t)R * kSelBins : 0);
-}
-
-template <int LEVEL>
-cudaError_t launch_select_level(const float *a, int64_t n, int R, const SelRankList &ranks, char *ws, float *t_out,
-                                int grid, cudaStream_t stream)
-{
-    const size_t smem = sel_smem_bytes(LEVEL, R);
-    // (the limit is set to the most that any call needs, so calls never lower it under one another)
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(select_kernel<LEVEL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)sel_smem_bytes(LEVEL, kSelRanks));
-        if (e != cudaSuccess) return e;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kSelThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, select_kernel<LEVEL>, a, n, R, ranks, ws, t_out);
-}
+size_t sel_smem_bytes(int R) { return (size_t)sel_counts(R) * sizeof(unsigned) + kSelBins0 + (size_t)R * kSelBins; }
 
 }  // namespace
 
@@ -461,9 +452,23 @@ cudaError_t launch_select(const float *a, int64_t n, const int64_t *m, int R, vo
     const int64_t want = (n + 4 * kSelThreads - 1) / (4 * kSelThreads);
     const int sms = fused_grid(kMaxGrid);
     const int grid = (int)(want < sms ? want : sms);
-    if ((e = launch_select_level<0>(a, n, R, ranks, base, t_dev, grid, stream)) != cudaSuccess) return e;
-    if ((e = launch_select_level<1>(a, n, R, ranks, base, t_dev, grid, stream)) != cudaSuccess) return e;
-    return launch_select_level<2>(a, n, R, ranks, base, t_dev, grid, stream);
+    const size_t smem = sel_smem_bytes(R);
+    // (the limit is set to the most that any call needs, so calls never lower it under one another)
+    if (smem > 48 * 1024) {
+        e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel_smem_bytes(kSelRanks));
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kSelThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;   // the CTAs wait for one another
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, select_kernel, a, n, R, ranks, base, t_dev);
 }
 
 }  // namespace sats
