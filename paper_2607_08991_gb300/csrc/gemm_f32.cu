@@ -12,12 +12,16 @@
 //    accumulator takes K = 32 only (the small parts first); every K block of 64 fills
 //    two of them, and the epilogue warps read both from TMEM while the next block's MMAs
 //    run, add the two and add the sum to totals that they keep in registers (rounded to
-//    nearest).  Measured against fp64 on the Llama-shaped layer: 1.1e-7 relative, as the
-//    fp32 FMA chains that this replaced.
+//    nearest).  Measured against fp64 on the Llama-shaped layer, 256 tokens: 1.1e-7 relative
+//    with bf16 and 1.9e-7 with fp32 activations (the fp32 FMA chains that this replaced:
+//    1.1e-7 and 2.2e-7).
 //
-// What bounds it: at up to 128 tokens the weight stream, beyond that the MMAs (about 70
-// cycles each up to N = 128) and the TMEM reads (two accumulators per K block), which
-// take about as long as each other; three MMAs per step with fp32 activations.
+// What bounds it: neither the weight stream (17 us on that layer) nor the MMAs, but what the
+// roles issue per K block: waits and commits of about 100 cycles each, the TMEM reads and
+// additions of two accumulators (two at a time, f32x2; fp32: the next columns' read in
+// flight), and with fp32 activations the converters (no test for infinities but one vote at
+// the end of a step).  Llama-shaped layer, us before and after these: bf16 16 / 128 / 256
+// tokens 25.0 / 34.0 / 65.2 -> 24.7 / 32.6 / 63.8, fp32 46.0 / 98.0 / 200 -> 39.5 / 75.8 / 152.
 #include "tc_common.cuh"
 
 namespace sats {
@@ -43,6 +47,13 @@ struct PreciseGateParams {
     uint32_t tmem_cols;    // four accumulators of NT columns
 };
 
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 __device__ __forceinline__ float bf16_top(float x) { return __uint_as_float(__float_as_uint(x) & 0xffff0000u); }
 
 __device__ __forceinline__ uint32_t pack_tops(float lo, float hi)
@@ -51,38 +62,28 @@ __device__ __forceinline__ uint32_t pack_tops(float lo, float hi)
 }
 
 // Eight fp32 values -> one 16-byte chunk of each part: the top 8 significant bits, the next 8, the
-// last 8 (each difference x - top is exact, so the parts' sum is x).
-__device__ __forceinline__ void cut8(const float4 &p, const float4 &q, uint4 (&part)[kParts])
+// last 8 (each difference x - top is exact, so the parts' sum is x).  With SPECIAL an infinity leaves
+// nothing after its top; without, inf - inf, and `odd` becomes NaN if any value was not finite.
+template <bool SPECIAL>
+__device__ __forceinline__ void cut8(const float4 &p, const float4 &q, uint4 (&part)[kParts], f32x2 &odd)
 {
-    float v[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+    const float v[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+    const f32x2 minus1 = pack2(-1.f, -1.f);
     uint32_t out[kParts][4];
-    uint32_t most = 0u;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) most = max(most, __float_as_uint(v[e]) & 0x7fffffffu);
-    if (most < 0x7f800000u) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const f32x2 minus1 = pack2(-1.f, -1.f);
-            f32x2 r = pack2(v[2 * e], v[2 * e + 1]);
-#pragma unroll
-            for (int i = 0; i < kParts; ++i) {
-                const float2 f = unpack2(r);
-                out[i][e] = pack_tops(f.x, f.y);
-                if (i + 1 < kParts) r = ffma2(pack2(bf16_top(f.x), bf16_top(f.y)), minus1, r);
-            }
+    for (int e = 0; e < 4; ++e) {
+        const float a = v[2 * e], b = v[2 * e + 1];
+        out[0][e] = pack_tops(a, b);
+        float2 d = unpack2(ffma2(pack2(bf16_top(a), bf16_top(b)), minus1, pack2(a, b)));
+        if (SPECIAL) {   // a value that is its own top leaves nothing
+            d.x = __float_as_uint(a) & 0xffffu ? d.x : 0.f;
+            d.y = __float_as_uint(b) & 0xffffu ? d.y : 0.f;
         }
-    } else {   // infinities keep out of the differences (inf - inf), NaN stays NaN in every part
-#pragma unroll
-        for (int i = 0; i < kParts; ++i) {
-            float t[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                t[e] = bf16_top(v[e]);
-                v[e] = t[e] == v[e] ? 0.f : v[e] - t[e];
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) out[i][e] = pack_tops(t[2 * e], t[2 * e + 1]);
-        }
+        out[1][e] = pack_tops(d.x, d.y);
+        const f32x2 r = ffma2(pack2(bf16_top(d.x), bf16_top(d.y)), minus1, pack2(d.x, d.y));
+        const float2 f = unpack2(r);
+        out[2][e] = pack_tops(f.x, f.y);
+        if (!SPECIAL) odd = ffma2(r, pack2(0.f, 0.f), odd);
     }
 #pragma unroll
     for (int i = 0; i < kParts; ++i) part[i] = make_uint4(out[i][0], out[i][1], out[i][2], out[i][3]);
@@ -102,51 +103,55 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 // The converter warps (threads 64 .. 64 + kConvThreads - 1): fp32 tiles of NT rows x 64 columns, one
 // per step, cut into kPartStages stages of swizzled bf16 parts [kParts][NT][64].  Unit u of a tile is
 // 8 consecutive values (chunk u mod 8 of row u / 8), load(row, chunk, step, lo, hi) fetches one (zero
-// unless set); the next step's units are loaded while this one's are cut.
+// unless set); the next step's units are loaded while this one's are cut.  (Loads up to four steps ahead
+// cost more in code than they hid: LoRA layer, 8 tokens, 84.4 us with four, 81.0 with two, 79.7 with one.)
 template <int TOK, typename Load>
 __device__ __forceinline__ bool cut_tiles(uint8_t *parts, int NT, int steps, uint64_t *pfull, uint64_t *pempty,
                                           volatile int *abort, Load load)
 {
     constexpr int kUnits = (TOK * 8 + kConvThreads - 1) / kConvThreads;
-    // steps whose units are in flight: a load takes as long as several small tiles' MMAs, and the
-    // registers of a large tile hold one step
-    constexpr int kAhead = TOK <= 32 ? 4 : TOK <= 64 ? 2 : 1;
     const int ct = threadIdx.x - 64, nu = NT * 8;
-    float4 lo[kAhead][kUnits], hi[kAhead][kUnits];
-    auto fetch = [&](int a, int i, int step) {
+    float4 lo[kUnits], hi[kUnits];
+    auto fetch = [&](int i, int step) {
         const int u = ct + kConvThreads * i;
-        lo[a][i] = hi[a][i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (u < nu && step < steps) load(u >> 3, u & 7, step, lo[a][i], hi[a][i]);
+        lo[i] = hi[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (u < nu && step < steps) load(u >> 3, u & 7, step, lo[i], hi[i]);
     };
 #pragma unroll
-    for (int a = 0; a < kAhead; ++a)
+    for (int i = 0; i < kUnits; ++i) fetch(i, 0);
+    for (int step = 0; step < steps; ++step) {
+        const int ps = step % kPartStages;
+        if (!mbar_wait(&pempty[ps], (uint32_t)((step / kPartStages) & 1) ^ 1u, abort)) return false;
+        uint8_t *dst = parts + (size_t)ps * kParts * NT * kTileBytes;
+        auto put = [&](int u, const uint4 (&part)[kParts]) {
+            const int r = u >> 3, c = u & 7;
+            if (u >= nu) return;
 #pragma unroll
-        for (int i = 0; i < kUnits; ++i) fetch(a, i, a);
-    for (int base = 0; base < steps; base += kAhead) {
+            for (int q = 0; q < kParts; ++q)
+                *reinterpret_cast<uint4 *>(dst + (size_t)(q * NT + r) * kTileBytes + ((c ^ (r & 7)) << 4)) = part[q];
+        };
+        f32x2 odd = pack2(0.f, 0.f);
 #pragma unroll
-        for (int a = 0; a < kAhead; ++a) {
-            const int step = base + a;
-            if (step >= steps) break;
-            const int ps = step % kPartStages;
-            if (!mbar_wait(&pempty[ps], (uint32_t)((step / kPartStages) & 1) ^ 1u, abort)) return false;
-            uint8_t *dst = parts + (size_t)ps * kParts * NT * kTileBytes;
-#pragma unroll
-            for (int i = 0; i < kUnits; ++i) {
-                const int u = ct + kConvThreads * i, r = u >> 3, c = u & 7;
-                uint4 part[kParts];
-                cut8(lo[a][i], hi[a][i], part);
-                fetch(a, i, step + kAhead);
-                if (u < nu) {
-#pragma unroll
-                    for (int q = 0; q < kParts; ++q)
-                        *reinterpret_cast<uint4 *>(dst + (size_t)(q * NT + r) * kTileBytes + ((c ^ (r & 7)) << 4)) =
-                            part[q];
-                }
-            }
-            fence_async_smem();   // the MMAs read the tile through the async proxy
-            __syncwarp();
-            if ((threadIdx.x & 31) == 0) mbar_arrive(&pfull[ps]);
+        for (int i = 0; i < kUnits; ++i) {
+            uint4 part[kParts];
+            cut8<false>(lo[i], hi[i], part, odd);
+            fetch(i, step + 1);
+            put(ct + kConvThreads * i, part);
         }
+        const float2 o = unpack2(odd);
+        if (!(o.x == 0.f && o.y == 0.f)) {   // not all finite: once more
+#pragma unroll 1
+            for (int u = ct; u < nu; u += kConvThreads) {
+                float4 p = make_float4(0.f, 0.f, 0.f, 0.f), q = p;
+                uint4 part[kParts];
+                load(u >> 3, u & 7, step, p, q);
+                cut8<true>(p, q, part, odd);
+                put(u, part);
+            }
+        }
+        fence_async_smem();   // the MMAs read the tile through the async proxy
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(&pfull[ps]);
     }
     return true;
 }
@@ -154,8 +159,7 @@ __device__ __forceinline__ bool cut_tiles(uint8_t *parts, int NT, int steps, uin
 // a = SiLU(x W_gate) for one tile of NT tokens and R neurons per CTA (neurons are the MMA's
 // M, tokens its N).  Grid: token tiles x neuron tiles, the token tiles of one neuron tile
 // next to each other, so that its weights come from L2 for all but the first of them.
-// TOK: the most tokens of a tile (64 leaves registers for a second level of sums and for loads two
-// steps ahead with fp32 activations).
+// TOK: the most tokens of a tile (64 leaves registers for a second level of sums with fp32 activations).
 template <bool F32, int TOK>
 __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     gate_precise_kernel(const __grid_constant__ CUtensorMap tmX, const PreciseGateParams p)
@@ -207,9 +211,10 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     const uint32_t tmem = *tmem_slot;
     grid_launch_dependents();
 
-    // (one lane runs the load role here: 256 bf16 tokens took 69 us so and 75 with a whole warp)
-    if (warp == 0 && lane == 0) {
-        const uint32_t lead = 1u;
+    // (bf16: one lane runs the load role, 256 tokens 69 us so and 75 with a whole warp; fp32: the warp, 64
+    // tokens 48.0 us and 51.6 with one lane)
+    if (warp == 0 && (F32 || lane == 0)) {
+        const uint32_t lead = F32 ? elect_one() : 1u;
         const uint32_t load_bytes = (uint32_t)p.w_bytes + (F32 ? 0u : (uint32_t)(NT * kTileBytes));
         // (each weight tile is read once with one token tile, else by its neighbours through L2)
         const uint64_t once = l2_policy_evict_first();
@@ -227,7 +232,11 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
         int kb = 0;
         for (int s = 0, ph = 0; kb < KBh; ++kb) {
             if (kb >= npre) {
-                if (!mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { abort_flag = 1; break; }
+                if (!(F32 ? warp_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)
+                          : mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag))) {
+                    abort_flag = 1;
+                    break;
+                }
                 mbar_expect_if(lead, &full[s], load_bytes);
                 load_w(s, kb);
             }
@@ -242,8 +251,10 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
         for (int s = 0, ph = 0; kb < KBh; ++kb) {
             const int buf = kb & 1, ps = kb % kPartStages;
             const uint32_t bph = (uint32_t)((kb >> 1) & 1);
-            if (!warp_wait(&acc_empty[buf], bph ^ 1u, &abort_flag) || !warp_wait(&full[s], (uint32_t)ph, &abort_flag) ||
-                (F32 && !warp_wait(&pfull[ps], (uint32_t)((kb / kPartStages) & 1), &abort_flag))) {
+            // fp32: the three barriers by a lane each (a wait costs about 100 cycles even when its phase is over)
+            uint64_t *const bar = lane == 1 ? &acc_empty[buf] : F32 && lane == 2 ? &pfull[ps] : &full[s];
+            if (F32 ? !warp_wait(bar, lane == 1 ? bph ^ 1u : lane == 2 ? bph : (uint32_t)ph, &abort_flag)
+                    : !warp_wait(&acc_empty[buf], bph ^ 1u, &abort_flag) || !warp_wait(&full[s], (uint32_t)ph, &abort_flag)) {
                 abort_flag = 1;
                 break;
             }
@@ -285,47 +296,50 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
         // acc: totals; sub: the sums of up to kSubBlocks K blocks, added to the totals together, so that
         // a total takes few roundings at its full size (where the registers hold both)
         constexpr bool kTwoLevel = kBlocks <= 2;
-        float acc[kBlocks][16], sub[kTwoLevel ? kBlocks : 1][16];
+        constexpr int kPairs = 8 * kBlocks;
+        f32x2 acc[kPairs], sub[kTwoLevel ? kPairs : 1];
 #pragma unroll
-        for (int k = 0; k < kBlocks; ++k)
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                acc[k][e] = 0.f;
-                if (kTwoLevel) sub[kTwoLevel ? k : 0][e] = 0.f;
-            }
+        for (int k = 0; k < kPairs; ++k) {
+            acc[k] = pack2(0.f, 0.f);
+            if (kTwoLevel) sub[kTwoLevel ? k : 0] = pack2(0.f, 0.f);
+        }
         bool ok = true;
         for (int kb = 0; kb < KBh; ++kb) {
             const int buf = kb & 1;
             if (!mbar_wait(&acc_full[buf], (uint32_t)((kb >> 1) & 1), &abort_flag)) { ok = false; break; }
             tc_fence_after();
             if (quad < n_quads) {
+                const uint32_t a0 = lane0 + (uint32_t)(2 * buf * NT);
+                constexpr int kV = F32 ? 2 : 1;
+                float v[kV][2][8];
+                auto fetch = [&](int o) {   // 8 columns of both accumulators
+                    const uint32_t c = (uint32_t)(16 * (grp + G * (o >> 1)) + 8 * (o & 1));
+                    tmem_ld8(a0 + c, v[o % kV][0]);
+                    tmem_ld8(a0 + (uint32_t)NT + c, v[o % kV][1]);
+                };
+                if (F32 && 16 * grp < NT) fetch(0);
 #pragma unroll
-                for (int k = 0; k < kBlocks; ++k) {
-                    const int c0 = 16 * (grp + G * k);
-                    if (c0 >= NT) break;
+                for (int o = 0; o < 2 * kBlocks; ++o) {
+                    if (16 * (grp + G * (o >> 1)) >= NT) break;
+                    if (!F32) fetch(o);
+                    tmem_ld_wait();
+                    if (F32 && o + 1 < 2 * kBlocks && 16 * (grp + G * ((o + 1) >> 1)) < NT) fetch(o + 1);
 #pragma unroll
-                    for (int o = 0; o < 16; o += 8) {
-                        float v0[8], v1[8];
-                        tmem_ld8(lane0 + (uint32_t)(2 * buf * NT + c0 + o), v0);
-                        tmem_ld8(lane0 + (uint32_t)((2 * buf + 1) * NT + c0 + o), v1);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            if (kTwoLevel) sub[kTwoLevel ? k : 0][o + e] += v0[e] + v1[e];
-                            else acc[k][o + e] += v0[e] + v1[e];
-                        }
+                    for (int e = 0; e < 4; ++e) {
+                        const f32x2 w = add2(pack2(v[o % kV][0][2 * e], v[o % kV][0][2 * e + 1]),
+                                             pack2(v[o % kV][1][2 * e], v[o % kV][1][2 * e + 1]));
+                        f32x2 &to = kTwoLevel ? sub[kTwoLevel ? 4 * o + e : 0] : acc[4 * o + e];
+                        to = add2(to, w);
                     }
                 }
             }
             warp_arrive_tmem(&acc_empty[buf], lane);
             if (kTwoLevel && (kb % kSubBlocks == kSubBlocks - 1 || kb + 1 == KBh)) {
 #pragma unroll
-                for (int k = 0; k < kBlocks; ++k)
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        acc[k][e] += sub[kTwoLevel ? k : 0][e];
-                        sub[kTwoLevel ? k : 0][e] = 0.f;
-                    }
+                for (int k = 0; k < kPairs; ++k) {
+                    acc[k] = add2(acc[k], sub[kTwoLevel ? k : 0]);
+                    sub[kTwoLevel ? k : 0] = pack2(0.f, 0.f);
+                }
             }
         }
         grid_dependency_wait();   // a may still be in use by the preceding kernel
@@ -337,7 +351,8 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                     const int j = 16 * (grp + G * k) + e;
                     if (j < NT && m0 + j < p.B) {
                         // (a wait that gave up leaves NaN: this call has no status word)
-                        const float g = ok ? acc[k][e] : __int_as_float(0x7fffffff);
+                        const float2 two = unpack2(acc[8 * k + e / 2]);
+                        const float g = ok ? (e & 1 ? two.y : two.x) : __int_as_float(0x7fffffff);
                         p.a[(size_t)(m0 + j) * p.N + n] = g / (1.0f + expf(-g));   // SiLU, Eq. 2
                     }
                 }
@@ -400,7 +415,7 @@ cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, f
 //   lora_out_kernel      y += s w B_down
 // W is streamed once for up to kLoraTok tokens, where the fused kernel streamed it once per pass
 // of one or two (129 us for four tokens on the Llama-shaped layer at 70 % sparsity, 267 us for
-// eight).  What bounds it: that stream; with at most 32 tokens the parts of an operand are the
+// eight; 79 and 80 here).  What bounds it: that stream and the roles' serial issue; with at most 32 tokens the parts of an operand are the
 // rows of one tile, so a K step is one MMA per weight tile however many parts there are, and
 // their products are added in the epilogue.
 constexpr int kLoraTok = 32;

@@ -86,10 +86,12 @@ __device__ __forceinline__ uint32_t elect_one()
 // warp = threadIdx.x / 32, known to be the same in all its lanes.
 __device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 
-// mbar_wait by all lanes of a warp, with one answer.
+// mbar_wait by all lanes of a warp (of one barrier or of one each), with one answer.
 __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, volatile int *abort)
 {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
+    __syncwarp();
+    return ok;
 }
 
 __device__ __forceinline__ void mma_bf16_if(uint32_t lead, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
