@@ -42,6 +42,7 @@
 // 4) + 31; the groups split the accumulator's columns; G = 1 in the down kernel of
 // batched decode, up to seven in its gate/up kernel, four in the prefill kernels).
 // Every wait is bounded in time and sets the status word when it gives up.
+#include <algorithm>
 #include "tc_common.cuh"
 
 namespace sats {
@@ -1390,8 +1391,32 @@ cudaError_t launch_down_wide(const sats_layer *layer, const uint16_t *hact, cons
     return lists.idx && !inside ? launch_keep_lists(lists, M, stream) : cudaSuccess;
 }
 
-// Which orientation a batch's gate/up takes.
+// Which orientation a batch takes.
 bool skinny_batch(int B, bool split) { return B <= (split ? kMaxSkinnySplit : kMaxSkinny); }
+
+// Whether a skinny batch's gate and up go through the prefill kernel all the same: the skinny one spends an MMA of
+// 128 rows per K step on its R-neuron tile, however few R are (N = 7168: 48), in a time that grows with the tokens.
+// Estimates in us: the epilogue's share, then the longer of the weight stream (the prefill kernel's over the SMs
+// that have a tile) and the MMAs.  The constants are a fit to 13 shapes from 304 x 997 to 8192 x 14336 at 112 to
+// 256 tokens, wrong by up to 6 % near the line, hence the 0.87; below kMinGateUpWide tokens they were not fitted,
+// and little is to be had.  Both sides, us: hidden 1024 / intermediate 4096, 256 bf16 tokens 30.9 skinny, 22.8 so;
+// 4096 / 7168, 160 fp32 tokens 78.1 and 64.2; 8192 / 7168, 128 fp32 tokens 124 and 83; 4096 / 14336, 192 bf16
+// tokens 81.7 (taken) and 90.4.
+constexpr int kMinGateUpWide = 97;
+
+bool gate_up_wide(const sats_layer *layer, int B, bool split)
+{
+    if (B < kMinGateUpWide) return false;
+    const int H = layer->H, N = layer->N, sms = sm_count(), mtiles = (B + BM - 1) / BM, NT = (B + 15) & ~15;
+    const int Rw = wide_rows(N, layer->tc_R, mtiles, sms, split);
+    const int tiles = mtiles * ((N + Rw - 1) / Rw), waves = (tiles + sms - 1) / sms;
+    const double steps = H / 64.0, stream = 4.0 * H * N / 6.7e6;
+    const double skinny_mma = (layer->tc_T + sms - 1) / sms * steps * 0.002354 * (NT * (split ? 2 : 1) - 14.4);
+    const double wide_mma = waves * steps * 0.001069 * (BM * (split ? 2 : 1) + 2 * Rw);
+    const double skinny = 0.0219 * NT + std::max(0.937 * stream, skinny_mma);
+    const double wide = 3.28 + std::max(1.232 * stream * waves * sms / tiles, wide_mma);
+    return wide < 0.87 * skinny;
+}
 }  // namespace
 
 // Gate and up projections of B fp32 inputs with every neuron kept: h in bf16 parts and a =
@@ -1534,7 +1559,9 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
         a.zero = out_mode == kOutY ? out : nullptr;   // the down projection adds into y
         a.ctl = ctl;
         if (skinny_batch(B, split)) {
-            if ((e = launch_gate_up_skinny(layer, a, stream)) != cudaSuccess) return e;
+            e = gate_up_wide(layer, B, split) ? launch_gate_up_wide(layer, a, stream)
+                                              : launch_gate_up_skinny(layer, a, stream);
+            if (e != cudaSuccess) return e;
             e = launch_down_skinny(layer, hact, hact_lo, B, out, perm, lists, ctl, stream);
         } else {
             if ((e = launch_gate_up_wide(layer, a, stream)) != cudaSuccess) return e;
