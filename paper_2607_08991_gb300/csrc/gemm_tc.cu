@@ -646,6 +646,7 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    grid_launch_dependents();   // the down projection may start prefetching its weights
 
     if (warp == 0) {
         const uint32_t lead = elect_one();
@@ -700,6 +701,7 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
             }
         };
         for (int j = 0; j < kWidePrefetch; ++j) prefetch_ahead();
+        grid_dependency_wait();   // x may belong to the preceding kernel
         int i = 0, s = 0, ph = 0;
         bool stop = false;
         for (int q = blockIdx.x; q < p.tiles && !stop; q += gridDim.x) {
@@ -767,6 +769,7 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
         consumed_s = i;
         mma_commit_if(lead, mma_done);
     } else if (warp >= 2) {
+        grid_dependency_wait();   // y, h and the keep bytes may still be in use by the preceding kernels
         if (p.zero) {
             // this CTA's share of y, cleared for the down projection's additions while the first
             // tile's MMAs run
@@ -926,6 +929,7 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    grid_launch_dependents();   // the next kernels may start their prologue as SMs free up
 
     if (warp == 0) {
         const uint32_t lead = elect_one();
@@ -934,7 +938,7 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
         // tiles by the CTAs of the first two token tiles, the h tiles by every fourth unit column;
         // the cursor's unit is decoded once per unit
         int pu = blockIdx.x, pkb = 0, pkb1 = 0, pm0 = 0, pd0 = 0;
-        bool pf_w = false, pf_h = false;
+        bool pf_w = false, pf_h = false, written = false;   // (h is not, before the preceding kernel ends)
         auto prefetch_unit = [&]() {
             if (pu >= p.units) return;
             unit(pu, pm0, pd0, pkb, pkb1);
@@ -947,7 +951,7 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
             if (pf_w)
                 for (int q = 0; q < p.dtiles; ++q)
                     bulk_prefetch_l2_if(lead, p.w + ((size_t)(pd0 + q) * KBn + pkb) * BM * BK, (uint32_t)kA);
-            if (pf_h) {
+            if (pf_h && written) {
                 tma_prefetch_l2_if(lead, &tmH, pkb * BK, pm0);
                 tma_prefetch_l2_if(lead, &tmH2, pkb * BK, pm0);
             }
@@ -957,6 +961,8 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
             }
         };
         for (int j = 0; j < kWidePrefetch; ++j) prefetch_ahead();
+        grid_dependency_wait();   // h is written by the preceding gate/up kernel
+        written = true;
         int i = 0, s = 0, ph = 0;
         bool stop = false;
         for (int u = blockIdx.x; u < p.units && !stop; u += gridDim.x) {
@@ -1017,6 +1023,7 @@ __global__ void __launch_bounds__(kWideMaxThreads, 1)
         consumed_s = i;
         mma_commit_if(lead, mma_done);
     } else if (warp >= 2) {
+        grid_dependency_wait();   // y is cleared, h and the keep bytes written by the preceding kernel
         __shared__ int warp_sums[kWideMaxThreads / 32];
         for (int m = blockIdx.x; p.lists.idx && m < p.M; m += gridDim.x)
             write_keep_list(p.lists, m, (int)threadIdx.x - 64, (int)blockDim.x - 64, warp_sums, 1);
@@ -1267,6 +1274,13 @@ cudaError_t launch_gate_up_skinny(const sats_layer *layer, const GateUpArgs &a, 
     return e == cudaSuccess ? e : fail(e, "gate/up kernel launch");
 }
 
+// Whether a prefill kernel starts, and asks for its first weights, while the preceding one ends: a fifth to a third
+// of a small layer's call (us: hidden 512 / intermediate 1408, 333 tokens 20.8 -> 15.1; 2048 / 8192, 333 tokens
+// 56.2 -> 46.8 and 1024 tokens 105.8 -> 98.1; 4096 / 14336, 333 tokens 131.3 -> 128.9).  Calls beyond about 200 us
+// do without: their ends are a small share, and kept busy through them the chip clocks lower (4096 / 14336, 2048
+// tokens in a loop 594 -> 600, 8192 / 7168 606 -> 615).
+bool wide_overlap(int M, int H, int N) { return (long long)M * H * N < 1LL << 35; }
+
 cudaError_t launch_gate_up_wide(const sats_layer *layer, const GateUpArgs &a, cudaStream_t stream)
 {
     const int H = layer->H, N = layer->N, R = layer->tc_R, B = a.B, sms = sm_count();
@@ -1309,9 +1323,8 @@ cudaError_t launch_gate_up_wide(const sats_layer *layer, const GateUpArgs &a, cu
     static std::atomic<int> cfg_gu[64];
     cudaError_t e = set_smem(gu_wide_kernel, smem_for(gp.stages, gp.stage_bytes), cfg_gu);
     if (e != cudaSuccess) return fail(e, "shared-memory attribute");
-    gu_wide_kernel<<<dim3(gp.tiles < sms ? gp.tiles : sms), 64 + 128 * gu_groups, smem_for(gp.stages, gp.stage_bytes),
-                     stream>>>(mX, mX2, gp);
-    e = cudaGetLastError();
+    e = launch_pdl_if(wide_overlap(B, H, N), gu_wide_kernel, dim3(gp.tiles < sms ? gp.tiles : sms), 64 + 128 * gu_groups,
+                      smem_for(gp.stages, gp.stage_bytes), stream, mX, mX2, gp);
     return e == cudaSuccess ? e : fail(e, "gate/up kernel launch");
 }
 
@@ -1357,7 +1370,7 @@ cudaError_t launch_down_skinny(const sats_layer *layer, const uint16_t *hact, co
 cudaError_t launch_down_wide(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
                              const int32_t *perm, const KeepLists &lists, int *ctl, cudaStream_t stream)
 {
-    const int N = layer->N, ldn = layer->ldn, sms = sm_count();
+    const int H = layer->H, N = layer->N, ldn = layer->ldn, sms = sm_count();
     CUtensorMap mH, mH2;
     if (!make_map(&mH, hact, M, N, (uint64_t)ldn * 2, BM) || !make_map(&mH2, hact_lo, M, N, (uint64_t)ldn * 2, BM))
         return fail(cudaErrorInvalidValue, "tensor map encoding");
@@ -1384,9 +1397,8 @@ cudaError_t launch_down_wide(const sats_layer *layer, const uint16_t *hact, cons
     static std::atomic<int> cfg_dn[64];
     cudaError_t e = set_smem(down_wide_kernel, smem_for(dp.stages, dp.stage_bytes), cfg_dn);
     if (e != cudaSuccess) return fail(e, "shared-memory attribute");
-    down_wide_kernel<<<dim3(grid), 64 + 128 * kWideDownGroups,
-                       smem_for(dp.stages, dp.stage_bytes), stream>>>(mH, mH2, dp);
-    e = cudaGetLastError();
+    e = launch_pdl_if(wide_overlap(M, H, N), down_wide_kernel, dim3(grid), 64 + 128 * kWideDownGroups,
+                      smem_for(dp.stages, dp.stage_bytes), stream, mH, mH2, dp);
     if (e != cudaSuccess) return fail(e, "down kernel launch");
     return lists.idx && !inside ? launch_keep_lists(lists, M, stream) : cudaSuccess;
 }

@@ -389,10 +389,11 @@ cudaError_t launch_pdl_threads(void (*kernel)(KArgs...), dim3 grid, int threads,
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// As launch_pdl, with `threads` per CTA and `smem` bytes of dynamic shared memory.
+// As launch_pdl, with `threads` per CTA and `smem` bytes of dynamic shared memory; overlap: whether to start
+// before the preceding kernel has ended.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl_cfg(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
-                           Args &&...args)
+cudaError_t launch_pdl_if(bool overlap, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem,
+                          cudaStream_t stream, Args &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -403,8 +404,15 @@ cudaError_t launch_pdl_cfg(void (*kernel)(KArgs...), dim3 grid, int threads, siz
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = overlap ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_cfg(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
+                           Args &&...args)
+{
+    return launch_pdl_if(true, kernel, grid, threads, smem, stream, std::forward<Args>(args)...);
 }
 
 // Dynamic shared memory of a launch: the stage ring, 1 KB of alignment slack and the barriers.
