@@ -1409,12 +1409,13 @@ bool skinny_batch(int B, bool split) { return B <= (split ? kMaxSkinnySplit : kM
 // Whether a skinny batch's gate and up go through the prefill kernel all the same: the skinny one spends an MMA of
 // 128 rows per K step on its R-neuron tile, however few R are (N = 7168: 48), in a time that grows with the tokens.
 // Estimates in us: the epilogue's share, then the longer of the weight stream (the prefill kernel's over the SMs
-// that have a tile) and the MMAs.  The constants are a fit to 13 shapes from 304 x 997 to 8192 x 14336 at 112 to
-// 256 tokens, wrong by up to 6 % near the line, hence the 0.87; below kMinGateUpWide tokens they were not fitted,
-// and little is to be had.  Both sides, us: hidden 1024 / intermediate 4096, 256 bf16 tokens 30.9 skinny, 22.8 so;
-// 4096 / 7168, 160 fp32 tokens 78.1 and 64.2; 8192 / 7168, 128 fp32 tokens 124 and 83; 4096 / 14336, 192 bf16
-// tokens 81.7 (taken) and 90.4.
-constexpr int kMinGateUpWide = 97;
+// that have a tile) and the MMAs.  The constants are a fit to 13 shapes from 304 x 997 to 8192 x 14336 at 64 to 256
+// tokens, wrong by up to 6 % near the line, hence the 0.95; below kMinGateUpWide tokens they were not fitted, and
+// nothing is to be had.  Over those the rule takes 13 % (bf16) and 17 % (fp32) off the time of the skinny kernel
+// alone, and no call got slower.  Both sides, us: hidden 512 / intermediate 1408, 96 bf16 tokens 12.9 skinny, 10.4 so;
+// 1024 / 4096, 256 bf16 31.0 and 19.1; 4096 / 7168, 160 fp32 76.3 and 60.0; 8192 / 7168, 128 fp32 123 and 77;
+// 4096 / 14336, 192 bf16 78.5 (taken) and 83.7.
+constexpr int kMinGateUpWide = 65;
 
 bool gate_up_wide(const sats_layer *layer, int B, bool split)
 {
@@ -1423,11 +1424,11 @@ bool gate_up_wide(const sats_layer *layer, int B, bool split)
     const int Rw = wide_rows(N, layer->tc_R, mtiles, sms, split);
     const int tiles = mtiles * ((N + Rw - 1) / Rw), waves = (tiles + sms - 1) / sms;
     const double steps = H / 64.0, stream = 4.0 * H * N / 6.7e6;
-    const double skinny_mma = (layer->tc_T + sms - 1) / sms * steps * 0.002354 * (NT * (split ? 2 : 1) - 14.4);
-    const double wide_mma = waves * steps * 0.001069 * (BM * (split ? 2 : 1) + 2 * Rw);
-    const double skinny = 0.0219 * NT + std::max(0.937 * stream, skinny_mma);
-    const double wide = 3.28 + std::max(1.232 * stream * waves * sms / tiles, wide_mma);
-    return wide < 0.87 * skinny;
+    const double skinny_mma = (layer->tc_T + sms - 1) / sms * steps * 0.001948 * (NT * (split ? 2 : 1) + 55.9);
+    const double wide_mma = waves * steps * 0.00109 * (BM * (split ? 2 : 1) + 2 * Rw);
+    const double skinny = 0.0263 * NT + std::max(0.899 * stream, skinny_mma);
+    const double wide = 0.968 + std::max(1.256 * stream * waves * sms / tiles, wide_mma);
+    return wide < 0.95 * skinny;
 }
 }  // namespace
 

@@ -1,4 +1,4 @@
-"""Batches of 97 to 256 tokens (224 with fp32 activations) around the line between the two gate/up
+"""Batches of 65 to 256 tokens (224 with fp32 activations) around the line between the two gate/up
 kernels: token counts at the tiles' edges, on layers that the rule sends each way, with the down
 projection of the smaller batches behind either.  Same bounds as the other tensor-core batches."""
 import pytest
@@ -18,12 +18,12 @@ def sats():
 
 
 @pytest.mark.parametrize("H,N", [
-    (512, 1408),     # prefill kernel from 112 (fp32) or about 130 tokens
+    (512, 1408),     # the prefill kernel throughout
     (72, 130),       # one tile of 16 neurons per SM and fewer; a partial K block
     (1024, 777),
     (128, 14600),    # more than one wave of tiles either way
 ])
-@pytest.mark.parametrize("B,f32", [(97, True), (112, True), (113, True), (128, False), (129, False), (129, True),
+@pytest.mark.parametrize("B,f32", [(65, False), (66, True), (97, True), (112, True), (113, True), (128, False), (129, False), (129, True),
                                    (208, False), (224, True), (256, False)])
 def test_either_gate_up_kernel(sats, oracle, H, N, B, f32):
     _run(sats, oracle, H, N, B, 0.6, f32=f32)
