@@ -28,10 +28,28 @@ constexpr size_t kErrKeep = (size_t)1 << 30;
 
 size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 
+// A launch that may start while the preceding kernel ends; the kernel waits for that before it reads or writes.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_after(void (*kernel)(KArgs...), dim3 grid, int threads, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // out[b] = x[b] / sqrt(mean_i x[b][i]^2 + eps) * w  (one CTA per row).
 __global__ void __launch_bounds__(256) rmsnorm_kernel(const float *__restrict__ x, int H, const float *__restrict__ w,
                                                       float eps, float *__restrict__ out)
 {
+    grid_dependency_wait();
+    grid_launch_dependents();
     const float *xr = x + (size_t)blockIdx.x * H;
     float *o = out + (size_t)blockIdx.x * H;
     __shared__ float red[8];
@@ -95,12 +113,17 @@ struct Candidates {
 __global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict__ a, const uint16_t *__restrict__ hhi,
                                                         const uint16_t *__restrict__ hlo, int C, int N, int ld,
                                                         const Candidates cand, int K, uint16_t *__restrict__ rhi,
-                                                        uint16_t *__restrict__ rlo, unsigned long long *counts)
+                                                        uint16_t *__restrict__ rlo, unsigned long long *counts,
+                                                        float4 *__restrict__ out, size_t n4)
 {
     __shared__ unsigned dropped[kErrGroup];
     if (threadIdx.x < kErrGroup) dropped[threadIdx.x] = 0u;
     grid_dependency_wait();   // h and a are the gate/up kernel's
     grid_launch_dependents();
+    // the rows' projection adds into out
+    for (size_t i = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 256 + threadIdx.x; i < n4;
+         i += (size_t)gridDim.x * gridDim.y * 256)
+        out[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
     const int c = blockIdx.x, n0 = (blockIdx.y * 256 + threadIdx.x) * 8;
     const bool in = n0 < N;
@@ -167,6 +190,8 @@ struct SquareSum {
 __global__ void __launch_bounds__(256) drop_err_kernel(const float *__restrict__ y, const float *__restrict__ d, int C,
                                                        int H, float eps, double *__restrict__ acc)
 {
+    grid_dependency_wait();
+    grid_launch_dependents();
     const int c = blockIdx.x, k = blockIdx.y;
     const float4 *yr = reinterpret_cast<const float4 *>(y + (size_t)c * H);
     const float4 *dr = reinterpret_cast<const float4 *>(d + ((size_t)k * C + c) * H);
@@ -283,11 +308,10 @@ sats_status enqueue_rows(const sats_layer *layer, const ErrInputs &in, int C, co
     const int H = layer->H, N = layer->N, ld = layer->ldn;
     int *ctl = reinterpret_cast<int *>(base + W.mlp + ws_layout(H, N, C).ctl);
     uint16_t *rhi = reinterpret_cast<uint16_t *>(base + W.rhi), *rlo = reinterpret_cast<uint16_t *>(base + W.rlo);
-    cudaError_t e = cudaMemsetAsync(out, 0, (size_t)kg * C * H * sizeof(float), st);
-    if (e != cudaSuccess) return cuda_fail(e, "layer error output clear");
-    drop_rows_kernel<<<dim3(C, (ld / 8 + 255) / 256), 256, 0, st>>>(in.a, in.hhi, in.hlo, C, N, ld, cand, kg, rhi, rlo,
-                                                                   dropped);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "dropped rows kernel launch");
+    const cudaError_t e = launch_after(drop_rows_kernel, dim3(C, (ld / 8 + 255) / 256), 256, st, (const float *)in.a,
+                                       (const uint16_t *)in.hhi, (const uint16_t *)in.hlo, C, N, ld, cand, kg, rhi, rlo,
+                                       dropped, reinterpret_cast<float4 *>(out), (size_t)kg * C * H / 4);
+    if (e != cudaSuccess) return cuda_fail(e, "dropped rows kernel launch");
     return run_tc_down(layer, rhi, rlo, kg * C, out, ctl, st) == cudaSuccess ? SATS_OK : SATS_ECUDA;
 }
 
@@ -324,8 +348,8 @@ sats_status enqueue_err(const sats_layer *layer, const ErrInputs &in, int C, con
         }
         const sats_status s = enqueue_rows(layer, in, C, cand, kg, sums.dropped + k0, out, base, W, st);
         if (s != SATS_OK) return s;
-        drop_err_kernel<<<dim3(C, kg), 256, 0, st>>>(in.y, out, C, layer->H, eps, sums.err + k0);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_after(drop_err_kernel, dim3(C, kg), 256, st, (const float *)in.y, (const float *)out,
+                                           C, layer->H, eps, sums.err + k0);
         if (e != cudaSuccess) return cuda_fail(e, "error reduction kernel launch");
     }
     return SATS_OK;
@@ -370,6 +394,8 @@ sats_status layer_err_tc(const sats_layer *layer, const float *x, int C, const f
 
 __global__ void __launch_bounds__(256) add_rows_kernel(float4 *__restrict__ x, const float4 *__restrict__ y, size_t n4)
 {
+    grid_dependency_wait();
+    grid_launch_dependents();
     const size_t i = blockIdx.x * (size_t)256 + threadIdx.x;
     if (i >= n4) return;
     const float4 a = x[i], b = y[i];
@@ -421,8 +447,7 @@ sats_status sats_rmsnorm(const float *x, int B, int H, const float *w, float eps
     if (B < 0 || H < 1 || std::isnan(eps) || eps < 0.0f) return SATS_EINVAL;
     if (B == 0) return SATS_OK;
     if (!x || !w || !out) return SATS_EINVAL;
-    rmsnorm_kernel<<<B, 256, 0, static_cast<cudaStream_t>(stream)>>>(x, H, w, eps, out);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_after(rmsnorm_kernel, dim3(B), 256, static_cast<cudaStream_t>(stream), x, H, w, eps, out);
     return e == cudaSuccess ? SATS_OK : cuda_fail(e, "rmsnorm kernel launch");
 }
 
@@ -623,9 +648,9 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
                                  err_eps, ErrSums(sums + l * sum_bytes, K), ews, E, st)) != SATS_OK)
                 return s;
             const size_t n4 = (size_t)C * H / 4;
-            add_rows_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(
-                reinterpret_cast<float4 *>(x), reinterpret_cast<const float4 *>(inputs_of(l).y), n4);
-            if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "residual kernel launch");
+            e = launch_after(add_rows_kernel, dim3((unsigned)((n4 + 255) / 256)), 256, st, reinterpret_cast<float4 *>(x),
+                             reinterpret_cast<const float4 *>(inputs_of(l).y), n4);
+            if (e != cudaSuccess) return cuda_fail(e, "residual kernel launch");
             continue;
         }
         // x <- x + MLP_l(n_l) with every neuron kept
@@ -867,6 +892,8 @@ __global__ void __launch_bounds__(32 * kTallyWarps) tally_kernel(const int32_t *
 __global__ void score_final_kernel(const double *__restrict__ total, const unsigned *__restrict__ count, int V,
                                    float *__restrict__ score)
 {
+    grid_dependency_wait();
+    grid_launch_dependents();
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= V) return;
     const int at = spread(v, spread_rows(V));
@@ -1068,16 +1095,7 @@ template <typename... KArgs, typename... Args>
 cudaError_t launch_search(void (*kernel)(KArgs...), int V, cudaStream_t st, Args... args)
 {
     const int want = (V + 2 * kTauThreads - 1) / (2 * kTauThreads), sms = fused_grid(kMaxGrid);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(want < sms ? want : sms);
-    cfg.blockDim = dim3(kTauThreads);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+    return launch_after(kernel, dim3(want < sms ? want : sms), kTauThreads, st, args...);
 }
 
 float score_of(uint32_t ordered)
@@ -1114,8 +1132,9 @@ sats_status sats_token_scores(const int32_t *ids, const float *l_base, const flo
     if (e != cudaSuccess) return cuda_fail(e, "score workspace clear");
     if (n > 0 && (e = launch_tally<true>(ids, l_base, l_sparse, n, V, total, count, status, st)) != cudaSuccess)
         return cuda_fail(e, "score kernel launch");
-    score_final_kernel<<<(V + 255) / 256, 256, 0, st>>>(total, count, V, score);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "score kernel launch");
+    e = launch_after(score_final_kernel, dim3((V + 255) / 256), 256, st, (const double *)total, (const unsigned *)count, V,
+                     score);
+    if (e != cudaSuccess) return cuda_fail(e, "score kernel launch");
     return read_status_word(status, st);
 }
 
