@@ -111,7 +111,7 @@ struct Candidates {
 // [K][C][ld]; ld is a multiple of 8, and columns N .. ld - 1 are never read as neurons.  Grid: (C,
 // column blocks of 8 x 256).  Bound by its writes (4 K C N bytes, mostly into L2).
 __global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict__ a, const uint16_t *__restrict__ hhi,
-                                                        const uint16_t *__restrict__ hlo, int C, int N, int ld,
+                                                        const uint16_t *__restrict__ hlo, int C, int N, int ld, int lda,
                                                         const Candidates cand, int K, uint16_t *__restrict__ rhi,
                                                         uint16_t *__restrict__ rlo, unsigned long long *counts,
                                                         float4 *__restrict__ out, size_t n4)
@@ -131,9 +131,15 @@ __global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict_
     uint4 hh = make_uint4(0u, 0u, 0u, 0u), hl = hh;
     if (in) {
         const size_t at = (size_t)c * ld + n0;
-        const float4 p = *reinterpret_cast<const float4 *>(a + at), q = *reinterpret_cast<const float4 *>(a + at + 4);
-        av[0] = p.x; av[1] = p.y; av[2] = p.z; av[3] = p.w;
-        av[4] = q.x; av[5] = q.y; av[6] = q.z; av[7] = q.w;
+        const float *ar = a + (size_t)c * lda + n0;
+        if ((lda & 7) == 0) {
+            const float4 p = reinterpret_cast<const float4 *>(ar)[0], q = reinterpret_cast<const float4 *>(ar)[1];
+            av[0] = p.x; av[1] = p.y; av[2] = p.z; av[3] = p.w;
+            av[4] = q.x; av[5] = q.y; av[6] = q.z; av[7] = q.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) av[e] = n0 + e < N ? ar[e] : 0.f;
+        }
         hh = *reinterpret_cast<const uint4 *>(hhi + at);
         hl = *reinterpret_cast<const uint4 *>(hlo + at);
     }
@@ -293,12 +299,15 @@ struct ErrSums {
 // What the candidates of one block are formed from.
 struct ErrInputs {
     float *y;                // [C][H]: the dense output
-    float *a;                // [C][ldn]: SiLU(x W_gate)
+    float *a;                // [C][lda]: SiLU(x W_gate)
     uint16_t *hhi, *hlo;     // [C][ldn]: a u of every neuron
+    int lda;                 // ldn, or N where a is given (of fp32 accuracy) rather than the gate/up kernel's
+    bool a_given;
     static size_t bytes(int H, int N, int C) { return al256((size_t)C * H * 4 + (size_t)C * ((N + 7) & ~7) * 8); }
-    ErrInputs(void *p, int H, int N, int C)
+    ErrInputs(void *p, int H, int N, int C, bool a_given)
         : y(static_cast<float *>(p)), a(y + (size_t)C * H),
-          hhi(reinterpret_cast<uint16_t *>(a + (size_t)C * ((N + 7) & ~7))), hlo(hhi + (size_t)C * ((N + 7) & ~7)) {}
+          hhi(reinterpret_cast<uint16_t *>(a + (size_t)C * ((N + 7) & ~7))), hlo(hhi + (size_t)C * ((N + 7) & ~7)),
+          lda(a_given ? N : (N + 7) & ~7), a_given(a_given) {}
 };
 
 // The rows of kg candidates (cand) and their product with W_down, into out [kg][C][H].
@@ -309,13 +318,13 @@ sats_status enqueue_rows(const sats_layer *layer, const ErrInputs &in, int C, co
     int *ctl = reinterpret_cast<int *>(base + W.mlp + ws_layout(H, N, C).ctl);
     uint16_t *rhi = reinterpret_cast<uint16_t *>(base + W.rhi), *rlo = reinterpret_cast<uint16_t *>(base + W.rlo);
     const cudaError_t e = launch_after(drop_rows_kernel, dim3(C, (ld / 8 + 255) / 256), 256, st, (const float *)in.a,
-                                       (const uint16_t *)in.hhi, (const uint16_t *)in.hlo, C, N, ld, cand, kg, rhi, rlo,
+                                       (const uint16_t *)in.hhi, (const uint16_t *)in.hlo, C, N, ld, in.lda, cand, kg, rhi, rlo,
                                        dropped, reinterpret_cast<float4 *>(out), (size_t)kg * C * H / 4);
     if (e != cudaSuccess) return cuda_fail(e, "dropped rows kernel launch");
     return run_tc_down(layer, rhi, rlo, kg * C, out, ctl, st) == cudaSuccess ? SATS_OK : SATS_ECUDA;
 }
 
-// h, a and the dense output of one block's inputs x.  The dense output is projected on its own: a stack's next
+// h, a (unless given) and the dense output of one block's inputs x.  The dense output is projected on its own: a stack's next
 // block starts from it, and up to 256 inputs take the batched-decode kernel, whose shorter accumulator chains
 // are the more accurate ones.
 sats_status enqueue_err_inputs(const sats_layer *layer, const float *x, int C, const ErrInputs &in, char *base,
@@ -324,7 +333,7 @@ sats_status enqueue_err_inputs(const sats_layer *layer, const float *x, int C, c
     const WsLayout M = ws_layout(layer->H, layer->N, C);
     char *mlp = base + W.mlp;
     int *ctl = reinterpret_cast<int *>(mlp + M.ctl);
-    if (run_tc_gate_up(layer, x, C, mlp + M.tc, in.hhi, in.hlo, in.a, ctl, st) != cudaSuccess) return SATS_ECUDA;
+    if (run_tc_gate_up(layer, x, C, mlp + M.tc, in.hhi, in.hlo, in.a_given ? nullptr : in.a, ctl, st) != cudaSuccess) return SATS_ECUDA;
     const cudaError_t e = cudaMemsetAsync(in.y, 0, (size_t)C * layer->H * sizeof(float), st);
     if (e != cudaSuccess) return cuda_fail(e, "layer error output clear");
     return run_tc_down(layer, in.hhi, in.hlo, C, in.y, ctl, st) == cudaSuccess ? SATS_OK : SATS_ECUDA;
@@ -377,7 +386,7 @@ sats_status layer_err_tc(const sats_layer *layer, const float *x, int C, const f
     cudaError_t e = clear_fused_state(mlp, layer->H, layer->N, C, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(base + W.acc, 0, sum_bytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "layer error workspace clear");
-    const ErrInputs in(base + W.a, layer->H, layer->N, C);
+    const ErrInputs in(base + W.a, layer->H, layer->N, C, false);
     sats_status s = enqueue_err_inputs(layer, x, C, in, base, W, st);
     if (s == SATS_OK)
         s = enqueue_err(layer, in, C, t, nullptr, [](int k) { return k; }, K, eps, ErrSums(base + W.acc, K), base, W, st);
@@ -602,7 +611,6 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     char *base = static_cast<char *>(ws);
     float *x = reinterpret_cast<float *>(base + W.x);
     float *nall = reinterpret_cast<float *>(base + W.n);
-    float *a = reinterpret_cast<float *>(base + W.a);
     void *sel = base + W.sel;
     float *q = reinterpret_cast<float *>(base + W.q);
     char *ews = base + W.err;
@@ -610,7 +618,13 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     char *sums = base + W.sums;
     const size_t sum_bytes = ErrSums::bytes(Kmax);
     const bool batched = use_tc_path(H, C);
-    auto inputs_of = [&](int l) { return ErrInputs(W.in_each ? base + W.in + l * W.in_each : ews + E.a, H, N, C); };
+    // The masks take the accurate gate activations that the thresholds are percentiles of: a neuron at a threshold
+    // falls on its own side (with the gate/up kernel's, 1.2e-5 off, the shares at the chosen thresholds were off by a
+    // few neurons).
+    auto inputs_of = [&](int l) {
+        return ErrInputs(W.in_each ? base + W.in + l * W.in_each : ews + E.a, H, N, C, true);
+    };
+    auto gate_of = [&](int l) { return batched ? inputs_of(l).a : reinterpret_cast<float *>(base + W.a); };
     const size_t ews_bytes = W.total - W.err;
     void *mlp = ews + E.mlp;
     auto n_of = [&](int l) { return nall + (size_t)l * C * H; };
@@ -629,6 +643,7 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     std::vector<int64_t> rank((size_t)K0 + 1);
     for (int l = 0; l < L; ++l) {
         if ((s = sats_rmsnorm(x, C, H, norm_w[l], eps, n_of(l), stream)) != SATS_OK) return s;
+        float *a = gate_of(l);
         if ((s = sats_gate_act_f32(layers[l], n_of(l), C, a, stream)) != SATS_OK) return s;
         // Eq. 3 at k / K0, the largest |a|, and the guardrail block's percentile at the target, all
         // from shared passes over |a|; read back once after the last block
@@ -725,9 +740,10 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
             ta[(size_t)l * Kt + Kc + k] = t;
         }
         if (K1 == 0) continue;
-        if (batched && W.in_each == 0 &&
-            (s = enqueue_err_inputs(layers[l], n_of(l), C, inputs_of(l), ews, E, st)) != SATS_OK)
-            return s;
+        if (batched && W.in_each == 0) {
+            if ((s = sats_gate_act_f32(layers[l], n_of(l), C, gate_of(l), stream)) != SATS_OK) return s;
+            if ((s = enqueue_err_inputs(layers[l], n_of(l), C, inputs_of(l), ews, E, st)) != SATS_OK) return s;
+        }
         s = batched ? enqueue_err(layers[l], inputs_of(l), C, tf.data() + (size_t)l * K1, nullptr, [](int k) { return k; },
                                   K1, err_eps, ErrSums(sums + l * sum_bytes, K1), ews, E, st)
                     : sats_layer_err(layers[l], n_of(l), C, tf.data() + (size_t)l * K1, K1, err_eps,

@@ -1432,8 +1432,8 @@ bool gate_up_wide(const sats_layer *layer, int B, bool split)
 }
 }  // namespace
 
-// Gate and up projections of B fp32 inputs with every neuron kept: h in bf16 parts and a =
-// SiLU(x W_gate) (all with row stride layer->ldn), for the calibration's masks.  tc_ws: the tensor-core
+// Gate and up projections of B fp32 inputs with every neuron kept: h in bf16 parts and, where
+// wanted, a = SiLU(x W_gate) (all with row stride layer->ldn), for the calibration's masks.  tc_ws: the tensor-core
 // region of a workspace for B tokens.  In passes of up to kGateUpTokens tokens
 // of the skinny kernel, whose epilogue has a thread per neuron and writes a in whole lines.
 constexpr int kGateUpTokens = 128;
@@ -1457,7 +1457,7 @@ cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void 
         a.B = B - m0 < per ? B - m0 : per;
         a.hact = hhi + m0 * ldn;
         a.hact_lo = hlo + m0 * ldn;
-        a.a_out = a_out + m0 * ldn;
+        a.a_out = a_out ? a_out + m0 * ldn : nullptr;
         a.ctl = ctl;
         if ((e = launch_gate_up_skinny(layer, a, stream)) != cudaSuccess) return e;
     }

@@ -137,7 +137,7 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
                          int out_mode, float *out, int32_t *active_idx, int32_t *active_cnt, uint8_t *keep_trace,
                          void *tc_ws, int *ctl, cudaStream_t stream, bool union_path = false);
 // The calibration's halves of it: gate and up of B fp32 inputs with every neuron kept (h in bf16
-// parts and a = SiLU(x W_gate), all with row stride ldn), and the down projection of any M rows of
+// parts and, unless a_out is null, a = SiLU(x W_gate), all with row stride ldn), and the down projection of any M rows of
 // h, added into out.
 cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void *tc_ws, uint16_t *hhi, uint16_t *hlo,
                            float *a_out, int *ctl, cudaStream_t stream);

@@ -1,7 +1,7 @@
 """Eq. 6 in groups of candidates, and the calibration with and without its blocks' inputs kept: sizes at
-which the candidates of a block do not fit one group, and at which what would be kept passes 1 GiB.  Every
-error in the calibration's table is that of a separate evaluation at the same thresholds, and Eq. 6 of a
-few inputs is the definition's."""
+which the candidates of a block do not fit one group, and at which what would be kept passes 1 GiB.  The shares in
+the calibration's table are the accurate gate activations', its errors those of separate evaluations, and
+Eq. 6 of a few inputs is the definition's."""
 import numpy as np
 import pytest
 import torch
@@ -22,6 +22,7 @@ def sats():
 
 @pytest.mark.parametrize("H,N,C,K0,K1", [
     (64, 264, 5, 36, 33),        # more candidates than a group holds
+    (72, 261, 5, 12, 5),         # rows of a that no vector load can take
     (16, 40000, 1700, 8, 2),     # groups of four candidates; 1.1 GB of inputs are not kept
 ])
 def test_table_equals_separate_evaluations(sats, H, N, C, K0, K1):
@@ -35,10 +36,16 @@ def test_table_equals_separate_evaluations(sats, H, N, C, K0, K1):
     n = torch.empty_like(x)
     sats.rmsnorm(x, gains[0], 1e-5, n)
     t, err, sp = (np.asarray(v[0]) for v in r["table"])
-    e2, s2 = sats.layer_err(layers[0], n, list(t), eps=1e-6)
-    # the same kernels on the same inputs: only the order of the output's fp32 additions differs
-    np.testing.assert_allclose(err, e2, rtol=1e-4, atol=1e-6)
-    np.testing.assert_allclose(sp, s2, rtol=0, atol=1e-12)
+    # the shares: exactly those of the accurate gate activations, from which the thresholds come
+    a = torch.empty(C, N, device="cuda")
+    sats.gate_act_f32(layers[0], n, a)
+    a = a.abs_()
+    np.testing.assert_allclose(sp, [float((a < float(v)).double().mean()) for v in t], rtol=0, atol=1e-12)
+    # the errors: between the separate evaluations a relative 1e-4 to either side, whose masks (from activations
+    # 1.2e-5 off) hold every neuron at the threshold on one side
+    lo, _ = sats.layer_err(layers[0], n, list(t * (1 - 1e-4)), eps=1e-6)
+    hi, _ = sats.layer_err(layers[0], n, list(t * (1 + 1e-4)), eps=1e-6)
+    assert (err >= np.minimum(lo, hi) * (1 - 2e-3) - 2e-5).all() and (err <= np.maximum(lo, hi) * (1 + 2e-3) + 2e-5).all()
     assert (np.diff(sp[np.argsort(t)]) >= 0).all()
     for l in layers:
         l.close()
