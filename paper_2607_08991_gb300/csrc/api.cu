@@ -269,13 +269,11 @@ sats_status sats_lora_create(const sats_layer *layer, const void *A_gate, const 
                              static_cast<const uint16_t *>(A_up), static_cast<const uint16_t *>(B_up),
                              static_cast<const uint16_t *>(A_down), static_cast<const uint16_t *>(B_down), l->H, l->N,
                              r, l, st);
-    if (e == cudaSuccess) e = lora_pack_tc(layer, static_cast<const uint16_t *>(A_down), l, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         cudaFree(l->blk);
         cudaFree(l->agu);
         cudaFree(l->bd);
-        cudaFree(l->ad_blk);
         delete l;
         return cuda_fail(e, "adapter allocation or repacking");
     }
@@ -290,11 +288,10 @@ sats_status sats_lora_destroy(sats_lora *lora)
     const cudaError_t e1 = cudaFree(lora->blk);
     const cudaError_t e2 = cudaFree(lora->agu);
     const cudaError_t e3 = cudaFree(lora->bd);
-    const cudaError_t e4 = cudaFree(lora->ad_blk);
     delete lora;
     if (e1 != cudaSuccess) return cuda_fail(e1, "cudaFree");
     if (e2 != cudaSuccess) return cuda_fail(e2, "cudaFree");
-    return from_cuda(e3 != cudaSuccess ? e3 : e4, "cudaFree");
+    return from_cuda(e3, "cudaFree");
 }
 
 static sats_status lora_common(const sats_layer *layer, const sats_lora *lora, int x_mode, const void *x, int B,

@@ -410,12 +410,11 @@ cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, f
 // The sparse path of a fine-tuned model (Sec. 4) for batches beyond one pass of the fused
 // kernel, in the arithmetic of that kernel:
 //   lora_z_kernel        z = x A_gate | x A_up, per slice of hidden rows
-//   lora_gate_up_kernel  g = x W_gate + s z B_gate[:, n], u likewise, h = keep ? SiLU(g) u : 0
-//   lora_down_kernel     y += h W_down, w += h A_down (one more tile of outputs)
-//   lora_out_kernel      y += s w B_down
+//   lora_gate_up_kernel  g = x W_gate + s z B_gate[:, n], u likewise, h = keep ? SiLU(g) u : 0, w += h A_down
+//   lora_down_kernel     y += h W_down + s w B_down
 // W is streamed once for up to kLoraTok tokens, where the fused kernel streamed it once per pass
 // of one or two (129 us for four tokens on the Llama-shaped layer at 70 % sparsity, 267 us for
-// eight; 79 and 80 here).  What bounds it: that stream and the roles' serial issue; with at most 32 tokens the parts of an operand are the
+// eight; 77 here; with A_down as one more tile of outputs and w B_down in a kernel of its own 79 and 80).  What bounds it: that stream and the roles' serial issue; with at most 32 tokens the parts of an operand are the
 // rows of one tile, so a K step is one MMA per weight tile however many parts there are, and
 // their products are added in the epilogue.
 constexpr int kLoraTok = 32;
@@ -425,10 +424,10 @@ constexpr int kLoraEpiThreads = 256;           // two groups of four warps, one 
 template <bool F32> constexpr int kLoraGuThreads = 64 + (F32 ? kConvThreads : 0) + kLoraEpiThreads;
 constexpr int kLoraDownThreads = 64 + kConvThreads + kLoraEpiThreads;
 
-// z[b][s][0 .. 2r) over the hidden rows of slice s.  Grid: (slices, B).
+// z[b][s][0 .. 2r) over the hidden rows of slice s, and w[b] cleared.  Grid: (slices, B).
 template <typename X>
 __global__ void __launch_bounds__(256) lora_z_kernel(const X *__restrict__ x, int H, const uint16_t *__restrict__ agu,
-                                                     int r, float *__restrict__ z)
+                                                     int r, float *__restrict__ z, float *__restrict__ wsum)
 {
     __shared__ float red[256][9];
     const int s = blockIdx.x, slices = gridDim.x, b = blockIdx.y, t = threadIdx.x;
@@ -437,6 +436,7 @@ __global__ void __launch_bounds__(256) lora_z_kernel(const X *__restrict__ x, in
     const int h0 = (int)((long long)H * s / slices), h1 = (int)((long long)H * (s + 1) / slices);
     grid_dependency_wait();
     grid_launch_dependents();
+    if (s == 0 && t < kLoraWRow) wsum[(size_t)b * kLoraWRow + t] = 0.f;   // the gate/up kernel adds into it
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
@@ -478,7 +478,7 @@ struct LoraGuParams {
     uint8_t *keep;          // [B][keep_stride] or nullptr
     int keep_stride;
     float *y;               // [B][H], cleared here for the down kernel's additions
-    float *wsum;            // [B][kLoraWRow], likewise
+    float *wsum;            // [B][kLoraWRow]: w = h A_down, added to
     int *ctl;
     int stages, stage_bytes, w_bytes, ring_bytes;
     uint32_t tmem_cols;
@@ -654,7 +654,6 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
         for (long long i = (long long)cta * kLoraEpiThreads + et; i < (long long)p.B * (p.H >> 2);
              i += (long long)ctas * kLoraEpiThreads)
             reinterpret_cast<float4 *>(p.y)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int i = cta * kLoraEpiThreads + et; i < p.B * kLoraWRow; i += ctas * kLoraEpiThreads) p.wsum[i] = 0.f;
         const int r = p.r, r2 = 2 * r;
         for (int i = et; i < NT * r2; i += kLoraEpiThreads) {
             const int j = i / r2, c = i % r2;
@@ -664,11 +663,15 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
             zs[j][c] = v;
         }
         named_barrier(1, kLoraEpiThreads);
-        if (ok && busy && 32 * quad + lane < R && n < p.N) {
+        const bool mine = ok && busy && 32 * quad + lane < R && n < p.N;
+        const uint16_t *col = p.blk + (size_t)n * 3 * r;
+        float hv[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) hv[e] = 0.f;
+        if (mine) {
             float lg[16], lu[16];
 #pragma unroll
             for (int e = 0; e < 16; ++e) lg[e] = lu[e] = 0.f;
-            const uint16_t *col = p.blk + (size_t)n * 3 * r;
             for (int q0 = 0; q0 < r; q0 += 8) {
                 float bg[8], bu[8];
                 unpack8(*reinterpret_cast<const uint4 *>(col + q0), bg);
@@ -689,9 +692,35 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
                     const float u = fmaf(p.scale, lu[e], acc[1][e]);
                     const float a = g / (1.0f + expf(-g));   // SiLU, Eq. 2
                     const bool keep = fabsf(a) >= p.t_l;     // Eqs. 4-5
-                    p.h[(size_t)j * p.ldh + n] = keep ? a * u : 0.f;
+                    hv[e] = keep ? a * u : 0.f;
+                    p.h[(size_t)j * p.ldh + n] = hv[e];
                     if (p.keep) p.keep[(size_t)j * p.keep_stride + n] = keep ? 1 : 0;
                 }
+            }
+        }
+        // w += h A_down: 4 tokens x 8 rank columns at a time, summed over the warp's neurons so that lane k is left
+        // with token k mod 4, column k / 4
+        for (int q0 = 0; busy && q0 < r; q0 += 8) {
+            float ad[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) ad[q] = 0.f;
+            if (mine) unpack8(*reinterpret_cast<const uint4 *>(col + 2 * r + q0), ad);
+#pragma unroll
+            for (int t0 = 0; t0 < 16; t0 += 4) {
+                if (m0 + c0 + t0 >= p.B) break;
+                float x[32];
+#pragma unroll
+                for (int k = 0; k < 32; ++k) x[k] = hv[t0 + (k & 3)] * ad[k >> 2];
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1)
+#pragma unroll
+                    for (int k = 0; k < o; ++k) {
+                        const bool up = lane & o;
+                        const float give = up ? x[k] : x[k + o], have = up ? x[k + o] : x[k];
+                        x[k] = have + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+                const int j = m0 + c0 + t0 + (lane & 3);
+                if (j < p.B && c0 + t0 + (lane & 3) < NT) atomicAdd(p.wsum + (size_t)j * kLoraWRow + q0 + (lane >> 2), x[0]);
             }
         }
     }
@@ -711,14 +740,15 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
 
 struct LoraDownParams {
     const uint16_t *w;      // wd_blk
-    const uint16_t *ad;     // ad_blk: A_down as one more hidden tile of kMaxLoraRank rows
     const float *h;         // [B][ldh] fp32
     int ldh, B, H, N;
     int NT, halves;
-    int KBn, dt, units;     // units = (dt + 1) KBn: (hidden tile or A_down, neuron block) pairs
+    int KBn, units;         // units = hidden tiles x KBn: (hidden tile, neuron block) pairs
+    const uint16_t *bd;     // B_down [r][H]
     int r;
+    float scale;
     float *y;               // [B][H], added to
-    float *wsum;            // [B][kLoraWRow], added to
+    const float *wsum;      // [B][kLoraWRow]
     int *ctl;
     int stages, ring_bytes;
     uint32_t tmem_cols;
@@ -726,7 +756,8 @@ struct LoraDownParams {
 };
 
 // CTA c takes units [c U / G, (c + 1) U / G) in order for the tokens of tile blockIdx.y; consecutive
-// units of one output tile are summed in registers and added into y (or w).
+// units of one output tile are summed in registers and added into y, with s w B_down by the CTA of the tile's
+// first unit.
 __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const LoraDownParams p)
 {
     constexpr int kEpi0 = 2 + kConvThreads / 32;
@@ -744,6 +775,7 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
     __shared__ int abort_flag, issued_s, consumed_s;
     __shared__ float tr[kLoraEpiThreads / 32][16][33];
+    __shared__ __align__(16) float ws[kLoraTok][kLoraWRow];   // s w
     const int warp = uniform_warp(), lane = threadIdx.x & 31;
     const int NT = p.NT, S = p.stages, KBn = p.KBn, halves = p.halves, NX = kParts * NT;
     const int m0 = (int)blockIdx.y * NT;
@@ -784,13 +816,10 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
         int i = 0;
         for (int s = 0, ph = 0; i < nu; ++i) {
             if (!warp_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)) { set_timeout(p.ctl, &abort_flag); break; }
-            const int u = u0 + i, d = u / KBn;
-            const bool ad = d == p.dt;
-            const uint32_t bytes = (uint32_t)((ad ? kMaxLoraRank : BM) * kTileBytes);
-            const uint16_t *src = ad ? p.ad + (size_t)(u - d * KBn) * kMaxLoraRank * BK : p.w + (size_t)u * BM * BK;
-            mbar_expect_if(lead, &full[s], bytes);
-            if (gridDim.y == 1) bulk_load_if(lead, ring + (size_t)s * kA, src, bytes, &full[s], once);
-            else bulk_load_shared_if(lead, ring + (size_t)s * kA, src, bytes, &full[s]);
+            const uint16_t *src = p.w + (size_t)(u0 + i) * BM * BK;
+            mbar_expect_if(lead, &full[s], (uint32_t)kA);
+            if (gridDim.y == 1) bulk_load_if(lead, ring + (size_t)s * kA, src, (uint32_t)kA, &full[s], once);
+            else bulk_load_shared_if(lead, ring + (size_t)s * kA, src, (uint32_t)kA, &full[s]);
             if (++s == S) { s = 0; ph ^= 1; }
         }
         issued_s = i;
@@ -843,11 +872,17 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
         };
         if (!cut_tiles<kLoraTok>(parts, NT, nu, pfull, pempty, &abort_flag, load)) set_timeout(p.ctl, &abort_flag);
     } else if (warp >= kEpi0) {
-        grid_dependency_wait();   // y and w are cleared, and the keep bytes written, by the preceding kernel
+        grid_dependency_wait();   // y is cleared, w and the keep bytes written by the preceding kernel
+        const int et = threadIdx.x - 32 * kEpi0;
+        for (int i = et; i < NT * kLoraWRow; i += kLoraEpiThreads) {
+            const int j = i / kLoraWRow, q = i % kLoraWRow;
+            ws[j][q] = m0 + j < p.B && q < p.r ? p.scale * p.wsum[(size_t)(m0 + j) * kLoraWRow + q] : 0.f;
+        }
+        named_barrier(1, kLoraEpiThreads);
         __shared__ int warp_sums[kLoraEpiThreads / 32];
         if (blockIdx.y == 0)
             for (int m = blockIdx.x; p.lists.idx && m < p.B; m += gridDim.x)
-                write_keep_list(p.lists, m, (int)threadIdx.x - 32 * kEpi0, kLoraEpiThreads, warp_sums, 1);
+                write_keep_list(p.lists, m, et, kLoraEpiThreads, warp_sums, 1);
         const int quad = warp & 3, grp = (warp - kEpi0) >> 2;
         const int c0 = 16 * grp;
         const bool busy = c0 < NT;
@@ -884,7 +919,25 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
             if (i + 1 < nu && (u + 1) / KBn == d) continue;
             // the last unit of this output tile: 32 rows x 16 tokens through shared memory, so that each
             // lane adds four vectors of four hidden units of one token
-            if (busy && d < p.dt) {
+            if (busy) {
+                const int row = d * BM + 32 * quad + lane;
+                if (d * KBn >= u0 && row < p.H) {   // this CTA has the tile's first unit
+                    float l[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) l[e] = 0.f;
+                    for (int q = 0; q < p.r; q += 4) {   // (ranks are multiples of 8)
+                        float b[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) b[k] = __uint_as_float((uint32_t)p.bd[(size_t)(q + k) * p.H + row] << 16);
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            const float4 w = *reinterpret_cast<const float4 *>(&ws[c0 + e][q]);
+                            l[e] = fmaf(w.w, b[3], fmaf(w.z, b[2], fmaf(w.y, b[1], fmaf(w.x, b[0], l[e]))));
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) acc[e] += l[e];
+                }
 #pragma unroll
                 for (int e = 0; e < 16; ++e) T[e][lane] = acc[e];
                 __syncwarp();
@@ -898,10 +951,6 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
                                        T[te][r0 + 4 * k + 3]);
                 }
                 __syncwarp();
-            } else if (busy && quad == 0 && lane < p.r) {   // row q of A_down's tile
-#pragma unroll
-                for (int e = 0; e < 16; ++e)
-                    if (m0 + c0 + e < p.B && c0 + e < NT) atomicAdd(p.wsum + (size_t)(m0 + c0 + e) * kLoraWRow + lane, acc[e]);
             }
 #pragma unroll
             for (int e = 0; e < 16; ++e) acc[e] = 0.f;
@@ -918,43 +967,6 @@ __global__ void __launch_bounds__(kLoraDownThreads, 1) lora_down_kernel(const Lo
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, p.tmem_cols);
-    }
-}
-
-// y[b] += scale w[b] B_down.  Grid: (blocks of 8 x 128 hidden units, B).
-__global__ void __launch_bounds__(128) lora_out_kernel(const float *__restrict__ wsum, const uint16_t *__restrict__ bd,
-                                                       int H, int r, float scale, float *__restrict__ y)
-{
-    const int b = blockIdx.y, h = (blockIdx.x * 128 + threadIdx.x) * 8;
-    grid_dependency_wait();
-    grid_launch_dependents();
-    if (h >= H) return;
-    float acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-#pragma unroll 8
-    for (int q = 0; q < r; ++q) {
-        float w[8];
-        unpack8(*reinterpret_cast<const uint4 *>(bd + (size_t)q * H + h), w);
-        const float v = scale * wsum[(size_t)b * kLoraWRow + q];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] = fmaf(v, w[e], acc[e]);
-    }
-    float4 *dst = reinterpret_cast<float4 *>(y + (size_t)b * H + h);
-    const float4 p = dst[0], q = dst[1];
-    dst[0] = make_float4(p.x + acc[0], p.y + acc[1], p.z + acc[2], p.w + acc[3]);
-    dst[1] = make_float4(q.x + acc[4], q.y + acc[5], q.z + acc[6], q.w + acc[7]);
-}
-
-// A_down [N][r] as tiles [kb][q][64] of kMaxLoraRank rows (row q, neuron kb 64 + c), 128-byte swizzled;
-// rows past r and neurons past N are zero.
-__global__ void pack_ad_kernel(const uint16_t *__restrict__ Ad, int N, int r, int KBn, uint16_t *__restrict__ dst)
-{
-    const size_t total = (size_t)KBn * kMaxLoraRank * BK;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % BK), q = (int)(i / BK % kMaxLoraRank), kb = (int)(i / BK / kMaxLoraRank);
-        const int n = kb * BK + c;
-        dst[(i / BK) * BK + (size_t)(((c / 8) ^ (q & 7)) * 8) + c % 8] = (n < N && q < r) ? Ad[(size_t)n * r + q] : (uint16_t)0;
     }
 }
 
@@ -1007,14 +1019,6 @@ bool lora_tc_ok(int H, int B)
     return use_tc_path(H, B) && B >= 3 && B <= 65535 && need <= 4 * H;
 }
 
-cudaError_t lora_pack_tc(const sats_layer *layer, const uint16_t *Ad, sats_lora *l, cudaStream_t stream)
-{
-    const cudaError_t e = cudaMalloc(&l->ad_blk, (size_t)layer->tc_kbn * kMaxLoraRank * tc::BK * 2);
-    if (e != cudaSuccess) return e;
-    tc::pack_ad_kernel<<<256, 256, 0, stream>>>(Ad, l->N, l->r, layer->tc_kbn, l->ad_blk);
-    return cudaGetLastError();
-}
-
 cudaError_t run_lora_tc(const sats_layer *layer, const sats_lora *lora, bool x_f32, const void *x, int B, float t_l,
                         float *y, int32_t *active_idx, int32_t *active_cnt, void *tc_ws, int *ctl, cudaStream_t stream)
 {
@@ -1033,10 +1037,10 @@ cudaError_t run_lora_tc(const sats_layer *layer, const sats_lora *lora, bool x_f
     };
     cudaError_t e =
         x_f32 ? launch_pdl_threads(lora_z_kernel<float>, dim3(slices, B), 256, stream, static_cast<const float *>(x), H,
-                                   static_cast<const uint16_t *>(lora->agu), lora->r, z)
+                                   static_cast<const uint16_t *>(lora->agu), lora->r, z, wsum)
               : launch_pdl_threads(lora_z_kernel<uint16_t>, dim3(slices, B), 256, stream,
                                    static_cast<const uint16_t *>(x), H, static_cast<const uint16_t *>(lora->agu),
-                                   lora->r, z);
+                                   lora->r, z, wsum);
     if (e != cudaSuccess) return failed(e, "adapter input kernel launch");
 
     const int mt = (B + kLoraTok - 1) / kLoraTok;
@@ -1067,7 +1071,6 @@ cudaError_t run_lora_tc(const sats_layer *layer, const sats_lora *lora, bool x_f
 
     LoraDownParams dp{};
     dp.w = layer->wd_blk;
-    dp.ad = lora->ad_blk;
     dp.h = h;
     dp.ldh = layer->ldn;
     dp.B = B;
@@ -1076,9 +1079,10 @@ cudaError_t run_lora_tc(const sats_layer *layer, const sats_lora *lora, bool x_f
     dp.NT = gp.NT;
     dp.halves = 2;
     dp.KBn = layer->tc_kbn;
-    dp.dt = layer->tc_dt;
-    dp.units = (dp.dt + 1) * dp.KBn;
+    dp.units = layer->tc_dt * dp.KBn;
+    dp.bd = lora->bd;
     dp.r = lora->r;
+    dp.scale = lora->scale;
     dp.y = y;
     dp.wsum = wsum;
     dp.lists = {keep, gp.keep_stride, N, active_idx, active_cnt, nullptr};
@@ -1092,10 +1096,7 @@ cudaError_t run_lora_tc(const sats_layer *layer, const sats_lora *lora, bool x_f
     if ((e = set_smem(lora_down_kernel, smem, cfg)) != cudaSuccess) return failed(e, "shared-memory attribute");
     const int sms = sm_count();
     e = launch_pdl_cfg(lora_down_kernel, dim3(dp.units < sms ? dp.units : sms, mt), kLoraDownThreads, smem, stream, dp);
-    if (e != cudaSuccess) return failed(e, "adapted down kernel launch");
-    e = launch_pdl_threads(lora_out_kernel, dim3((H + 1023) / 1024, B), 128, stream, static_cast<const float *>(wsum),
-                           static_cast<const uint16_t *>(lora->bd), H, lora->r, lora->scale, y);
-    return e == cudaSuccess ? e : failed(e, "adapter output kernel launch");
+    return e == cudaSuccess ? e : failed(e, "adapted down kernel launch");
 }
 
 }  // namespace sats

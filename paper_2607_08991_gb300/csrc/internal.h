@@ -34,7 +34,6 @@ struct sats_lora {
     uint16_t *blk = nullptr;      // [ceil(N / 8)][8][3 r]: neuron j's B_gate[:, j], B_up[:, j], A_down[j, :]
     uint16_t *agu = nullptr;      // [H][2 r]: A_gate[h, :], A_up[h, :]
     uint16_t *bd = nullptr;       // [r][H]: B_down
-    uint16_t *ad_blk = nullptr;   // [ceil(N / 64)][32][64]: A_down as a weight tile of the down projection (batches)
 };
 
 namespace sats {
@@ -149,10 +148,8 @@ struct TcRegions {
     size_t x, h, keep;
 };
 TcRegions tc_regions(int H, int N, int B);
-// gemm_f32.cu: LoRA batches beyond one pass of the fused kernel.  lora_pack_tc allocates and fills
-// ad_blk; lora_tc_ok says whether a batch's scratch fits its workspace (hidden sizes of 96 and more).
+// gemm_f32.cu: LoRA batches beyond one pass of the fused kernel.  lora_tc_ok says whether a batch's scratch fits its workspace (hidden sizes of 96 and more).
 bool lora_tc_ok(int H, int B);
-cudaError_t lora_pack_tc(const sats_layer *layer, const uint16_t *Ad, sats_lora *l, cudaStream_t stream);
 cudaError_t run_lora_tc(const sats_layer *layer, const sats_lora *lora, bool x_f32, const void *x, int B, float t_l,
                         float *y, int32_t *active_idx, int32_t *active_cnt, void *tc_ws, int *ctl, cudaStream_t stream);
 cudaError_t launch_wait_timeout(int *ctl, cudaStream_t stream);
