@@ -339,7 +339,7 @@ __device__ void gate_producer(const FusedParams &p, Shared<BT> &S, uint8_t *grin
     for (int seq = 0;; ++seq) {
         const int buf = seq % kBufs;
         // the buffer's previous list has been formed (first kBufs uses pass)
-        if (!mbar_wait(&S.bfree[buf], ((uint32_t)(seq / kBufs) & 1u) ^ 1u, &S.abort)) { ok = false; break; }
+        if (!mbar_wait<LORA>(&S.bfree[buf], ((uint32_t)(seq / kBufs) & 1u) ^ 1u, &S.abort)) { ok = false; break; }
         const bool fixed = seq < kStatic && static_chunk(seq) < nch;
         int k;
         if (fixed) {
@@ -359,7 +359,7 @@ __device__ void gate_producer(const FusedParams &p, Shared<BT> &S, uint8_t *grin
         S.chunkrows[buf] = rows;
         for (int r0 = 0; r0 < rows; r0 += rows_per_stage) {
             const int nr = min(rows_per_stage, rows - r0);
-            if (!mbar_wait(&S.gempty[stage], phase ^ 1u, &S.abort)) { ok = false; break; }
+            if (!mbar_wait<LORA>(&S.gempty[stage], phase ^ 1u, &S.abort)) { ok = false; break; }
             GateDesc &d = S.gdesc[stage];
             d.kind = kRows;
             d.nrows = nr;
@@ -385,7 +385,7 @@ __device__ void gate_producer(const FusedParams &p, Shared<BT> &S, uint8_t *grin
             // first chunk's mask came 1.3 us after the dependency was released (instrumented).
             // (each ring slot on the latest phase this loop issued: only this thread re-arms a slot)
             for (int s2 = 0; s2 < kGateStages && ok; ++s2)
-                if (S.gissued[s2] > 0) ok = mbar_wait(&S.gfull[s2], (uint32_t)(S.gissued[s2] - 1), &S.abort);
+                if (S.gissued[s2] > 0) ok = mbar_wait<LORA>(&S.gfull[s2], (uint32_t)(S.gissued[s2] - 1), &S.abort);
             if (!ok) break;
             prefetch_fixed();
         }
@@ -406,7 +406,7 @@ __device__ void gate_producer(const FusedParams &p, Shared<BT> &S, uint8_t *grin
             next_k = claim();
         }
     }
-    if (ok && mbar_wait(&S.gempty[stage], phase ^ 1u, &S.abort)) {
+    if (ok && mbar_wait<LORA>(&S.gempty[stage], phase ^ 1u, &S.abort)) {
         S.gdesc[stage].kind = kEnd;
         mbar_arrive(&S.gfull[stage]);
     } else {
@@ -818,8 +818,8 @@ __device__ void list_producer(const FusedParams &p, Shared<BT> &S, uint8_t *urin
         for (int j = j0 + lane; j < j1; j += 32) p.flags[j] = 0ull;
     }
     __threadfence();
-    bool ok = mbar_wait(&S.xloaded, 0u, &S.abort);
-    if constexpr (LORA) ok = ok && mbar_wait(&lora_of(S).zdone, 0u, &S.abort);   // this CTA's slice of x A is added
+    bool ok = mbar_wait<LORA>(&S.xloaded, 0u, &S.abort);
+    if constexpr (LORA) ok = ok && mbar_wait<LORA>(&lora_of(S).zdone, 0u, &S.abort);   // this CTA's slice of x A is added
     __syncwarp();
     if (ok && lane == 0) {
         // this CTA has read its activations, zeroed its slice of y and cleared its flags
@@ -851,7 +851,7 @@ __device__ void list_producer(const FusedParams &p, Shared<BT> &S, uint8_t *urin
     };
     for (int seq = 0; ok; ++seq) {
         const int buf = seq % kBufs;
-        if (!mbar_wait(&S.gsync[buf], (uint32_t)(seq / kBufs) & 1u, &S.abort)) { ok = false; break; }
+        if (!mbar_wait<LORA>(&S.gsync[buf], (uint32_t)(seq / kBufs) & 1u, &S.abort)) { ok = false; break; }
         __syncwarp();
         const int n0 = S.chunkq[buf];
         if (n0 < 0) break;
@@ -901,7 +901,7 @@ __device__ void list_producer(const FusedParams &p, Shared<BT> &S, uint8_t *urin
         const int nid = n0 + lane;
         for (int k0 = 0; k0 < cnt; k0 += geo.rows) {
             const int nr = min(geo.rows, cnt - k0);
-            if (!mbar_wait(&S.uempty[stage], phase ^ 1u, &S.abort)) { ok = false; break; }
+            if (!mbar_wait<LORA>(&S.uempty[stage], phase ^ 1u, &S.abort)) { ok = false; break; }
             UdDesc<BT> &d = S.udesc[stage];
             const bool in_stage = mine && pos >= k0 && pos < k0 + nr;
             if (in_stage) {
@@ -944,7 +944,7 @@ __device__ void list_producer(const FusedParams &p, Shared<BT> &S, uint8_t *urin
         S.seen = flags_open ? 1 : 0;
     }
     __syncwarp();
-    if (ok && mbar_wait(&S.uempty[stage], phase ^ 1u, &S.abort)) {
+    if (ok && mbar_wait<LORA>(&S.uempty[stage], phase ^ 1u, &S.abort)) {
         if (lane == 0) {
             S.udesc[stage].kind = kEnd;
             mbar_arrive(&S.ufull[stage]);
@@ -1129,7 +1129,7 @@ __device__ bool updown_warps(const FusedParams &p, Shared<BT> &S, const uint8_t 
     // still to do (done while waiting on the next stage's barrier)
     int pend_stage = -1, pend_nr = 0, pend_ub = 0;
     for (;;) {
-        if (!mbar_wait(&S.ufull[stage], phase, &S.abort)) {
+        if (!mbar_wait<LORA>(&S.ufull[stage], phase, &S.abort)) {
             S.abort = 1;
             flag_status(p.ctl, kStatusTimeout);
             return false;
