@@ -106,12 +106,12 @@ struct Candidates {
     const float *dev;
 };
 
-// Row (k, c) of the dropped neurons' h, in bf16 parts: h where |a| < t_k, 0 elsewhere, for the K
-// candidates of a group; counts[k] += the neurons dropped.  h (hi, lo) and a are [C][ld], the rows
-// [K][C][ld]; ld is a multiple of 8, and columns N .. ld - 1 are never read as neurons.  Grid: (C,
+// The rows of a group of K candidates, in bf16 parts: row (0, c) is h of every neuron (for the dense output), row
+// (k + 1, c) is h where |a| < t_k, 0 elsewhere; counts[k] += the neurons dropped.  h (hi, lo) is [C][ld], a [C][N],
+// the rows [K + 1][C][ld]; ld is a multiple of 8, and columns N .. ld - 1 are never read as neurons.  Grid: (C,
 // column blocks of 8 x 256).  Bound by its writes (4 K C N bytes, mostly into L2).
 __global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict__ a, const uint16_t *__restrict__ hhi,
-                                                        const uint16_t *__restrict__ hlo, int C, int N, int ld, int lda,
+                                                        const uint16_t *__restrict__ hlo, int C, int N, int ld,
                                                         const Candidates cand, int K, uint16_t *__restrict__ rhi,
                                                         uint16_t *__restrict__ rlo, unsigned long long *counts,
                                                         float4 *__restrict__ out, size_t n4)
@@ -131,8 +131,8 @@ __global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict_
     uint4 hh = make_uint4(0u, 0u, 0u, 0u), hl = hh;
     if (in) {
         const size_t at = (size_t)c * ld + n0;
-        const float *ar = a + (size_t)c * lda + n0;
-        if ((lda & 7) == 0) {
+        const float *ar = a + (size_t)c * N + n0;
+        if ((N & 7) == 0) {
             const float4 p = reinterpret_cast<const float4 *>(ar)[0], q = reinterpret_cast<const float4 *>(ar)[1];
             av[0] = p.x; av[1] = p.y; av[2] = p.z; av[3] = p.w;
             av[4] = q.x; av[5] = q.y; av[6] = q.z; av[7] = q.w;
@@ -142,6 +142,8 @@ __global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict_
         }
         hh = *reinterpret_cast<const uint4 *>(hhi + at);
         hl = *reinterpret_cast<const uint4 *>(hlo + at);
+        *reinterpret_cast<uint4 *>(rhi + at) = hh;
+        *reinterpret_cast<uint4 *>(rlo + at) = hl;
     }
     for (int k = 0; k < K; ++k) {
         const float t = cand.dev ? cand.dev[cand.at[k]] : cand.t[k];
@@ -154,7 +156,7 @@ __global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict_
                 cnt += drop ? 1u : 0u;
                 m[e / 2] |= drop ? (e & 1 ? 0xffff0000u : 0xffffu) : 0u;
             }
-            const size_t at = ((size_t)k * C + c) * ld + n0;
+            const size_t at = ((size_t)(k + 1) * C + c) * ld + n0;
             *reinterpret_cast<uint4 *>(rhi + at) = make_uint4(hh.x & m[0], hh.y & m[1], hh.z & m[2], hh.w & m[3]);
             *reinterpret_cast<uint4 *>(rlo + at) = make_uint4(hl.x & m[0], hl.y & m[1], hl.z & m[2], hl.w & m[3]);
         }
@@ -165,93 +167,119 @@ __global__ void __launch_bounds__(256) drop_rows_kernel(const float *__restrict_
     if (threadIdx.x < K && dropped[threadIdx.x]) atomicAdd(counts + threadIdx.x, (unsigned long long)dropped[threadIdx.x]);
 }
 
-// A sum of squares carried as an unevaluated pair of floats (error-free product and sums), about
-// 48 bits: this GPU's 64-bit rate is 1/64 of its 32-bit one.
+// A sum of squares as an unevaluated sum of three floats (the product's error by FMA, the sums' by Knuth's TwoSum),
+// more than the 53 bits of a double: this GPU's 64-bit rate is 1/64 of its 32-bit one (1344 rows of 4096: 33 us in
+// doubles, 10 so).
 struct SquareSum {
-    float hi = 0.f, lo = 0.f;
-    __device__ void join(float v, float rest)   // += v + rest, |rest| far below |v|
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+    static __device__ float two_sum(float &s, float v)   // s += v; returns what the sum was rounded by
     {
-        const float s = __fadd_rn(hi, v), b = __fadd_rn(s, -hi);
-        lo += (__fadd_rn(hi, -__fadd_rn(s, -b)) + __fadd_rn(v, -b)) + rest;
-        hi = s;
+        const float t = __fadd_rn(s, v), b = __fadd_rn(t, -s);
+        const float e = __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -b)), __fadd_rn(v, -b));
+        s = t;
+        return e;
+    }
+    __device__ void join(float v0, float v1, float v2)
+    {
+        const float e0 = two_sum(s1, two_sum(s0, v0)), e1 = two_sum(s1, v1);
+        s2 += (e0 + e1) + v2;
     }
     __device__ void add(float v)
     {
         const float p = __fmul_rn(v, v);
-        join(p, __fmaf_rn(v, v, -p));
+        join(p, __fmaf_rn(v, v, -p), 0.f);
     }
-    __device__ void over_warp()
-    {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
-            join(h, l);
-        }
-    }
-    __device__ double value() const { return (double)hi + (double)lo; }
+    __device__ double value() const { return ((double)s2 + (double)s1) + (double)s0; }
 };
 
-// Token c, candidate k: acc[k] += ||d_kc|| / (||y_c|| + eps), with d = y - y~_t (the dropped
-// neurons' output, rows [K][C][H]) and y the dense output [C][H].  Grid: (C, K).
-__global__ void __launch_bounds__(256) drop_err_kernel(const float *__restrict__ y, const float *__restrict__ d, int C,
-                                                       int H, float eps, double *__restrict__ acc)
+// sq[r] = ||row r||^2 of the group's outputs [rows][H].  Grid: rows.
+__global__ void __launch_bounds__(256) row_squares_kernel(const float *__restrict__ out, int H, double *__restrict__ sq)
 {
     grid_dependency_wait();
     grid_launch_dependents();
-    const int c = blockIdx.x, k = blockIdx.y;
-    const float4 *yr = reinterpret_cast<const float4 *>(y + (size_t)c * H);
-    const float4 *dr = reinterpret_cast<const float4 *>(d + ((size_t)k * C + c) * H);
-    SquareSum sd, sy;
+    const float *row = out + (size_t)blockIdx.x * H;
+    SquareSum s;
     for (int i = threadIdx.x; i < (H >> 2); i += 256) {   // H is a multiple of 8
-        const float4 p = dr[i], q = yr[i];
-        sd.add(p.x); sd.add(p.y); sd.add(p.z); sd.add(p.w);
-        sy.add(q.x); sy.add(q.y); sy.add(q.z); sy.add(q.w);
+        const float4 p = reinterpret_cast<const float4 *>(row)[i];
+        s.add(p.x); s.add(p.y); s.add(p.z); s.add(p.w);
     }
-    __shared__ float part[2][8][2];
-    __shared__ double sums[2];
-    sd.over_warp();
-    sy.over_warp();
-    if ((threadIdx.x & 31) == 0) {
-        const int w = threadIdx.x >> 5;
-        part[0][w][0] = sd.hi; part[0][w][1] = sd.lo;
-        part[1][w][0] = sy.hi; part[1][w][1] = sy.lo;
-    }
-    __syncthreads();
-    if (threadIdx.x < 2) {
-        SquareSum s;
-        for (int w = 0; w < 8; ++w) s.join(part[threadIdx.x][w][0], part[threadIdx.x][w][1]);
-        sums[threadIdx.x] = s.value();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        s.join(__shfl_xor_sync(0xffffffffu, s.s0, o), __shfl_xor_sync(0xffffffffu, s.s1, o),
+               __shfl_xor_sync(0xffffffffu, s.s2, o));
+    __shared__ float part[8][3];
+    __shared__ double wide[8];
+    __shared__ bool again;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane == 0) {
+        part[warp][0] = s.s0;
+        part[warp][1] = s.s1;
+        part[warp][2] = s.s2;
     }
     __syncthreads();
-    auto in_range = [](double v) { return v > 1e-24 && v < 1e36; };
-    if (!in_range(sums[0]) || !in_range(sums[1])) {   // 32-bit squares may have over- or underflown
-        double dd = 0.0, yy = 0.0;
-        for (int i = threadIdx.x; i < H; i += 256) {
-            const double p = d[((size_t)k * C + c) * H + i], q = y[(size_t)c * H + i];
-            dd += p * p;
-            yy += q * q;
-        }
-        __syncthreads();   // every thread has read the sums
-        if (threadIdx.x < 2) sums[threadIdx.x] = 0.0;
-        __syncthreads();
-        atomicAdd(&sums[0], dd);
-        atomicAdd(&sums[1], yy);
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) s.join(part[w][0], part[w][1], part[w][2]);
+        const double v = s.value();
+        again = !(v > 1e-24 && v < 1e36);   // 32-bit squares may have over- or underflown
+        sq[blockIdx.x] = v;
     }
-    if (threadIdx.x == 0) atomicAdd(acc + k, sqrt(sums[0]) / (sqrt(sums[1]) + (double)eps));
+    __syncthreads();
+    if (!again) return;
+    double d = 0.0;
+    for (int i = threadIdx.x; i < H; i += 256) d += (double)row[i] * (double)row[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if (lane == 0) wide[warp] = d;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) d += wide[w];
+        sq[blockIdx.x] = d;
+    }
 }
+
+// err[k] += sum_c ||d_kc|| / (||y_c|| + eps), with d = y - y~_t (the dropped neurons' output) and y the dense one:
+// sq is [K + 1][C], the dense rows first.  Grid: K.
+__global__ void __launch_bounds__(256) err_ratio_kernel(const double *__restrict__ sq, int C, float eps,
+                                                        double *__restrict__ err)
+{
+    grid_dependency_wait();
+    grid_launch_dependents();
+    const double *d = sq + (size_t)(blockIdx.x + 1) * C;
+    double s = 0.0;
+    for (int c = threadIdx.x; c < C; c += 256) s += sqrt(d[c]) / (sqrt(sq[c]) + (double)eps);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    __shared__ double part[8];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) s += part[w];
+        err[blockIdx.x] += s;   // (the groups and their kernels follow one another)
+    }
+}
+
+// What the candidates of one block are formed from.
+struct ErrInputs {
+    float *a;                // [C][N]: SiLU(x W_gate)
+    uint16_t *hhi, *hlo;     // [C][ldn]: a u of every neuron
+    static size_t bytes(int N, int C) { return al256((size_t)C * ((N + 7) & ~7) * 8); }
+    ErrInputs(void *p, int N, int C)
+        : a(static_cast<float *>(p)),
+          hhi(reinterpret_cast<uint16_t *>(a + (size_t)C * ((N + 7) & ~7))), hlo(hhi + (size_t)C * ((N + 7) & ~7)) {}
+};
 
 // Workspace of Eq. 6.  Batches on the fused kernel (at most two tokens) compare whole outputs
 // (yd, yk, idx, cnt); batches on the tensor cores project the dropped neurons of a group of
-// candidates (a: ErrInputs, rows, y: the group's outputs).
+// candidates (a: ErrInputs, rows, y: the group's outputs, sq: their squared norms).
 struct ErrLayout {
-    size_t mlp, yd, yk, idx, cnt, a, rhi, rlo, y, acc, total;
+    size_t mlp, yd, yk, idx, cnt, a, rhi, rlo, y, sq, acc, total;
 };
 
-// Candidates per group: at most kErrGroup, and about kErrRows rows of h at most (but one candidate's).
+// Candidates per group: at most kErrGroup, and about kErrRows rows of h at most (but one candidate's), the dense
+// rows among them.
 int err_group(int C, int K)
 {
-    const int fit = kErrRows / C;
+    const int fit = kErrRows / C - 1;
     return std::max(1, std::min(std::min(fit, kErrGroup), K));
 }
 
@@ -266,11 +294,12 @@ ErrLayout err_layout(int H, int N, int C, int K)
     };
     L.mlp = take(ws_layout(H, N, C).total);
     if (use_tc_path(H, C)) {
-        const size_t ldn = ((size_t)N + 7) & ~(size_t)7, rows = (size_t)err_group(C, K) * C;
-        L.a = take((size_t)C * H * 4 + (size_t)C * ldn * 8);   // ErrInputs
+        const size_t ldn = ((size_t)N + 7) & ~(size_t)7, rows = (size_t)(err_group(C, K) + 1) * C;
+        L.a = take(ErrInputs::bytes(N, C));
         L.rhi = take(rows * ldn * 2);
         L.rlo = take(rows * ldn * 2);
         L.y = take(rows * H * sizeof(float));
+        L.sq = take(rows * sizeof(double));
         L.acc = take((size_t)std::max(K, 1) * (sizeof(double) + sizeof(unsigned long long)));   // ErrSums
     } else {
         L.yd = take((size_t)C * H * sizeof(float));
@@ -283,12 +312,16 @@ ErrLayout err_layout(int H, int N, int C, int K)
     return L;
 }
 
-// Eq. 6 on the tensor cores: h = a u of every neuron once, then y - y~_t = (h where |a| < t)
-// W_down directly, for all candidates of a group as the rows of one GEMM.  That is one pass over
-// W_gate and W_up and one over W_down per group instead of both per candidate (20 passes of 72 us
-// for 19 candidates of 64 inputs on the Llama-shaped layer), and the small difference is formed
-// without cancellation.  What bounds it: the down projection's MMAs (two per product: h's high and
-// low parts).
+// Eq. 6 on the tensor cores: a and h = a u of every neuron once, in fp32 accuracy, then y - y~_t = (h where |a| < t)
+// W_down directly, for all candidates of a group as the rows of one GEMM, and y itself as C more of its rows.
+// That is one pass over W_gate and W_up and one over W_down per group instead of both per candidate (20 passes of
+// 72 us for 19 candidates of 64 inputs on the Llama-shaped layer).  What its accuracy rests on: an accumulator that is
+// truncated after every K = 16 step comes out short, the shorter the longer its chain.  g and u short by 1e-5 change a
+// and h of small and of large |a| by different shares, so they are taken in fp32 accuracy; y and y - y~_t take the same
+// chains and keep little of it in their ratio.  Against 64 bits (2-norm over the candidates), with both / with h from
+// the batched gate/up kernel and y from a GEMM of its own: that layer 2.6e-7 / 1.6e-6, hidden 2048 / intermediate
+// 5633, 48 inputs 2.8e-7 / 2.4e-6.  What bounds it: the down projection's MMAs (two per product: h's high and low
+// parts).
 struct ErrSums {
     double *err;                     // [K]
     unsigned long long *dropped;     // [K]
@@ -296,21 +329,7 @@ struct ErrSums {
     ErrSums(void *p, int K) : err(static_cast<double *>(p)), dropped(reinterpret_cast<unsigned long long *>(err + K)) {}
 };
 
-// What the candidates of one block are formed from.
-struct ErrInputs {
-    float *y;                // [C][H]: the dense output
-    float *a;                // [C][lda]: SiLU(x W_gate)
-    uint16_t *hhi, *hlo;     // [C][ldn]: a u of every neuron
-    int lda;                 // ldn, or N where a is given (of fp32 accuracy) rather than the gate/up kernel's
-    bool a_given;
-    static size_t bytes(int H, int N, int C) { return al256((size_t)C * H * 4 + (size_t)C * ((N + 7) & ~7) * 8); }
-    ErrInputs(void *p, int H, int N, int C, bool a_given)
-        : y(static_cast<float *>(p)), a(y + (size_t)C * H),
-          hhi(reinterpret_cast<uint16_t *>(a + (size_t)C * ((N + 7) & ~7))), hlo(hhi + (size_t)C * ((N + 7) & ~7)),
-          lda(a_given ? N : (N + 7) & ~7), a_given(a_given) {}
-};
-
-// The rows of kg candidates (cand) and their product with W_down, into out [kg][C][H].
+// The dense rows and those of kg candidates (cand), and their product with W_down, into out [kg + 1][C][H].
 sats_status enqueue_rows(const sats_layer *layer, const ErrInputs &in, int C, const Candidates &cand, int kg,
                          unsigned long long *dropped, float *out, char *base, const ErrLayout &W, cudaStream_t st)
 {
@@ -318,25 +337,36 @@ sats_status enqueue_rows(const sats_layer *layer, const ErrInputs &in, int C, co
     int *ctl = reinterpret_cast<int *>(base + W.mlp + ws_layout(H, N, C).ctl);
     uint16_t *rhi = reinterpret_cast<uint16_t *>(base + W.rhi), *rlo = reinterpret_cast<uint16_t *>(base + W.rlo);
     const cudaError_t e = launch_after(drop_rows_kernel, dim3(C, (ld / 8 + 255) / 256), 256, st, (const float *)in.a,
-                                       (const uint16_t *)in.hhi, (const uint16_t *)in.hlo, C, N, ld, in.lda, cand, kg, rhi, rlo,
-                                       dropped, reinterpret_cast<float4 *>(out), (size_t)kg * C * H / 4);
+                                       (const uint16_t *)in.hhi, (const uint16_t *)in.hlo, C, N, ld, cand, kg, rhi, rlo,
+                                       dropped, reinterpret_cast<float4 *>(out), (size_t)(kg + 1) * C * H / 4);
     if (e != cudaSuccess) return cuda_fail(e, "dropped rows kernel launch");
-    return run_tc_down(layer, rhi, rlo, kg * C, out, ctl, st) == cudaSuccess ? SATS_OK : SATS_ECUDA;
+    return run_tc_down(layer, rhi, rlo, (kg + 1) * C, out, ctl, st) == cudaSuccess ? SATS_OK : SATS_ECUDA;
 }
 
-// h, a (unless given) and the dense output of one block's inputs x.  The dense output is projected on its own: a stack's next
-// block starts from it, and up to 256 inputs take the batched-decode kernel, whose shorter accumulator chains
-// are the more accurate ones.
-sats_status enqueue_err_inputs(const sats_layer *layer, const float *x, int C, const ErrInputs &in, char *base,
-                               const ErrLayout &W, cudaStream_t st)
+__global__ void __launch_bounds__(256) add_rows_kernel(float4 *__restrict__ x, const float4 *__restrict__ y, size_t n4)
 {
-    const WsLayout M = ws_layout(layer->H, layer->N, C);
-    char *mlp = base + W.mlp;
-    int *ctl = reinterpret_cast<int *>(mlp + M.ctl);
-    if (run_tc_gate_up(layer, x, C, mlp + M.tc, in.hhi, in.hlo, in.a_given ? nullptr : in.a, ctl, st) != cudaSuccess) return SATS_ECUDA;
-    const cudaError_t e = cudaMemsetAsync(in.y, 0, (size_t)C * layer->H * sizeof(float), st);
-    if (e != cudaSuccess) return cuda_fail(e, "layer error output clear");
-    return run_tc_down(layer, in.hhi, in.hlo, C, in.y, ctl, st) == cudaSuccess ? SATS_OK : SATS_ECUDA;
+    grid_dependency_wait();
+    grid_launch_dependents();
+    const size_t i = blockIdx.x * (size_t)256 + threadIdx.x;
+    if (i >= n4) return;
+    const float4 a = x[i], b = y[i];
+    x[i] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+
+// x += the dense output, projected on its own: up to 256 inputs take the batched-decode kernel, whose shorter
+// accumulator chains are the more accurate ones.
+sats_status enqueue_residual(const sats_layer *layer, float *x, int C, const ErrInputs &in, char *base,
+                             const ErrLayout &W, cudaStream_t st)
+{
+    const size_t n = (size_t)C * layer->H;
+    float *y = reinterpret_cast<float *>(base + W.y);
+    int *ctl = reinterpret_cast<int *>(base + W.mlp + ws_layout(layer->H, layer->N, C).ctl);
+    cudaError_t e = cudaMemsetAsync(y, 0, n * sizeof(float), st);
+    if (e != cudaSuccess) return cuda_fail(e, "dense output clear");
+    if (run_tc_down(layer, in.hhi, in.hlo, C, y, ctl, st) != cudaSuccess) return SATS_ECUDA;
+    e = launch_after(add_rows_kernel, dim3((unsigned)((n / 4 + 255) / 256)), 256, st, reinterpret_cast<float4 *>(x),
+                     reinterpret_cast<const float4 *>(y), n / 4);
+    return e == cudaSuccess ? SATS_OK : cuda_fail(e, "residual kernel launch");
 }
 
 // Enqueues the sums for K candidates: thresholds t (host), or q[at(k)] on the device where q is given.
@@ -357,8 +387,10 @@ sats_status enqueue_err(const sats_layer *layer, const ErrInputs &in, int C, con
         }
         const sats_status s = enqueue_rows(layer, in, C, cand, kg, sums.dropped + k0, out, base, W, st);
         if (s != SATS_OK) return s;
-        const cudaError_t e = launch_after(drop_err_kernel, dim3(C, kg), 256, st, (const float *)in.y, (const float *)out,
-                                           C, layer->H, eps, sums.err + k0);
+        double *sq = reinterpret_cast<double *>(base + W.sq);
+        cudaError_t e = launch_after(row_squares_kernel, dim3((kg + 1) * C), 256, st, (const float *)out, layer->H, sq);
+        if (e == cudaSuccess)
+            e = launch_after(err_ratio_kernel, dim3(kg), 256, st, (const double *)sq, C, eps, sums.err + k0);
         if (e != cudaSuccess) return cuda_fail(e, "error reduction kernel launch");
     }
     return SATS_OK;
@@ -386,10 +418,11 @@ sats_status layer_err_tc(const sats_layer *layer, const float *x, int C, const f
     cudaError_t e = clear_fused_state(mlp, layer->H, layer->N, C, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(base + W.acc, 0, sum_bytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "layer error workspace clear");
-    const ErrInputs in(base + W.a, layer->H, layer->N, C, false);
-    sats_status s = enqueue_err_inputs(layer, x, C, in, base, W, st);
-    if (s == SATS_OK)
-        s = enqueue_err(layer, in, C, t, nullptr, [](int k) { return k; }, K, eps, ErrSums(base + W.acc, K), base, W, st);
+    const ErrInputs in(base + W.a, layer->N, C);
+    e = launch_gate_act_f32(layer, x, C, in.a, st);
+    if (e == cudaSuccess) e = launch_up_f32(layer, x, C, in.a, in.hhi, in.hlo, st);
+    if (e != cudaSuccess) return cuda_fail(e, "gate and up kernels launch");
+    sats_status s = enqueue_err(layer, in, C, t, nullptr, [](int k) { return k; }, K, eps, ErrSums(base + W.acc, K), base, W, st);
     if (s != SATS_OK) return s;
     std::vector<char> h(sum_bytes);
     e = cudaMemcpyAsync(h.data(), base + W.acc, sum_bytes, cudaMemcpyDeviceToHost, st);
@@ -399,16 +432,6 @@ sats_status layer_err_tc(const sats_layer *layer, const float *x, int C, const f
     if (s != SATS_OK) return s;
     err_means(h.data(), K, C, layer->N, err, sp);
     return SATS_OK;
-}
-
-__global__ void __launch_bounds__(256) add_rows_kernel(float4 *__restrict__ x, const float4 *__restrict__ y, size_t n4)
-{
-    grid_dependency_wait();
-    grid_launch_dependents();
-    const size_t i = blockIdx.x * (size_t)256 + threadIdx.x;
-    if (i >= n4) return;
-    const float4 a = x[i], b = y[i];
-    x[i] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
 
 struct SatsLayout {
@@ -432,7 +455,7 @@ SatsLayout sats_layout(int H, int N, int C, int L, int K0, int K)
     S.sums = off;   // every block's ErrSums
     off += al256((size_t)L * ErrSums::bytes(K));
     // every block's ErrInputs, kept from the coarse candidates for the fine ones, up to kErrKeep bytes
-    const size_t each = use_tc_path(H, C) ? ErrInputs::bytes(H, N, C) : 0;
+    const size_t each = use_tc_path(H, C) ? ErrInputs::bytes(N, C) : 0;
     S.in = off;
     S.in_each = each * L <= kErrKeep ? each : 0;
     off += S.in_each * L;
@@ -618,16 +641,18 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     char *sums = base + W.sums;
     const size_t sum_bytes = ErrSums::bytes(Kmax);
     const bool batched = use_tc_path(H, C);
-    // The masks take the accurate gate activations that the thresholds are percentiles of: a neuron at a threshold
-    // falls on its own side (with the gate/up kernel's, 1.2e-5 off, the shares at the chosen thresholds were off by a
-    // few neurons).
+    // (the masks take the gate activations that the thresholds are percentiles of)
     auto inputs_of = [&](int l) {
-        return ErrInputs(W.in_each ? base + W.in + l * W.in_each : ews + E.a, H, N, C, true);
+        return ErrInputs(W.in_each ? base + W.in + l * W.in_each : ews + E.a, N, C);
+    };
+    auto n_of = [&](int l) { return nall + (size_t)l * C * H; };
+    auto up_of = [&](int l) {
+        const ErrInputs in = inputs_of(l);
+        return launch_up_f32(layers[l], n_of(l), C, in.a, in.hhi, in.hlo, st);
     };
     auto gate_of = [&](int l) { return batched ? inputs_of(l).a : reinterpret_cast<float *>(base + W.a); };
     const size_t ews_bytes = W.total - W.err;
     void *mlp = ews + E.mlp;
-    auto n_of = [&](int l) { return nall + (size_t)l * C * H; };
     const int guard = guardrail ? L - 1 : -1;
 
     // 1-2: the dense stack gives each block's MLP inputs; coarse candidates from |SiLU(n W_gate)|
@@ -656,16 +681,13 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
                 return cuda_fail(e, "percentile kernels launch");
         if (batched) {
             // 3: Eq. 6 for every coarse candidate (and, with them, the guardrail's CATS threshold), the
-            // thresholds read on the device; x <- x + MLP_l(n_l) takes the dense output from it
+            // thresholds read on the device; then x <- x + MLP_l(n_l)
             const int K = l == guard ? Kc + 1 : Kc;
-            if ((s = enqueue_err_inputs(layers[l], n_of(l), C, inputs_of(l), ews, E, st)) != SATS_OK) return s;
+            if ((e = up_of(l)) != cudaSuccess) return cuda_fail(e, "up kernel launch");
             if ((s = enqueue_err(layers[l], inputs_of(l), C, nullptr, ql, [&](int k) { return k < Kc ? k : Kc + 1; }, K,
                                  err_eps, ErrSums(sums + l * sum_bytes, K), ews, E, st)) != SATS_OK)
                 return s;
-            const size_t n4 = (size_t)C * H / 4;
-            e = launch_after(add_rows_kernel, dim3((unsigned)((n4 + 255) / 256)), 256, st, reinterpret_cast<float4 *>(x),
-                             reinterpret_cast<const float4 *>(inputs_of(l).y), n4);
-            if (e != cudaSuccess) return cuda_fail(e, "residual kernel launch");
+            if ((s = enqueue_residual(layers[l], x, C, inputs_of(l), ews, E, st)) != SATS_OK) return s;
             continue;
         }
         // x <- x + MLP_l(n_l) with every neuron kept
@@ -742,7 +764,7 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
         if (K1 == 0) continue;
         if (batched && W.in_each == 0) {
             if ((s = sats_gate_act_f32(layers[l], n_of(l), C, gate_of(l), stream)) != SATS_OK) return s;
-            if ((s = enqueue_err_inputs(layers[l], n_of(l), C, inputs_of(l), ews, E, st)) != SATS_OK) return s;
+            if ((e = up_of(l)) != cudaSuccess) return cuda_fail(e, "up kernel launch");
         }
         s = batched ? enqueue_err(layers[l], inputs_of(l), C, tf.data() + (size_t)l * K1, nullptr, [](int k) { return k; },
                                   K1, err_eps, ErrSums(sums + l * sum_bytes, K1), ews, E, st)

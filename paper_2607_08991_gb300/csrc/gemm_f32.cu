@@ -1,6 +1,6 @@
 // gemm_f32.cu -- products on the tensor cores of sm_103a whose results are as
 // accurate as fp32 FMAs, for the paths that promise fp32 arithmetic: the post-gate
-// activations of the calibrations (Sec. 2, Eqs. 1-3; Sec. 3.1).
+// activations of the calibrations (Sec. 2, Eqs. 1-3; Sec. 3.1), and a u of Eq. 6.
 //
 // Two things keep tcgen05.mma (bf16 operands, fp32 accumulator) from that accuracy:
 //  - its operands.  The weights are bf16 as they are; an fp32 activation is cut into
@@ -42,7 +42,9 @@ struct PreciseGateParams {
     const float *x;        // fp32 activations [B][H] (the converter warps read them; bf16 ones come by TMA)
     int B, H, N, R, KBh;
     int NT;                // tokens per tile, a multiple of 16
-    float *a;              // [B][N]
+    float *a;              // [B][N]: written, or read for h (UP)
+    uint16_t *hhi, *hlo;   // UP: [B][ldh] bf16
+    int ldh;
     int stages, stage_bytes, w_bytes, ring_bytes;
     uint32_t tmem_cols;    // four accumulators of NT columns
 };
@@ -160,7 +162,8 @@ __device__ __forceinline__ bool cut_tiles(uint8_t *parts, int NT, int steps, uin
 // M, tokens its N).  Grid: token tiles x neuron tiles, the token tiles of one neuron tile
 // next to each other, so that its weights come from L2 for all but the first of them.
 // TOK: the most tokens of a tile (64 leaves registers for a second level of sums with fp32 activations).
-template <bool F32, int TOK>
+// UP: u = x W_up instead, and from it and the a of an earlier launch h = a u in two bf16 parts.
+template <bool F32, int TOK, bool UP>
 __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     gate_precise_kernel(const __grid_constant__ CUtensorMap tmX, const PreciseGateParams p)
 {
@@ -219,7 +222,7 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
         // (each weight tile is read once with one token tile, else by its neighbours through L2)
         const uint64_t once = l2_policy_evict_first();
         auto load_w = [&](int s, int kb) {
-            const uint16_t *src = p.w + (size_t)((size_t)t * KBh + kb) * 2 * R * BK;
+            const uint16_t *src = p.w + ((size_t)((size_t)t * KBh + kb) * 2 + (UP ? 1 : 0)) * R * BK;
             if (gridDim.x == 1) bulk_load_if(lead, ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s], once);
             else bulk_load_shared_if(lead, ring + (size_t)s * p.stage_bytes, src, (uint32_t)p.w_bytes, &full[s]);
         };
@@ -342,10 +345,17 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                 }
             }
         }
-        grid_dependency_wait();   // a may still be in use by the preceding kernel
+        grid_dependency_wait();   // a (h) may still be in use by the preceding kernel
         if (32 * quad + lane < R && n < p.N) {
 #pragma unroll
-            for (int k = 0; k < kBlocks; ++k)
+            for (int k = 0; k < kBlocks; ++k) {
+                float av[UP ? 16 : 1];
+                if (UP)
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const int j = 16 * (grp + G * k) + e;
+                        av[UP ? e : 0] = j < NT && m0 + j < p.B ? p.a[(size_t)(m0 + j) * p.N + n] : 0.f;
+                    }
 #pragma unroll
                 for (int e = 0; e < 16; ++e) {
                     const int j = 16 * (grp + G * k) + e;
@@ -353,9 +363,17 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                         // (a wait that gave up leaves NaN: this call has no status word)
                         const float2 two = unpack2(acc[8 * k + e / 2]);
                         const float g = ok ? (e & 1 ? two.y : two.x) : __int_as_float(0x7fffffff);
-                        p.a[(size_t)(m0 + j) * p.N + n] = g / (1.0f + expf(-g));   // SiLU, Eq. 2
+                        if (!UP) {
+                            p.a[(size_t)(m0 + j) * p.N + n] = g / (1.0f + expf(-g));   // SiLU, Eq. 2
+                        } else {
+                            const float h = av[UP ? e : 0] * g;
+                            const uint16_t hb = bf16_bits(h);
+                            p.hhi[(size_t)(m0 + j) * p.ldh + n] = hb;
+                            p.hlo[(size_t)(m0 + j) * p.ldh + n] = bf16_bits(h - __uint_as_float((uint32_t)hb << 16));
+                        }
                     }
                 }
+            }
         }
     }
     __syncthreads();
@@ -373,8 +391,9 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     }
 }
 
-template <bool F32, int TOK>
-cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, float *a, cudaStream_t stream)
+template <bool F32, int TOK, bool UP = false>
+cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, float *a, cudaStream_t stream,
+                                uint16_t *hhi = nullptr, uint16_t *hlo = nullptr)
 {
     PreciseGateParams p{};
     p.w = layer->gu_blk;
@@ -387,6 +406,9 @@ cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, f
     const int mt = (B + kPreciseTok - 1) / kPreciseTok;
     p.NT = ((B + mt - 1) / mt + 15) & ~15;   // the tokens evenly over the fewest tiles
     p.a = a;
+    p.hhi = hhi;
+    p.hlo = hlo;
+    p.ldh = layer->ldn;
     p.tmem_cols = tmem_cols_for(4 * p.NT);
     p.w_bytes = p.R * kTileBytes;
     p.stage_bytes = p.w_bytes + (F32 ? 0 : p.NT * kTileBytes);
@@ -401,9 +423,9 @@ cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, f
         return cudaErrorInvalidValue;
     static std::atomic<int> cfg[64];
     const size_t smem = smem_for(1, p.ring_bytes + parts);
-    const cudaError_t e = set_smem(gate_precise_kernel<F32, TOK>, smem, cfg);
+    const cudaError_t e = set_smem(gate_precise_kernel<F32, TOK, UP>, smem, cfg);
     if (e != cudaSuccess) return e;
-    return launch_pdl_cfg(gate_precise_kernel<F32, TOK>, dim3(mt, layer->tc_T), kPreciseThreads<F32>, smem, stream, mX, p);
+    return launch_pdl_cfg(gate_precise_kernel<F32, TOK, UP>, dim3(mt, layer->tc_T), kPreciseThreads<F32>, smem, stream, mX, p);
 }
 
 // ---------------------------------------------------------------------- LoRA batches
@@ -1005,6 +1027,14 @@ cudaError_t launch_gate_act_f32(const sats_layer *layer, const float *x, int B, 
 {
     return B <= 64 ? tc::launch_gate_precise<true, 64>(layer, x, B, a, stream)
                    : tc::launch_gate_precise<true, tc::kPreciseTok>(layer, x, B, a, stream);
+}
+
+cudaError_t launch_up_f32(const sats_layer *layer, const float *x, int B, const float *a, uint16_t *hhi, uint16_t *hlo,
+                          cudaStream_t stream)
+{
+    float *const in = const_cast<float *>(a);   // (read only)
+    return B <= 64 ? tc::launch_gate_precise<true, 64, true>(layer, x, B, in, stream, hhi, hlo)
+                   : tc::launch_gate_precise<true, tc::kPreciseTok, true>(layer, x, B, in, stream, hhi, hlo);
 }
 
 // Scratch of a LoRA batch inside the tensor-core region of a workspace: z and w where the other

@@ -183,7 +183,6 @@ struct SkinnyGuParams {
     uint8_t *keep;                // [M][keep_stride] or nullptr
     int keep_stride;
     uint8_t *keep_trace;          // [M][N] or nullptr
-    float *a_out;                 // ACT: [M][ldh] fp32: SiLU(g) of every neuron (the calibration's masks)
     int *ctl;
     float *zero;                  // y [M][H] to clear for the down projection's additions, or nullptr
     int zero_count;               // M H (a multiple of 8)
@@ -200,9 +199,7 @@ struct SkinnyGuParams {
 // lane r, column j (gate) and NT + j (up).  Grid: tc_T CTAs.  In gate-only mode
 // only the gate rows are read and multiplied.  The epilogue runs once all MMAs
 // are done, on G groups of four warps (blockDim 64 + 128 G): group g takes the
-// 16-token column blocks g, g + G, ... of every row (G = 1 in gate-only mode).  ACT: SiLU(g) is written too
-// (a template flag: tested per element in the epilogue it cost 1-2.5 % of calls of 100-250 tokens).
-template <bool ACT>
+// 16-token column blocks g, g + G, ... of every row (G = 1 in gate-only mode).
 __global__ void __launch_bounds__(kSkinnyMaxThreads, 1)
     gu_skinny_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmX2,
                      const SkinnyGuParams p)
@@ -362,7 +359,6 @@ __global__ void __launch_bounds__(kSkinnyMaxThreads, 1)
                     p.hact_lo[(size_t)j * p.ldh + n] = bf16_bits(h - __uint_as_float((uint32_t)hb << 16));
                     if (p.keep) p.keep[(size_t)j * p.keep_stride + n] = keep ? 1 : 0;
                     if (p.keep_trace) p.keep_trace[(size_t)(p.perm ? p.perm[j] : j) * p.N + n] = keep ? 1 : 0;
-                    if (ACT) p.a_out[(size_t)j * p.ldh + n] = a;
                 }
             }
         }
@@ -1198,7 +1194,6 @@ struct GateUpArgs {
     uint16_t *hact, *hact_lo;
     uint8_t *keep;               // [B][keep_stride] or nullptr
     uint8_t *keep_trace;
-    float *a_out;                // [B][ldn] (skinny kernel only) or nullptr
     float *zero;                 // y [B][H] to clear, or nullptr
     int *ctl;
 };
@@ -1244,7 +1239,6 @@ cudaError_t launch_gate_up_skinny(const sats_layer *layer, const GateUpArgs &a, 
     gp.keep = a.keep;
     gp.keep_stride = keep_stride_of(N);
     gp.keep_trace = a.keep_trace;
-    gp.a_out = a.a_out;
     gp.ctl = a.ctl;
     gp.zero = a.zero;
     gp.zero_count = B * H;
@@ -1260,17 +1254,15 @@ cudaError_t launch_gate_up_skinny(const sats_layer *layer, const GateUpArgs &a, 
     gp.ring_bytes = gp.stages * gp.stage_bytes + slack;
     gp.merge = split && NT <= 128 ? 1 : 0;
     gp.tmem_cols = tmem_cols_for((gp.merge ? 4 : 2) * NT);
-    static std::atomic<int> cfg_act[64];
-    cudaError_t e = a.a_out ? set_smem(gu_skinny_kernel<true>, smem_for(1, gp.ring_bytes), cfg_act)
-                            : set_smem(gu_skinny_kernel<false>, smem_for(1, gp.ring_bytes), cfg_gu_skinny);
+    cudaError_t e = set_smem(gu_skinny_kernel, smem_for(1, gp.ring_bytes), cfg_gu_skinny);
     if (e != cudaSuccess) return fail(e, "shared-memory attribute");
     // epilogue groups: one per 16-token column block, at most kSkinnyMaxGroups where the last of them saves
     // a turn, else one less (the epilogue runs after the last MMA, so its time adds to the call's)
     const int blocks16 = NT / 16, G = kSkinnyMaxGroups;
     const int most = (blocks16 + G - 1) / G < (blocks16 + G - 2) / (G - 1) ? G : G - 1;
     const int groups = blocks16 < most ? blocks16 : most;
-    e = launch_pdl_cfg(a.a_out ? gu_skinny_kernel<true> : gu_skinny_kernel<false>, dim3(layer->tc_T), 64 + 128 * groups,
-                       smem_for(1, gp.ring_bytes), stream, mX, mX2, gp);
+    e = launch_pdl_cfg(gu_skinny_kernel, dim3(layer->tc_T), 64 + 128 * groups, smem_for(1, gp.ring_bytes), stream, mX, mX2,
+                       gp);
     return e == cudaSuccess ? e : fail(e, "gate/up kernel launch");
 }
 
@@ -1432,38 +1424,6 @@ bool gate_up_wide(const sats_layer *layer, int B, bool split)
 }
 }  // namespace
 
-// Gate and up projections of B fp32 inputs with every neuron kept: h in bf16 parts and, where
-// wanted, a = SiLU(x W_gate) (all with row stride layer->ldn), for the calibration's masks.  tc_ws: the tensor-core
-// region of a workspace for B tokens.  In passes of up to kGateUpTokens tokens
-// of the skinny kernel, whose epilogue has a thread per neuron and writes a in whole lines.
-constexpr int kGateUpTokens = 128;
-
-cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void *tc_ws, uint16_t *hhi, uint16_t *hlo,
-                           float *a_out, int *ctl, cudaStream_t stream)
-{
-    const int H = layer->H;
-    const size_t ldn = layer->ldn;
-    const TcLayout W = tc_layout(H, layer->N, B);
-    uint8_t *base = static_cast<uint8_t *>(tc_ws);
-    uint16_t *xhi = reinterpret_cast<uint16_t *>(base + W.xhi), *xlo = reinterpret_cast<uint16_t *>(base + W.xlo);
-    cudaError_t e = launch_pdl_threads(split_kernel, dim3(B), 256, stream, x, H, static_cast<const float *>(nullptr), 0.f,
-                                       xhi, xlo, static_cast<const int32_t *>(nullptr));
-    if (e != cudaSuccess) return fail(e, "split kernel launch");
-    const int passes = (B + kGateUpTokens - 1) / kGateUpTokens, per = (B + passes - 1) / passes;
-    for (int m0 = 0; m0 < B; m0 += per) {
-        GateUpArgs a{};
-        a.xhi = xhi + (size_t)m0 * H;
-        a.xlo = xlo + (size_t)m0 * H;
-        a.B = B - m0 < per ? B - m0 : per;
-        a.hact = hhi + m0 * ldn;
-        a.hact_lo = hlo + m0 * ldn;
-        a.a_out = a_out ? a_out + m0 * ldn : nullptr;
-        a.ctl = ctl;
-        if ((e = launch_gate_up_skinny(layer, a, stream)) != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
 // out[m] += (hact + hact_lo)[m] W_down for M rows of h (row stride layer->ldn).
 cudaError_t run_tc_down(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
                         int *ctl, cudaStream_t stream)
@@ -1547,9 +1507,9 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
         gp.ring_bytes = gp.stages * gp.stage_bytes + slack;
         gp.merge = split && NT <= 128 ? 1 : 0;
         gp.tmem_cols = tmem_cols_for(gp.merge ? 2 * NT : NT);
-        if ((e = set_smem(gu_skinny_kernel<false>, smem_for(1, gp.ring_bytes), cfg_gu_skinny)) != cudaSuccess)
+        if ((e = set_smem(gu_skinny_kernel, smem_for(1, gp.ring_bytes), cfg_gu_skinny)) != cudaSuccess)
             return fail(e, "shared-memory attribute");
-        e = launch_pdl_cfg(gu_skinny_kernel<false>, dim3(layer->tc_T), 64 + 128, smem_for(1, gp.ring_bytes), stream, mX, mX2,
+        e = launch_pdl_cfg(gu_skinny_kernel, dim3(layer->tc_T), 64 + 128, smem_for(1, gp.ring_bytes), stream, mX, mX2,
                            gp);
         if (e != cudaSuccess) return fail(e, "gate kernel launch");
         e = launch_union_tail(layer, B, xa, split ? xlo : nullptr, uflag, ulist, ucount, a_keep, ldn, u, ldn, out, ctl,

@@ -135,11 +135,7 @@ cudaError_t run_tc_layer(const sats_layer *layer, int x_mode, const void *x, int
                          float eps, const uint8_t *dense_flags, const int32_t *perm, const int32_t *n_dense,
                          int out_mode, float *out, int32_t *active_idx, int32_t *active_cnt, uint8_t *keep_trace,
                          void *tc_ws, int *ctl, cudaStream_t stream, bool union_path = false);
-// The calibration's halves of it: gate and up of B fp32 inputs with every neuron kept (h in bf16
-// parts and, unless a_out is null, a = SiLU(x W_gate), all with row stride ldn), and the down projection of any M rows of
-// h, added into out.
-cudaError_t run_tc_gate_up(const sats_layer *layer, const float *x, int B, void *tc_ws, uint16_t *hhi, uint16_t *hlo,
-                           float *a_out, int *ctl, cudaStream_t stream);
+// The down projection of any M rows of h (two bf16 parts with row stride ldn), added into out.
 cudaError_t run_tc_down(const sats_layer *layer, const uint16_t *hact, const uint16_t *hact_lo, int M, float *out,
                         int *ctl, cudaStream_t stream);
 // Byte offsets of the tensor-core region's parts that other paths reuse: the bf16 copies of x
@@ -158,6 +154,9 @@ cudaError_t launch_route(const int32_t *ids, int B, const uint8_t *lut, int V, i
 cudaError_t launch_gate_act(const sats_layer *layer, const uint16_t *x, int B, float *a,
                             cudaStream_t stream);
 cudaError_t launch_gate_act_f32(const sats_layer *layer, const float *x, int B, float *a, cudaStream_t stream);
+// h = a u of every neuron, u = x W_up in the same accuracy, in two bf16 parts with row stride ldn.
+cudaError_t launch_up_f32(const sats_layer *layer, const float *x, int B, const float *a, uint16_t *hhi, uint16_t *hlo,
+                          cudaStream_t stream);
 
 // One block over B tokens (fused kernel or tensor cores), as the C ABI calls run it
 // (api.cu).  ws: a workspace of ws_layout(H, N, B).total bytes with zeroed control words.
