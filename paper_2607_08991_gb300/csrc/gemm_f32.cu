@@ -11,17 +11,25 @@
 //    sum came out 1.2e-5 short (256 steps of half a unit of the 24th bit).  Here an
 //    accumulator takes K = 32 only (the small parts first); every K block of 64 fills
 //    two of them, and the epilogue warps read both from TMEM while the next block's MMAs
-//    run, add the two and add the sum to totals that they keep in registers (rounded to
-//    nearest).  Measured against fp64 on the Llama-shaped layer, 256 tokens: 1.1e-7 relative
-//    with bf16 and 1.9e-7 with fp32 activations (the fp32 FMA chains that this replaced:
-//    1.1e-7 and 2.2e-7).
+//    run, add the two, and add the sums (rounded to nearest) in two levels or, up to hidden
+//    2048 with bf16 activations, to totals whose roundings are summed beside them.
+//
+// The error of a = SiLU(x W_gate) against fp64 (2-norm, units of 1e-8), before the tensor cores (fp32 FMA
+// chains) / with sums in two levels of 8 blocks, fp32 tiles of more than 64 tokens in one, and a plain SiLU / now:
+//   hidden                 256              512               1024              2048               4096               8192
+//   bf16              7.1 /      6.7   7.7 /  9.0 / 6.8   8.5 /  9.5 /  6.8   9.5 / 10.1 /  6.7  10.9 / 11.0 / 10.5  13.5 / 12.2 / 11.8
+//   fp32,  64 tokens  9.3 /      8.9  10.7 / 10.4 / 9.5  13.1 / 10.9 / 10.2  16.9 / 11.4 / 11.1  22.5 / 12.1 / 11.7  30.7 / 13.3 / 12.9
+//   fp32, 256 tokens  9.3 /      8.9  10.7 / 10.4 / 9.5  13.1 / 12.2 / 10.2  16.9 / 14.9 / 11.1  22.5 / 18.8 / 11.7  30.7 / 24.3 / 12.8
+// The worst of the elements, in units of the result's rms, 1e-6: 4096 bf16 1.4 / 1.8 / 1.6, fp32 2.2 / 3.7 / 1.7;
+// 8192 bf16 1.3 / 1.7 / 1.7, fp32 2.8 / 4.0 / 1.8.  An Eq. 3 threshold of the Llama-shaped layer, 256 bf16
+// tokens: 1.1e-7 / 9.5e-8 / 9.3e-8 of its value on average over 27 quantiles, 5.7e-7 / 5.0e-7 / 4.3e-7 at worst.
 //
 // What bounds it: neither the weight stream (17 us on that layer) nor the MMAs, but what the
 // roles issue per K block: waits and commits of about 100 cycles each, the TMEM reads and
 // additions of two accumulators (two at a time, f32x2; fp32: the next columns' read in
 // flight), and with fp32 activations the converters (no test for infinities but one vote at
-// the end of a step).  Llama-shaped layer, us before and after these: bf16 16 / 128 / 256
-// tokens 25.0 / 34.0 / 65.2 -> 24.7 / 32.6 / 63.8, fp32 46.0 / 98.0 / 200 -> 39.5 / 75.8 / 152.
+// the end of a step).  Llama-shaped layer, us: bf16 16 / 128 / 256 tokens 24.6 / 34.1 / 67.1, fp32 40.1 / 84.0 / 170.
+// Without the accuracy that the last column above has over the middle one: 24.6 / 32.7 / 63.9 and 39.2 / 75.5 / 153.
 #include "tc_common.cuh"
 
 namespace sats {
@@ -33,9 +41,13 @@ constexpr int kConvThreads = 192;    // converter warps (fp32 activations)
 // copy and MMA warps, converters, epilogue groups (fp32: two of 64 totals a thread within the
 // 128 registers that 16 warps leave; bf16: four of 32)
 template <bool F32> constexpr int kPreciseThreads = F32 ? 64 + kConvThreads + 256 : 64 + 512;
+// Largest hidden size at which bf16 totals keep their roundings: above it sums in two levels are as near to 64 bits as
+// FMA chains were (the table above), and keeping them everywhere costs 36 % (Llama-shaped layer, 256 tokens 67.1 -> 87.3 us;
+// here hidden 1024 / intermediate 4096 24.8 -> 32.1).
+constexpr int kKeepH = 2048;
 constexpr int kPartStages = 2;       // cut tiles in shared memory
 constexpr int kParts = 3;
-constexpr int kSubBlocks = 8;        // K blocks summed before they join the totals
+constexpr int kBarrierBytes = 256;   // the barriers and the TMEM slot, after the operand tiles
 
 struct PreciseGateParams {
     const uint16_t *w;     // gu_blk
@@ -45,6 +57,7 @@ struct PreciseGateParams {
     float *a;              // [B][N]: written, or read for h (UP)
     uint16_t *hhi, *hlo;   // UP: [B][ldh] bf16
     int ldh;
+    int sub;               // K blocks summed before they join the totals
     int stages, stage_bytes, w_bytes, ring_bytes;
     uint32_t tmem_cols;    // four accumulators of NT columns
 };
@@ -54,6 +67,16 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
     f32x2 d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
+}
+
+// SiLU(g) = g / (1 + e^-g), Eq. 2, with the quotient's remainder and what 1 + e^-g was rounded by brought back in.
+__device__ __forceinline__ float silu_rounded(float g)
+{
+    const float e = expf(-g), d = 1.0f + e, b = __fadd_rn(d, -1.0f);
+    const float rest = __fadd_rn(1.0f, -__fadd_rn(d, -b)) + __fadd_rn(e, -b);   // d + rest = 1 + e
+    const float q = g / d;
+    const float c = __fdividef(fmaf(-q, rest, fmaf(-q, d, g)), d);
+    return fabsf(c) < INFINITY ? q + c : q;   // (not a number where e or g is infinite)
 }
 
 __device__ __forceinline__ float bf16_top(float x) { return __uint_as_float(__float_as_uint(x) & 0xffff0000u); }
@@ -163,7 +186,8 @@ __device__ __forceinline__ bool cut_tiles(uint8_t *parts, int NT, int steps, uin
 // next to each other, so that its weights come from L2 for all but the first of them.
 // TOK: the most tokens of a tile (64 leaves registers for a second level of sums with fp32 activations).
 // UP: u = x W_up instead, and from it and the a of an earlier launch h = a u in two bf16 parts.
-template <bool F32, int TOK, bool UP>
+// KEEP: what a total is rounded by is summed beside it and added at the end (bf16 activations).
+template <bool F32, int TOK, bool UP, bool KEEP>
 __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     gate_precise_kernel(const __grid_constant__ CUtensorMap tmX, const PreciseGateParams p)
 {
@@ -296,22 +320,30 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
         const int quad = warp & 3, grp = (warp - kEpi0) >> 2;
         const uint32_t lane0 = tmem + ((uint32_t)(32 * quad) << 16);
         const int n = t * R + 32 * quad + lane;
-        // acc: totals; sub: the sums of up to kSubBlocks K blocks, added to the totals together, so that
-        // a total takes few roundings at its full size (where the registers hold both)
-        constexpr bool kTwoLevel = kBlocks <= 2;
+        // sum: the sums of up to p.sub K blocks, which join the totals together, so that a total takes few roundings at
+        // its full size; with KEEP every K block joins, and sum holds what the totals were rounded by.  64 totals a
+        // thread (fp32 activations, tiles of more than 64 tokens) are kept in shared memory.
+        constexpr bool kShared = kBlocks > 2;
         constexpr int kPairs = 8 * kBlocks;
-        f32x2 acc[kPairs], sub[kTwoLevel ? kPairs : 1];
+        static_assert(!KEEP || !(kShared || UP), "kept roundings need the totals in registers");
+        f32x2 sum[kPairs], tot[kShared ? 1 : kPairs];
+        f32x2 *const shared_tot = reinterpret_cast<f32x2 *>(reinterpret_cast<uint8_t *>(full) + kBarrierBytes) +
+                                  (threadIdx.x - 32 * kEpi0);   // [kPairs] of this thread, 128 G apart
+        const bool busy = quad < n_quads;   // (uniform in the warp, as is the next)
+        auto in_tile = [&](int pair) { return 16 * (grp + G * (pair >> 3)) < NT; };
 #pragma unroll
         for (int k = 0; k < kPairs; ++k) {
-            acc[k] = pack2(0.f, 0.f);
-            if (kTwoLevel) sub[kTwoLevel ? k : 0] = pack2(0.f, 0.f);
+            sum[k] = pack2(0.f, 0.f);
+            if (!kShared) tot[kShared ? 0 : k] = sum[k];
+            else if (in_tile(k)) shared_tot[k * 128 * G] = sum[k];
         }
+        int since = 0;
         bool ok = true;
         for (int kb = 0; kb < KBh; ++kb) {
             const int buf = kb & 1;
             if (!mbar_wait(&acc_full[buf], (uint32_t)((kb >> 1) & 1), &abort_flag)) { ok = false; break; }
             tc_fence_after();
-            if (quad < n_quads) {
+            if (busy) {
                 const uint32_t a0 = lane0 + (uint32_t)(2 * buf * NT);
                 constexpr int kV = F32 ? 2 : 1;
                 float v[kV][2][8];
@@ -331,17 +363,26 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                     for (int e = 0; e < 4; ++e) {
                         const f32x2 w = add2(pack2(v[o % kV][0][2 * e], v[o % kV][0][2 * e + 1]),
                                              pack2(v[o % kV][1][2 * e], v[o % kV][1][2 * e + 1]));
-                        f32x2 &to = kTwoLevel ? sub[kTwoLevel ? 4 * o + e : 0] : acc[4 * o + e];
-                        to = add2(to, w);
+                        f32x2 &s = sum[4 * o + e], &t0 = tot[kShared ? 0 : 4 * o + e];
+                        if (KEEP) {
+                            const f32x2 minus1 = pack2(-1.f, -1.f), t1 = add2(t0, w);
+                            s = add2(s, ffma2(ffma2(t0, minus1, t1), minus1, w));   // += w - (t1 - t0)
+                            t0 = t1;
+                        } else {
+                            s = add2(s, w);
+                        }
                     }
                 }
             }
             warp_arrive_tmem(&acc_empty[buf], lane);
-            if (kTwoLevel && (kb % kSubBlocks == kSubBlocks - 1 || kb + 1 == KBh)) {
+            if (!KEEP && (++since == p.sub || kb + 1 == KBh)) {
+                since = 0;
 #pragma unroll
                 for (int k = 0; k < kPairs; ++k) {
-                    acc[k] = add2(acc[k], sub[kTwoLevel ? k : 0]);
-                    sub[kTwoLevel ? k : 0] = pack2(0.f, 0.f);
+                    if (!busy || !in_tile(k)) break;
+                    f32x2 &to = kShared ? shared_tot[k * 128 * G] : tot[kShared ? 0 : k];
+                    to = add2(to, sum[k]);
+                    sum[k] = pack2(0.f, 0.f);
                 }
             }
         }
@@ -361,10 +402,16 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                     const int j = 16 * (grp + G * k) + e;
                     if (j < NT && m0 + j < p.B) {
                         // (a wait that gave up leaves NaN: this call has no status word)
-                        const float2 two = unpack2(acc[8 * k + e / 2]);
-                        const float g = ok ? (e & 1 ? two.y : two.x) : __int_as_float(0x7fffffff);
+                        const int pair = 8 * k + e / 2;
+                        const float2 two = unpack2(kShared ? shared_tot[pair * 128 * G] : tot[kShared ? 0 : pair]);
+                        float g = e & 1 ? two.y : two.x;
+                        if (KEEP && fabsf(g) < INFINITY) {   // (what an infinite total was rounded by is no number)
+                            const float2 r = unpack2(sum[pair]);
+                            g += e & 1 ? r.y : r.x;
+                        }
+                        if (!ok) g = __int_as_float(0x7fffffff);
                         if (!UP) {
-                            p.a[(size_t)(m0 + j) * p.N + n] = g / (1.0f + expf(-g));   // SiLU, Eq. 2
+                            p.a[(size_t)(m0 + j) * p.N + n] = silu_rounded(g);
                         } else {
                             const float h = av[UP ? e : 0] * g;
                             const uint16_t hb = bf16_bits(h);
@@ -391,7 +438,10 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     }
 }
 
-template <bool F32, int TOK, bool UP = false>
+// K blocks summed before they join the totals.
+int sub_blocks(int KBh) { return KBh <= 32 ? 4 : 8; }
+
+template <bool F32, int TOK, bool UP = false, bool KEEP = false>
 cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, float *a, cudaStream_t stream,
                                 uint16_t *hhi = nullptr, uint16_t *hlo = nullptr)
 {
@@ -412,20 +462,22 @@ cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, f
     p.tmem_cols = tmem_cols_for(4 * p.NT);
     p.w_bytes = p.R * kTileBytes;
     p.stage_bytes = p.w_bytes + (F32 ? 0 : p.NT * kTileBytes);
+    p.sub = sub_blocks(p.KBh);
     const int parts = F32 ? kPartStages * kParts * p.NT * kTileBytes : 0;
+    const int totals = F32 && TOK > 64 ? TOK * BM * 4 : 0;
     // the MMAs read 128 rows from a stage's start (rows R..127 of D are not used)
     const int over = BM * kTileBytes - p.stage_bytes;
     const int slack = over > 0 ? ((over + 1023) & ~1023) : 0;
-    p.stages = stages_for(p.stage_bytes, wide_budget() - parts - slack);
+    p.stages = stages_for(p.stage_bytes, wide_budget() - parts - slack - totals);
     p.ring_bytes = p.stages * p.stage_bytes + slack;
     CUtensorMap mX{};
     if (!F32 && !make_map(&mX, x, (uint64_t)B, (uint64_t)p.H, (uint64_t)p.H * 2, (uint32_t)p.NT))
         return cudaErrorInvalidValue;
     static std::atomic<int> cfg[64];
-    const size_t smem = smem_for(1, p.ring_bytes + parts);
-    const cudaError_t e = set_smem(gate_precise_kernel<F32, TOK, UP>, smem, cfg);
+    const size_t smem = smem_for(1, p.ring_bytes + parts + totals);
+    const cudaError_t e = set_smem(gate_precise_kernel<F32, TOK, UP, KEEP>, smem, cfg);
     if (e != cudaSuccess) return e;
-    return launch_pdl_cfg(gate_precise_kernel<F32, TOK, UP>, dim3(mt, layer->tc_T), kPreciseThreads<F32>, smem, stream, mX, p);
+    return launch_pdl_cfg(gate_precise_kernel<F32, TOK, UP, KEEP>, dim3(mt, layer->tc_T), kPreciseThreads<F32>, smem, stream, mX, p);
 }
 
 // ---------------------------------------------------------------------- LoRA batches
@@ -1020,7 +1072,8 @@ cudaError_t launch_lora_gate_up(LoraGuParams &p, const sats_layer *layer, const 
 
 cudaError_t launch_gate_act(const sats_layer *layer, const uint16_t *x, int B, float *a, cudaStream_t stream)
 {
-    return tc::launch_gate_precise<false, tc::kPreciseTok>(layer, x, B, a, stream);
+    return layer->H <= tc::kKeepH ? tc::launch_gate_precise<false, tc::kPreciseTok, false, true>(layer, x, B, a, stream)
+                                  : tc::launch_gate_precise<false, tc::kPreciseTok>(layer, x, B, a, stream);
 }
 
 cudaError_t launch_gate_act_f32(const sats_layer *layer, const float *x, int B, float *a, cudaStream_t stream)
