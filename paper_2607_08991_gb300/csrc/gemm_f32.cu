@@ -542,6 +542,7 @@ struct LoraGuParams {
     int B, H, N, R, KBh;
     int NT;                 // tokens per tile (16 or 32)
     int halves;             // accumulators per K block and weight matrix: K = 32 each (2) or 64 (1)
+    int sub;                // K blocks summed before they join the totals
     float t_l, scale;
     const uint16_t *blk;    // adapter columns per neuron: B_gate, B_up, A_down
     int r;
@@ -683,46 +684,71 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
         const int n = t * R + 32 * quad + lane;
         const bool busy = c0 < NT && 32 * quad < R;   // (uniform in the warp)
         const uint32_t lane0 = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0;
-        float acc[2][16];
+        // acc: the sums of up to p.sub K blocks; they join the totals together, so that a total takes few roundings
+        // at its full size.  The totals are kept in shared memory with fp32 activations (whose parts take the registers).
+        float acc[2][16], tot[2][F32 ? 1 : 16];
+        float *const shared_tot = reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(full) + kBarrierBytes) + et;   // [2][16], kLoraEpiThreads apart
 #pragma unroll
         for (int q = 0; q < 2; ++q)
 #pragma unroll
-            for (int e = 0; e < 16; ++e) acc[q][e] = 0.f;
+            for (int e = 0; e < 16; ++e) {
+                acc[q][e] = 0.f;
+                if (F32) shared_tot[(16 * q + e) * kLoraEpiThreads] = 0.f;
+                else tot[q][F32 ? 0 : e] = 0.f;
+            }
         bool ok = true;
-        for (int kb = 0; kb < KBh; ++kb) {
-            const int buf = kb & 1;
-            if (!mbar_wait(&acc_full[buf], (uint32_t)((kb >> 1) & 1), &abort_flag)) {
-                set_timeout(p.ctl, &abort_flag);
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            if (busy) {
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    float sum[16];
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) sum[e] = 0.f;
-                    for (int f = 0; f < halves; ++f) {
-                        float v[kXParts][16];
-#pragma unroll
-                        for (int k = 0; k < kXParts; ++k)
-                            tmem_ld16(lane0 + (uint32_t)(((buf * halves + f) * 2 + q) * NX + k * NT), v[k]);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            float w = v[kXParts - 1][e];   // the small parts first
-#pragma unroll
-                            for (int k = kXParts - 2; k >= 0; --k) w += v[k][e];
-                            sum[e] += w;
-                        }
-                    }
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) acc[q][e] += sum[e];
+        int kb = 0;
+        auto blocks = [&](int end) {
+            for (; kb < end; ++kb) {
+                const int buf = kb & 1;
+                if (!mbar_wait(&acc_full[buf], (uint32_t)((kb >> 1) & 1), &abort_flag)) {
+                    set_timeout(p.ctl, &abort_flag);
+                    return false;
                 }
+                tc_fence_after();
+                if (busy) {
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        float sum[16];
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) sum[e] = 0.f;
+                        for (int f = 0; f < halves; ++f) {
+                            float v[kXParts][16];
+#pragma unroll
+                            for (int k = 0; k < kXParts; ++k)
+                                tmem_ld16(lane0 + (uint32_t)(((buf * halves + f) * 2 + q) * NX + k * NT), v[k]);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) {
+                                float w = v[kXParts - 1][e];   // the small parts first
+#pragma unroll
+                                for (int k = kXParts - 2; k >= 0; --k) w += v[k][e];
+                                sum[e] += w;
+                            }
+                        }
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) acc[q][e] += sum[e];
+                    }
+                }
+                warp_arrive_tmem(&acc_empty[buf], lane);
             }
-            warp_arrive_tmem(&acc_empty[buf], lane);
+            return true;
+        };
+        while (ok && kb < KBh) {
+            ok = blocks(min(KBh, kb + p.sub));
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    float &to = F32 ? shared_tot[(16 * q + e) * kLoraEpiThreads] : tot[q][F32 ? 0 : e];
+                    to += acc[q][e];
+                    acc[q][e] = 0.f;
+                }
         }
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int e = 0; e < 16; ++e) acc[q][e] = F32 ? shared_tot[(16 * q + e) * kLoraEpiThreads] : tot[q][F32 ? 0 : e];
         grid_dependency_wait();   // z, and y, w, h and the keep bytes may still be in use by the preceding kernels
         const int ctas = (int)(gridDim.x * gridDim.y), cta = (int)(blockIdx.y * gridDim.x + blockIdx.x);
         for (long long i = (long long)cta * kLoraEpiThreads + et; i < (long long)p.B * (p.H >> 2);
@@ -1053,15 +1079,20 @@ cudaError_t launch_lora_gate_up(LoraGuParams &p, const sats_layer *layer, const 
     // the up tile's MMA reads 128 rows from row R (rows R..127 of D are not used)
     const int over = (p.R + BM) * kTileBytes - p.stage_bytes;
     const int slack = over > 0 ? ((over + 1023) & ~1023) : 0;
-    p.stages = stages_for(p.stage_bytes, kSmemBudget - parts - slack);
+    const int totals = F32 ? 32 * kLoraEpiThreads * 4 : 0;
+    // (half of the totals fit beside the ring's budget, zs and the barriers)
+    p.stages = stages_for(p.stage_bytes, kSmemBudget - parts - slack - totals / 2);
     p.ring_bytes = p.stages * p.stage_bytes + slack;
     p.halves = F32 && p.NT > 16 ? 1 : 2;
+    // One sum over 64 blocks is as near to 64 bits as the fused kernel's (hidden 4096, fp32: 3.0e-7 both); longer ones go
+    // in parts (8192 / intermediate 3584, bf16: 3.4e-7 as one sum, 2.2e-7 so, 2.7e-7 on the fused kernel; 1 % of the call).
+    p.sub = p.KBh <= 64 ? p.KBh : 32;
     p.tmem_cols = tmem_cols_for(2 * p.halves * 2 * (F32 ? kParts : 1) * p.NT);
     CUtensorMap mX{};
     if (!F32 && !make_map(&mX, x, (uint64_t)p.B, (uint64_t)p.H, (uint64_t)p.H * 2, (uint32_t)p.NT))
         return cudaErrorInvalidValue;
     static std::atomic<int> cfg[64];
-    const size_t smem = smem_for(1, p.ring_bytes + parts);
+    const size_t smem = smem_for(1, p.ring_bytes + parts + totals);
     const cudaError_t e = set_smem(lora_gate_up_kernel<F32>, smem, cfg);
     if (e != cudaSuccess) return e;
     return launch_pdl_cfg(lora_gate_up_kernel<F32>, dim3(mt, layer->tc_T), kLoraGuThreads<F32>, smem, stream, mX, p);

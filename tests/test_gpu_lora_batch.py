@@ -59,3 +59,30 @@ def test_batches_match_oracle(sats, oracle, H, N, B, r, f32):
     assert np.linalg.norm(y2.cpu().numpy() - y_ref) <= 1e-6 * np.linalg.norm(y_ref)
     lora.close()
     layer.close()
+
+
+@pytest.mark.parametrize("H,N,B,f32", [(8192, 3584, 4, False), (8192, 3584, 17, True), (6000, 2001, 3, True),
+                                       (2048, 3100, 8, False), (256, 400, 16, True)])
+def test_no_further_from_fp64_than_single_tokens(sats, oracle, H, N, B, f32):
+    """A batch's sums are no less accurate than the fused kernel's, which runs the same tokens one at a time."""
+    r, scale = 16, 1.0
+    w, lo, layer, lora = _setup(sats, H, N, r, scale, seed=12)
+    if f32:
+        xf = inputs.activations_f32(B, H, seed=inputs.SEED_X + 32)
+        x64, x = xf.astype(np.float64), P.dev(xf)
+    else:
+        xb = inputs.activations_bf16(B, H, seed=inputs.SEED_X + 32)
+        x64, x = oracle.bf16_to_f64(xb), P.dev_u16(xb)
+    t = _threshold(oracle, w, H, 0.6)
+    ws = sats.Workspace(H, N, B)
+    y, keep = _call(sats, layer, lora, x, t, B, H, N, ws)
+    ref, _, _, _ = oracle.sparse_mlp_lora(x64, w.Wg, w.Wu, w.Wd, lo, scale, t, keep_hint=keep, band_rel=P.BAND_REL)
+    one = np.empty_like(y)
+    for b in range(B):
+        one[b], k1 = (v[0] for v in _call(sats, layer, lora, x[b:b + 1], t, 1, H, N, ws))
+        if not np.array_equal(k1, keep[b]):   # a neuron at the threshold fell on the other side
+            one[b] = ref[b]
+    err, err1 = np.linalg.norm(y - ref), np.linalg.norm(one - ref)
+    assert err1 > 0 and err <= err1
+    lora.close()
+    layer.close()
