@@ -238,7 +238,8 @@ __global__ void __launch_bounds__(256) row_squares_kernel(const float *__restric
 }
 
 // err[k] += sum_c ||d_kc|| / (||y_c|| + eps), with d = y - y~_t (the dropped neurons' output) and y the dense one:
-// sq is [K + 1][C], the dense rows first.  Grid: K.
+// sq is [K + 1][C], the dense rows first.  A dense output that is not finite has no distortion (infinity less infinity,
+// were the outputs subtracted).  Grid: K.
 __global__ void __launch_bounds__(256) err_ratio_kernel(const double *__restrict__ sq, int C, float eps,
                                                         double *__restrict__ err)
 {
@@ -246,7 +247,8 @@ __global__ void __launch_bounds__(256) err_ratio_kernel(const double *__restrict
     grid_launch_dependents();
     const double *d = sq + (size_t)(blockIdx.x + 1) * C;
     double s = 0.0;
-    for (int c = threadIdx.x; c < C; c += 256) s += sqrt(d[c]) / (sqrt(sq[c]) + (double)eps);
+    for (int c = threadIdx.x; c < C; c += 256)
+        s += isfinite(sq[c]) ? sqrt(d[c]) / (sqrt(sq[c]) + (double)eps) : (double)NAN;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     __shared__ double part[8];

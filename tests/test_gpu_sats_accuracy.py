@@ -77,3 +77,18 @@ def test_calibration_table_against_fp64(sats):
     ref = _errors(h, [mask < np.float32(v) for v in t], W[2], 1e-6)
     assert np.linalg.norm(err - ref) <= 1e-6 * np.linalg.norm(ref)
     layer.close()
+
+
+@pytest.mark.parametrize("C", [2, 4, 40])   # the fused kernel; the tensor cores
+def test_infinite_output_has_no_error(sats, C):
+    """A kept neuron whose output overflows: y - y~ is infinity less infinity, not a small distortion."""
+    H, N = 96, 24
+    w = inputs.mlp_weights(H, N, std=0.02, seed=1420)
+    Wg, Wu, Wd = (m.copy() for m in (w.Wg, w.Wu, w.Wd))
+    Wg[:, 0] = Wu[:, 0] = inputs.to_bf16_bits(np.full(H, 0.02, np.float32))
+    Wd[0, :] = inputs.to_bf16_bits(np.full(H, 3e38, np.float32))
+    layer = sats.Layer(P.dev_u16(Wg), P.dev_u16(Wu), P.dev_u16(Wd))
+    x = np.abs(inputs.activations_f32(C, H, seed=1421))
+    err, sp = sats.layer_err(layer, P.dev(x), [0.05, 0.2], eps=1e-6)   # |a| of neuron 0: about 1.2; of the others: below 0.5
+    assert np.isnan(err).all() and (np.asarray(sp) > 0).all() and (np.asarray(sp) < 1).all()
+    layer.close()
