@@ -25,7 +25,9 @@
  *     enqueued.  Errors found by a kernel (a token id outside the vocabulary, a
  *     wait that ran out of time) are recorded in a status word in the
  *     workspace (or in the caller's status word for sats_route) and returned by
- *     sats_get_error.  No call aborts, throws, or traps on the device.
+ *     sats_get_error; a call that synchronises returns them itself.
+ *     sats_gate_act and sats_gate_act_f32 have no status word: a wait that
+ *     runs out leaves NaN in a.  No call aborts, throws, or traps on the device.
  *   - Calls never allocate device memory, except sats_layer_create.
  *   - Requirements: H a multiple of 8 and 8 <= H <= 8192; N >= 1; B >= 0.
  *   - SM occupancy: the single-token / two-token decode kernel (the small-batch
@@ -322,7 +324,9 @@ SATS_API sats_status sats_gate_act(const sats_layer *layer, const void *x, int B
  *   a      : device fp32 [n] (NaN not allowed)
  *   t_out  : host fp32 [1], written.
  *   ws     : device workspace of at least sats_select_workspace_bytes() bytes.
- * Synchronises `stream` (the result is returned on the host).
+ * Synchronises `stream` (the result is returned on the host).  Its CTAs (a
+ * cooperative launch) wait, bounded, for one another: SATS_ETIMEOUT, with
+ * *t_out NaN, if one does not come within 2 s.
  */
 SATS_API size_t sats_select_workspace_bytes(void);
 SATS_API sats_status sats_percentile_threshold(const float *a, int64_t n, double k, float *t_out,
@@ -426,6 +430,15 @@ SATS_API sats_status sats_route_calibrate(const float *score, int V, const int32
  * shape (at least 256 bytes), not in use by another call.
  */
 SATS_API sats_status sats_selftest_wait_timeout(void *ws, size_t ws_bytes, void *stream);
+
+/*
+ * sats_selftest_select_timeout -- the same for sats_percentile_threshold: its
+ * selection over a (device fp32 [n], n >= 1) at k = 1, waiting for one CTA
+ * more than there are.  Returns SATS_ETIMEOUT after about 2 s, with *t_out NaN;
+ * arguments and workspace as there.
+ */
+SATS_API sats_status sats_selftest_select_timeout(const float *a, int64_t n, float *t_out, void *ws,
+                                                  size_t ws_bytes, void *stream);
 
 /*
  * sats_get_error -- synchronises `stream`, reads the status word in the

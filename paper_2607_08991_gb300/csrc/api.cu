@@ -494,8 +494,8 @@ sats_status sats_gate_act(const sats_layer *layer, const void *x, int B, float *
 
 size_t sats_select_workspace_bytes(void) { return select_ws_bytes(); }
 
-sats_status sats_percentile_threshold(const float *a, int64_t n, double k, float *t_out, void *ws, size_t ws_bytes,
-                                      void *stream)
+static sats_status percentile_threshold(const float *a, int64_t n, double k, float *t_out, void *ws, size_t ws_bytes,
+                                        void *stream, int absent)
 {
     if (!t_out || n < 0 || std::isnan(k)) return SATS_EINVAL;
     if (n == 0 || !(k > 0.0)) { *t_out = 0.0f; return SATS_OK; }
@@ -503,11 +503,25 @@ sats_status sats_percentile_threshold(const float *a, int64_t n, double k, float
     if (!a || !ws || ws_bytes < select_ws_bytes() || !aligned16(ws)) return SATS_EINVAL;
     const int64_t m = percentile_rank(n, k);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    float *t_dev = reinterpret_cast<float *>(static_cast<char *>(ws) + select_ws_bytes() - 128);
-    cudaError_t e = launch_select(a, n, &m, 1, ws, t_dev, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(t_out, t_dev, sizeof(float), cudaMemcpyDeviceToHost, st);
+    struct {
+        int32_t status;
+        float t;
+    } got;
+    static_assert(kSelResultWord == kSelStatusWord + 1, "read back together");
+    int *words = static_cast<int *>(ws);
+    cudaError_t e = launch_select(a, n, &m, 1, ws, reinterpret_cast<float *>(words + kSelResultWord),
+                                  words + kSelStatusWord, st, absent);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&got, words + kSelStatusWord, sizeof got, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    return from_cuda(e);
+    if (e != cudaSuccess) return from_cuda(e);
+    *t_out = got.t;
+    return (got.status & kStatusTimeout) ? SATS_ETIMEOUT : SATS_OK;
+}
+
+sats_status sats_percentile_threshold(const float *a, int64_t n, double k, float *t_out, void *ws, size_t ws_bytes,
+                                      void *stream)
+{
+    return percentile_threshold(a, n, k, t_out, ws, ws_bytes, stream, 0);
 }
 
 static sats_status read_status(int32_t *word, cudaStream_t st)
@@ -526,6 +540,13 @@ sats_status sats_selftest_wait_timeout(void *ws, size_t ws_bytes, void *stream)
 {
     if (!ws || ws_bytes < (size_t)kCtlInts * sizeof(int)) return SATS_EINVAL;
     return from_cuda(launch_wait_timeout(static_cast<int *>(ws), static_cast<cudaStream_t>(stream)));
+}
+
+sats_status sats_selftest_select_timeout(const float *a, int64_t n, float *t_out, void *ws, size_t ws_bytes,
+                                         void *stream)
+{
+    if (n < 1) return SATS_EINVAL;
+    return percentile_threshold(a, n, 1.0, t_out, ws, ws_bytes, stream, 1);
 }
 
 sats_status sats_get_error(void *ws, size_t ws_bytes, void *stream)

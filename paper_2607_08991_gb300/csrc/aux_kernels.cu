@@ -118,8 +118,9 @@ __global__ void __launch_bounds__(kRouteThreads) route_kernel(const int32_t *ids
 // levels 1 and 2 count the next 10 bits of the values that share their leading bits
 // with one of the ranks (a slot each; ranks in one bin share its slot).  At each level
 // a CTA counts its values in shared memory and adds the non-zero counts to the level's
-// histogram; once all CTAs have, every one of them finds every rank's bin by itself.
-// The three levels are one cooperative launch, whose CTAs meet twice.
+// histogram; once all CTAs have, every one of them finds every rank's bin by itself (after
+// the last level the first CTA alone).  The three levels are one cooperative launch; a CTA whose
+// bounded wait for the others runs out records it in *status, and the results are then NaN.
 //
 // What bounds it: passes over values that sit in L2, and the meetings.  Post-gate
 // magnitudes fall into a few dozen of the top bins, so counting them with atomics in
@@ -135,7 +136,7 @@ constexpr int kSelThreads = 1024, kSelWarps = kSelThreads / 32;
 
 // Workspace of a selection of R ranks; cleared as a whole before it.
 struct SelWs {
-    int *done;              // [3] CTAs finished per level
+    int *done;              // [3] CTAs finished per level; the words behind them are the caller's (kSelStatusWord)
     unsigned *hist0;        // [kSelBins0]
     unsigned *hist;         // [2][R][kSelBins] levels 1 and 2
 };
@@ -148,7 +149,7 @@ __host__ __device__ inline size_t sel_layout(char *base, int R, SelWs *w)
         off += (bytes + 255) & ~(size_t)255;
         return p;
     };
-    w->done = reinterpret_cast<int *>(take(3 * sizeof(int)));
+    w->done = reinterpret_cast<int *>(take((kSelResultWord + kSelRanks) * sizeof(int)));
     w->hist0 = reinterpret_cast<unsigned *>(take(kSelBins0 * sizeof(unsigned)));
     w->hist = reinterpret_cast<unsigned *>(take((size_t)2 * R * kSelBins * sizeof(unsigned)));
     return off;
@@ -233,17 +234,23 @@ struct SelRankList {
     long long m[kSelRanks];
 };
 
-// All CTAs of the (cooperative) grid have added their counts of a level; false if they do not within kWaitLimitNs.
-__device__ __forceinline__ bool sel_meet(int *done, bool *met)
+// This CTA has added its counts of a level.
+__device__ __forceinline__ void sel_arrive(int *done)
 {
     __threadfence();
     __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(done, 1);
+}
+
+// `ctas` CTAs of the (cooperative) grid have; false, and a timeout in *status, if they do not within kWaitLimitNs.
+__device__ __forceinline__ bool sel_meet(const int *done, int ctas, int *status, bool *met)
+{
     if (threadIdx.x == 0) {
-        atomicAdd(done, 1);
         const unsigned long long t0 = global_ns();
         bool ok = true;
-        while (ld_acquire_gpu(done) < (int)gridDim.x)
+        while (ld_acquire_gpu(done) < ctas)
             if (global_ns() - t0 > kWaitLimitNs) { ok = false; break; }
+        if (!ok) atomicOr(status, kStatusTimeout);
         *met = ok;
     }
     __syncthreads();
@@ -251,7 +258,7 @@ __device__ __forceinline__ bool sel_meet(int *done, bool *met)
 }
 
 __global__ void __launch_bounds__(kSelThreads) select_kernel(const float *__restrict__ a, int64_t n, int R,
-                                                             const SelRankList ranks, char *ws,
+                                                             const SelRankList ranks, char *ws, int ctas, int *status,
                                                              float *__restrict__ t_out)
 {
     extern __shared__ unsigned sel_smem[];
@@ -303,11 +310,13 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float *__rest
             for (int i = tid; i < nh; i += kSelThreads)
                 if (h[i]) atomicAdd(gh + i, h[i]);
         }
-        if (!sel_meet(w.done + level, &met)) {
-            if (tid < R) t_out[tid] = __int_as_float(0x7fffffff);
+        sel_arrive(w.done + level);
+        if (level == 2 && blockIdx.x != 0) return;
+        if (!sel_meet(w.done + level, ctas, status, &met)) {
+            // (where another CTA gives up, the first one does at the last level)
+            if (blockIdx.x == 0 && tid < R) t_out[tid] = __int_as_float(0x7fffffff);
             return;
         }
-        if (level == 2 && blockIdx.x != 0) return;
         // all CTAs' counts (past L1: the other CTAs wrote them)
         for (int i = tid; i < (level == 0 ? kSelBins0 : nh) / 4; i += kSelThreads)
             reinterpret_cast<uint4 *>(h)[i] = __ldcg(reinterpret_cast<const uint4 *>(gh) + i);
@@ -438,9 +447,11 @@ size_t select_multi_ws_bytes(int R)
 }
 
 // t_dev[i] = the m[i]-th smallest of |a_0 .. a_{n-1}| for R <= kSelRanks ranks in [1, n];
-// ws: select_multi_ws_bytes(R) bytes, 16-byte aligned.
-cudaError_t launch_select(const float *a, int64_t n, const int64_t *m, int R, void *ws, float *t_dev,
-                          cudaStream_t stream)
+// ws: select_multi_ws_bytes(R) bytes, 16-byte aligned.  A wait that gives up sets kStatusTimeout in *status (device; a
+// word of its own, or ws's word kSelStatusWord, which is cleared here).  absent: CTAs that are waited for and do not exist (the
+// self-test's; 0).
+cudaError_t launch_select(const float *a, int64_t n, const int64_t *m, int R, void *ws, float *t_dev, int *status,
+                          cudaStream_t stream, int absent)
 {
     if (R < 1 || R > kSelRanks) return cudaErrorInvalidValue;
     SelRankList ranks;
@@ -468,7 +479,7 @@ cudaError_t launch_select(const float *a, int64_t n, const int64_t *m, int R, vo
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, select_kernel, a, n, R, ranks, base, t_dev);
+    return cudaLaunchKernelEx(&cfg, select_kernel, a, n, R, ranks, base, grid + absent, status, t_dev);
 }
 
 }  // namespace sats

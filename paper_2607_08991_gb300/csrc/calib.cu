@@ -421,8 +421,9 @@ sats_status layer_err_tc(const sats_layer *layer, const float *x, int C, const f
     if (e == cudaSuccess) e = cudaMemsetAsync(base + W.acc, 0, sum_bytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "layer error workspace clear");
     const ErrInputs in(base + W.a, layer->N, C);
-    e = launch_gate_act_f32(layer, x, C, in.a, st);
-    if (e == cudaSuccess) e = launch_up_f32(layer, x, C, in.a, in.hhi, in.hlo, st);
+    int *status = reinterpret_cast<int *>(mlp + ws_layout(layer->H, layer->N, C).ctl) + kCtlStatus;
+    e = launch_gate_act_f32(layer, x, C, in.a, status, st);
+    if (e == cudaSuccess) e = launch_up_f32(layer, x, C, in.a, in.hhi, in.hlo, status, st);
     if (e != cudaSuccess) return cuda_fail(e, "gate and up kernels launch");
     sats_status s = enqueue_err(layer, in, C, t, nullptr, [](int k) { return k; }, K, eps, ErrSums(base + W.acc, K), base, W, st);
     if (s != SATS_OK) return s;
@@ -490,7 +491,7 @@ sats_status sats_gate_act_f32(const sats_layer *layer, const float *x, int B, fl
     if (!layer || B < 0) return SATS_EINVAL;
     if (B == 0) return SATS_OK;
     if (!x || !a || (reinterpret_cast<uintptr_t>(x) & 15u)) return SATS_EINVAL;
-    const cudaError_t e = launch_gate_act_f32(layer, x, B, a, static_cast<cudaStream_t>(stream));
+    const cudaError_t e = launch_gate_act_f32(layer, x, B, a, nullptr, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? SATS_OK : cuda_fail(e, "gate activation kernel launch");
 }
 
@@ -647,14 +648,16 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     auto inputs_of = [&](int l) {
         return ErrInputs(W.in_each ? base + W.in + l * W.in_each : ews + E.a, N, C);
     };
+    char *mlp = ews + E.mlp;
+    // every bounded wait of the call reports here
+    int *status = reinterpret_cast<int *>(mlp + ws_layout(H, N, C).ctl) + kCtlStatus;
     auto n_of = [&](int l) { return nall + (size_t)l * C * H; };
     auto up_of = [&](int l) {
         const ErrInputs in = inputs_of(l);
-        return launch_up_f32(layers[l], n_of(l), C, in.a, in.hhi, in.hlo, st);
+        return launch_up_f32(layers[l], n_of(l), C, in.a, in.hhi, in.hlo, status, st);
     };
     auto gate_of = [&](int l) { return batched ? inputs_of(l).a : reinterpret_cast<float *>(base + W.a); };
     const size_t ews_bytes = W.total - W.err;
-    void *mlp = ews + E.mlp;
     const int guard = guardrail ? L - 1 : -1;
 
     // 1-2: the dense stack gives each block's MLP inputs; coarse candidates from |SiLU(n W_gate)|
@@ -671,7 +674,8 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     for (int l = 0; l < L; ++l) {
         if ((s = sats_rmsnorm(x, C, H, norm_w[l], eps, n_of(l), stream)) != SATS_OK) return s;
         float *a = gate_of(l);
-        if ((s = sats_gate_act_f32(layers[l], n_of(l), C, a, stream)) != SATS_OK) return s;
+        if ((e = launch_gate_act_f32(layers[l], n_of(l), C, a, status, st)) != cudaSuccess)
+            return cuda_fail(e, "gate activation kernel launch");
         // Eq. 3 at k / K0, the largest |a|, and the guardrail block's percentile at the target, all
         // from shared passes over |a|; read back once after the last block
         float *ql = q + (size_t)l * (K0 + 1);
@@ -679,7 +683,8 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
         for (int k = 0; k < nq; ++k)
             rank[(size_t)k] = percentile_rank(n, k < Kc ? (double)(k + 1) / K0 : k == Kc ? 1.0 : s_tar);
         for (int k = 0; k < nq; k += kSelRanks)
-            if ((e = launch_select(a, n, rank.data() + k, std::min(kSelRanks, nq - k), sel, ql + k, st)) != cudaSuccess)
+            if ((e = launch_select(a, n, rank.data() + k, std::min(kSelRanks, nq - k), sel, ql + k, status, st)) !=
+                cudaSuccess)
                 return cuda_fail(e, "percentile kernels launch");
         if (batched) {
             // 3: Eq. 6 for every coarse candidate (and, with them, the guardrail's CATS threshold), the
@@ -709,7 +714,7 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
         amax[(size_t)l] = ql[Kc];
         if (l == guard) g_t = s_tar > 0.0 ? ql[Kc + 1] : 0.f;
     }
-    if (batched && (s = sats_get_error(mlp, ws_layout(H, N, C).total, stream)) != SATS_OK) return s;
+    if ((s = sats_get_error(mlp, ws_layout(H, N, C).total, stream)) != SATS_OK) return s;
     // 3 (without a batch): Eq. 6 block by block
     std::vector<float> tf((size_t)Kmax);
     std::vector<double> eb((size_t)Kmax), sb((size_t)Kmax);
@@ -765,7 +770,8 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
         }
         if (K1 == 0) continue;
         if (batched && W.in_each == 0) {
-            if ((s = sats_gate_act_f32(layers[l], n_of(l), C, gate_of(l), stream)) != SATS_OK) return s;
+            if ((e = launch_gate_act_f32(layers[l], n_of(l), C, gate_of(l), status, st)) != cudaSuccess)
+                return cuda_fail(e, "gate activation kernel launch");
             if ((e = up_of(l)) != cudaSuccess) return cuda_fail(e, "up kernel launch");
         }
         s = batched ? enqueue_err(layers[l], inputs_of(l), C, tf.data() + (size_t)l * K1, nullptr, [](int k) { return k; },

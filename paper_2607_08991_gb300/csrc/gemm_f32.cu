@@ -57,6 +57,7 @@ struct PreciseGateParams {
     float *a;              // [B][N]: written, or read for h (UP)
     uint16_t *hhi, *hlo;   // UP: [B][ldh] bf16
     int ldh;
+    int *status;           // takes kStatusTimeout if a wait gives up, or nullptr
     int sub;               // K blocks summed before they join the totals
     int stages, stage_bytes, w_bytes, ring_bytes;
     uint32_t tmem_cols;    // four accumulators of NT columns
@@ -211,6 +212,10 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
     const int R = p.R, NT = p.NT, S = p.stages, KBh = p.KBh;
     const int m0 = (int)blockIdx.x * NT, t = blockIdx.y;
     const int n_quads = (R + 31) / 32;   // TMEM lane quarters that hold neurons
+    auto give_up = [&]() {
+        abort_flag = 1;
+        if (p.status) atomicOr(p.status, kStatusTimeout);
+    };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
@@ -261,7 +266,7 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
             if (kb >= npre) {
                 if (!(F32 ? warp_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag)
                           : mbar_wait(&empty[s], (uint32_t)ph ^ 1u, &abort_flag))) {
-                    abort_flag = 1;
+                    give_up();
                     break;
                 }
                 mbar_expect_if(lead, &full[s], load_bytes);
@@ -282,7 +287,7 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
             uint64_t *const bar = lane == 1 ? &acc_empty[buf] : F32 && lane == 2 ? &pfull[ps] : &full[s];
             if (F32 ? !warp_wait(bar, lane == 1 ? bph ^ 1u : lane == 2 ? bph : (uint32_t)ph, &abort_flag)
                     : !warp_wait(&acc_empty[buf], bph ^ 1u, &abort_flag) || !warp_wait(&full[s], (uint32_t)ph, &abort_flag)) {
-                abort_flag = 1;
+                give_up();
                 break;
             }
             tc_fence_after();
@@ -315,7 +320,7 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                 hi = src[1];
             }
         };
-        if (!cut_tiles<TOK>(parts, NT, KBh, pfull, pempty, &abort_flag, load)) abort_flag = 1;
+        if (!cut_tiles<TOK>(parts, NT, KBh, pfull, pempty, &abort_flag, load)) give_up();
     } else if (warp >= kEpi0) {
         const int quad = warp & 3, grp = (warp - kEpi0) >> 2;
         const uint32_t lane0 = tmem + ((uint32_t)(32 * quad) << 16);
@@ -341,7 +346,11 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
         bool ok = true;
         for (int kb = 0; kb < KBh; ++kb) {
             const int buf = kb & 1;
-            if (!mbar_wait(&acc_full[buf], (uint32_t)((kb >> 1) & 1), &abort_flag)) { ok = false; break; }
+            if (!mbar_wait(&acc_full[buf], (uint32_t)((kb >> 1) & 1), &abort_flag)) {
+                give_up();
+                ok = false;
+                break;
+            }
             tc_fence_after();
             if (busy) {
                 const uint32_t a0 = lane0 + (uint32_t)(2 * buf * NT);
@@ -401,7 +410,6 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                 for (int e = 0; e < 16; ++e) {
                     const int j = 16 * (grp + G * k) + e;
                     if (j < NT && m0 + j < p.B) {
-                        // (a wait that gave up leaves NaN: this call has no status word)
                         const int pair = 8 * k + e / 2;
                         const float2 two = unpack2(kShared ? shared_tot[pair * 128 * G] : tot[kShared ? 0 : pair]);
                         float g = e & 1 ? two.y : two.x;
@@ -409,7 +417,7 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
                             const float2 r = unpack2(sum[pair]);
                             g += e & 1 ? r.y : r.x;
                         }
-                        if (!ok) g = __int_as_float(0x7fffffff);
+                        if (!ok) g = __int_as_float(0x7fffffff);   // (some callers have no status word)
                         if (!UP) {
                             p.a[(size_t)(m0 + j) * p.N + n] = silu_rounded(g);
                         } else {
@@ -442,8 +450,8 @@ __global__ void __launch_bounds__(kPreciseThreads<F32>, 1)
 int sub_blocks(int KBh) { return KBh <= 32 ? 4 : 8; }
 
 template <bool F32, int TOK, bool UP = false, bool KEEP = false>
-cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, float *a, cudaStream_t stream,
-                                uint16_t *hhi = nullptr, uint16_t *hlo = nullptr)
+cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, float *a, int *status,
+                                cudaStream_t stream, uint16_t *hhi = nullptr, uint16_t *hlo = nullptr)
 {
     PreciseGateParams p{};
     p.w = layer->gu_blk;
@@ -459,6 +467,7 @@ cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, f
     p.hhi = hhi;
     p.hlo = hlo;
     p.ldh = layer->ldn;
+    p.status = status;
     p.tmem_cols = tmem_cols_for(4 * p.NT);
     p.w_bytes = p.R * kTileBytes;
     p.stage_bytes = p.w_bytes + (F32 ? 0 : p.NT * kTileBytes);
@@ -1103,22 +1112,23 @@ cudaError_t launch_lora_gate_up(LoraGuParams &p, const sats_layer *layer, const 
 
 cudaError_t launch_gate_act(const sats_layer *layer, const uint16_t *x, int B, float *a, cudaStream_t stream)
 {
-    return layer->H <= tc::kKeepH ? tc::launch_gate_precise<false, tc::kPreciseTok, false, true>(layer, x, B, a, stream)
-                                  : tc::launch_gate_precise<false, tc::kPreciseTok>(layer, x, B, a, stream);
+    return layer->H <= tc::kKeepH ? tc::launch_gate_precise<false, tc::kPreciseTok, false, true>(layer, x, B, a, nullptr, stream)
+                                  : tc::launch_gate_precise<false, tc::kPreciseTok>(layer, x, B, a, nullptr, stream);
 }
 
-cudaError_t launch_gate_act_f32(const sats_layer *layer, const float *x, int B, float *a, cudaStream_t stream)
+cudaError_t launch_gate_act_f32(const sats_layer *layer, const float *x, int B, float *a, int *status,
+                                cudaStream_t stream)
 {
-    return B <= 64 ? tc::launch_gate_precise<true, 64>(layer, x, B, a, stream)
-                   : tc::launch_gate_precise<true, tc::kPreciseTok>(layer, x, B, a, stream);
+    return B <= 64 ? tc::launch_gate_precise<true, 64>(layer, x, B, a, status, stream)
+                   : tc::launch_gate_precise<true, tc::kPreciseTok>(layer, x, B, a, status, stream);
 }
 
 cudaError_t launch_up_f32(const sats_layer *layer, const float *x, int B, const float *a, uint16_t *hhi, uint16_t *hlo,
-                          cudaStream_t stream)
+                          int *status, cudaStream_t stream)
 {
     float *const in = const_cast<float *>(a);   // (read only)
-    return B <= 64 ? tc::launch_gate_precise<true, 64, true>(layer, x, B, in, stream, hhi, hlo)
-                   : tc::launch_gate_precise<true, tc::kPreciseTok, true>(layer, x, B, in, stream, hhi, hlo);
+    return B <= 64 ? tc::launch_gate_precise<true, 64, true>(layer, x, B, in, status, stream, hhi, hlo)
+                   : tc::launch_gate_precise<true, tc::kPreciseTok, true>(layer, x, B, in, status, stream, hhi, hlo);
 }
 
 // Scratch of a LoRA batch inside the tensor-core region of a workspace: z and w where the other

@@ -153,10 +153,12 @@ cudaError_t launch_route(const int32_t *ids, int B, const uint8_t *lut, int V, i
                          int32_t *n_dense, uint8_t *flags, int32_t *status, cudaStream_t stream);
 cudaError_t launch_gate_act(const sats_layer *layer, const uint16_t *x, int B, float *a,
                             cudaStream_t stream);
-cudaError_t launch_gate_act_f32(const sats_layer *layer, const float *x, int B, float *a, cudaStream_t stream);
+// (status: a device word that takes kStatusTimeout if a wait gives up, or nullptr; a is then NaN in places)
+cudaError_t launch_gate_act_f32(const sats_layer *layer, const float *x, int B, float *a, int *status,
+                                cudaStream_t stream);
 // h = a u of every neuron, u = x W_up in the same accuracy, in two bf16 parts with row stride ldn.
 cudaError_t launch_up_f32(const sats_layer *layer, const float *x, int B, const float *a, uint16_t *hhi, uint16_t *hlo,
-                          cudaStream_t stream);
+                          int *status, cudaStream_t stream);
 
 // One block over B tokens (fused kernel or tensor cores), as the C ABI calls run it
 // (api.cu).  ws: a workspace of ws_layout(H, N, B).total bytes with zeroed control words.
@@ -171,7 +173,9 @@ constexpr int kSelRanks = 32;   // ranks that one selection finds together
 int64_t percentile_rank(int64_t n, double k);   // Eq. 3's rank of the k-th quantile, 0 < k <= 1
 size_t select_ws_bytes();
 size_t select_multi_ws_bytes(int R);
-cudaError_t launch_select(const float *a, int64_t n, const int64_t *m, int R, void *ws, float *t_dev,
-                          cudaStream_t stream);
+// Words of a selection's workspace for a caller who reads them back together: its status, its first result.
+constexpr int kSelStatusWord = 3, kSelResultWord = 4;
+cudaError_t launch_select(const float *a, int64_t n, const int64_t *m, int R, void *ws, float *t_dev, int *status,
+                          cudaStream_t stream, int absent = 0);
 
 }  // namespace sats

@@ -79,6 +79,7 @@ def lib() -> ctypes.CDLL:
             "sats_get_error": (I, [P, Z, P]),
             "sats_get_status_word": (I, [P, P]),
             "sats_selftest_wait_timeout": (I, [P, Z, P]),
+            "sats_selftest_select_timeout": (I, [P, I64, ctypes.POINTER(F), P, Z, P]),
         }
         for name, (res, args) in sig.items():
             fn = getattr(L, name)
@@ -99,7 +100,8 @@ def exported_symbols() -> Sequence[str]:
             "sats_select_workspace_bytes", "sats_percentile_threshold", "sats_rmsnorm", "sats_gate_act_f32",
             "sats_layer_err_workspace_bytes", "sats_layer_err", "sats_sats_select", "sats_sats_workspace_bytes",
             "sats_sats_calibrate", "sats_route_calib_workspace_bytes", "sats_token_scores", "sats_route_calibrate",
-            "sats_get_error", "sats_get_status_word", "sats_selftest_wait_timeout")
+            "sats_get_error", "sats_get_status_word", "sats_selftest_wait_timeout",
+            "sats_selftest_select_timeout")
 
 
 def status_string(s: int) -> str:
@@ -427,6 +429,15 @@ def selftest_wait_timeout(ws: Workspace, stream: Optional[torch.cuda.Stream] = N
     """Runs the library's bounded device waits against conditions nothing satisfies; the
     next get_error(ws) reads ETIMEOUT (takes about 4 s)."""
     _check(lib().sats_selftest_wait_timeout(ws.buf.data_ptr(), ws.nbytes, _stream(stream)), "sats_selftest_wait_timeout")
+
+
+def selftest_select_timeout(a: torch.Tensor, sel_ws: torch.Tensor, stream: Optional[torch.cuda.Stream] = None):
+    """Runs percentile_threshold's selection with one CTA missing; returns the status (ETIMEOUT, after about 2 s) and
+    what it left as the threshold."""
+    out = ctypes.c_float()
+    s = lib().sats_selftest_select_timeout(_ptr(a, "a", 4), a.numel(), ctypes.byref(out), _ptr(sel_ws, "sel_ws"),
+                                           sel_ws.numel() * sel_ws.element_size(), _stream(stream))
+    return int(s), float(out.value)
 
 
 def get_error(ws: Workspace, stream: Optional[torch.cuda.Stream] = None) -> int:

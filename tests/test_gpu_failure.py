@@ -52,3 +52,13 @@ def test_bounded_waits_time_out_and_the_workspace_recovers(sats, oracle):
     P.assert_keep_match(keep, keep_ref, a_ref, t)
     P.assert_close(y.cpu().numpy(), y_ref)
     layer.close()
+
+
+@pytest.mark.parametrize("n", [8, 300000])   # one CTA, and many, short of one
+def test_selection_reports_a_missing_cta(sats, n):
+    a = torch.arange(1, n + 1, dtype=torch.float32, device="cuda")
+    sel = torch.zeros(sats.select_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    assert sats.percentile_threshold(a, 0.5, sel) == n // 2
+    status, t = sats.selftest_select_timeout(a, sel)
+    assert status == sats.ETIMEOUT and np.isnan(t)
+    assert sats.percentile_threshold(a, 1.0, sel) == n   # the workspace stays usable
