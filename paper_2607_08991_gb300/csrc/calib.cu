@@ -554,7 +554,7 @@ sats_status sats_sats_select(const double *t, const double *err, const double *s
 {
     if (L < 1 || K < 0 || !t_out || !b_out || !S_out || std::isnan(s_tar)) return SATS_EINVAL;
     if (K > 0 && (!t || !err || !sp)) return SATS_EINVAL;
-    if (guard >= L) return SATS_EINVAL;
+    if (guard >= L || (guard >= 0 && (std::isnan(guard_t) || std::isnan(guard_sp)))) return SATS_EINVAL;
     // per block, candidate indices by decreasing threshold (stable: the first listed wins a tie)
     std::vector<std::vector<int>> order((size_t)L);
     std::vector<double> budgets(1, 0.0);

@@ -48,3 +48,8 @@ def test_select_rejects_bad_arguments(sats):
         sats.sats_select([[float("nan")]], [[0.1]], [[0.5]], 0.5)
     with pytest.raises(sats.SatsError):
         sats.sats_select([[0.1]], [[0.1]], [[0.5]], 0.5, guard=3)
+    nan = float("nan")
+    for guard_t, guard_sp in ((nan, 0.5), (0.1, nan)):   # the guarded block's own choice and share
+        with pytest.raises(sats.SatsError):
+            sats.sats_select([[0.1]], [[0.1]], [[0.5]], 0.5, guard=0, guard_t=guard_t, guard_sp=guard_sp)
+    sats.sats_select([[0.1]], [[0.1]], [[0.5]], 0.5, guard=-1, guard_t=nan, guard_sp=nan)   # not used
