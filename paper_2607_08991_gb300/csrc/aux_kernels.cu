@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float *__rest
                                                              const SelRankList ranks, char *ws, int ctas, int *status,
                                                              float *__restrict__ t_out)
 {
-    extern __shared__ unsigned sel_smem[];
+    extern __shared__ __align__(16) unsigned sel_smem[];   // (stored to in 16-byte vectors)
     __shared__ int bins[kSelRanks], slot[kSelRanks], nslots;
     __shared__ long long rest[kSelRanks];        // rank within the bins chosen so far (1-based)
     __shared__ uint32_t prefix[kSelRanks];       // bits chosen so far
