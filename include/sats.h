@@ -349,7 +349,8 @@ SATS_API sats_status sats_percentile_threshold(const float *a, int64_t n, double
  *     sp[k]  = (1/C) sum_c (neurons with |a| < t_k) / N
  *   y is the dense output (Eq. 1), y~_t the thresholded one (Eqs. 4-5), both
  *   computed by the library's MLP kernels.  err, sp: host double [K].  ws:
- *   device workspace of sats_layer_err_workspace_bytes(H, N, C, K) bytes,
+ *   device workspace of sats_layer_err_workspace_bytes(H, N, C, K) bytes (an
+ *   ordinary workspace for C tokens, 4 C N bytes and at most 512 MiB),
  *   256-byte aligned (no initialisation needed).  Synchronises `stream`.
  *
  * sats_sats_select -- Eqs. 7-10 on the host over a candidate table t, err,
@@ -373,7 +374,9 @@ SATS_API sats_status sats_percentile_threshold(const float *a, int64_t n, double
  *   the last block keeps the CATS threshold (the Eq. 3 percentile at s_tar),
  *   as Sec. 4 does.  Writes t_out (host fp32 [L]), b* and S(b*), and, if all
  *   three are given, the candidate table (host double [L][K0 - 1 + K1]).
- *   ws: sats_sats_workspace_bytes(H, N, C, L, K0, K1) bytes, 256-byte aligned.
+ *   ws: sats_sats_workspace_bytes(H, N, C, L, K0, K1) bytes (as sats_layer_err,
+ *   4 (L + 1) C H bytes, and at most 1 GiB of values kept between steps 3 and
+ *   6), 256-byte aligned.
  *   Synchronises `stream`.
  */
 SATS_API sats_status sats_rmsnorm(const float *x, int B, int H, const float *w, float eps, float *out,

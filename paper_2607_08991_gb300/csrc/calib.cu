@@ -21,10 +21,9 @@ namespace sats {
 namespace {
 
 constexpr int kErrGroup = 32;     // candidate thresholds per group of Eq. 6
-// Rows of h per group (candidates x inputs): enough to fill the GPU for several waves, and at most
-// about 470 MB of rows at the largest layers' 14336 neurons
-constexpr int kErrRows = 8192;
-constexpr size_t kErrKeep = (size_t)1 << 30;
+// Bytes of a group's rows (candidates x inputs: h's two parts and the output) at most
+constexpr size_t kErrRowBytes = (size_t)512 << 20;
+constexpr size_t kErrKeep = (size_t)1 << 30;   // of a calibration's kept inputs, at most
 
 size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -264,28 +263,36 @@ __global__ void __launch_bounds__(256) err_ratio_kernel(const double *__restrict
 struct ErrInputs {
     float *a;                // [C][N]: SiLU(x W_gate)
     uint16_t *hhi, *hlo;     // [C][ldn]: a u of every neuron
-    static size_t bytes(int N, int C) { return al256((size_t)C * ((N + 7) & ~7) * 8); }
-    ErrInputs(void *p, int N, int C)
-        : a(static_cast<float *>(p)),
-          hhi(reinterpret_cast<uint16_t *>(a + (size_t)C * ((N + 7) & ~7))), hlo(hhi + (size_t)C * ((N + 7) & ~7)) {}
+    static size_t a_bytes(int N, int C) { return al256((size_t)C * N * 4); }
+    static size_t h_bytes(int N, int C) { return al256((size_t)C * ((N + 7) & ~7) * 4); }
+    ErrInputs(void *a, void *h, int N, int C)
+        : a(static_cast<float *>(a)), hhi(static_cast<uint16_t *>(h)), hlo(hhi + (size_t)C * ((N + 7) & ~7)) {}
 };
 
 // Workspace of Eq. 6.  Batches on the fused kernel (at most two tokens) compare whole outputs
 // (yd, yk, idx, cnt); batches on the tensor cores project the dropped neurons of a group of
-// candidates (a: ErrInputs, rows, y: the group's outputs, sq: their squared norms).
+// candidates (a: the gate activations of a call that has no other place for them; rows, y: the group's outputs, sq: their
+// squared norms).  mlp is an ordinary workspace; h takes the place of its h.
 struct ErrLayout {
-    size_t mlp, yd, yk, idx, cnt, a, rhi, rlo, y, sq, acc, total;
+    size_t mlp, yd, yk, idx, cnt, a, h, rhi, rlo, y, sq, acc, total;
 };
 
-// Candidates per group: at most kErrGroup, and about kErrRows rows of h at most (but one candidate's), the dense
-// rows among them.
-int err_group(int C, int K)
+// Candidates of a group and inputs of a chunk: as many candidates as a launch takes, and inputs within kErrRowBytes (but
+// one, whose rows are 140 MB at the largest layer), the dense rows among them.
+struct ErrGroup {
+    int candidates, inputs;
+    size_t rows() const { return (size_t)(candidates + 1) * inputs; }
+};
+
+ErrGroup err_group(int H, int N, int C, int K)
 {
-    const int fit = kErrRows / C - 1;
-    return std::max(1, std::min(std::min(fit, kErrGroup), K));
+    const int g = std::max(1, std::min(K, kErrGroup));
+    const size_t row = ((size_t)((N + 7) & ~7) + H) * 4, fit = std::max<size_t>(1, kErrRowBytes / (row * (g + 1)));
+    const int chunks = (int)((C + fit - 1) / fit);
+    return {g, (C + chunks - 1) / chunks};
 }
 
-ErrLayout err_layout(int H, int N, int C, int K)
+ErrLayout err_layout(int H, int N, int C, int K, bool own_a)
 {
     ErrLayout L{};
     size_t off = 0;
@@ -296,8 +303,9 @@ ErrLayout err_layout(int H, int N, int C, int K)
     };
     L.mlp = take(ws_layout(H, N, C).total);
     if (use_tc_path(H, C)) {
-        const size_t ldn = ((size_t)N + 7) & ~(size_t)7, rows = (size_t)(err_group(C, K) + 1) * C;
-        L.a = take(ErrInputs::bytes(N, C));
+        const size_t ldn = ((size_t)N + 7) & ~(size_t)7, rows = err_group(H, N, C, K).rows();
+        if (own_a) L.a = take(ErrInputs::a_bytes(N, C));
+        L.h = L.mlp + ws_layout(H, N, C).tc + tc_regions(H, N, C).h;
         L.rhi = take(rows * ldn * 2);
         L.rlo = take(rows * ldn * 2);
         L.y = take(rows * H * sizeof(float));
@@ -332,15 +340,14 @@ struct ErrSums {
 };
 
 // The dense rows and those of kg candidates (cand), and their product with W_down, into out [kg + 1][C][H].
-sats_status enqueue_rows(const sats_layer *layer, const ErrInputs &in, int C, const Candidates &cand, int kg,
-                         unsigned long long *dropped, float *out, char *base, const ErrLayout &W, cudaStream_t st)
+sats_status enqueue_rows(const sats_layer *layer, const float *a, const uint16_t *hhi, const uint16_t *hlo, int C,
+                         const Candidates &cand, int kg, unsigned long long *dropped, float *out, char *base,
+                         const ErrLayout &W, int *ctl, cudaStream_t st)
 {
     const int H = layer->H, N = layer->N, ld = layer->ldn;
-    int *ctl = reinterpret_cast<int *>(base + W.mlp + ws_layout(H, N, C).ctl);
     uint16_t *rhi = reinterpret_cast<uint16_t *>(base + W.rhi), *rlo = reinterpret_cast<uint16_t *>(base + W.rlo);
-    const cudaError_t e = launch_after(drop_rows_kernel, dim3(C, (ld / 8 + 255) / 256), 256, st, (const float *)in.a,
-                                       (const uint16_t *)in.hhi, (const uint16_t *)in.hlo, C, N, ld, cand, kg, rhi, rlo,
-                                       dropped, reinterpret_cast<float4 *>(out), (size_t)(kg + 1) * C * H / 4);
+    const cudaError_t e = launch_after(drop_rows_kernel, dim3(C, (ld / 8 + 255) / 256), 256, st, a, hhi, hlo, C, N, ld, cand,
+                                       kg, rhi, rlo, dropped, reinterpret_cast<float4 *>(out), (size_t)(kg + 1) * C * H / 4);
     if (e != cudaSuccess) return cuda_fail(e, "dropped rows kernel launch");
     return run_tc_down(layer, rhi, rlo, (kg + 1) * C, out, ctl, st) == cudaSuccess ? SATS_OK : SATS_ECUDA;
 }
@@ -356,44 +363,53 @@ __global__ void __launch_bounds__(256) add_rows_kernel(float4 *__restrict__ x, c
 }
 
 // x += the dense output, projected on its own: up to 256 inputs take the batched-decode kernel, whose shorter
-// accumulator chains are the more accurate ones.
-sats_status enqueue_residual(const sats_layer *layer, float *x, int C, const ErrInputs &in, char *base,
-                             const ErrLayout &W, cudaStream_t st)
+// accumulator chains are the more accurate ones.  In chunks of what the groups' output holds (rows).
+sats_status enqueue_residual(const sats_layer *layer, float *x, int C, const ErrInputs &in, size_t rows, char *base,
+                             const ErrLayout &W, int *ctl, cudaStream_t st)
 {
-    const size_t n = (size_t)C * layer->H;
+    const int H = layer->H;
     float *y = reinterpret_cast<float *>(base + W.y);
-    int *ctl = reinterpret_cast<int *>(base + W.mlp + ws_layout(layer->H, layer->N, C).ctl);
-    cudaError_t e = cudaMemsetAsync(y, 0, n * sizeof(float), st);
-    if (e != cudaSuccess) return cuda_fail(e, "dense output clear");
-    if (run_tc_down(layer, in.hhi, in.hlo, C, y, ctl, st) != cudaSuccess) return SATS_ECUDA;
-    e = launch_after(add_rows_kernel, dim3((unsigned)((n / 4 + 255) / 256)), 256, st, reinterpret_cast<float4 *>(x),
-                     reinterpret_cast<const float4 *>(y), n / 4);
-    return e == cudaSuccess ? SATS_OK : cuda_fail(e, "residual kernel launch");
+    for (size_t c0 = 0; c0 < (size_t)C; c0 += rows) {
+        const int m = (int)std::min(rows, C - c0);
+        const size_t n = (size_t)m * H, at = c0 * layer->ldn;
+        cudaError_t e = cudaMemsetAsync(y, 0, n * sizeof(float), st);
+        if (e != cudaSuccess) return cuda_fail(e, "dense output clear");
+        if (run_tc_down(layer, in.hhi + at, in.hlo + at, m, y, ctl, st) != cudaSuccess) return SATS_ECUDA;
+        e = launch_after(add_rows_kernel, dim3((unsigned)((n / 4 + 255) / 256)), 256, st,
+                         reinterpret_cast<float4 *>(x + c0 * H), reinterpret_cast<const float4 *>(y), n / 4);
+        if (e != cudaSuccess) return cuda_fail(e, "residual kernel launch");
+    }
+    return SATS_OK;
 }
 
-// Enqueues the sums for K candidates: thresholds t (host), or q[at(k)] on the device where q is given.
-// sums: cleared device memory of ErrSums::bytes(K).
+// Enqueues the sums for K candidates: thresholds t (host), or q[at(k)] on the device where q is given; group: that of the
+// call's workspace.  sums: cleared device memory of ErrSums::bytes(K).
 template <typename At>
 sats_status enqueue_err(const sats_layer *layer, const ErrInputs &in, int C, const float *t, const float *q, At at, int K,
-                        float eps, const ErrSums &sums, char *base, const ErrLayout &W, cudaStream_t st)
+                        float eps, const ErrSums &sums, const ErrGroup &group, char *base, const ErrLayout &W, int *ctl,
+                        cudaStream_t st)
 {
     float *out = reinterpret_cast<float *>(base + W.y);
-    const int group = err_group(C, K);
-    for (int k0 = 0; k0 < K; k0 += group) {
-        const int kg = std::min(group, K - k0);
-        Candidates cand{};
-        cand.dev = q;
-        for (int k = 0; k < kg; ++k) {
-            cand.t[k] = q ? 0.f : t[k0 + k];
-            cand.at[k] = at(k0 + k);
+    double *sq = reinterpret_cast<double *>(base + W.sq);
+    for (int c0 = 0; c0 < C; c0 += group.inputs) {
+        const int cc = std::min(group.inputs, C - c0);
+        const size_t h0 = (size_t)c0 * layer->ldn;
+        for (int k0 = 0; k0 < K; k0 += group.candidates) {
+            const int kg = std::min(group.candidates, K - k0);
+            Candidates cand{};
+            cand.dev = q;
+            for (int k = 0; k < kg; ++k) {
+                cand.t[k] = q ? 0.f : t[k0 + k];
+                cand.at[k] = at(k0 + k);
+            }
+            const sats_status s = enqueue_rows(layer, in.a + (size_t)c0 * layer->N, in.hhi + h0, in.hlo + h0, cc, cand, kg,
+                                               sums.dropped + k0, out, base, W, ctl, st);
+            if (s != SATS_OK) return s;
+            cudaError_t e = launch_after(row_squares_kernel, dim3((kg + 1) * cc), 256, st, (const float *)out, layer->H, sq);
+            if (e == cudaSuccess)
+                e = launch_after(err_ratio_kernel, dim3(kg), 256, st, (const double *)sq, cc, eps, sums.err + k0);
+            if (e != cudaSuccess) return cuda_fail(e, "error reduction kernel launch");
         }
-        const sats_status s = enqueue_rows(layer, in, C, cand, kg, sums.dropped + k0, out, base, W, st);
-        if (s != SATS_OK) return s;
-        double *sq = reinterpret_cast<double *>(base + W.sq);
-        cudaError_t e = launch_after(row_squares_kernel, dim3((kg + 1) * C), 256, st, (const float *)out, layer->H, sq);
-        if (e == cudaSuccess)
-            e = launch_after(err_ratio_kernel, dim3(kg), 256, st, (const double *)sq, C, eps, sums.err + k0);
-        if (e != cudaSuccess) return cuda_fail(e, "error reduction kernel launch");
     }
     return SATS_OK;
 }
@@ -420,12 +436,13 @@ sats_status layer_err_tc(const sats_layer *layer, const float *x, int C, const f
     cudaError_t e = clear_fused_state(mlp, layer->H, layer->N, C, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(base + W.acc, 0, sum_bytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "layer error workspace clear");
-    const ErrInputs in(base + W.a, layer->N, C);
-    int *status = reinterpret_cast<int *>(mlp + ws_layout(layer->H, layer->N, C).ctl) + kCtlStatus;
-    e = launch_gate_act_f32(layer, x, C, in.a, status, st);
-    if (e == cudaSuccess) e = launch_up_f32(layer, x, C, in.a, in.hhi, in.hlo, status, st);
+    const ErrInputs in(base + W.a, base + W.h, layer->N, C);
+    int *ctl = reinterpret_cast<int *>(mlp + ws_layout(layer->H, layer->N, C).ctl);
+    e = launch_gate_act_f32(layer, x, C, in.a, ctl + kCtlStatus, st);
+    if (e == cudaSuccess) e = launch_up_f32(layer, x, C, in.a, in.hhi, in.hlo, ctl + kCtlStatus, st);
     if (e != cudaSuccess) return cuda_fail(e, "gate and up kernels launch");
-    sats_status s = enqueue_err(layer, in, C, t, nullptr, [](int k) { return k; }, K, eps, ErrSums(base + W.acc, K), base, W, st);
+    sats_status s = enqueue_err(layer, in, C, t, nullptr, [](int k) { return k; }, K, eps, ErrSums(base + W.acc, K),
+                                err_group(layer->H, layer->N, C, K), base, W, ctl, st);
     if (s != SATS_OK) return s;
     std::vector<char> h(sum_bytes);
     e = cudaMemcpyAsync(h.data(), base + W.acc, sum_bytes, cudaMemcpyDeviceToHost, st);
@@ -438,7 +455,7 @@ sats_status layer_err_tc(const sats_layer *layer, const float *x, int C, const f
 }
 
 struct SatsLayout {
-    size_t x, n, a, sel, q, sums, in, in_each, err, total;   // in_each: 0 if the blocks share one
+    size_t x, n, sel, q, sums, a, in_each, err, total;   // in_each: 0 if the blocks share one
 };
 
 SatsLayout sats_layout(int H, int N, int C, int L, int K0, int K)
@@ -449,21 +466,20 @@ SatsLayout sats_layout(int H, int N, int C, int L, int K0, int K)
     off += al256((size_t)C * H * sizeof(float));
     S.n = off;
     off += al256((size_t)L * C * H * sizeof(float));
-    S.a = off;
-    off += al256((size_t)C * N * sizeof(float));
     S.sel = off;
     off += al256(select_multi_ws_bytes(kSelRanks));
     S.q = off;   // every block's percentiles: the coarse candidates, the largest |a|, the guardrail's
     off += al256((size_t)L * (K0 + 1) * sizeof(float));
     S.sums = off;   // every block's ErrSums
     off += al256((size_t)L * ErrSums::bytes(K));
-    // every block's ErrInputs, kept from the coarse candidates for the fine ones, up to kErrKeep bytes
-    const size_t each = use_tc_path(H, C) ? ErrInputs::bytes(N, C) : 0;
-    S.in = off;
+    // every block's a and h, kept from the coarse candidates for the fine ones, up to kErrKeep bytes; else one a (and the
+    // h of Eq. 6's workspace)
+    const size_t each = use_tc_path(H, C) ? ErrInputs::a_bytes(N, C) + ErrInputs::h_bytes(N, C) : 0;
     S.in_each = each * L <= kErrKeep ? each : 0;
-    off += S.in_each * L;
+    S.a = off;
+    off += S.in_each ? S.in_each * L : ErrInputs::a_bytes(N, C);
     S.err = off;
-    off += err_layout(H, N, C, K).total;
+    off += err_layout(H, N, C, K, false).total;
     S.total = off;
     return S;
 }
@@ -498,7 +514,7 @@ sats_status sats_gate_act_f32(const sats_layer *layer, const float *x, int B, fl
 size_t sats_layer_err_workspace_bytes(int H, int N, int C, int K)
 {
     if (H < 8 || H > kMaxH || (H % 8) != 0 || N < 1 || N > kMaxN || C < 1 || K < 0) return 0;
-    return err_layout(H, N, C, K).total;
+    return err_layout(H, N, C, K, true).total;
 }
 
 sats_status sats_layer_err(const sats_layer *layer, const float *x, int C, const float *t, int K, float eps,
@@ -512,7 +528,7 @@ sats_status sats_layer_err(const sats_layer *layer, const float *x, int C, const
     for (int k = 0; k < K; ++k)
         if (bad_t(t[k])) return SATS_EINVAL;
     const int H = layer->H, N = layer->N;
-    const ErrLayout W = err_layout(H, N, C, K);
+    const ErrLayout W = err_layout(H, N, C, K, true);
     if (ws_bytes < W.total) return SATS_ENOSPACE;
     if (K == 0) return SATS_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -640,17 +656,19 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     void *sel = base + W.sel;
     float *q = reinterpret_cast<float *>(base + W.q);
     char *ews = base + W.err;
-    const ErrLayout E = err_layout(H, N, C, Kmax);
+    const ErrLayout E = err_layout(H, N, C, Kmax, false);
+    const ErrGroup group = err_group(H, N, C, Kmax);
     char *sums = base + W.sums;
     const size_t sum_bytes = ErrSums::bytes(Kmax);
     const bool batched = use_tc_path(H, C);
     // (the masks take the gate activations that the thresholds are percentiles of)
     auto inputs_of = [&](int l) {
-        return ErrInputs(W.in_each ? base + W.in + l * W.in_each : ews + E.a, N, C);
+        char *a = base + W.a + l * W.in_each;
+        return ErrInputs(a, W.in_each ? a + ErrInputs::a_bytes(N, C) : ews + E.h, N, C);
     };
     char *mlp = ews + E.mlp;
     // every bounded wait of the call reports here
-    int *status = reinterpret_cast<int *>(mlp + ws_layout(H, N, C).ctl) + kCtlStatus;
+    int *ctl = reinterpret_cast<int *>(mlp + ws_layout(H, N, C).ctl), *status = ctl + kCtlStatus;
     auto n_of = [&](int l) { return nall + (size_t)l * C * H; };
     auto up_of = [&](int l) {
         const ErrInputs in = inputs_of(l);
@@ -663,7 +681,7 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
     // 1-2: the dense stack gives each block's MLP inputs; coarse candidates from |SiLU(n W_gate)|
     cudaError_t e = cudaMemcpyAsync(x, x_cal, (size_t)C * H * sizeof(float), cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = clear_fused_state(mlp, H, N, C, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, W.in - W.q, st);   // (the sums follow the percentiles)
+    if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, W.a - W.q, st);   // (the sums follow the percentiles)
     if (e != cudaSuccess) return cuda_fail(e, "calibration set-up");
     std::vector<double> tc((size_t)L * Kc), amax((size_t)L), errc((size_t)L * Kc), spc((size_t)L * Kc);
     double g_t = 0.0, g_sp = 0.0;
@@ -692,9 +710,10 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
             const int K = l == guard ? Kc + 1 : Kc;
             if ((e = up_of(l)) != cudaSuccess) return cuda_fail(e, "up kernel launch");
             if ((s = enqueue_err(layers[l], inputs_of(l), C, nullptr, ql, [&](int k) { return k < Kc ? k : Kc + 1; }, K,
-                                 err_eps, ErrSums(sums + l * sum_bytes, K), ews, E, st)) != SATS_OK)
+                                 err_eps, ErrSums(sums + l * sum_bytes, K), group, ews, E, ctl, st)) != SATS_OK)
                 return s;
-            if ((s = enqueue_residual(layers[l], x, C, inputs_of(l), ews, E, st)) != SATS_OK) return s;
+            if ((s = enqueue_residual(layers[l], x, C, inputs_of(l), group.rows(), ews, E, ctl, st)) != SATS_OK)
+                return s;
             continue;
         }
         // x <- x + MLP_l(n_l) with every neuron kept
@@ -775,7 +794,7 @@ sats_status sats_sats_calibrate(const sats_layer *const *layers, const float *co
             if ((e = up_of(l)) != cudaSuccess) return cuda_fail(e, "up kernel launch");
         }
         s = batched ? enqueue_err(layers[l], inputs_of(l), C, tf.data() + (size_t)l * K1, nullptr, [](int k) { return k; },
-                                  K1, err_eps, ErrSums(sums + l * sum_bytes, K1), ews, E, st)
+                                  K1, err_eps, ErrSums(sums + l * sum_bytes, K1), group, ews, E, ctl, st)
                     : sats_layer_err(layers[l], n_of(l), C, tf.data() + (size_t)l * K1, K1, err_eps,
                                      ea.data() + (size_t)l * Kt + Kc, sa.data() + (size_t)l * Kt + Kc, ews, ews_bytes,
                                      stream);

@@ -99,3 +99,17 @@ def test_every_entry_rejects_missing_arguments_before_any_cuda_call(libsats):
     assert L.sats_route_calib_workspace_bytes(151936) >= 151936
     assert L.sats_sats_workspace_bytes(4096, 14336, 32, 64, 20, 8) >= L.sats_layer_err_workspace_bytes(4096, 14336,
                                                                                                          64, 20)
+
+
+@pytest.mark.parametrize("H,N,C,K", [(8192, 1 << 20, 512, 20), (8192, 1 << 20, 4096, 40), (8192, 28672, 4096, 32),
+                                     (4096, 14336, 64, 19), (96, 5, 100000, 33)])
+def test_calibration_workspaces_are_bounded(libsats, H, N, C, K):
+    """Eq. 6 asks for an ordinary workspace, the gate activations and at most 512 MiB of rows, however wide the layer and
+    however many inputs and candidates; a calibration for every block's inputs and at most 1 GiB of kept values more."""
+    from paper_2607_08991_gb300 import sats
+    L = sats.lib()
+    small = 8 << 20   # sums, histograms, alignment
+    one = L.sats_workspace_bytes(H, N, C) + 4 * C * N + (512 << 20) + small
+    assert L.sats_layer_err_workspace_bytes(H, N, C, K) <= one
+    blocks = 3
+    assert L.sats_sats_workspace_bytes(H, N, C, blocks, K, 8) <= one + (1 + blocks) * 4 * C * H + (1 << 30)

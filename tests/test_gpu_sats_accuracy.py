@@ -47,7 +47,8 @@ def _gap(v, s):
 
 
 @pytest.mark.parametrize("H,N,C,K", [(2048, 5633, 48, 12), (1024, 2816, 120, 12), (4096, 6000, 9, 3), (512, 1408, 300, 4),
-                                     (96, 261, 5, 7)])
+                                     (96, 261, 5, 7), (96, 40001, 400, 9), (104, 9, 3, 40)])   # several chunks of
+                                     # inputs; several groups of candidates
 def test_layer_err_against_fp64(sats, H, N, C, K):
     layer, W = _block(sats, H, N, 1400)
     x = inputs.activations_f32(C, H, seed=1401)
