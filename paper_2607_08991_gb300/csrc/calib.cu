@@ -835,9 +835,14 @@ namespace {
 // Zipf ids in order of rank: 57 us, most of it on the first few lines).
 constexpr int kSpread = 64;
 
-__host__ __device__ inline int spread_rows(int V) { return (V + kSpread - 1) / kSpread; }
+__host__ __device__ inline int spread_rows(int V) { return V / kSpread + (V % kSpread != 0); }
 
-__device__ __forceinline__ int spread(int v, int rows) { return (v & (kSpread - 1)) * rows + v / kSpread; }
+__device__ __forceinline__ size_t spread(int v, int rows)
+{
+    return (size_t)(v & (kSpread - 1)) * rows + v / kSpread;   // (up to V + 62, beyond int for the largest V)
+}
+
+int blocks_of(int V, int per) { return (int)(((int64_t)V + per - 1) / per); }
 
 // A warp's table of the token ids it has met: sums of the occurrences it has seen, added to the
 // device totals once at the end.  Token frequencies are far from even (a corpus' most common token
@@ -961,7 +966,7 @@ __global__ void score_final_kernel(const double *__restrict__ total, const unsig
     grid_launch_dependents();
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= V) return;
-    const int at = spread(v, spread_rows(V));
+    const size_t at = spread(v, spread_rows(V));
     const unsigned c = count[at];
     if (c == 0u) {
         score[v] = INFINITY;
@@ -1019,8 +1024,8 @@ __global__ void __launch_bounds__(kTauThreads) tau_level_kernel(const float *__r
     const uint32_t prefix = LEVEL == 0 ? 0u : S->prefix;
     const int rows = spread_rows(V);
     __syncthreads();
-    for (int v = blockIdx.x * kTauThreads + tid; v < V; v += gridDim.x * kTauThreads) {
-        const unsigned f = freq[spread(v, rows)];
+    for (unsigned v = blockIdx.x * kTauThreads + tid; v < (unsigned)V; v += gridDim.x * kTauThreads) {   // (int would overflow)
+        const unsigned f = freq[spread((int)v, rows)];
         const uint32_t b = ordered_bits(score[v]);
         const bool in = LEVEL == 0 || (LEVEL == 1 ? (b >> 21) == (prefix >> 21) : (b >> 10) == (prefix >> 10));
         if (f && in) atomicAdd(h + ((b >> kShift) & (kBins - 1)), (unsigned long long)f);
@@ -1078,8 +1083,8 @@ __global__ void __launch_bounds__(kTauThreads) tau_sums_kernel(const float *__re
     const uint32_t at = S->prefix, zero = 0x80000000u, inf = 0xff800000u;
     unsigned long long s[4] = {0ull, 0ull, 0ull, 0ull};
     uint32_t na = 0u;
-    for (int v = blockIdx.x * kTauThreads + threadIdx.x; v < V; v += gridDim.x * kTauThreads) {
-        const unsigned f = freq[spread(v, rows)];
+    for (unsigned v = blockIdx.x * kTauThreads + threadIdx.x; v < (unsigned)V; v += gridDim.x * kTauThreads) {
+        const unsigned f = freq[spread((int)v, rows)];
         if (!f) continue;
         const uint32_t b = ordered_bits(score[v]);
         s[0] += b < at ? f : 0u;
@@ -1159,7 +1164,7 @@ cudaError_t launch_tally(const int32_t *ids, const float *lb, const float *ls, i
 template <typename... KArgs, typename... Args>
 cudaError_t launch_search(void (*kernel)(KArgs...), int V, cudaStream_t st, Args... args)
 {
-    const int want = (V + 2 * kTauThreads - 1) / (2 * kTauThreads), sms = fused_grid(kMaxGrid);
+    const int want = blocks_of(V, 2 * kTauThreads), sms = fused_grid(kMaxGrid);
     return launch_after(kernel, dim3(want < sms ? want : sms), kTauThreads, st, args...);
 }
 
@@ -1197,7 +1202,7 @@ sats_status sats_token_scores(const int32_t *ids, const float *l_base, const flo
     if (e != cudaSuccess) return cuda_fail(e, "score workspace clear");
     if (n > 0 && (e = launch_tally<true>(ids, l_base, l_sparse, n, V, total, count, status, st)) != cudaSuccess)
         return cuda_fail(e, "score kernel launch");
-    e = launch_after(score_final_kernel, dim3((V + 255) / 256), 256, st, (const double *)total, (const unsigned *)count, V,
+    e = launch_after(score_final_kernel, dim3(blocks_of(V, 256)), 256, st, (const double *)total, (const unsigned *)count, V,
                      score);
     if (e != cudaSuccess) return cuda_fail(e, "score kernel launch");
     return read_status_word(status, st);
@@ -1272,7 +1277,7 @@ sats_status sats_route_calibrate(const float *score, int V, const int32_t *heldo
     *tau_out = best_tau;
     if (R_out) *R_out = best_R;
     if (lut) {
-        lut_kernel<<<(V + 255) / 256, 256, 0, st>>>(score, V, best_tau, lut);
+        lut_kernel<<<blocks_of(V, 256), 256, 0, st>>>(score, V, best_tau, lut);
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "table kernel launch");
     }
     return SATS_OK;

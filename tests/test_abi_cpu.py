@@ -113,3 +113,11 @@ def test_calibration_workspaces_are_bounded(libsats, H, N, C, K):
     assert L.sats_layer_err_workspace_bytes(H, N, C, K) <= one
     blocks = 3
     assert L.sats_sats_workspace_bytes(H, N, C, blocks, K, 8) <= one + (1 + blocks) * 4 * C * H + (1 << 30)
+
+
+@pytest.mark.parametrize("V", [1, 63, 64, 65, 151936, 2**31 - 78000, 2**31 - 65, 2**31 - 64, 2**31 - 1])
+def test_route_calibration_workspace_of_any_vocabulary(libsats, V):
+    """A double and a count per token, in rows of 64; sizes near the largest int do not wrap around."""
+    from paper_2607_08991_gb300 import sats
+    n = sats.lib().sats_route_calib_workspace_bytes(V)
+    assert 12 * V <= n <= 12 * (V + 63) + (1 << 16)
