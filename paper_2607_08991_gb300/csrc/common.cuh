@@ -56,8 +56,8 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
 }
 
 // Tests the phase; if it is not complete the thread is suspended (not spinning) until it completes or a limit:
-// the hardware's own, or with HINT about kSuspendHintNs.  Without one wake-ups come earlier (0.5 to 1 % of every
-// batched call and of the decode call; spinning on test_wait is slower still, the roles share their schedulers).
+// the hardware's own, or with HINT about kSuspendHintNs.  Without one wake-ups come earlier (0.5 to 1 % of a
+// batched call, the decode call within noise; spinning on test_wait is slower still, the roles share their schedulers).
 // The producers and the list and up/down warps of decode with an adapter, which wait for the whole grid's sums
 // first, keep the hint: hidden 536 / intermediate 1209, rank 32, 2 tokens 16.2 us with it, 17.4 without.
 constexpr uint32_t kSuspendHintNs = 100000;
@@ -119,14 +119,6 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
         : "memory");
 }
 
-// As bulk_load, with the default L2 policy (data that other CTAs read too).
-__device__ __forceinline__ void bulk_load_shared(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar))
-                 : "memory");
-}
-
 // Starts bringing `bytes` (a multiple of 16) at a 16-byte aligned global
 // address into L2; no completion to wait for.
 __device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes)
@@ -178,11 +170,6 @@ __device__ __forceinline__ uint64_t ld_relaxed_gpu_u64(const uint64_t *p)
 __device__ __forceinline__ void st_relaxed_gpu_u64(uint64_t *p, uint64_t v)
 {
     asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ void st_release_gpu(int *p, int v)
-{
-    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // bf16 pair (one 32-bit word, element 2i in the low half) -> two floats.
