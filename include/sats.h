@@ -242,10 +242,15 @@ SATS_API sats_status sats_sparse_mlp_union_f32(const sats_layer *layer, const fl
  *   u = x W_up + scale (x A_up) B_up,        h = keep ? a u : 0
  *   y = h W_down + scale (h A_down) B_down
  * in the decode kernel: the gate's low-rank term for every neuron, the up and
- * down terms only for kept neurons.  Larger batches (where sats_uses_tensor_cores
- * says so, from hidden size 96) stream the weights once through the tensor cores
- * in that kernel's fp32 arithmetic: activations and h enter as three bf16 parts
- * and sums are rounded every 32 products.
+ * down terms only for kept neurons.  Batches of 3 to 65535 tokens that
+ * sats_uses_tensor_cores puts there, from hidden size 96, run on the tensor
+ * cores in that kernel's fp32 accuracy and stream the weights once per 32
+ * tokens: fp32 activations and h enter as three bf16 parts, and sums are
+ * rounded to fp32 every 32 products (every 64 with fp32 activations in tiles
+ * of more than 16 tokens).  Other batches run as passes of the decode kernel.
+ * On the tensor cores a dropped neuron's W_down row is multiplied by zero
+ * rather than not read, so it has to be finite there, as in sats_sparse_mlp's
+ * batches.
  * Arguments, index outputs, workspace and errors are those of sats_sparse_mlp
  * (x bf16) and sats_sparse_mlp_f32 (x fp32); the adapter must match the
  * layer's H and N (else SATS_ESHAPE).

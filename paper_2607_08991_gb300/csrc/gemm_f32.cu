@@ -490,16 +490,16 @@ cudaError_t launch_gate_precise(const sats_layer *layer, const void *x, int B, f
 }
 
 // ---------------------------------------------------------------------- LoRA batches
-// The sparse path of a fine-tuned model (Sec. 4) for batches beyond one pass of the fused
-// kernel, in the arithmetic of that kernel:
+// The sparse path of a fine-tuned model (Sec. 4) for batches of three tokens and more, in the
+// accuracy of the fused kernel, which runs the smaller ones:
 //   lora_z_kernel        z = x A_gate | x A_up, per slice of hidden rows
 //   lora_gate_up_kernel  g = x W_gate + s z B_gate[:, n], u likewise, h = keep ? SiLU(g) u : 0, w += h A_down
 //   lora_down_kernel     y += h W_down + s w B_down
-// W is streamed once for up to kLoraTok tokens, where the fused kernel streamed it once per pass
-// of one or two (129 us for four tokens on the Llama-shaped layer at 70 % sparsity, 267 us for
-// eight; 77 here; with A_down as one more tile of outputs and w B_down in a kernel of its own 79 and 80).  What bounds it: that stream and the roles' serial issue; with at most 32 tokens the parts of an operand are the
-// rows of one tile, so a K step is one MMA per weight tile however many parts there are, and
-// their products are added in the epilogue.
+// W is streamed once for up to kLoraTok tokens, where the fused kernel streamed it once per pass of one or two
+// (129 us for four tokens on the Llama-shaped layer at 70 % sparsity, 267 us for eight; 77 here; with A_down as one
+// more tile of outputs and w B_down in a kernel of its own 79 and 80).  What bounds it: that stream and the roles'
+// serial issue; with at most 32 tokens the parts of an operand are the rows of one tile, so a K step is one MMA per
+// weight tile however many parts there are, and their products are added in the epilogue.
 constexpr int kLoraTok = 32;
 constexpr int kLoraWRow = kMaxLoraRank;        // row pitch of w
 constexpr int kLoraZRow = 2 * kMaxLoraRank;    // row pitch of z
@@ -696,7 +696,8 @@ __global__ void __launch_bounds__(kLoraGuThreads<F32>, 1)
         // acc: the sums of up to p.sub K blocks; they join the totals together, so that a total takes few roundings
         // at its full size.  The totals are kept in shared memory with fp32 activations (whose parts take the registers).
         float acc[2][16], tot[2][F32 ? 1 : 16];
-        float *const shared_tot = reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(full) + kBarrierBytes) + et;   // [2][16], kLoraEpiThreads apart
+        float *const shared_tot = reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(full) + kBarrierBytes) +
+                                  et;   // [2][16] of this thread, kLoraEpiThreads apart
 #pragma unroll
         for (int q = 0; q < 2; ++q)
 #pragma unroll

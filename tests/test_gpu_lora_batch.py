@@ -1,7 +1,8 @@
 """LoRA batches beyond one pass of the fused kernel, at token counts around the tile edges, neuron
 counts that do not fill a tile or a K block, the smallest hidden size of the path and every rank,
 against the oracle element by element.  The bound is fp32 arithmetic's (both matrix products are
-summed in segments of 32 rounded once each, a few units of 2^-24): 1e-6 relative, which a plain
+summed in segments of 32 products, of 64 with fp32 activations in tiles of more than 16 tokens, rounded once
+each, a few units of 2^-24): 1e-6 relative, which a plain
 accumulator chain on the tensor cores (1e-5) or h rounded to two bf16 parts (4e-6) does not meet."""
 import numpy as np
 import pytest
