@@ -74,7 +74,8 @@ __host__ __device__ constexpr uint32_t instr_desc(int M, int N)
 // elected lane.  With a role's loop in one lane's branch every address and descriptor had to be moved into uniform
 // registers before each instruction: about 100 cycles per MMA, commit or copy, more than the MMAs of a batched-
 // decode K block or the eight copies of a prefill stage leave (the same box, us; before -> MMA role -> both roles):
-// Llama-shaped layer 8 bf16 tokens 57.5 -> 54.3 -> 53.5 and 2048 610 -> 601 -> 560, hidden 8192 / intermediate 7168
+// Llama-shaped layer 8 bf16 tokens 57.5 -> 54.3 -> 53.5 and 2048 (a few calls; in a loop at the power limit about 600
+// either way) 610 -> 601 -> 560, hidden 8192 / intermediate 7168
 // 8 tokens 75 -> 61 -> 54, hidden 2048 / intermediate 8192 25.4 -> 22.5 -> 20.1.
 __device__ __forceinline__ uint32_t elect_one()
 {
